@@ -68,7 +68,9 @@ enum {
 
 /* Arithmetic of the sweeps (App. C series). */
 enum {
-  DYSON_PREC_F64 = 0,           /* complex128 sweeps on the FP64 pipes                   */
+  DYSON_PREC_F64 = 0,           /* complex128 sweeps, FP64-accurate: BF16 slice products
+                                   on the tensor cores, or the FP64 pipes where the
+                                   slices of Lambda do not fit in device memory          */
   DYSON_PREC_TF32X3_F64REF = 1  /* complex FP32 sweeps as 3xTF32 tcgen05 products with
                                    FP32 accumulation, refined by FP64 Dyson residuals     */
 };
@@ -289,7 +291,7 @@ const char* dyson_last_error(const dyson_ctx* ctx);
 
 /* Kernel kinds timed by the optional per-launch CUDA-event profiler. */
 enum {
-  DYSON_KERNEL_SWEEP_F64 = 0,     /* FP64 series sweep (gather + complex GEMM)               */
+  DYSON_KERNEL_SWEEP_F64 = 0,     /* FP64 series sweep (gather, slicing and complex GEMM)    */
   DYSON_KERNEL_SWEEP_F32 = 1,     /* FP32 CUDA-core sweep                                    */
   DYSON_KERNEL_SWEEP_TC = 2,      /* 3xTF32 tcgen05 sweep GEMM (split + MMA + epilogue)      */
   DYSON_KERNEL_RESIDUAL_F64 = 3,  /* FP64 Dyson residual r = Lambda delta + K G - G          */

@@ -10,6 +10,7 @@
 #include "detail.cuh"
 #include "gmres.cuh"
 #include "oz.cuh"
+#include "oz64.cuh"
 #include "symmetry.cuh"
 #include "tc.cuh"
 
@@ -140,9 +141,13 @@ int solve_f64(dyson_ctx* c, int ncol, int gs, double tol, int max_sweeps, double
     DY_CUDA(c, cudaMemsetAsync(c->d_norm, 0, (size_t)ng * sizeof(unsigned long long), c->stream));
     {
       KernelTimer t(c, DYSON_KERNEL_SWEEP_F64);
-      launch_sweep_f64(c->d_lam, c->d_JW, c->d_nbr, c->d_nbond, Ga, Gb, nullptr, c->d_src_site, c->d_src_time,
-                       c->Nr, c->Nc, ncol, gs, 0, c->d_norm, c->stream);
-      c->launches += 1;
+      if (c->use_oz64) {
+        if ((rc = oz64_sweep(c, ncol, gs, Ga, Gb, nullptr, 0))) return rc;
+      } else {
+        launch_sweep_f64(c->d_lam, c->d_JW, c->d_nbr, c->d_nbond, Ga, Gb, nullptr, c->d_src_site, c->d_src_time,
+                         c->Nr, c->Nc, ncol, gs, 0, c->d_norm, c->stream);
+        c->launches += 1;
+      }
     }
     DY_CUDA(c, cudaGetLastError());
     if ((rc = read_norms(c, ng, false))) return rc;
@@ -152,6 +157,7 @@ int solve_f64(dyson_ctx* c, int ncol, int gs, double tol, int max_sweeps, double
     r->gemm_flops += sweep_flops(c, ncol);
     r->update = upd;
     if (!(upd < kDivergedF64)) {
+      if (c->use_oz64 && (rc = oz64_check_error(c))) return rc;
       status = DYSON_ERR_DIVERGED;
       break;
     }
@@ -571,9 +577,13 @@ int solve_mixed(dyson_ctx* c, int ncol, int gs, int precision, double tol, int m
       if ((rc = oz_residual(c, ncol, gs, G, r32, tol))) return rc;
     } else {
       KernelTimer t(c, DYSON_KERNEL_RESIDUAL_F64);
-      launch_sweep_f64(c->d_lam, c->d_JW, c->d_nbr, c->d_nbond, G, nullptr, r32, c->d_src_site, c->d_src_time,
-                       c->Nr, c->Nc, ncol, gs, 1, c->d_norm, c->stream);
-      c->launches += 1;
+      if (c->use_oz64) {
+        if ((rc = oz64_sweep(c, ncol, gs, G, nullptr, r32, 1))) return rc;
+      } else {
+        launch_sweep_f64(c->d_lam, c->d_JW, c->d_nbr, c->d_nbond, G, nullptr, r32, c->d_src_site, c->d_src_time,
+                         c->Nr, c->Nc, ncol, gs, 1, c->d_norm, c->stream);
+        c->launches += 1;
+      }
     }
     DY_CUDA(c, cudaGetLastError());
     if (c->use_oz && (rc = oz_error_enqueue(c))) return rc;   // read with the norms: one synchronisation
@@ -585,6 +595,7 @@ int solve_mixed(dyson_ctx* c, int ncol, int gs, int precision, double tol, int m
     rep->residual = res;
     for (int q = 0; q < ng; ++q) rref[q] = std::max(bits_to_double(c->h_norm[q]), 1e-300);
     if (!(res < kDivergedGrowth)) {
+      if (c->use_oz64 && (rc = oz64_check_error(c))) return rc;
       status = DYSON_ERR_DIVERGED;
       break;
     }
@@ -723,6 +734,7 @@ int dyson_build_sigma(dyson_ctx* c) {
   c->sigma_built = true;
   c->lam32_built = c->lam_split_built = false;
   oz_invalidate(c);
+  oz64_invalidate(c);
   se_invalidate(c);                                      // Sigma = 0: Lambda is the atomic G0 again
   return DYSON_OK;
 }
@@ -743,9 +755,19 @@ namespace dyson_detail {
 
 // Build the reduced-precision copies of Lambda a solve needs and pick the sweep
 // and residual kernels (sets c->use_tc, c->use_oz).
+// FP64 sweeps and residuals on the tensor cores where the slices of Lambda fit (sets c->use_oz64);
+// the FP64-pipe kernel otherwise
+int prepare_oz64(dyson_ctx* c) {
+  c->use_oz64 = oz64_usable(c);
+  if (!c->use_oz64) return DYSON_OK;
+  const int rc = oz64_prepare(c);
+  if (rc == DYSON_ERR_OOM) c->use_oz64 = false;
+  return rc == DYSON_ERR_OOM ? DYSON_OK : rc;
+}
+
 int prepare_tables(dyson_ctx* c, int precision) {
-  c->use_tc = c->use_oz = false;
-  if (precision == DYSON_PREC_F64) return DYSON_OK;
+  c->use_tc = c->use_oz = c->use_oz64 = false;
+  if (precision == DYSON_PREC_F64) return prepare_oz64(c);
   const bool tc = c->tc_enabled && tc_supported(c, c->Nc);
   if (!tc && !c->lam32_built) {
     if (!c->d_lam32) DY_CUDA(c, dalloc(&c->d_lam32, (size_t)c->Nr * c->Nc * c->Nc));
@@ -763,19 +785,22 @@ int prepare_tables(dyson_ctx* c, int precision) {
   }
   c->use_tc = tc;
   c->use_oz = tc && c->oz_enabled && oz_supported(c);
-  return DYSON_OK;
+  return c->use_oz ? DYSON_OK : prepare_oz64(c);
 }
 
 // Largest number of vector columns, a multiple of `unit` and at most `want`, whose
 // work state fits in 85 % of the free device memory.  F64: two complex128 states;
-// mixed: complex128 G + three FP32 states (+ the FP32 gather buffer of the
-// tensor-core sweep, + the BF16 slices of the split-product residual).
-int64_t chunk_columns(dyson_ctx* c, int precision, int64_t unit, int64_t want, size_t* bytes_per_col) {
-  const double per_el = precision == DYSON_PREC_F64
-                            ? 32.0
-                            : (c->use_tc ? 48.0 : 40.0) + (c->use_oz ? (double)oz_bytes_per_element() : 0.0);
+// mixed: complex128 G + three FP32 states (*bytes_per_col: these, the work buffer); besides it
+// the FP32 gather buffer of the tensor-core sweep and the BF16 slices of the split-product
+// residual or FP64 sweep (*total_per_col: all).
+int64_t chunk_columns(dyson_ctx* c, int precision, int64_t unit, int64_t want, size_t* bytes_per_col,
+                      size_t* total_per_col) {
+  const double state = precision == DYSON_PREC_F64 ? 32.0 : 40.0;
+  const double per_el = state + (c->use_tc ? 8.0 : 0.0) + (c->use_oz ? (double)oz_bytes_per_element() : 0.0) +
+                        (c->use_oz64 ? oz64_bytes_per_element(c) : 0.0);
   const double col_bytes = per_el * c->Nr * (double)c->Nc;
-  *bytes_per_col = (size_t)col_bytes;
+  *bytes_per_col = (size_t)(state * c->Nr * (double)c->Nc);
+  if (total_per_col) *total_per_col = (size_t)col_bytes;
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return 0;
   const double budget = 0.85 * (double)(free_b + c->work_bytes);
@@ -1083,6 +1108,7 @@ int dyson_transpose_sigma(dyson_ctx* c) {
   c->sigma_transposed = !c->sigma_transposed;
   c->lam32_built = c->lam_split_built = false;
   oz_invalidate(c);
+  oz64_invalidate(c);
   return DYSON_OK;
 }
 
@@ -1149,7 +1175,8 @@ int dyson_set_wait_limit(dyson_ctx* c, double seconds) {
   const unsigned long long ns = seconds == 0.0 ? 2000000000ull : (unsigned long long)(seconds * 1e9);
   int rc = tc_set_wait_limit(c, ns);
   if (rc) return rc;
-  return oz_set_wait_limit(c, ns);
+  if ((rc = oz_set_wait_limit(c, ns))) return rc;
+  return oz64_set_wait_limit(c, ns);
 }
 
 int dyson_set_graph_sweeps(dyson_ctx* c, int sweeps) {
@@ -1174,6 +1201,7 @@ void dyson_destroy(dyson_ctx* c) {
   flush_timers(c);
   tc_release(c);
   oz_release(c);
+  oz64_release(c);
   gmres_release(c);
   se_release(c);
   if (c->d_sym_perm) cudaFree(c->d_sym_perm);

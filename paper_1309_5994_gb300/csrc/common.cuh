@@ -177,6 +177,9 @@ struct dyson_ctx {
   bool se_installed = false;         // Lambda holds the local block of a self-energy step
   bool oz_enabled = true;            // split-product residual allowed where 2 Nc <= 512
   bool use_oz = false;               // chosen for the current solve
+  void* oz64 = nullptr;              // split-product FP64 sweep state (slices, scales, maps)
+  bool oz64_enabled = true;          // split-product FP64 sweeps allowed (memory permitting)
+  bool use_oz64 = false;             // chosen for the current solve: FP64 sweeps and residuals on the tensor cores
 
   std::string err;
 };

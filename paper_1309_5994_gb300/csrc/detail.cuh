@@ -104,6 +104,7 @@ int prepare_tables(dyson_ctx* c, int precision);
 int solve_mixed(dyson_ctx* c, int ncol, int gs, int precision, double tol, int max_sweeps, double2** result,
                 dyson_report* rep);
 // vector columns per chunk that fit in device memory (multiple of unit, at most want)
-int64_t chunk_columns(dyson_ctx* c, int precision, int64_t unit, int64_t want, size_t* bytes_per_col);
+int64_t chunk_columns(dyson_ctx* c, int precision, int64_t unit, int64_t want, size_t* bytes_per_col,
+                      size_t* total_per_col = nullptr);
 
 }  // namespace dyson_detail

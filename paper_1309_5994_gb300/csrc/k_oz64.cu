@@ -1,0 +1,633 @@
+// FP64 series sweep of App. C (and the FP64 Dyson residual) on the BF16 tensor cores:
+//     out = B + (Lambda W) X,   X_i(n, k) = sum_{j in NN(i)} J_ij(k) G_j(n, k).
+//
+// GB300's FP64 pipe does 2 FMA per SM and clock (1.1 TFLOP/s measured), its BF16 tensor cores
+// three orders more, so the contraction is done in integer slices (the Ozaki scheme): every
+// row of A = [[Re, -Im], [Im, Re]] of Lambda W and every column of X is scaled by a power of two
+// below 1 and cut into S = 8 signed 7-bit digits, v = 2^e sum_s q_s 2^{-7 s}, the first 56 bits
+// below the row's (column's) largest value.  The digits are small integers, exact in BF16, and
+// the products of digits s and t of one diagonal d = s + t accumulate in FP32 in a TMEM block of
+// their own: the eight blocks d = 2..9 hold integers.  With |q_1| <= 128, |q_s| <= 64 and at
+// most 512 terms (a K segment) the sums of diagonals 2..7 stay within 2^24 and are exact; a sum
+// of diagonals 8 and 9 that passed 2^24 would be rounded at 2^-24 of itself, 2^-65 of the
+// largest product.  The 36 products with s + t <= 9 leave out terms below 2^-58 of
+// max|A_row| max|X_col| each.  The epilogue adds the blocks in int64 at 2^-53 of
+// max|A_row| max|X_col| and rounds once to FP64.
+//
+// Both embeddings are interleaved (row 2 z + part, column 2 z' + part'): an FP64 chunk state
+// [i][n][z] complex128 is then a plain real column of 2 Nc entries, the epilogue's stores are
+// coalesced, and the two parts of one entry sit in neighbouring lanes (the update norm is the
+// complex modulus).
+//
+// Kernels: k_oz64_aprep (once per Lambda), k_oz64_xprep (gather, scale, digits of X),
+// k_oz64_gemm (persistent: TMA + tcgen05.mma kind::f16, 128 x 64 tiles).
+#include <algorithm>
+
+#include <cuda_bf16.h>
+#include <cudaTypedefs.h>
+
+#include "common.cuh"
+#include "oz64.cuh"
+#include "ptx.cuh"
+
+namespace {
+
+constexpr int S = 8;                                      // digits of 7 bits
+constexpr int FIX = 7 * S;
+constexpr int BM = 128, BN = 64, BK = 32;                 // 32 bf16 = 64-byte rows (64-byte swizzle)
+constexpr int A_TILE = BM * BK * 2;                       // 8 KB per A slice
+constexpr int X_TILE = BN * BK * 2;                       // 4 KB per X slice
+constexpr int STAGE_BYTES = S * (A_TILE + X_TILE);        // 96 KB
+constexpr int STAGES = 2;
+constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024;
+constexpr int SEG_KB = 512 / BK;                          // k-blocks of one exact K segment
+constexpr int THREADS = 384;                              // warp 0 TMA, warp 1 MMA, warps 4-11 epilogue
+constexpr int COLS_PER_WARP = BN / 2;
+constexpr uint32_t TMEM_COLS = S * BN;                    // one block of 64 columns per diagonal
+constexpr int E_BAD = 1 << 20;                            // scale exponent of a row or column with inf or NaN
+
+// kind::f16, D = F32, A = B = BF16, K-major, M = 128 (N set per MMA)
+constexpr uint32_t IDESC0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BM >> 4) << 24);
+
+struct Oz64State {
+  CUtensorMap amap, xmap;
+  __nv_bfloat16* as = nullptr;        // [S][Nr][2Nc][Kp]
+  int* esig = nullptr;                // [Nr][2Nc] row scale exponents
+  size_t a_bytes = 0;
+  bool a_ready = false;
+  __nv_bfloat16* xs = nullptr;        // [S][Nr][ncol][Kp]
+  int* etau = nullptr;                // [Nr][ncol] column scale exponents
+  size_t x_bytes = 0, tau_bytes = 0;
+  const void* xmap_ptr = nullptr;
+  int xmap_ncol = -1;
+  int* d_err = nullptr;
+  int num_sms = 1;
+  bool smem_set = false;
+};
+
+int k_pad(int Nc) { return (2 * Nc + BK - 1) / BK * BK; }
+
+// digits of |x| 2^{FIX - e} (|x| < 2^e) in one pass: with 64 added in every digit position below
+// the top, digit s of the sum in base 128, less 64, is the balanced digit in [-64, 63]
+__device__ __forceinline__ unsigned long long biased_digits(double x, int e) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int E = (int)((b >> 52) & 0x7FF);
+  const unsigned long long M = E == 0 ? 0 : ((b & 0xFFFFFFFFFFFFFull) | (1ull << 52));
+  const int sh = E - 1075 + FIX - e;                       // <= 3
+  unsigned long long v;
+  if (sh >= 0) {
+    v = M << min(sh, 8);
+  } else {
+    const int r = min(-sh, 63);
+    v = (M + ((1ull << r) >> 1)) >> r;
+  }
+  constexpr unsigned long long BIAS = [] {
+    unsigned long long s = 0;
+    for (int k = 2; k <= S; ++k) s += 64ull << (7 * (S - k));
+    return s;
+  }();
+  return v + BIAS;
+}
+__device__ __forceinline__ float digit(unsigned long long A, int s, bool neg) {
+  const int sh = 7 * (S - s);
+  const int q = s == 1 ? (int)(A >> sh) : (int)((unsigned)(A >> sh) & 127u) - 64;
+  return __int2float_rn(neg ? -q : q);
+}
+__device__ __forceinline__ bool sign_of(double x) { return __double2hiint(x) < 0; }
+
+// exponent e with |v| < 2^e for every v whose |high word| is at most mb; E_BAD for inf or NaN
+__device__ __forceinline__ int scale_exponent(unsigned int mb) {
+  const int E = (int)(mb >> 20);
+  return E == 0x7FF ? E_BAD : (E == 0 ? 0 : E - 1022);
+}
+
+// One warp per (site i, contour row z): the two rows 2 z (Re, -Im) and 2 z + 1 (Im, Re) of the
+// embedding share their digits and their scale.  Jrow (hopping equal on every bond): column z'
+// also carries J(t(z')), so that X is the plain sum of the neighbours' columns.
+__global__ void __launch_bounds__(256) k_oz64_aprep(const double2* __restrict__ lam, const double* __restrict__ Jrow,
+                                                    int Nr, int Nt, int Nm, double dt, double beta, int Kp,
+                                                    __nv_bfloat16* __restrict__ as, int* __restrict__ esig) {
+  const int Nc = 2 * Nt + Nm, N2 = 2 * Nc;
+  const size_t row = (size_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+  const int lane = threadIdx.x & 31;
+  if (row >= (size_t)Nr * Nc) return;
+  const double2* lrow = lam + row * Nc;
+  auto value = [&](int k) {
+    double2 v = cmul(lrow[k], contour_weight(k, Nt, Nm, dt, beta));
+    if (Jrow) {
+      const double j = Jrow[contour_time_index(k, Nt)];
+      v.x *= j;
+      v.y *= j;
+    }
+    return v;
+  };
+  unsigned int mb = 0;
+  for (int k = lane; k < Nc; k += 32) {
+    const double2 v = value(k);
+    mb = max(mb, max((unsigned)__double2hiint(v.x) & 0x7FFFFFFFu, (unsigned)__double2hiint(v.y) & 0x7FFFFFFFu));
+  }
+  for (int o = 16; o > 0; o >>= 1) mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, o));
+  const int e = scale_exponent(mb);
+  const size_t r0 = 2 * row;                               // = i N2 + 2 z
+  if (lane < 2) esig[r0 + lane] = e;
+  const size_t stride = (size_t)Nr * N2 * Kp;
+  for (int k = lane; 2 * k < Kp; k += 32) {
+    const double2 v = k < Nc ? value(k) : make_double2(0.0, 0.0);
+    const unsigned long long Ar = biased_digits(v.x, e), Ai = biased_digits(v.y, e);
+    const bool nr = sign_of(v.x), ni = sign_of(v.y);
+#pragma unroll
+    for (int s = 1; s <= S; ++s) {
+      const float qr = digit(Ar, s, nr), qi = digit(Ai, s, ni);
+      __nv_bfloat162* d = reinterpret_cast<__nv_bfloat162*>(as + (s - 1) * stride + r0 * Kp) + k;
+      d[0] = __floats2bfloat162_rn(qr, -qi);
+      d[Kp / 2] = __floats2bfloat162_rn(qi, qr);
+    }
+  }
+}
+
+// One warp per (site i, vector column n), sites fastest (the four reads of a neighbour's column
+// meet in L2): X = sum_j J_ij G_j in FP64, column scale, digits.  UNIFORM: J sits in the Lambda
+// slices.  PER_LANE contour points per lane in registers; PER_LANE = 0: any Nc, X summed twice.
+template <bool UNIFORM, int PER_LANE>
+__global__ void __launch_bounds__(256) k_oz64_xprep(const double2* __restrict__ G, const double* __restrict__ Jtab,
+                                                    const int* __restrict__ nbr, const int* __restrict__ nbond, int Nr,
+                                                    int Nt, int Nc, int ncol, int Kp, __nv_bfloat16* __restrict__ xs,
+                                                    int* __restrict__ etau) {
+  const size_t wi = (size_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+  const int lane = threadIdx.x & 31;
+  if (wi >= (size_t)Nr * ncol) return;
+  const int i = (int)(wi % Nr), n = (int)(wi / Nr);
+  const size_t w = (size_t)i * ncol + n;
+  const double2* col[4];
+  const double* jrow[4];
+  bool has[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int j = nbr[i * 4 + q];
+    has[q] = j >= 0;
+    col[q] = G + ((size_t)(has[q] ? j : i) * ncol + n) * Nc;
+    if (!UNIFORM) jrow[q] = Jtab + (size_t)(has[q] ? nbond[i * 4 + q] : 0) * Nt;
+  }
+  auto gather = [&](int z) {
+    double2 x = make_double2(0.0, 0.0);
+    const int tk = UNIFORM ? 0 : contour_time_index(z, Nt);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (!has[q]) continue;
+      const double2 g = col[q][z];
+      if (UNIFORM) {
+        x.x += g.x;
+        x.y += g.y;
+      } else {
+        const double j = jrow[q][tk];
+        x.x = fma(j, g.x, x.x);
+        x.y = fma(j, g.y, x.y);
+      }
+    }
+    return x;
+  };
+  constexpr int NREG = PER_LANE > 0 ? PER_LANE : 1;
+  double2 x[NREG];
+  unsigned int mb = 0;
+  auto fold = [&](double2 v) {
+    mb = max(mb, max((unsigned)__double2hiint(v.x) & 0x7FFFFFFFu, (unsigned)__double2hiint(v.y) & 0x7FFFFFFFu));
+  };
+  if (PER_LANE > 0) {
+#pragma unroll
+    for (int u = 0; u < NREG; ++u) {
+      const int z = lane + 32 * u;
+      x[u] = z < Nc ? gather(z) : make_double2(0.0, 0.0);
+      fold(x[u]);
+    }
+  } else {
+    for (int z = lane; z < Nc; z += 32) fold(gather(z));
+  }
+  for (int o = 16; o > 0; o >>= 1) mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, o));
+  const int e = scale_exponent(mb);
+  if (lane == 0) etau[w] = e;
+  const size_t stride = (size_t)Nr * ncol * Kp;
+  __nv_bfloat162* dst = reinterpret_cast<__nv_bfloat162*>(xs + w * Kp);
+  auto put = [&](int z, double2 v) {
+    const unsigned long long Ar = biased_digits(v.x, e), Ai = biased_digits(v.y, e);
+    const bool nr = sign_of(v.x), ni = sign_of(v.y);
+#pragma unroll
+    for (int s = 1; s <= S; ++s)
+      dst[(s - 1) * (stride / 2) + z] = __floats2bfloat162_rn(digit(Ar, s, nr), digit(Ai, s, ni));
+  };
+  if (PER_LANE > 0) {
+#pragma unroll
+    for (int u = 0; u < NREG; ++u) {
+      const int z = lane + 32 * u;
+      if (2 * z < Kp) put(z, x[u]);
+    }
+  } else {
+    for (int z = lane; 2 * z < Kp; z += 32) put(z, z < Nc ? gather(z) : make_double2(0.0, 0.0));
+  }
+}
+
+// V 2^e as FP64, rounded to nearest (halves away from zero); 0 below the normal range, inf above it
+__device__ __forceinline__ double fixed_to_double(long long V, int e) {
+  const unsigned long long a = (unsigned long long)(V < 0 ? -V : V);
+  const int lz = __clzll((long long)a);
+  const unsigned long long m = a << (lz & 63);              // leading bit at 63
+  const unsigned long long q = (m >> 11) + ((m >> 10) & 1);  // 53 bits, the leading one adds 1 to the exponent
+  const int ex = 1085 - lz + e;
+  unsigned long long bits = ((unsigned long long)(unsigned)ex << 52) + q;
+  if (ex >= 2045) bits = 0x7FF0000000000000ull;
+  if (ex < 1 || a == 0) bits = 0;
+  if (e >= E_BAD / 2) bits = 0x7FF8000000000000ull;
+  return __longlong_as_double((long long)(bits | ((unsigned long long)V & 0x8000000000000000ull)));
+}
+
+// |(d, partner lane's d)| as FP32
+__device__ __forceinline__ float pair_modulus(double d) {
+  const float a = fabsf((float)d);
+  const float b = __shfl_xor_sync(0xffffffffu, a, 1);
+  const float mx = fmaxf(a, b), mn = fminf(a, b);
+  const float t = mx > 0.f ? __fdividef(mn, mx) : 0.f;
+  const float m = mx * sqrtf(fmaf(t, t, 1.f));
+  return (a == a && b == b && m == m) ? m : __int_as_float(0x7f800000);
+}
+
+// Persistent: one CTA per SM walks 128 x 64 output tiles (row tile fastest, then column tile, then
+// site).  A stage is a 32-deep k-block of all eight slices of both operands.  Per k16 step,
+// slice s of A times slices 1..9-s of X (back to back in the stage) lands in the TMEM blocks of
+// diagonals s+1..9: twelve MMAs of N <= 256 for the 36 products.
+// What bounds it: the MMAs' 1152 columns per k16 step (and the same step's shared-memory reads).
+// The eight accumulators fill TMEM, so the MMAs of a tile wait until the epilogue has read the
+// previous tile's into int64 registers; its FP64 part overlaps them.  64 columns
+// per tile, because at 32 (two sets) each A slice would be read from L2 twice as often.
+template <int MODE>
+__global__ void __launch_bounds__(THREADS, 1)
+    k_oz64_gemm(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap xmap,
+                const int* __restrict__ esig, const int* __restrict__ etau, const double* __restrict__ Gin,
+                const double2* __restrict__ lam, const int* __restrict__ src_site, const int* __restrict__ src_time,
+                int Nr, int Nc, int KB, int ncol, int gs, double* __restrict__ out, float* __restrict__ r32,
+                unsigned long long* __restrict__ norm, int* __restrict__ err) {
+  using namespace ptx;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], acc_full, acc_empty, drain;
+  __shared__ uint32_t tmem_holder;
+  __shared__ WaitCtl wctl;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int N2 = 2 * Nc;
+  const int MT = (N2 + BM - 1) / BM, NT = (ncol + BN - 1) / BN;
+  const int tiles = MT * NT * Nr;
+  const int nseg = (KB + SEG_KB - 1) / SEG_KB;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(&acc_full, 1);
+    mbar_init(&acc_empty, 256);
+    mbar_init(&drain, 1);
+    wait_ctl_init(&wctl);
+    fence_barrier_init();
+  }
+  if (warp == 1) tmem_alloc(&tmem_holder, TMEM_COLS);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_holder;
+  volatile WaitCtl* abort_p = &wctl;
+  auto stage_ptr = [&](int s) { return smem + (size_t)s * STAGE_BYTES; };
+
+  if (warp == 0) {
+    if (lane == 0) {
+      // ---------------- TMA producer ----------------
+      int g = 0;
+      bool ok = true;
+      for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
+        const int mt = tile % MT, nt = (tile / MT) % NT, site = tile / (MT * NT);
+        for (int kb = 0; kb < KB; ++kb, ++g) {
+          const int s = g % STAGES;
+          if (g >= STAGES && !mbar_wait(&empty[s], ((g / STAGES) - 1) & 1, abort_p)) {
+            ok = false;
+            break;
+          }
+          uint8_t* st = stage_ptr(s);
+          mbar_expect_tx(&full[s], STAGE_BYTES);
+          for (int q = 0; q < S; ++q) {
+            tma_load_4d(st + q * A_TILE, &amap, &full[s], kb * BK, mt * BM, site, q);
+            tma_load_4d(st + S * A_TILE + q * X_TILE, &xmap, &full[s], kb * BK, nt * BN, site, q);
+          }
+        }
+      }
+      for (int q = g > STAGES ? g - STAGES : 0; q < g; ++q)
+        mbar_wait(&full[q % STAGES], (q / STAGES) & 1, abort_p, false);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      // ---------------- MMA issuer ----------------
+      int g = 0, t = 0;
+      bool ok = true, any = false;
+      for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
+        for (int kb = 0; kb < KB; ++kb, ++g) {
+          const bool first = kb % SEG_KB == 0;
+          if (first) {                                      // a new segment overwrites the accumulators
+            if (t >= 1 && !mbar_wait(&acc_empty, (t - 1) & 1, abort_p)) {
+              ok = false;
+              break;
+            }
+            ++t;
+            tc_fence_after();
+          }
+          const int s = g % STAGES;
+          if (!mbar_wait(&full[s], (g / STAGES) & 1, abort_p)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t base = smem_u32(stage_ptr(s));
+#pragma unroll
+          for (int k16 = 0; k16 < BK / 16; ++k16) {
+#pragma unroll
+            for (int sl = 0; sl < S; ++sl) {
+              const uint64_t ad = sdesc_sw64(base + sl * A_TILE + k16 * 32);
+#pragma unroll
+              for (int t0 = 0; t0 < S - sl; t0 += 256 / BN) {
+                const int nblk = (S - sl - t0) < 256 / BN ? (S - sl - t0) : 256 / BN;
+                const uint32_t idesc = IDESC0 | ((uint32_t)(nblk * BN >> 3) << 17);
+                const uint64_t xd = sdesc_sw64(base + S * A_TILE + t0 * X_TILE + k16 * 32);
+                mma<0>(tmem + (uint32_t)((sl + t0) * BN), ad, xd, idesc, (first && k16 == 0 && sl == 0) ? 0u : 1u);
+              }
+            }
+          }
+          mma_commit(&empty[s]);
+          any = true;
+          if (kb + 1 == KB || (kb + 1) % SEG_KB == 0) mma_commit(&acc_full);
+        }
+      }
+      if (any) {
+        mma_commit(&drain);
+        mbar_wait(&drain, 0, abort_p, false);
+      }
+    }
+  } else if (warp >= 4) {
+    // ---------------- epilogue: warps 4-11, two per TMEM lane quarter ----------------
+    const int q4 = warp & 3, half = (warp - 4) >> 2;
+    const uint32_t tacc = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(half * COLS_PER_WARP);
+    // int64 unit 2^-53 of the scales' product, coarser by the bits that several segments add
+    int extra = 0;
+    while ((1 << extra) < nseg) ++extra;
+    int t = 0;
+    bool go = true;
+    for (int tile = blockIdx.x; tile < tiles && go; tile += gridDim.x) {
+      const int mt = tile % MT, nt = (tile / MT) % NT, site = tile / (MT * NT);
+      const int m = mt * BM + q4 * 32 + lane;
+      const int n_first = nt * BN + half * COLS_PER_WARP;
+      const bool row_ok = m < N2;
+      const int es = row_ok ? esig[(size_t)site * N2 + m] : 0;
+      long long V[COLS_PER_WARP];
+      for (int seg = 0; seg < nseg; ++seg, ++t) {
+        go = mbar_wait(&acc_full, t & 1, abort_p);
+        go = __all_sync(0xffffffffu, go);                   // tcgen05.ld below is warp-collective
+        if (!go) break;
+        tc_fence_after();
+#pragma unroll
+        for (int c = 0; c < COLS_PER_WARP / 4; ++c) {
+          uint32_t r[S][4];
+#pragma unroll
+          for (int d = 0; d < S; ++d) tmem_ld4(tacc + (uint32_t)(d * BN + c * 4), r[d]);
+          tmem_wait_ld();
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            auto f = [&](int d) { return __uint_as_float(r[d][j]); };
+            // diagonals 2..7 are integers; 8 and 9 are below the unit's last bits
+            long long v = (long long)__float2int_rn(fmaf(f(7), 0x1p-10f, f(6) * 0x1p-3f));
+            v += (long long)__float2int_rn(f(5)) * (1ll << 4) + (long long)__float2int_rn(f(4)) * (1ll << 11);
+            v += (long long)__float2int_rn(f(3)) * (1ll << 18) + (long long)__float2int_rn(f(2)) * (1ll << 25);
+            v += ((long long)__float2int_rn(f(1)) + (long long)__float2int_rn(f(0)) * (1ll << 7)) * (1ll << 32);
+            if (extra) v = (v + (1ll << (extra - 1))) >> extra;
+            V[c * 4 + j] = seg ? V[c * 4 + j] + v : v;
+          }
+        }
+        tc_fence_before();
+        mbar_arrive(&acc_empty);                            // the next segment's MMAs may start
+      }
+      if (!go) break;
+      int qcur = n_first / gs;
+      int left = gs - (n_first - qcur * gs);                // columns until the next norm group
+      float runmax = 0.f;
+#pragma unroll
+      for (int j = 0; j < COLS_PER_WARP; ++j) {
+        const int n = n_first + j;
+        if (n < ncol) {                                     // warp-uniform
+          if (left == 0) {
+            float mm = runmax;
+            for (int o = 16; o > 0; o >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, o));
+            if (lane == 0) atomicMax(norm + qcur, (unsigned long long)__double_as_longlong((double)mm));
+            ++qcur;
+            left = gs;
+            runmax = 0.f;
+          }
+          --left;
+          const size_t cidx = (size_t)site * ncol + n;
+          double y = fixed_to_double(V[j], es + __ldg(etau + cidx) - 53 + extra);
+          if (__builtin_expect(__ldg(src_site + n) == site, 0) && row_ok) {   // B = Lambda_s e_{z'}
+            const double2 b = lam[((size_t)site * Nc + (m >> 1)) * Nc + src_time[n]];
+            y += (m & 1) ? b.y : b.x;
+          }
+          const size_t off = cidx * N2 + m;
+          double d = 0.0;
+          if (row_ok) {
+            d = y - Gin[off];
+            if (MODE == 0) out[off] = y;
+            else r32[cidx * N2 + (m >> 1) + ((m & 1) ? Nc : 0)] = (float)d;
+          }
+          runmax = fmaxf(runmax, pair_modulus(d));
+        }
+      }
+      float mm = runmax;
+      for (int o = 16; o > 0; o >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, o));
+      if (lane == 0 && n_first < ncol) atomicMax(norm + qcur, (unsigned long long)__double_as_longlong((double)mm));
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    __syncwarp();
+    tc_fence_after();
+    tmem_dealloc(tmem, TMEM_COLS);
+  }
+  // a wait that ran out raises the flag and makes the norm infinite, so that the host looks at the
+  // flag only where a norm is not finite
+  if (threadIdx.x == 0 && wctl.abort) {
+    atomicExch(err, 1);
+    atomicMax(norm, 0x7FF0000000000000ull);
+  }
+}
+
+PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
+  static PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
+    return static_cast<PFN_cuTensorMapEncodeTiled_v12000>(nullptr);
+  }();
+  return fn;
+}
+
+// 4D bf16 map [d3][d2][d1][d0] with a (32 x rows x 1 x 1) box and 64-byte swizzle
+bool make_map4(CUtensorMap* m, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t d3, uint32_t rows) {
+  auto fn = encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[4] = {d0, d1, d2, d3};
+  cuuint64_t strides[3] = {d0 * 2, d0 * d1 * 2, d0 * d1 * d2 * 2};
+  cuuint32_t box[4] = {(cuuint32_t)BK, rows, 1, 1};
+  cuuint32_t es[4] = {1, 1, 1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, es,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+Oz64State* state(dyson_ctx* c) {
+  if (!c->oz64) c->oz64 = new Oz64State();
+  return static_cast<Oz64State*>(c->oz64);
+}
+
+template <class T>
+int grow(dyson_ctx* c, T** p, size_t* have, size_t bytes, const char* what) {
+  if (*have >= bytes) return DYSON_OK;
+  if (*p) cudaFree(*p);
+  *p = nullptr;
+  *have = 0;
+  cudaError_t e = cudaMalloc((void**)p, bytes);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return ctx_fail(c, DYSON_ERR_OOM, std::string(what) + ": " + cudaGetErrorString(e));
+  }
+  *have = bytes;
+  return DYSON_OK;
+}
+
+size_t a_slice_bytes(const dyson_ctx* c) { return (size_t)S * c->Nr * 2 * c->Nc * k_pad(c->Nc) * 2; }
+
+const double* uniform_hopping(const dyson_ctx* c) { return c->j_uniform && c->Nb > 0 ? c->dJ : nullptr; }
+
+template <bool UNIFORM>
+void launch_xprep(dyson_ctx* c, int ncol, const double2* G, Oz64State* st) {
+  const size_t warps = (size_t)c->Nr * ncol;
+  const unsigned blocks = (unsigned)((warps + 7) / 8);
+  const int Kp = k_pad(c->Nc), pts = Kp / 2;               // padded points per column
+  auto go = [&](auto kernel) {
+    kernel<<<blocks, 256, 0, c->stream>>>(G, c->dJ, c->d_nbr, c->d_nbond, c->Nr, c->Nt, c->Nc, ncol, Kp, st->xs,
+                                          st->etau);
+  };
+  if (pts <= 32) go(k_oz64_xprep<UNIFORM, 1>);
+  else if (pts <= 64) go(k_oz64_xprep<UNIFORM, 2>);
+  else if (pts <= 128) go(k_oz64_xprep<UNIFORM, 4>);
+  else if (pts <= 256) go(k_oz64_xprep<UNIFORM, 8>);
+  else go(k_oz64_xprep<UNIFORM, 0>);
+}
+
+}  // namespace
+
+bool oz64_usable(dyson_ctx* c) {
+  if (!c->oz64_enabled || !encode_fn()) return false;
+  Oz64State* st = static_cast<Oz64State*>(c->oz64);
+  if (st && st->a_bytes >= a_slice_bytes(c)) return true;
+  size_t free_b = 0, total_b = 0;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;
+  return a_slice_bytes(c) <= (free_b + c->work_bytes) / 3;
+}
+
+double oz64_bytes_per_element(const dyson_ctx* c) {
+  return (double)S * 2 * k_pad(c->Nc) / c->Nc + 4.0 / c->Nc;
+}
+
+void oz64_invalidate(dyson_ctx* c) {
+  if (c->oz64) static_cast<Oz64State*>(c->oz64)->a_ready = false;
+}
+
+int oz64_prepare(dyson_ctx* c) {
+  Oz64State* st = state(c);
+  const int Nr = c->Nr, Nc = c->Nc, N2 = 2 * Nc, Kp = k_pad(Nc);
+  int rc;
+  if (!st->d_err) {
+    DY_CUDA(c, cudaMalloc(&st->d_err, sizeof(int)));
+    DY_CUDA(c, cudaMemsetAsync(st->d_err, 0, sizeof(int), c->stream));
+    DY_CUDA(c, cudaDeviceGetAttribute(&st->num_sms, cudaDevAttrMultiProcessorCount, c->device));
+  }
+  if (!st->smem_set) {
+    DY_CUDA(c, cudaFuncSetAttribute(k_oz64_gemm<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
+    DY_CUDA(c, cudaFuncSetAttribute(k_oz64_gemm<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
+    st->smem_set = true;
+  }
+  if (!st->a_ready) {
+    if ((rc = grow(c, &st->as, &st->a_bytes, a_slice_bytes(c), "FP64 slices of Lambda"))) return rc;
+    if (!st->esig) DY_CUDA(c, cudaMalloc(&st->esig, (size_t)Nr * N2 * sizeof(int)));
+    const size_t rows = (size_t)Nr * Nc;
+    k_oz64_aprep<<<(unsigned)((rows + 7) / 8), 256, 0, c->stream>>>(c->d_lam, uniform_hopping(c), Nr, c->Nt, c->Nm,
+                                                                   c->dt, c->beta, Kp, st->as, st->esig);
+    DY_CUDA(c, cudaGetLastError());
+    c->launches += 1;
+    if (!make_map4(&st->amap, st->as, Kp, N2, Nr, S, BM))
+      return ctx_fail(c, DYSON_ERR_CUDA, "cuTensorMapEncodeTiled failed for the FP64 Lambda slices");
+    st->a_ready = true;
+  }
+  return DYSON_OK;
+}
+
+int oz64_sweep(dyson_ctx* c, int ncol, int gs, const double2* Gin, double2* out, float* r32, int mode) {
+  int rc = oz64_prepare(c);
+  if (rc) return rc;
+  Oz64State* st = state(c);
+  const int Nr = c->Nr, Nc = c->Nc, N2 = 2 * Nc, Kp = k_pad(Nc);
+  if ((rc = grow(c, &st->xs, &st->x_bytes, (size_t)S * Nr * ncol * Kp * 2, "FP64 slices of X"))) return rc;
+  if ((rc = grow(c, &st->etau, &st->tau_bytes, (size_t)Nr * ncol * sizeof(int), "FP64 column scales"))) return rc;
+  if (st->xmap_ptr != st->xs || st->xmap_ncol != ncol) {
+    if (!make_map4(&st->xmap, st->xs, Kp, ncol, Nr, S, BN))
+      return ctx_fail(c, DYSON_ERR_CUDA, "cuTensorMapEncodeTiled failed for the FP64 X slices");
+    st->xmap_ptr = st->xs;
+    st->xmap_ncol = ncol;
+  }
+  if (uniform_hopping(c)) launch_xprep<true>(c, ncol, Gin, st);
+  else launch_xprep<false>(c, ncol, Gin, st);
+  DY_CUDA(c, cudaGetLastError());
+  const long long tiles = (long long)((N2 + BM - 1) / BM) * ((ncol + BN - 1) / BN) * Nr;
+  const int grid = (int)std::min<long long>(tiles, st->num_sms);
+  auto go = [&](auto kernel) {
+    kernel<<<grid, THREADS, SMEM_BYTES, c->stream>>>(
+        st->amap, st->xmap, st->esig, st->etau, reinterpret_cast<const double*>(Gin), c->d_lam, c->d_src_site,
+        c->d_src_time, Nr, Nc, Kp / BK, ncol, gs, reinterpret_cast<double*>(out), r32, c->d_norm, st->d_err);
+  };
+  if (mode == 0) go(k_oz64_gemm<0>);
+  else go(k_oz64_gemm<1>);
+  DY_CUDA(c, cudaGetLastError());
+  c->launches += 2;
+  return DYSON_OK;
+}
+
+int oz64_set_wait_limit(dyson_ctx* c, unsigned long long ns) {
+  DY_CUDA(c, cudaMemcpyToSymbolAsync(ptx::g_wait_limit_ns, &ns, sizeof ns, 0, cudaMemcpyHostToDevice, c->stream));
+  DY_CUDA(c, cudaStreamSynchronize(c->stream));
+  return DYSON_OK;
+}
+
+int oz64_check_error(dyson_ctx* c) {
+  Oz64State* st = static_cast<Oz64State*>(c->oz64);
+  if (!st || !st->d_err) return DYSON_OK;
+  int flag = 0;
+  DY_CUDA(c, cudaMemcpyAsync(&flag, st->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+  DY_CUDA(c, cudaStreamSynchronize(c->stream));
+  if (!flag) return DYSON_OK;
+  DY_CUDA(c, cudaMemsetAsync(st->d_err, 0, sizeof(int), c->stream));
+  return ctx_fail(c, DYSON_ERR_TIMEOUT, "an FP64 sweep pipeline wait exceeded its time limit");
+}
+
+void oz64_release(dyson_ctx* c) {
+  Oz64State* st = static_cast<Oz64State*>(c->oz64);
+  if (!st) return;
+  void* ptrs[] = {st->as, st->esig, st->xs, st->etau, st->d_err};
+  for (void* p : ptrs)
+    if (p) cudaFree(p);
+  delete st;
+  c->oz64 = nullptr;
+}

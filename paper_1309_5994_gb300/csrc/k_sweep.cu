@@ -40,7 +40,8 @@ __device__ __forceinline__ unsigned long long nonneg_bits(double v) {
   return (unsigned long long)__double_as_longlong(v);
 }
 
-// K3: FP64 sweep (MODE 0) or FP64 Dyson residual (MODE 1).  Tile 64 rows z x 64
+// K3: FP64 sweep (MODE 0) or FP64 Dyson residual (MODE 1) on the FP64 pipe, where the slices of
+// Lambda that k_oz64 needs (64 bytes per entry) do not fit in device memory.  Tile 64 rows z x 64
 // vector columns n per CTA, 256 threads, 4x4 complex outputs per thread.
 template <int MODE>
 __global__ __launch_bounds__(256) void k_sweep_f64(

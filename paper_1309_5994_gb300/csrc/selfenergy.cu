@@ -49,6 +49,7 @@
 using namespace dyson_detail;
 
 void oz_invalidate(dyson_ctx* c);
+void oz64_invalidate(dyson_ctx* c);
 
 namespace {
 
@@ -976,6 +977,7 @@ extern "C" int dyson_selfenergy_step(dyson_ctx* c, const double* gloc, double mi
   DY_CUDA(c, cudaStreamSynchronize(c->stream));
   c->lam32_built = c->lam_split_built = false;
   oz_invalidate(c);
+  oz64_invalidate(c);
   c->se_installed = true;
   double ss = 0.0, mx = 0.0;
   for (int b = 0; b < MIX_BLOCKS; ++b) {

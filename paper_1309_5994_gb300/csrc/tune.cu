@@ -77,9 +77,9 @@ int dyson_autotune(dyson_ctx* c, int32_t max_block_columns, dyson_tuning* out) {
   int rc;
   if ((rc = prepare_tables(c, DYSON_PREC_TF32X3_F64REF))) return rc;
   if (!c->use_tc) return ctx_fail(c, DYSON_ERR_INVALID_ARG, "the tensor-core sweep needs Nc % 64 == 0");
-  size_t col_bytes = 0;
+  size_t col_bytes = 0, col_total = 0;
   const int64_t cap = chunk_columns(c, DYSON_PREC_TF32X3_F64REF, c->Nc, (int64_t)max_block_columns * c->Nc,
-                                    &col_bytes) / c->Nc;
+                                    &col_bytes, &col_total) / c->Nc;
   if (cap < 1) return ctx_fail(c, DYSON_ERR_OOM, "one block column does not fit in device memory");
   // a chunk whose inner solve may switch to GMRES (DYSON_INNER_AUTO or _GMRES) must leave
   // room for the Krylov basis of the full restart length (restart + 4 FP32 states), or
@@ -89,7 +89,7 @@ int dyson_autotune(dyson_ctx* c, int32_t max_block_columns, dyson_tuning* out) {
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess) {
       const int m = c->gmres_restart > 0 ? c->gmres_restart : 40;
-      const double per_block = (double)c->Nc * ((double)col_bytes + (m + 4.0) * c->Nr * 2.0 * c->Nc * sizeof(float));
+      const double per_block = (double)c->Nc * ((double)col_total + (m + 4.0) * c->Nr * 2.0 * c->Nc * sizeof(float));
       const double avail = 0.8 * (double)(free_b + c->work_bytes);
       cap_gm = std::max<int64_t>(1, std::min<int64_t>(cap, (int64_t)(avail / per_block)));
     }
