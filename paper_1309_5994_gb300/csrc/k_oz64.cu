@@ -22,6 +22,7 @@
 // Kernels: k_oz64_aprep (once per Lambda), k_oz64_xprep (gather, scale, digits of X),
 // k_oz64_gemm (persistent: TMA + tcgen05.mma kind::f16, 128 x 64 tiles).
 #include <algorithm>
+#include <type_traits>
 
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
@@ -41,8 +42,8 @@ constexpr int STAGE_BYTES = S * (A_TILE + X_TILE);        // 96 KB
 constexpr int STAGES = 2;
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024;
 constexpr int SEG_KB = 512 / BK;                          // k-blocks of one exact K segment
-constexpr int THREADS = 384;                              // warp 0 TMA, warp 1 MMA, warps 4-11 epilogue
-constexpr int COLS_PER_WARP = BN / 2;
+constexpr int THREADS = 640;                              // warp 0 TMA, warp 1 MMA, warps 4-19 epilogue
+constexpr int COLS_PER_WARP = BN / 4;
 constexpr uint32_t TMEM_COLS = S * BN;                    // one block of 64 columns per diagonal
 constexpr int E_BAD = 1 << 20;                            // scale exponent of a row or column with inf or NaN
 
@@ -88,10 +89,29 @@ __device__ __forceinline__ unsigned long long biased_digits(double x, int e) {
   }();
   return v + BIAS;
 }
-__device__ __forceinline__ float digit(unsigned long long A, int s, bool neg) {
-  const int sh = 7 * (S - s);
-  const int q = s == 1 ? (int)(A >> sh) : (int)((unsigned)(A >> sh) & 127u) - 64;
-  return __int2float_rn(neg ? -q : q);
+// Digit s (1..S) of two values as packed bf16 integers, signs applied.  The bits 0x4300 + j are
+// the bf16 number 128 + j for j = 0..128, so one exact packed FMA by +-1 subtracts the offset
+// (128 for the top digit, 128 + 64 for the balanced ones) and sets the sign: six instructions a
+// pair, where integer-to-float conversions took sixteen.
+struct PairSigns {
+  __nv_bfloat162 one, top, low;                            // +-1, -+128, -+192 per half
+};
+__device__ __forceinline__ __nv_bfloat162 as_bf162(unsigned int u) { return *reinterpret_cast<__nv_bfloat162*>(&u); }
+__device__ __forceinline__ PairSigns pair_signs(bool neg_lo, bool neg_hi) {
+  const unsigned int f = (neg_lo ? 0x8000u : 0u) | (neg_hi ? 0x80000000u : 0u);
+  return {as_bf162(0x3F803F80u ^ f), as_bf162(0xC300C300u ^ f), as_bf162(0xC340C340u ^ f)};
+}
+template <int s>
+__device__ __forceinline__ __nv_bfloat162 digit_pair(unsigned long long lo, unsigned long long hi, PairSigns g) {
+  constexpr int sh = 7 * (S - s);
+  constexpr unsigned int mask = s == 1 ? 0xFFu : 0x7Fu;
+  const unsigned int j = ((unsigned int)(lo >> sh) & mask) | (((unsigned int)(hi >> sh) & mask) << 16);
+  return __hfma2(as_bf162(j + 0x43004300u), g.one, s == 1 ? g.top : g.low);
+}
+template <int s = 1, class F>
+__device__ __forceinline__ void each_digit(F&& f) {
+  f(std::integral_constant<int, s>());
+  if constexpr (s < S) each_digit<s + 1>(f);
 }
 __device__ __forceinline__ bool sign_of(double x) { return __double2hiint(x) < 0; }
 
@@ -135,13 +155,13 @@ __global__ void __launch_bounds__(256) k_oz64_aprep(const double2* __restrict__ 
     const double2 v = k < Nc ? value(k) : make_double2(0.0, 0.0);
     const unsigned long long Ar = biased_digits(v.x, e), Ai = biased_digits(v.y, e);
     const bool nr = sign_of(v.x), ni = sign_of(v.y);
-#pragma unroll
-    for (int s = 1; s <= S; ++s) {
-      const float qr = digit(Ar, s, nr), qi = digit(Ai, s, ni);
+    const PairSigns top = pair_signs(nr, !ni), bot = pair_signs(ni, nr);
+    each_digit([&](auto sc) {
+      constexpr int s = decltype(sc)::value;
       __nv_bfloat162* d = reinterpret_cast<__nv_bfloat162*>(as + (s - 1) * stride + r0 * Kp) + k;
-      d[0] = __floats2bfloat162_rn(qr, -qi);
-      d[Kp / 2] = __floats2bfloat162_rn(qi, qr);
-    }
+      d[0] = digit_pair<s>(Ar, Ai, top);
+      d[Kp / 2] = digit_pair<s>(Ai, Ar, bot);
+    });
   }
 }
 
@@ -209,10 +229,11 @@ __global__ void __launch_bounds__(256) k_oz64_xprep(const double2* __restrict__ 
   __nv_bfloat162* dst = reinterpret_cast<__nv_bfloat162*>(xs + w * Kp);
   auto put = [&](int z, double2 v) {
     const unsigned long long Ar = biased_digits(v.x, e), Ai = biased_digits(v.y, e);
-    const bool nr = sign_of(v.x), ni = sign_of(v.y);
-#pragma unroll
-    for (int s = 1; s <= S; ++s)
-      dst[(s - 1) * (stride / 2) + z] = __floats2bfloat162_rn(digit(Ar, s, nr), digit(Ai, s, ni));
+    const PairSigns g = pair_signs(sign_of(v.x), sign_of(v.y));
+    each_digit([&](auto sc) {
+      constexpr int s = decltype(sc)::value;
+      dst[(s - 1) * (stride / 2) + z] = digit_pair<s>(Ar, Ai, g);
+    });
   };
   if (PER_LANE > 0) {
 #pragma unroll
@@ -239,24 +260,31 @@ __device__ __forceinline__ double fixed_to_double(long long V, int e) {
   return __longlong_as_double((long long)(bits | ((unsigned long long)V & 0x8000000000000000ull)));
 }
 
-// |(d, partner lane's d)| as FP32
-__device__ __forceinline__ float pair_modulus(double d) {
-  const float a = fabsf((float)d);
-  const float b = __shfl_xor_sync(0xffffffffu, a, 1);
-  const float mx = fmaxf(a, b), mn = fminf(a, b);
-  const float t = mx > 0.f ? __fdividef(mn, mx) : 0.f;
-  const float m = mx * sqrtf(fmaf(t, t, 1.f));
-  return (a == a && b == b && m == m) ? m : __int_as_float(0x7f800000);
+// |d| as FP32 from its bits (truncated; no conversion on the FP64 pipe): 0 below 2^-126, inf from 2^127
+// and for NaN
+__device__ __forceinline__ float magnitude(double d) {
+  const unsigned int hi = (unsigned int)__double2hiint(d) & 0x7FFFFFFFu, lo = (unsigned int)__double2loint(d);
+  const unsigned int f = __funnelshift_l(lo, hi, 3) - (896u << 23);
+  return __uint_as_float(hi < 0x38100000u ? 0u : (hi >= 0x47E00000u ? 0x7F800000u : f));
+}
+// sqrt of a running maximum of squares (inf stays inf)
+__device__ __forceinline__ void flush_norm(float sq, unsigned long long* norm, int lane) {
+  for (int o = 16; o > 0; o >>= 1) sq = fmaxf(sq, __shfl_xor_sync(0xffffffffu, sq, o));
+  if (lane == 0) atomicMax(norm, (unsigned long long)__double_as_longlong(sqrt((double)sq)));
 }
 
 // Persistent: one CTA per SM walks 128 x 64 output tiles (row tile fastest, then column tile, then
 // site).  A stage is a 32-deep k-block of all eight slices of both operands.  Per k16 step,
 // slice s of A times slices 1..9-s of X (back to back in the stage) lands in the TMEM blocks of
 // diagonals s+1..9: twelve MMAs of N <= 256 for the 36 products.
-// What bounds it: the MMAs' 1152 columns per k16 step (and the same step's shared-memory reads).
 // The eight accumulators fill TMEM, so the MMAs of a tile wait until the epilogue has read the
-// previous tile's into int64 registers; its FP64 part overlaps them.  64 columns
-// per tile, because at 32 (two sets) each A slice would be read from L2 twice as often.
+// previous tile's into int64 registers; the rest of the epilogue overlaps them.  64 columns per
+// tile, because at 32 (two sets) each A slice would be read from L2 twice as often.
+// Measured on 10x10, Nc = 128, 512 columns (6.7 GFLOP of FP64): 0.19 ms, against 6.33 ms of the FP64-pipe
+// kernel.  A k-block's 24 MMAs take about 2600 cycles; reading the accumulators out takes
+// 4400 of a tile's 31000 cycles, and loads of the slices from DRAM another 6000 that two stages do
+// not hide.  Sixteen epilogue warps, their G loaded ahead and integer forms of the FP64
+// conversions: with eight warps that loaded G as they went the epilogue alone took 0.39 ms.
 template <int MODE>
 __global__ void __launch_bounds__(THREADS, 1)
     k_oz64_gemm(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap xmap,
@@ -282,7 +310,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       mbar_init(&empty[s], 1);
     }
     mbar_init(&acc_full, 1);
-    mbar_init(&acc_empty, 256);
+    mbar_init(&acc_empty, 512);
     mbar_init(&drain, 1);
     wait_ctl_init(&wctl);
     fence_barrier_init();
@@ -367,9 +395,9 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
     }
   } else if (warp >= 4) {
-    // ---------------- epilogue: warps 4-11, two per TMEM lane quarter ----------------
-    const int q4 = warp & 3, half = (warp - 4) >> 2;
-    const uint32_t tacc = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(half * COLS_PER_WARP);
+    // ---------------- epilogue: warps 4-19, four per TMEM lane quarter ----------------
+    const int q4 = warp & 3, part = (warp - 4) >> 2;
+    const uint32_t tacc = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(part * COLS_PER_WARP);
     // int64 unit 2^-53 of the scales' product, coarser by the bits that several segments add
     int extra = 0;
     while ((1 << extra) < nseg) ++extra;
@@ -378,9 +406,22 @@ __global__ void __launch_bounds__(THREADS, 1)
     for (int tile = blockIdx.x; tile < tiles && go; tile += gridDim.x) {
       const int mt = tile % MT, nt = (tile / MT) % NT, site = tile / (MT * NT);
       const int m = mt * BM + q4 * 32 + lane;
-      const int n_first = nt * BN + half * COLS_PER_WARP;
+      const int n_first = nt * BN + part * COLS_PER_WARP;
       const bool row_ok = m < N2;
       const int es = row_ok ? esig[(size_t)site * N2 + m] : 0;
+      const int cols = max(0, min(COLS_PER_WARP, ncol - n_first));
+      // lane j < 16: scale exponent and source of the warp's column j (read by shuffle below)
+      static_assert(COLS_PER_WARP == 16, "one column per lane of a half warp");
+      const int et_l = lane < cols ? __ldg(etau + (size_t)site * ncol + n_first + lane) : 0;
+      const unsigned src_here = __ballot_sync(0xffffffffu, lane < cols && __ldg(src_site + n_first + lane) == site);
+      const size_t off0 = ((size_t)site * ncol + n_first) * N2 + (row_ok ? m : 0);
+      // G of this lane's row, eight columns at a time (the first ones before the wait)
+      double gin[8];
+      auto load_g = [&](int c) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) gin[j] = c + j < cols ? __ldg(Gin + off0 + (size_t)(c + j) * N2) : 0.0;
+      };
+      load_g(0);
       long long V[COLS_PER_WARP];
       for (int seg = 0; seg < nseg; ++seg, ++t) {
         go = mbar_wait(&acc_full, t & 1, abort_p);
@@ -410,40 +451,34 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
       if (!go) break;
       int qcur = n_first / gs;
-      int left = gs - (n_first - qcur * gs);                // columns until the next norm group
-      float runmax = 0.f;
+      int left = min(COLS_PER_WARP, (qcur + 1) * gs - n_first);   // columns to the next norm group
+      float sq = 0.f;                                       // running max |d|^2 of the group
 #pragma unroll
       for (int j = 0; j < COLS_PER_WARP; ++j) {
-        const int n = n_first + j;
-        if (n < ncol) {                                     // warp-uniform
-          if (left == 0) {
-            float mm = runmax;
-            for (int o = 16; o > 0; o >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, o));
-            if (lane == 0) atomicMax(norm + qcur, (unsigned long long)__double_as_longlong((double)mm));
-            ++qcur;
-            left = gs;
-            runmax = 0.f;
-          }
-          --left;
-          const size_t cidx = (size_t)site * ncol + n;
-          double y = fixed_to_double(V[j], es + __ldg(etau + cidx) - 53 + extra);
-          if (__builtin_expect(__ldg(src_site + n) == site, 0) && row_ok) {   // B = Lambda_s e_{z'}
-            const double2 b = lam[((size_t)site * Nc + (m >> 1)) * Nc + src_time[n]];
-            y += (m & 1) ? b.y : b.x;
-          }
-          const size_t off = cidx * N2 + m;
-          double d = 0.0;
-          if (row_ok) {
-            d = y - Gin[off];
-            if (MODE == 0) out[off] = y;
-            else r32[cidx * N2 + (m >> 1) + ((m & 1) ? Nc : 0)] = (float)d;
-          }
-          runmax = fmaxf(runmax, pair_modulus(d));
+        if (j == 8) load_g(8);
+        const int et = __shfl_sync(0xffffffffu, et_l, j);
+        double y = fixed_to_double(V[j], es + et - 53 + extra);
+        if (j >= cols) continue;                            // warp-uniform
+        if (j == left) {
+          flush_norm(sq, norm + qcur, lane);
+          ++qcur;
+          left = j + gs;
+          sq = 0.f;
         }
+        if ((src_here >> j & 1) && row_ok) {                // B = Lambda_s e_{z'}
+          const double2 b = lam[((size_t)site * Nc + (m >> 1)) * Nc + src_time[n_first + j]];
+          y += (m & 1) ? b.y : b.x;
+        }
+        const double d = y - gin[j % 8];
+        const float a = row_ok ? magnitude(d) : 0.f;
+        if (row_ok) {
+          if (MODE == 0) out[off0 + (size_t)j * N2] = y;
+          else r32[((size_t)site * ncol + n_first + j) * N2 + (m >> 1) + ((m & 1) ? Nc : 0)] = (float)d;
+        }
+        const float a2 = a * a;
+        sq = fmaxf(sq, a2 + __shfl_xor_sync(0xffffffffu, a2, 1));
       }
-      float mm = runmax;
-      for (int o = 16; o > 0; o >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, o));
-      if (lane == 0 && n_first < ncol) atomicMax(norm + qcur, (unsigned long long)__double_as_longlong((double)mm));
+      if (cols > 0) flush_norm(sq, norm + qcur, lane);
     }
   }
 
