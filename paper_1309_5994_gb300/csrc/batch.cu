@@ -92,6 +92,7 @@ __global__ void k_batch_check(const BatchCheck* __restrict__ chk, int n, int* __
       S.hist[S.sweeps % kStallSweeps] = upd;
       stop = (upd <= S.target && (upd < S.peak || upd == 0.0)) ||
              (S.since_best >= kStallSweeps && S.best < kStallDrop * S.peak) ||
+             (S.since_best >= kPlateauSweeps && S.best < kPlateauDrop * S.peak) ||
              (S.since_peak >= kStallSweeps && upd < kStallDrop * S.peak && upd > kFlatRatio * ago) ||
              S.sweeps >= C.max_sweeps;
     }

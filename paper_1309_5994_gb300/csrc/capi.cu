@@ -228,6 +228,7 @@ __global__ void k_series_check(unsigned long long* __restrict__ norm, const doub
   if (S->peak > abort_peak) out = SERIES_ABORTED;
   else if ((upd <= target && (upd < S->peak || upd == 0.0)) ||
            (S->since_best >= kStallSweeps && S->best < kStallDrop * S->peak) ||
+           (S->since_best >= kPlateauSweeps && S->best < kPlateauDrop * S->peak) ||
            (S->since_peak >= kStallSweeps && upd < kStallDrop * S->peak && upd > kFlatRatio * ago))
     out = SERIES_STOPPED;
   else if (sweep >= max_sweeps)
@@ -331,6 +332,7 @@ int inner_solve(dyson_ctx* c, int ncol, int gs, int precision, float* r32, float
     }
     if ((upd <= target && (upd < S.peak || upd == 0.0)) ||  // on the decay, not before the peak
         (S.since_best >= kStallSweeps && S.best < kStallDrop * S.peak) ||
+        (S.since_best >= kPlateauSweeps && S.best < kPlateauDrop * S.peak) ||
         (S.since_peak >= kStallSweeps && upd < kStallDrop * S.peak && upd > kFlatRatio * ago)) {
       S.run = 0;
       S.outcome = SERIES_STOPPED;

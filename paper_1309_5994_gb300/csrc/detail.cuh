@@ -52,6 +52,12 @@ constexpr int kStallSweeps = 4;
 // kFlatRatio over the last kStallSweeps sweeps (the decay after the peak is factorial:
 // a factor 3 to 10 over four sweeps until the floor).
 constexpr double kFlatRatio = 0.8;
+// Where the transient amplifies the rounding, the floor can lie above kStallDrop of the peak,
+// and both rules above would let the series run through its whole budget on it.  It also stops
+// after kPlateauSweeps sweeps without a new minimum once it has come below kPlateauDrop of the
+// peak: a series that still converges, however slowly, keeps making new minima.
+constexpr int kPlateauSweeps = 10;
+constexpr double kPlateauDrop = 1e-2;
 
 // Refinement that grows the residual: a residual above kRefineContract times the
 // previous one, kRefineStrikes times, means the series of App. C does not
