@@ -79,7 +79,13 @@ int ensure_cols(dyson_ctx* c, int ncol, int ng) {
     c->d_norm = nullptr;
     c->h_norm = nullptr;
     c->norm_cap = 0;
+    if (c->d_xscale) cudaFree(c->d_xscale);
+    if (c->d_rref) cudaFree(c->d_rref);
+    c->d_xscale = nullptr;
+    c->d_rref = nullptr;
     DY_CUDA(c, dalloc(&c->d_norm, 2 * (size_t)ng));
+    DY_CUDA(c, dalloc(&c->d_xscale, ng));
+    DY_CUDA(c, dalloc(&c->d_rref, ng));
     DY_CUDA(c, cudaMallocHost((void**)&c->h_norm, 2 * (size_t)ng * sizeof(unsigned long long)));
     c->norm_cap = ng;
   }
@@ -182,11 +188,13 @@ struct SeriesState {
 enum { SERIES_RUNNING = 0, SERIES_STOPPED, SERIES_EXHAUSTED, SERIES_ABORTED, SERIES_NOT_FINITE };
 
 // After one sweep of a captured series: the update max_q norm_q / rref_q (norm words
-// cleared for the next sweep) and the stopping rule of inner_solve's host loop, in the
-// same order.  One warp; returns at once once the series has stopped.
+// cleared for the next sweep), the next sweep's FP16 scales, and the stopping rule of
+// inner_solve's host loop, in the same order.  One warp; returns at once once the series has stopped.
 __global__ void k_series_check(unsigned long long* __restrict__ norm, const double* __restrict__ rref, int ng,
-                               int max_sweeps, double target, double abort_peak, SeriesState* __restrict__ S) {
+                               int max_sweeps, double target, double abort_peak, SeriesState* __restrict__ S,
+                               TcScale* __restrict__ xscale, float jbound) {
   if (!S->run) return;
+  for (int q = threadIdx.x; q < ng; q += 32) set_scale(xscale + q, __uint_as_float(xscale[q].ymax), jbound);
   double m = 0.0;
   int bad = 0;
   for (int q = threadIdx.x; q < ng; q += 32) {
@@ -284,6 +292,12 @@ int inner_solve(dyson_ctx* c, int ncol, int gs, int precision, float* r32, float
   S.best = std::numeric_limits<double>::infinity();
   S.run = 1;
   int rc;
+  if (precision == DYSON_PREC_TF32X3_F64REF && c->use_tc && tc_uses_fused(c)) {
+    // the series starts from d = r: its scales come from the reference norms max|r|
+    DY_CUDA(c, cudaMemcpyAsync(c->d_rref, rref.data(), (size_t)ng * sizeof(double), cudaMemcpyHostToDevice,
+                               c->stream));                // pageable: complete when the call returns
+    if ((rc = tc_seed_scale(c, ng, c->d_rref, 0.0))) return rc;
+  }
   while (S.run && S.sweeps < std::min(max_sweeps, eager_until)) {
     const int sweep = S.sweeps + 1;
     DY_CUDA(c, cudaMemsetAsync(c->d_norm, 0, (size_t)ng * sizeof(unsigned long long), c->stream));
@@ -349,19 +363,11 @@ int inner_solve(dyson_ctx* c, int ncol, int gs, int precision, float* r32, float
       DY_CUDA(c, cudaMalloc(&c->d_series, sizeof(SeriesState)));
       DY_CUDA(c, cudaMallocHost(&c->h_series, sizeof(SeriesState)));
     }
-    if (c->rref_cap < ng) {
-      if (c->d_rref) cudaFree(c->d_rref);
-      c->d_rref = nullptr;
-      c->rref_cap = 0;
-      DY_CUDA(c, cudaMalloc(&c->d_rref, (size_t)ng * sizeof(double)));
-      c->rref_cap = ng;
-    }
     SeriesState* hS = static_cast<SeriesState*>(c->h_series);
     SeriesState* dS = static_cast<SeriesState*>(c->d_series);
     *hS = S;
     if ((rc = tc_prepare_sweep(c, ncol))) return rc;     // nothing to allocate or encode while capturing
-    DY_CUDA(c, cudaMemcpyAsync(c->d_rref, rref.data(), (size_t)ng * sizeof(double), cudaMemcpyHostToDevice,
-                               c->stream));                // pageable: complete when the call returns
+    if ((rc = tc_set_scale(c, ng))) return rc;
     DY_CUDA(c, cudaMemcpyAsync(dS, hS, sizeof(SeriesState), cudaMemcpyHostToDevice, c->stream));
     DY_CUDA(c, cudaMemsetAsync(c->d_norm, 0, (size_t)ng * sizeof(unsigned long long), c->stream));
     const int64_t launches0 = c->launches;
@@ -379,7 +385,8 @@ int inner_solve(dyson_ctx* c, int ncol, int gs, int precision, float* r32, float
     for (int k = 0; k < Sg && cap_rc == DYSON_OK; ++k) {
       cap_rc = tc_sweep(c, ncol, gs, r32, k % 2 ? db : da, k % 2 ? da : db, TC_GATHER | TC_GEMM, act, 0, rform);
       if (cap_rc == DYSON_OK)
-        k_series_check<<<1, 32, 0, c->stream>>>(c->d_norm, c->d_rref, ng, max_sweeps, target, abort_peak, dS);
+        k_series_check<<<1, 32, 0, c->stream>>>(c->d_norm, c->d_rref, ng, max_sweeps, target, abort_peak, dS,
+                                                   c->d_xscale, tc_jbound(c));
     }
     c->sweep_run = nullptr;
     c->sweep_count = nullptr;
@@ -446,10 +453,14 @@ int inner_solve(dyson_ctx* c, int ncol, int gs, int precision, float* r32, float
   return DYSON_OK;
 }
 
-// out = zero + K in: one FP32 sweep with a zero right-hand side (the GMRES matvec)
-int matvec_f32(dyson_ctx* c, int ncol, int gs, int precision, const float* zero, const float* in, float* out) {
+// out = zero + K in: one FP32 sweep with a zero right-hand side (the GMRES matvec);
+// bound: an upper bound of |in|, or 0 to read it from the state
+int matvec_f32(dyson_ctx* c, int ncol, int gs, int precision, const float* zero, const float* in, float* out,
+               double bound) {
   int rc;
   if (precision == DYSON_PREC_TF32X3_F64REF && c->use_tc) {
+    if ((rc = bound > 0.0 ? tc_seed_scale(c, ncol / gs, nullptr, bound) : tc_seed_scale_scan(c, ncol, gs, in)))
+      return rc;
     if ((rc = tc_timed_sweep(c, ncol, gs, zero, in, out, nullptr, 0, TC_R_ZERO))) return rc;
   } else {
     KernelTimer t(c, DYSON_KERNEL_SWEEP_F32);
@@ -538,8 +549,8 @@ int solve_mixed(dyson_ctx* c, int ncol, int gs, int precision, double tol, int m
   // digit, it uses its whole sweep budget, or the refined residual grows.
   bool gmres = c->inner_solver == DYSON_INNER_GMRES;
   const bool may_switch = c->inner_solver == DYSON_INNER_AUTO;
-  const MatvecFn mv = [&](const float* zero, const float* in, float* out) {
-    return matvec_f32(c, ncol, gs, precision, zero, in, out);
+  const MatvecFn mv = [&](const float* zero, const float* in, float* out, double bound) {
+    return matvec_f32(c, ncol, gs, precision, zero, in, out, bound);
   };
   for (int ref = 0; ref < c->max_refinements; ++ref) {
     float* d = nullptr;
@@ -680,6 +691,7 @@ int dyson_init(dyson_ctx** out, const dyson_lattice* L, const dyson_contour* C, 
       delete c;
       return fail_noctx(DYSON_ERR_INVALID_ARG, "J table holds a non-finite value");
     }
+  for (double v : c->J) c->j_max = std::max(c->j_max, (float)(std::fabs(v) * 1.000001));
   c->j_uniform = true;
   for (int b = 1; b < c->Nb && c->j_uniform; ++b)
     c->j_uniform = std::equal(c->J.begin() + (size_t)b * c->Nt, c->J.begin() + (size_t)(b + 1) * c->Nt, c->J.begin());
@@ -734,7 +746,7 @@ int dyson_build_sigma(dyson_ctx* c) {
   DY_CUDA(c, cudaGetLastError());
   DY_CUDA(c, cudaStreamSynchronize(c->stream));
   c->sigma_built = true;
-  c->lam32_built = c->lam_split_built = false;
+  c->lam32_built = c->lam_split_built = c->lam16_built = false;
   oz_invalidate(c);
   oz64_invalidate(c);
   se_invalidate(c);                                      // Sigma = 0: Lambda is the atomic G0 again
@@ -767,7 +779,7 @@ int prepare_oz64(dyson_ctx* c) {
   return rc == DYSON_ERR_OOM ? DYSON_OK : rc;
 }
 
-int prepare_tables(dyson_ctx* c, int precision) {
+int prepare_tables(dyson_ctx* c, int precision, bool unfused) {
   c->use_tc = c->use_oz = c->use_oz64 = false;
   if (precision == DYSON_PREC_F64) return prepare_oz64(c);
   const bool tc = c->tc_enabled && tc_supported(c, c->Nc);
@@ -777,7 +789,17 @@ int prepare_tables(dyson_ctx* c, int precision) {
     c->launches += 1;
     c->lam32_built = true;
   }
-  if (tc && !c->lam_split_built) {
+  if (tc && tc_uses_fused(c) && !c->lam16_built) {
+    const size_t n = (size_t)c->Nr * 4 * c->Nc * c->Nc;
+    if (!c->d_lam16_hi) DY_CUDA(c, dalloc(&c->d_lam16_hi, n));
+    if (!c->d_lam16_lo) DY_CUDA(c, dalloc(&c->d_lam16_lo, n));
+    if (!c->d_a_down) DY_CUDA(c, dalloc(&c->d_a_down, (size_t)c->Nr * 2 * c->Nc));
+    launch_lam_split16(c->d_lam, c->Nr, c->Nt, c->Nm, c->dt, c->beta, c->d_lam16_hi, c->d_lam16_lo, c->d_a_down,
+                       c->stream);
+    c->launches += 1;
+    c->lam16_built = true;
+  }
+  if (tc && (unfused || !tc_uses_fused(c)) && !c->lam_split_built) {
     size_t n = (size_t)c->Nr * 4 * c->Nc * c->Nc;
     if (!c->d_lam_hi) DY_CUDA(c, dalloc(&c->d_lam_hi, n));
     if (!c->d_lam_lo) DY_CUDA(c, dalloc(&c->d_lam_lo, n));
@@ -1108,7 +1130,7 @@ int dyson_transpose_sigma(dyson_ctx* c) {
   DY_CUDA(c, cudaGetLastError());
   DY_CUDA(c, cudaStreamSynchronize(c->stream));
   c->sigma_transposed = !c->sigma_transposed;
-  c->lam32_built = c->lam_split_built = false;
+  c->lam32_built = c->lam_split_built = c->lam16_built = false;
   oz_invalidate(c);
   oz64_invalidate(c);
   return DYSON_OK;
@@ -1209,7 +1231,8 @@ void dyson_destroy(dyson_ctx* c) {
   if (c->d_sym_perm) cudaFree(c->d_sym_perm);
   void* ptrs[] = {c->dU, c->dJ, c->d_nbr, c->d_nbond, c->d_eps, c->d_phase, c->d_lam, c->d_JW, c->d_Jz,
                   c->d_lam32, c->d_lam_hi, c->d_lam_lo, c->d_obs, c->work, c->d_src_site, c->d_src_time,
-                  c->d_norm, c->adj, c->d_act, c->d_series, c->d_rref};
+                  c->d_norm, c->adj, c->d_act, c->d_series, c->d_rref, c->d_xscale, c->d_lam16_hi,
+                  c->d_lam16_lo, c->d_a_down};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (c->h_norm) cudaFreeHost(c->h_norm);

@@ -1,6 +1,7 @@
 // Internal declarations shared by the translation units of the Dyson library.
 #pragma once
 
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -52,6 +53,11 @@ void launch_lam_c64(const double2* lam, int Nr, int Nt, int Nm, double dt, doubl
 void launch_lam_emb_split(const double2* lam, int Nr, int Nt, int Nm, double dt, double beta,
                           float* hi, float* lo, cudaStream_t s);
 
+// The same embedding as FP16 hi + lo, each row scaled by a power of two to a largest entry in
+// [2^14, 2^15); down [Nr][2Nc]: the inverse powers.
+void launch_lam_split16(const double2* lam, int Nr, int Nt, int Nm, double dt, double beta, __half* hi, __half* lo,
+                        float* down, cudaStream_t s);
+
 // transpose every Nc x Nc block of lam in place
 void launch_transpose_blocks(double2* lam, int Nr, int Nc, cudaStream_t s);
 
@@ -93,6 +99,26 @@ void launch_export(const double2* G, int Nr, int Nc, int nq, double2* out, cudaS
 // context
 // ---------------------------------------------------------------------------
 
+// Scale of one column group's X in the fused tensor-core sweep (FP16 operands): the power of two
+// applied, its inverse, and the bits of max|d_out| that the sweep leaves for the next one's.
+struct TcScale {
+  float up, down;
+  unsigned int ymax;
+};
+
+// Powers of two of the FP16 operands.  A group's X is multiplied by up = 2^u before it is split into
+// FP16 hi + lo, with 4 max|J| max|d| up in (2^14, 2^15], so that no sum of four neighbours
+// overflows; dmax: max|d| of the state the sweep reads, jbound = 4 max|J|.  (No finite bound: 1, and
+// infinities or NaNs of d reach the result as they are.)
+__device__ __forceinline__ void set_scale(TcScale* s, float dmax, float jbound) {
+  const float b = dmax * jbound;
+  int u = 0;
+  if (b > 0.f && b < __int_as_float(0x7f800000)) u = max(-100, min(100, 14 - ilogbf(b)));
+  s->up = ldexpf(1.f, u);
+  s->down = ldexpf(1.f, -u);
+  s->ymax = 0u;
+}
+
 struct dyson_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
@@ -108,8 +134,7 @@ struct dyson_ctx {
   cudaStream_t cap_stream = nullptr; // private stream the series graph is captured on (lazy)
   void* d_series = nullptr;          // device stopping state of the captured series
   void* h_series = nullptr;          // pinned mirror
-  double* d_rref = nullptr;          // reference norms of the current inner solve
-  int rref_cap = 0;
+  double* d_rref = nullptr;          // [norm_cap] reference norms of the current inner solve
 
   // device tables
   double* dU = nullptr;              // [Nr][Nt]
@@ -124,6 +149,12 @@ struct dyson_ctx {
   float2* d_lam32 = nullptr;         // [Nr][Nc][Nc] (lazy)
   float* d_lam_hi = nullptr;         // [Nr][2Nc][2Nc] (lazy)
   float* d_lam_lo = nullptr;
+  __half* d_lam16_hi = nullptr;      // [Nr][2Nc][2Nc] FP16 halves of the scaled embedding (fused sweep; lazy)
+  __half* d_lam16_lo = nullptr;
+  float* d_a_down = nullptr;         // [Nr][2Nc] powers of two that undo the rows' scales
+  bool lam16_built = false;
+  float j_max = 0.f;                 // max |J_b(t_k)|
+  TcScale* d_xscale = nullptr;       // [norm_cap] scales of the FP16 X per column group
   double* d_obs = nullptr;           // [3][Nr][Nt]
   bool sigma_built = false;
   bool sigma_transposed = false;     // every Lambda_i block transposed: solves give rows of G

@@ -5,8 +5,8 @@
 #include "common.cuh"
 
 // out = zero + K in over the FP32 planar chunk state (one series sweep with a zero
-// right-hand side); returns a DYSON_ERR_* code
-using MatvecFn = std::function<int(const float* zero, const float* in, float* out)>;
+// right-hand side); bound: an upper bound of |in|, or 0 for none known; returns a DYSON_ERR_* code
+using MatvecFn = std::function<int(const float* zero, const float* in, float* out, double bound)>;
 
 // Restart length that fits the free device memory for ncol columns (0: none fits).
 int gmres_restart_length(dyson_ctx* c, int ncol);

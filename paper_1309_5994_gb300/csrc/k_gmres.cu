@@ -452,7 +452,7 @@ int gmres_inner_solve(dyson_ctx* c, int ncol, const float* r, float* x, int max_
   double rel = INFINITY;
   while (its < max_iters) {
     // residue of the iterate: z0 = r - (I - K) x = r - x + K x
-    if ((rc = matvec(st->zero, x, st->u))) return rc;
+    if ((rc = matvec(st->zero, x, st->u, 0.0))) return rc;
     rep->sweeps += 1;
     rep->gemm_flops += sweep_flops(c, ncol);
     k_gm_lin3<<<lin_grid, 256, 0, s>>>(r, x, st->u, st->w, n4);
@@ -465,8 +465,8 @@ int gmres_inner_solve(dyson_ctx* c, int ncol, const float* r, float* x, int max_
     for (int j = 0; j < m && its < max_iters; ++j) {
       ++its;
       float* qj = st->Q + (size_t)j * vsz;
-      // u = K q_j, so w = (I - K) q_j = q_j - u
-      if ((rc = matvec(st->zero, qj, st->u))) return rc;
+      // u = K q_j, so w = (I - K) q_j = q_j - u (|q_j| <= 1: every column has unit length)
+      if ((rc = matvec(st->zero, qj, st->u, 1.0001))) return rc;
       rep->sweeps += 1;
       rep->gemm_flops += sweep_flops(c, ncol);
       // classical Gram-Schmidt: h = <Q, q_j - u>, w = q_j - u - Q h; then, for the

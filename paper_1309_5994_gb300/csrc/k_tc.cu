@@ -25,6 +25,7 @@
 // Every mbarrier wait is bounded (2 s of %globaltimer); on expiry the CTA
 // raises an error flag, lets in-flight copies and MMAs land, frees TMEM and
 // exits, and the host returns DYSON_ERR_TIMEOUT.
+#include <cuda_fp16.h>
 #include <cudaTypedefs.h>
 
 #include <algorithm>
@@ -70,7 +71,11 @@ struct TcState {
   int xh_ncol = -1;
   const float* xh_ptr = nullptr;
   int pair_clusters = -1;
-  // fused gather + GEMM (k_tc_fused<GT>): co-resident clusters per GT (-1: not yet asked)
+  // fused gather + GEMM (k_tc_fused<GT>): maps of the FP16 Lambda halves, co-resident clusters
+  // per GT (-1: not yet asked)
+  CUtensorMap h_hi, h_lo;
+  const void* h_hi_ptr = nullptr;
+  const void* h_lo_ptr = nullptr;
   int fused_clusters[2] = {-1, -1};
   // one-entry instance table of the single-context sweep (pinned host copy and device copy)
   TcInst* h_inst = nullptr;
@@ -204,6 +209,15 @@ __global__ __launch_bounds__(256) void k_tc_gather(const TcInst* __restrict__ ta
   }
 }
 
+// (a, b) = hi + lo in FP16, packed with a in the low halves; the difference a - hi is exact in FP32
+__device__ __forceinline__ void split_f16(float a, float b, unsigned int& hi, unsigned int& lo) {
+  const __half2 h = __floats2half2_rn(a, b);
+  const float2 f = __half22float2(h);
+  const __half2 l = __floats2half2_rn(a - f.x, b - f.y);
+  hi = *reinterpret_cast<const unsigned int*>(&h);
+  lo = *reinterpret_cast<const unsigned int*>(&l);
+}
+
 // split an fp32 tile (float4 granules e = tt, tt + 128, ...) into TF32 hi in place and lo at x + bytes
 template <int BYTES>
 __device__ __forceinline__ void split_tile(uint8_t* x, int tt) {
@@ -221,18 +235,49 @@ __device__ __forceinline__ void split_tile(uint8_t* x, int tt) {
   }
 }
 
+__device__ __forceinline__ void fold_ymax(TcScale* s, float y, int lane) {
+  unsigned int u = __float_as_uint(y);                    // y >= 0 (fmaxf drops NaN: the norm reports it)
+  u = __reduce_max_sync(0xffffffffu, u);
+  if (lane == 0) atomicMax(&s->ymax, u);
+}
+
+// scale of the next sweep from the maxima that the last one (or a seed) left
+__global__ void k_tc_scale(TcScale* __restrict__ sc, int ng, float jbound) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q < ng) set_scale(sc + q, __uint_as_float(sc[q].ymax), jbound);
+}
+// seeds of the maxima: a bound common to all groups, or a bound per group
+__global__ void k_tc_seed(TcScale* __restrict__ sc, int ng, const double* __restrict__ ref, float bound) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  // (1 + 1e-6: an FP32 state may exceed an FP64 bound by its rounding)
+  if (q < ng) sc[q].ymax = __float_as_uint(ref ? (float)(ref[q] * 1.000001) : bound);
+}
+// seed by reading the state: one warp per (site, vector column)
+__global__ void __launch_bounds__(256) k_tc_seed_scan(const float* __restrict__ d, int Nr, int Nc, int ncol, int gs,
+                                                      TcScale* __restrict__ sc) {
+  const size_t w = (size_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+  const int lane = threadIdx.x & 31;
+  if (w >= (size_t)Nr * ncol) return;
+  const int n = (int)(w % ncol);
+  const float4* p = reinterpret_cast<const float4*>(d + w * 2 * Nc);
+  float m = 0.f;
+  for (int k = lane; k < Nc / 2; k += 32) {
+    const float4 v = p[k];
+    m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+  }
+  const unsigned int u = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+  if (lane == 0 && u > sc[n / gs].ymax) atomicMax(&sc[n / gs].ymax, u);
+}
+
 // epilogue of one warp's 32 accumulator lanes x BN columns (TMEM address tacc):
 // y = r + acc at planar row mg, columns n_first.., store y, and fold max|y - d_in|
 // into norm[] per group of gs columns (gs a multiple of 32)
-// (CH = 32 or 16 columns per tcgen05.ld; 16 keeps the register count of the 512-thread
-// fused kernel below its limit)
-// (RZERO: r is zero on this tile, its loads are skipped)
-template <int CH = 32, bool RZERO = false>
 __device__ __forceinline__ void epilogue_rows(uint32_t tacc, int mg, int n_first, int site, int ncol, int gs,
                                               size_t N2, const float* __restrict__ r, const float* __restrict__ din,
                                               float* __restrict__ dout, unsigned long long* __restrict__ norm,
                                               int lane) {
   using namespace ptx;
+  constexpr int CH = 32;                            // columns per tcgen05.ld
   int qcur = n_first / gs;
   float runmax = 0.f;
   for (int c = 0; c < BN / CH; ++c) {
@@ -252,11 +297,10 @@ __device__ __forceinline__ void epilogue_rows(uint32_t tacc, int mg, int n_first
     const size_t base = ((size_t)site * ncol + n0) * N2 + mg;
 #pragma unroll
     for (int j = 0; j < CH; ++j) {
-      rv[j] = RZERO ? 0.f : __ldcs(r + base + (size_t)j * N2);
+      rv[j] = __ldcs(r + base + (size_t)j * N2);
       dv[j] = __ldcs(din + base + (size_t)j * N2);
     }
-    if (CH == 32) tmem_ld32(tacc + (uint32_t)(c * CH), v);
-    else tmem_ld16(tacc + (uint32_t)(c * CH), v);
+    tmem_ld32(tacc + (uint32_t)(c * CH), v);
     tmem_wait_ld();
 #pragma unroll
     for (int j = 0; j < CH; ++j) {
@@ -681,19 +725,35 @@ __global__ void __launch_bounds__(THREADS, 1)
 // ---------------------------------------------------------------------------
 // Fused sweep on CTA pairs: the neighbour gather is the producer of the MMA's
 // B operand.  Eight warps per CTA read the four neighbour rows of d_in
-// (coalesced float4 loads, all sixteen of a k-block issued back to back and one
-// k-block ahead of their sums), scale them by J(k), sum, round the sum to TF32
+// (coalesced float4 loads, sixteen issued back to back and half a k-block
+// ahead of their sums), scale them by J(k), sum, split the sum into FP16
 // hi + lo and write both straight into the 128-byte-swizzled stage, so X never
 // exists in global memory and only Lambda hi/lo travel by TMA.  The epilogue
 // forms d_out = r + K d_in and the update norm max|d_out - d_in| as the unfused
 // sweeps do (GMRES matvecs use it with r = 0).
-// A tile is (site, 256-column tile, GT row groups of 256 rows):
-//   GT = 1  tiles also run over the 2Nc / 256 row groups (each group-tile
-//           gathers its own copy of X; the copies meet in L2); two TMEM
-//           accumulators, so a tile's epilogue overlaps the next tile's MMAs;
-//   GT = 2  one tile covers 512 rows (2Nc = 512 or a multiple): X is gathered
-//           once per (site, column tile), the A stage holds both groups, and
-//           the two accumulators fill TMEM, so the epilogue does not overlap.
+// Operands: FP16 has the 11 significant bits of TF32 at half the bytes and twice the MMA
+// rate; its range is made up by powers of two, one per row of Lambda W (2^14 <= max < 2^15)
+// and one per column group of X (set_scale), taken out again in the epilogue.  hi + lo keeps
+// 22 bits of every entry down to 2^-16 of the row's (group's) largest and 2^-39 of the
+// largest below that, under the FP32 accumulation's own rounding.
+// The kernel is bound by the traffic between L2 and the SMs (10 to 12 TB/s were the most seen), so
+// the two forms differ in what they read there.  Both have two accumulator sets of 256 TMEM
+// columns, so that a tile's epilogue overlaps the next tile's MMAs:
+//   <2>  a tile is (site, 128 vector columns, 256 contour points z): its two accumulators are the
+//        real and the imaginary rows of those points.  A k-block is 64 complex points; the tiles
+//        Re and Im of Lambda are loaded once and serve both halves of the embedding
+//        [[Re, -Im], [Im, Re]] (the minus sign is the MMA's negate bit), and X is gathered once
+//        per ceil(Nc / 256) tiles.  Two stages of 96 KB.  Nc >= 256.
+//   <1>  a tile is (site, 256 vector columns, 256 rows of the embedding); a k-block is 64 real
+//        values, three stages of 64 KB.  Nc = 128, where <2> would fill half of its rows.
+// Bytes from L2 per sweep at 16x16, Nc = 256, 4096 columns: X 8.6 GB, Lambda 4.3, epilogue 4.3
+// and 2.1 written (<1>: X 17.2, Lambda 4.3; with the embedding in 512-row tiles: X 8.6, Lambda 8.6).
+// Measured there: 2.10 ms per sweep, 9.1 TB/s from L2; 2.67 ms as <1> and 2.37 with the embedding in
+// 512-row tiles; 2.66 ms in 3xTF32 with the traffic of <1>.  Each gather step waits for one loaded
+// memory latency (about 2.3 us, 64 KB in flight per SM); fetching the next tile's neighbour rows
+// into L2 ahead adds requests and cost 25 %.
+// Error of one inner solve against the FP64 residual, 8x8 to 24x24, six contours: 0.45 to 0.95 of the
+// 3xTF32 form's in every case (fewer roundings: twice the products per MMA).
 // Sites are visited in bands of two lattice rows, column by column, so that
 // a site's neighbours are read while they are still in L2.
 // Warp roles (512 threads per CTA, both CTAs of the pair):
@@ -710,7 +770,10 @@ __global__ void __launch_bounds__(THREADS, 1)
 constexpr int F_THREADS = 512;
 constexpr int F_PROD_W0 = 4, F_PROD_WARPS = 8;
 constexpr int F_EPI_W0 = 12;
-constexpr int F_A_GROUP = 2 * A_TILE;                   // Lambda hi + lo, one row group, this CTA's 128 rows
+constexpr int F_BK = 64;                                // k-block: 64 FP16 = one 128-byte swizzle row
+static_assert(A_TILE == BM * F_BK * 2 && PX_TILE == (BN / 2) * F_BK * 2, "FP16 tiles of 64 fill the TF32 tiles of 32");
+constexpr int F_A_GROUP = 2 * A_TILE;                   // Lambda hi + lo, this CTA's 128 rows of one accumulator
+constexpr uint32_t F_NEGATE_A = 1u << 13;               // instruction descriptor: D += (-A) B
 constexpr int F_SITE_BAND = 2;                          // lattice rows per band of the site order
 constexpr int F_RELAY_W = 2;                            // warp 2: relays "Lambda landed" to the even CTA
 // registers per thread of each warpgroup once the roles split: the producers keep sixteen
@@ -724,11 +787,17 @@ static_assert(F_PROD_W0 == 4 && F_PROD_WARPS == 8 && F_EPI_W0 == 12 && F_THREADS
               "the register split assumes warpgroups {0-3: control, 4-11: producers, 12-15: epilogue}");
 template <int GT>
 struct FusedCfg {
-  static constexpr int STAGE = GT * F_A_GROUP + 2 * PX_TILE;
+  static constexpr int NB = 256 / GT;                   // vector columns of a tile
+  static constexpr int X_TILE = (NB / 2) * F_BK * 2;    // one CTA's half of X hi (or lo)
+  // GT = 2: Re hi, Re lo, Im hi, Im lo | Xr hi, Xr lo, Xi hi, Xi lo;  GT = 1: hi, lo | X hi, X lo
+  static constexpr int STAGE = GT * F_A_GROUP + GT * 2 * X_TILE;
   static constexpr int STAGES = GT == 1 ? 3 : 2;
   static constexpr int SMEM = STAGES * STAGE + 1024;
-  static constexpr int NBUF = 2 / GT;                   // accumulator sets of GT x 256 columns
-  static_assert(NBUF * GT * BN <= 512, "TMEM holds 512 columns");
+  static constexpr int NBUF = 2;                        // accumulator sets of GT x NB columns
+  // kind::f16, D = F32, A = B = F16, K-major, M = 256, N = NB
+  static constexpr uint32_t IDESC = (1u << 4) | ((uint32_t)(NB >> 3) << 17) | ((uint32_t)(PM >> 4) << 24);
+  static_assert(NBUF * GT * NB <= 512, "TMEM holds 512 columns");
+  static_assert(TC_TILE_COLS % NB == 0, "a tile lies in one column tile of the support table");
 };
 
 // site of visit index v: bands of F_SITE_BAND lattice rows, walked column by column
@@ -744,15 +813,81 @@ struct FTile {
   int site, nt, gt;
   bool active;
 };
+// (act has one entry per site and TC_TILE_COLS columns, nact of them a site)
+template <int NB>
 __device__ __forceinline__ FTile fused_tile(int tile, int NGT, int NT, int Lx, int Ly, const int* __restrict__ act,
-                                            int sweep) {
+                                            int nact, int sweep) {
   FTile T;
   T.gt = tile % NGT;
   T.nt = (tile / NGT) % NT;
   T.site = band_site(tile / (NGT * NT), Lx, Ly);
-  T.active = !(act && act[T.site * NT + T.nt] > sweep);
+  T.active = !(act && act[T.site * nact + T.nt / (TC_TILE_COLS / NB)] > sweep);
   return T;
 }
+
+// Epilogue of one warp's 32 accumulator lanes: GT accumulators x NB columns in chunks of 16 columns.  The
+// accumulators hold 2^(a + x) times the product, the row's and the column group's powers of two:
+// y = r + acc adown sc[q].down; y is stored, max|y - d_in| folded into norm[] and max|y| into
+// sc[].ymax (for the next sweep's scale) per group of gs columns.  The loads of r and d_in run one
+// chunk ahead, the first ones before the accumulators are complete: a chunk costs no DRAM latency.
+// RZERO: r is zero on this tile.
+template <int GT, bool RZERO>
+struct FusedEpilogue {
+  static constexpr int NB = FusedCfg<GT>::NB, CH = 16, PER = NB / CH, CHUNKS = GT * PER;
+  const float* __restrict__ r;
+  const float* __restrict__ din;
+  float* __restrict__ dout;
+  int n_first, ncol, N2, row_gap;
+  size_t base0;                                          // element of (site, column n_first, this lane's first row)
+  float rv[2][CH], dv[2][CH];
+
+  __device__ __forceinline__ size_t at(int e) const {
+    return base0 + (size_t)(e % PER) * CH * N2 + (size_t)(e / PER) * row_gap;
+  }
+  template <int B>
+  __device__ __forceinline__ void load(int e) {
+    if (n_first + (e % PER) * CH >= ncol) return;        // warp-uniform (ncol is a multiple of 32)
+    const size_t o = at(e);
+#pragma unroll
+    for (int j = 0; j < CH; ++j) {
+      if (!RZERO) rv[B][j] = __ldcs(r + o + (size_t)j * N2);
+      dv[B][j] = __ldcs(din + o + (size_t)j * N2);
+    }
+  }
+  float runmax = 0.f, ymax = 0.f, down = 0.f;
+  int qcur = -1;
+  __device__ __forceinline__ void flush(unsigned long long* norm, TcScale* sc, int lane) {
+    const unsigned int m = __reduce_max_sync(0xffffffffu, __float_as_uint(runmax));
+    if (lane == 0) atomicMax(norm + qcur, nonneg_bits(__uint_as_float(m)));
+    fold_ymax(sc + qcur, ymax, lane);
+    runmax = ymax = 0.f;
+  }
+  template <int B>
+  __device__ __forceinline__ void chunk(int e, uint32_t tacc, float adown, int gs, unsigned long long* norm,
+                                        TcScale* sc, int lane) {
+    const int n0 = n_first + (e % PER) * CH;
+    if (n0 >= ncol) return;
+    const int q = n0 / gs;
+    if (q != qcur) {
+      if (qcur >= 0) flush(norm, sc, lane);
+      qcur = q;
+      down = adown * sc[q].down;
+    }
+    uint32_t v[CH];
+    ptx::tmem_ld16(tacc + (uint32_t)(e * CH), v);
+    ptx::tmem_wait_ld();
+    const size_t o = at(e);
+#pragma unroll
+    for (int j = 0; j < CH; ++j) {
+      const float y = RZERO ? __uint_as_float(v[j]) * down : fmaf(__uint_as_float(v[j]), down, rv[B][j]);
+      float d = fabsf(y - dv[B][j]);
+      d = (d == d) ? d : __int_as_float(0x7f800000);
+      __stcs(dout + o + (size_t)j * N2, y);
+      runmax = fmaxf(runmax, d);
+      ymax = fmaxf(ymax, fabsf(y));
+    }
+  }
+};
 
 template <int GT>
 __global__ void __launch_bounds__(F_THREADS, 1)
@@ -762,7 +897,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
                const int* __restrict__ nbond, int Lx,
                int Ly, int Nc, int ncol, int gs, unsigned long long* __restrict__ norm, int* __restrict__ err,
                const int* __restrict__ act, int sweep, const int* __restrict__ run,
-               const int* __restrict__ sweeps_done) {
+               const int* __restrict__ sweeps_done, const float* __restrict__ adown, TcScale* __restrict__ sc) {
   using namespace ptx;
   using Cfg = FusedCfg<GT>;
   // a sweep of a captured graph after the series has stopped: nothing to do (every CTA
@@ -781,9 +916,12 @@ __global__ void __launch_bounds__(F_THREADS, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
-  const int N2 = 2 * Nc, KB = N2 / BK;
-  const int NGT = N2 / (PM * GT);
-  const int NT = (ncol + BN - 1) / BN;
+  constexpr int NB = Cfg::NB, X_TILE = Cfg::X_TILE;
+  const int N2 = 2 * Nc;
+  const int KB = (GT == 2 ? Nc : N2) / F_BK;            // k-blocks of 64 complex points or 64 real values
+  const int NGT = GT == 2 ? (Nc + PM - 1) / PM : N2 / PM;
+  const int row_gap = GT == 2 ? Nc : 0;                 // rows of the two accumulators: z and Nc + z
+  const int NT = (ncol + NB - 1) / NB, nact = (ncol + TC_TILE_COLS - 1) / TC_TILE_COLS;
   const int tiles = Lx * Ly * NT * NGT;
 
   if (threadIdx.x == 0) {
@@ -820,15 +958,8 @@ __global__ void __launch_bounds__(F_THREADS, 1)
         int g = 0;
         bool ok = true;
         for (int tile = pair; tile < tiles && ok; tile += npairs) {
-          const FTile T = fused_tile(tile, NGT, NT, Lx, Ly, act, sweep);
+          const FTile T = fused_tile<NB>(tile, NGT, NT, Lx, Ly, act, nact, sweep);
           if (!T.active) continue;
-          int t2 = tile + npairs;
-          FTile N;
-          N.active = false;
-          for (; t2 < tiles; t2 += npairs) {
-            N = fused_tile(t2, NGT, NT, Lx, Ly, act, sweep);
-            if (N.active) break;
-          }
           for (int kb = 0; kb < KB; ++kb, ++g) {
             const int s = g % STAGES;
             if (g >= STAGES && !mbar_wait(&empty[s], ((g / STAGES) - 1) & 1, abort_p)) {
@@ -839,20 +970,9 @@ __global__ void __launch_bounds__(F_THREADS, 1)
             mbar_expect_tx(&full_a[s], GT * F_A_GROUP);
 #pragma unroll
             for (int gi = 0; gi < GT; ++gi) {
-              const int row0 = (T.gt * GT + gi) * PM + (int)rank * BM;
-              tma_load_3d(st + gi * F_A_GROUP, &map_ahi, &full_a[s], kb * BK, row0, T.site);
-              tma_load_3d(st + gi * F_A_GROUP + A_TILE, &map_alo, &full_a[s], kb * BK, row0, T.site);
-            }
-            const int ahead = kb + PREFETCH;
-            const FTile* P = ahead < KB ? &T : (N.active && ahead - KB < KB ? &N : nullptr);
-            if (P) {
-              const int k2 = ahead < KB ? ahead : ahead - KB;
-#pragma unroll
-              for (int gi = 0; gi < GT; ++gi) {
-                const int row0 = (P->gt * GT + gi) * PM + (int)rank * BM;
-                tma_prefetch_3d(&map_ahi, k2 * BK, row0, P->site);
-                tma_prefetch_3d(&map_alo, k2 * BK, row0, P->site);
-              }
+              const int row0 = T.gt * PM + (int)rank * BM + gi * row_gap;
+              tma_load_3d(st + gi * F_A_GROUP, &map_ahi, &full_a[s], kb * F_BK, row0, T.site);
+              tma_load_3d(st + gi * F_A_GROUP + A_TILE, &map_alo, &full_a[s], kb * F_BK, row0, T.site);
             }
           }
         }
@@ -865,7 +985,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
         int g = 0, t = 0;
         bool ok = true, any = false;
         for (int tile = pair; tile < tiles && ok; tile += npairs) {
-          const FTile T = fused_tile(tile, NGT, NT, Lx, Ly, act, sweep);
+          const FTile T = fused_tile<NB>(tile, NGT, NT, Lx, Ly, act, nact, sweep);
           if (!T.active) continue;
           const int buf = t % NBUF;
           if (t >= NBUF && !mbar_wait_cluster(&acc_empty[buf], ((t / NBUF) - 1) & 1, abort_p)) break;
@@ -879,19 +999,25 @@ __global__ void __launch_bounds__(F_THREADS, 1)
             }
             tc_fence_after();
             const uint32_t st = smem_u32(stage_ptr(s));
-            const uint32_t x_hi = st + GT * F_A_GROUP, x_lo = x_hi + PX_TILE;
+            const uint32_t xb = st + GT * F_A_GROUP;
 #pragma unroll
-            for (int k8 = 0; k8 < BK / 8; ++k8) {
-              const uint32_t off = k8 * 32;
-              const uint64_t dxh = sdesc_sw128(x_hi + off), dxl = sdesc_sw128(x_lo + off);
-#pragma unroll
-              for (int gi = 0; gi < GT; ++gi) {
-                const uint32_t a_hi = st + gi * F_A_GROUP, a_lo = a_hi + A_TILE;
-                const uint64_t dah = sdesc_sw128(a_hi + off), dal = sdesc_sw128(a_lo + off);
-                const uint32_t dacc = tmem + (uint32_t)((buf * GT + gi) * BN);
-                mma_pair_tf32(dacc, dah, dxh, P_IDESC, (kb | k8) ? 1u : 0u);
-                mma_pair_tf32(dacc, dah, dxl, P_IDESC, 1u);
-                mma_pair_tf32(dacc, dal, dxh, P_IDESC, 1u);
+            for (int k16 = 0; k16 < F_BK / 16; ++k16) {
+              const uint32_t off = k16 * 32;
+              const uint32_t first = (kb | k16) ? 1u : 0u;
+              auto three = [&](uint32_t dacc, uint32_t a, uint32_t x, uint32_t idesc, uint32_t accumulate) {
+                const uint64_t ah = sdesc_sw128(a + off), al = sdesc_sw128(a + A_TILE + off);
+                const uint64_t xh = sdesc_sw128(x + off), xl = sdesc_sw128(x + X_TILE + off);
+                mma_pair_f16(dacc, ah, xh, idesc, accumulate);
+                mma_pair_f16(dacc, ah, xl, idesc, 1u);
+                mma_pair_f16(dacc, al, xh, idesc, 1u);
+              };
+              const uint32_t d0 = tmem + (uint32_t)(buf * GT * NB);
+              three(d0, st, xb, Cfg::IDESC, first);                                       // Re Xr (or A X)
+              if constexpr (GT == 2) {
+                const uint32_t im = st + F_A_GROUP, xi = xb + 2 * X_TILE, d1 = d0 + NB;
+                three(d0, im, xi, Cfg::IDESC | F_NEGATE_A, 1u);                             // - Im Xi
+                three(d1, im, xb, Cfg::IDESC, first);                                     // Im Xr
+                three(d1, st, xi, Cfg::IDESC, 1u);                                        // Re Xi
               }
             }
             mma_commit_pair_mc(&empty[s], 0x3);
@@ -911,7 +1037,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
         int g = 0;
         bool ok = true;
         for (int tile = pair; tile < tiles && ok; tile += npairs) {
-          const FTile T = fused_tile(tile, NGT, NT, Lx, Ly, act, sweep);
+          const FTile T = fused_tile<NB>(tile, NGT, NT, Lx, Ly, act, nact, sweep);
           if (!T.active) continue;
           for (int kb = 0; kb < KB; ++kb, ++g) {
             const int s = g % STAGES;
@@ -927,14 +1053,17 @@ __global__ void __launch_bounds__(F_THREADS, 1)
   } else if (warp < F_EPI_W0) {
     reg_budget<F_REG_PROD, F_REGS_AT_LAUNCH>();
     // ---------------- gather producers (both CTAs) ----------------
-    // thread pt: 16-byte chunk j of the k-block row (k = 32 kb + 4 j .. + 3) for the
-    // tile columns c0 + 32 i, i = 0..3, of this CTA's half
+    // thread pt: the float4 groups k = 4 j .. + 3 and 32 + 4 j .. + 3 of 64 values (so that eight
+    // lanes read 128 contiguous bytes) for the tile columns c0 + 32 i, i < NB / 64, of this CTA's half.
+    // c0: the two columns of a half warp differ in bit 2, so that their 8-byte stores, which the
+    // 128-byte swizzle places in one 64-byte half of a row each, meet in different banks.
     const int pt = threadIdx.x - F_PROD_W0 * 32;
-    const int j = pt & 7, c0 = pt >> 3;
+    const int j = pt & 7, r4 = (pt >> 3) & 3, wv = pt >> 5;
+    const int c0 = (wv >> 1) * 8 + (wv & 1) * 2 + (r4 >> 1) + (r4 & 1) * 4;
     int g = 0;
     int ok = 1;
     for (int tile = pair; tile < tiles && ok; tile += npairs) {
-      const FTile T = fused_tile(tile, NGT, NT, Lx, Ly, act, sweep);
+      const FTile T = fused_tile<NB>(tile, NGT, NT, Lx, Ly, act, nact, sweep);
       if (!T.active) continue;
       int nb[4], bd[4];
 #pragma unroll
@@ -942,66 +1071,98 @@ __global__ void __launch_bounds__(F_THREADS, 1)
         nb[q] = __ldg(nbr + T.site * 4 + q);
         bd[q] = nb[q] >= 0 ? __ldg(nbond + T.site * 4 + q) : 0;
       }
-      const int col0 = T.nt * BN + (int)rank * (BN / 2);
+      const int col0 = T.nt * NB + (int)rank * (NB / 2);
       // this thread's columns col0 + c0 + 32 i, i < ni, lie before the end
-      const int ni = max(0, min(4, (ncol - col0 - c0 + 31) / 32));
+      const int ni = max(0, min(NB / 64, (ncol - col0 - c0 + 31) / 32));
+      float up[NB / 64];
+#pragma unroll
+      for (int i = 0; i < NB / 64; ++i) up[i] = i < ni ? __ldg(&sc[(col0 + c0 + 32 * i) / gs].up) : 0.f;
       // row of neighbour q at the first column (a valid address also where the neighbour is missing)
       const float* nbp[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q)
         nbp[q] = din + (nb[q] >= 0 && ni > 0 ? ((size_t)nb[q] * ncol + col0 + c0) * N2 : 0) + 4 * j;
       const size_t cstride = (size_t)32 * N2;            // 32 columns further
-      // sixteen neighbour loads and four hopping loads per k-block, issued back to back
-      // (no load behind a branch) one k-block ahead of their sums, so that their latency
-      // overlaps the previous k-block's stage wait and shared-memory stores
-      float4 v[4][4], jv[4];
-      auto issue = [&](int kb) {
-        const int k = kb * BK + 4 * j;
-        const int kz = k < Nc ? k : k - Nc;
+      // A k-block is gathered in two steps of two columns: GT = 2, the real, then the imaginary parts
+      // of both columns; GT = 1, two columns after the other two.  The sixteen neighbour loads of a
+      // step are issued back to back (no load behind a branch) one step ahead of their sums, so that
+      // their latency overlaps the previous step's sums, stores and stage wait.
+      float4 v[4][2][2], jv[4][2];
+      auto issue = [&](int kb, int h) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          jv[q] = __ldg(reinterpret_cast<const float4*>(Jz + (size_t)bd[q] * Nc + kz));
+        for (int q = 0; q < 4; ++q)
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const bool ok_qi = nb[q] >= 0 && i < ni;
-            v[q][i] = __ldg(reinterpret_cast<const float4*>(ok_qi ? nbp[q] + i * cstride + kb * BK : nbp[q]));
+          for (int i = 0; i < 2; ++i) {
+            const int ci = GT == 2 ? i : 2 * h + i;
+            const bool ok_qi = nb[q] >= 0 && ci < ni;
+            const float* p = ok_qi ? nbp[q] + ci * cstride + kb * F_BK + (GT == 2 ? h * Nc : 0) : nbp[q];
+            v[q][i][0] = __ldg(reinterpret_cast<const float4*>(p));
+            v[q][i][1] = __ldg(reinterpret_cast<const float4*>(p + 32));
+          }
+      };
+      auto issue_j = [&](int kb) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int k = kb * F_BK + 32 * u + 4 * j;
+          const int kz = k < Nc ? k : k - Nc;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            jv[q][u] = __ldg(reinterpret_cast<const float4*>(Jz + (size_t)bd[q] * Nc + kz));
+            if (nb[q] < 0) jv[q][u] = make_float4(0.f, 0.f, 0.f, 0.f);
           }
         }
       };
-      issue(0);
+      issue(0, 0);
+      issue_j(0);
       for (int kb = 0; kb < KB; ++kb, ++g) {
         const int s = g % STAGES;
-        float4 acc[4];
+        uint8_t* xs = stage_ptr(s) + GT * F_A_GROUP;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int h = 0; h < 2; ++h) {
+          float4 acc[2][2];
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            if (nb[q] >= 0 && i < ni) {
-              acc[i].x = fmaf(jv[q].x, v[q][i].x, acc[i].x);
-              acc[i].y = fmaf(jv[q].y, v[q][i].y, acc[i].y);
-              acc[i].z = fmaf(jv[q].z, v[q][i].z, acc[i].z);
-              acc[i].w = fmaf(jv[q].w, v[q][i].w, acc[i].w);
+          for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                if (nb[q] >= 0 && (GT == 2 ? i : 2 * h + i) < ni) {
+                  a.x = fmaf(jv[q][u].x, v[q][i][u].x, a.x);
+                  a.y = fmaf(jv[q][u].y, v[q][i][u].y, a.y);
+                  a.z = fmaf(jv[q][u].z, v[q][i][u].z, a.z);
+                  a.w = fmaf(jv[q][u].w, v[q][i][u].w, a.w);
+                }
+              }
+              acc[i][u] = a;
+            }
+          if (h == 0) issue(kb, 1);
+          else if (kb + 1 < KB) {
+            issue(kb + 1, 0);
+            issue_j(kb + 1);
+          }
+          if (h == 0) {
+            if (g >= STAGES && !mbar_wait(&empty[s], ((g / STAGES) - 1) & 1, abort_p)) ok = 0;
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+          }
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const int ci = GT == 2 ? i : 2 * h + i, c = c0 + 32 * ci;
+            uint8_t* xd = xs + (GT == 2 ? h * 2 * X_TILE : 0);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              const float f = up[ci];
+              const int off = c * 128 + (((4 * u + (j >> 1)) ^ (c & 7)) << 4) + (j & 1) * 8;
+              uint2 hi, lo;
+              split_f16(acc[i][u].x * f, acc[i][u].y * f, hi.x, lo.x);
+              split_f16(acc[i][u].z * f, acc[i][u].w * f, hi.y, lo.y);
+              *reinterpret_cast<uint2*>(xd + off) = hi;
+              *reinterpret_cast<uint2*>(xd + X_TILE + off) = lo;
             }
           }
         }
-        if (kb + 1 < KB) issue(kb + 1);
-        if (g >= STAGES && !mbar_wait(&empty[s], ((g / STAGES) - 1) & 1, abort_p)) ok = 0;
-        ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
-        uint8_t* xs = stage_ptr(s) + GT * F_A_GROUP;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int c = c0 + 32 * i;
-          const int off = c * 128 + ((j ^ (c & 7)) << 4);
-          float4 h, l;
-          h.x = to_tf32(acc[i].x); l.x = to_tf32(acc[i].x - h.x);
-          h.y = to_tf32(acc[i].y); l.y = to_tf32(acc[i].y - h.y);
-          h.z = to_tf32(acc[i].z); l.z = to_tf32(acc[i].z - h.z);
-          h.w = to_tf32(acc[i].w); l.w = to_tf32(acc[i].w - h.w);
-          *reinterpret_cast<float4*>(xs + off) = h;
-          *reinterpret_cast<float4*>(xs + PX_TILE + off) = l;
-        }
         fence_async_smem();
         __syncwarp();
         if (lane == 0) mbar_arrive(&xready[s]);
@@ -1014,32 +1175,52 @@ __global__ void __launch_bounds__(F_THREADS, 1)
     const uint32_t empty_bar0 = mapa(smem_u32(&acc_empty[0]), 0);
     int t = 0;
     for (int tile = pair; tile < tiles; tile += npairs) {
-      const FTile T = fused_tile(tile, NGT, NT, Lx, Ly, act, sweep);
+      const FTile T = fused_tile<NB>(tile, NGT, NT, Lx, Ly, act, nact, sweep);
       if (!T.active) continue;
       const int buf = t % NBUF;
-      bool go = mbar_wait(&acc_full[buf], (t / NBUF) & 1, abort_p);
-      ++t;
-      go = __all_sync(0xffffffffu, go);
-      if (!go) break;
-      tc_fence_after();
       // r = 0 (a matvec), or r non-zero only on the rows of each column's source site
       // (the first right-hand side Lambda delta_s) and no column of the tile has its
       // source here: its loads are skipped
+      const int n_first = T.nt * NB;
       bool rz = r == nullptr;
       if (!rz && rsrc) {
         bool here = false;
-        for (int n = T.nt * BN + lane; n < min(ncol, T.nt * BN + BN); n += 32) here |= __ldg(rsrc + n) == T.site;
+        for (int n = n_first + lane; n < min(ncol, n_first + NB); n += 32) here |= __ldg(rsrc + n) == T.site;
         rz = !__any_sync(0xffffffffu, here);
       }
-#pragma unroll
-      for (int gi = 0; gi < GT; ++gi) {
-        const uint32_t tacc = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)((buf * GT + gi) * BN);
-        const int mg = (T.gt * GT + gi) * PM + (int)rank * BM + q4 * 32 + lane;
-        if (rz)
-          epilogue_rows<16, true>(tacc, mg, T.nt * BN, T.site, ncol, gs, (size_t)N2, r, din, dout, norm, lane);
-        else
-          epilogue_rows<16, false>(tacc, mg, T.nt * BN, T.site, ncol, gs, (size_t)N2, r, din, dout, norm, lane);
-      }
+      const int mg = T.gt * PM + (int)rank * BM + q4 * 32 + lane;
+      const bool rows = GT == 1 || T.gt * PM + (int)rank * BM < Nc;   // Nc = 384: the last tile's odd CTA has none
+      const float ad = rows ? __ldg(adown + (size_t)T.site * N2 + mg) : 0.f;   // one scale for rows z and Nc + z
+      const size_t base0 = ((size_t)T.site * ncol + n_first) * N2 + mg;
+      const uint32_t tacc = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(buf * GT * NB);
+      bool go = true;
+      auto body = [&](auto E) {
+        E.r = r;
+        E.din = din;
+        E.dout = dout;
+        E.n_first = n_first;
+        E.ncol = rows ? ncol : 0;
+        E.row_gap = row_gap;
+        E.N2 = N2;
+        E.base0 = base0;
+        E.template load<0>(0);
+        go = mbar_wait(&acc_full[buf], (t / NBUF) & 1, abort_p);
+        go = __all_sync(0xffffffffu, go);                 // tcgen05.ld below is warp-collective
+        if (!go) return;
+        tc_fence_after();
+        constexpr int CHUNKS = decltype(E)::CHUNKS;
+        for (int e = 0; e < CHUNKS; e += 2) {
+          E.template load<1>(e + 1);
+          E.template chunk<0>(e, tacc, ad, gs, norm, sc, lane);
+          if (e + 2 < CHUNKS) E.template load<0>(e + 2);
+          E.template chunk<1>(e + 1, tacc, ad, gs, norm, sc, lane);
+        }
+        if (E.qcur >= 0) E.flush(norm, sc, lane);
+      };
+      if (rz) body(FusedEpilogue<GT, true>{});
+      else body(FusedEpilogue<GT, false>{});
+      ++t;
+      if (!go) break;
       tc_fence_before();
       mbar_arrive_remote(empty_bar0 + (uint32_t)(buf * sizeof(uint64_t)));
     }
@@ -1081,6 +1262,19 @@ bool make_map(CUtensorMap* m, const float* base, uint64_t d0, uint64_t d1, uint6
   cuuint32_t es[3] = {1, 1, 1};
   return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, (void*)base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// 3D map over an fp16 array [d2][d1][d0] with a (64 x box1 x 1) box, 128-byte swizzle
+bool make_map16(CUtensorMap* m, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint32_t box1) {
+  auto fn = encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[3] = {d0, d1, d2};
+  cuuint64_t strides[2] = {d0 * 2, d0 * d1 * 2};
+  cuuint32_t box[3] = {(cuuint32_t)F_BK, box1, 1};
+  cuuint32_t es[3] = {1, 1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void*>(base), dims, strides, box, es,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -1153,10 +1347,11 @@ int fused_clusters(dyson_ctx* c, TcState* st) {
 // row groups per fused tile for the context's variant (0: the fused kernel does not serve it)
 int fused_gt(dyson_ctx* c) {
   if (c->Nc % 128 != 0 || c->Lx * c->Ly != c->Nr) return 0;
-  if (c->tc_variant == DYSON_SWEEP_FUSED_PAIR) return fused_clusters<1>(c, state(c)) > 0 ? 1 : 0;
-  if (c->tc_variant == DYSON_SWEEP_FUSED_PAIR_WIDE && c->Nc % 256 == 0)
-    return fused_clusters<2>(c, state(c)) > 0 ? 2 : 0;
-  return 0;
+  if (c->tc_variant != DYSON_SWEEP_FUSED_PAIR && c->tc_variant != DYSON_SWEEP_FUSED_PAIR_WIDE) return 0;
+  if (c->tc_variant == DYSON_SWEEP_FUSED_PAIR_WIDE && c->Nc % 256 != 0) return 0;
+  // tiles of complex points wherever they are at least three quarters full
+  if (c->Nc >= 256 && fused_clusters<2>(c, state(c)) > 0) return 2;
+  return fused_clusters<1>(c, state(c)) > 0 ? 1 : 0;
 }
 
 }  // namespace
@@ -1183,6 +1378,15 @@ int tc_prepare(dyson_ctx* c, int ncol, bool need_x = true) {
     DY_CUDA(c, cudaMemsetAsync(st->d_err, 0, sizeof(int), c->stream));
     DY_CUDA(c, cudaDeviceGetAttribute(&st->num_sms, cudaDevAttrMultiProcessorCount, c->device));
   }
+  if (!need_x) {                                         // the fused sweep gathers in shared memory
+    if (st->h_hi_ptr != c->d_lam16_hi || st->h_lo_ptr != c->d_lam16_lo) {
+      if (!make_map16(&st->h_hi, c->d_lam16_hi, N2, N2, Nr, BM) || !make_map16(&st->h_lo, c->d_lam16_lo, N2, N2, Nr, BM))
+        return ctx_fail(c, DYSON_ERR_CUDA, "cuTensorMapEncodeTiled failed for the FP16 Lambda");
+      st->h_hi_ptr = c->d_lam16_hi;
+      st->h_lo_ptr = c->d_lam16_lo;
+    }
+    return DYSON_OK;
+  }
   if (st->a_hi_ptr != c->d_lam_hi || st->a_lo_ptr != c->d_lam_lo || st->a_Nr != Nr || st->a_Nc != Nc) {
     if (!make_map(&st->a_hi, c->d_lam_hi, N2, N2, Nr, BM) || !make_map(&st->a_lo, c->d_lam_lo, N2, N2, Nr, BM))
       return ctx_fail(c, DYSON_ERR_CUDA, "cuTensorMapEncodeTiled failed for Lambda");
@@ -1198,7 +1402,6 @@ int tc_prepare(dyson_ctx* c, int ncol, bool need_x = true) {
                                     SMEM_BYTES));
     st->smem_set = true;
   }
-  if (!need_x) return DYSON_OK;                          // the fused sweep gathers in shared memory
   size_t xbytes = (size_t)Nr * ncol * N2 * sizeof(float);
   if (st->xbuf_bytes < xbytes) {
     if (st->xbuf) cudaFree(st->xbuf);
@@ -1226,7 +1429,9 @@ template <int GT>
 int launch_fused(dyson_ctx* c, int ncol, int gs, const float* r, const float* din, float* dout, const int* act,
                  int sweep, const int* rsrc) {
   TcState* st = state(c);
-  const long long tiles = (long long)c->Nr * ((ncol + BN - 1) / BN) * ((2 * c->Nc) / (PM * GT));
+  const int NB = FusedCfg<GT>::NB;
+  const int row_tiles = GT == 2 ? (c->Nc + PM - 1) / PM : 2 * c->Nc / PM;
+  const long long tiles = (long long)c->Nr * ((ncol + NB - 1) / NB) * row_tiles;
   const int pairs = (int)std::min<long long>(tiles, fused_clusters<GT>(c, st));
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[1];
@@ -1240,16 +1445,50 @@ int launch_fused(dyson_ctx* c, int ncol, int gs, const float* r, const float* di
   cfg.stream = c->stream;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  DY_CUDA(c, cudaLaunchKernelEx(&cfg, k_tc_fused<GT>, st->a_hi, st->a_lo, r, din, dout, rsrc,
+  const int ng = ncol / gs;
+  if (!c->sweep_run) {                                   // (in a captured series the check kernel sets the scales)
+    k_tc_scale<<<(ng + 127) / 128, 128, 0, c->stream>>>(c->d_xscale, ng, tc_jbound(c));
+    c->launches += 1;
+  }
+  DY_CUDA(c, cudaLaunchKernelEx(&cfg, k_tc_fused<GT>, st->h_hi, st->h_lo, r, din, dout, rsrc,
                                 (const float*)c->d_Jz,
                                 (const int*)c->d_nbr, (const int*)c->d_nbond, c->Lx, c->Ly, c->Nc, ncol, gs,
-                                c->d_norm, st->d_err, act, sweep, c->sweep_run, c->sweep_count));
+                                c->d_norm, st->d_err, act, sweep, c->sweep_run, c->sweep_count,
+                                (const float*)c->d_a_down, c->d_xscale));
   DY_CUDA(c, cudaGetLastError());
   c->launches += 1;
   return DYSON_OK;
 }
 
 }  // namespace
+
+float tc_jbound(const dyson_ctx* c) { return 4.f * c->j_max; }
+
+int tc_seed_scale(dyson_ctx* c, int ng, const double* ref, double bound) {
+  if (!tc_uses_fused(c)) return DYSON_OK;
+  k_tc_seed<<<(ng + 127) / 128, 128, 0, c->stream>>>(c->d_xscale, ng, ref, (float)bound);
+  c->launches += 1;
+  DY_CUDA(c, cudaGetLastError());
+  return DYSON_OK;
+}
+
+int tc_seed_scale_scan(dyson_ctx* c, int ncol, int gs, const float* d) {
+  if (!tc_uses_fused(c)) return DYSON_OK;
+  int rc = tc_seed_scale(c, ncol / gs, nullptr, 0.0);
+  if (rc) return rc;
+  const size_t warps = (size_t)c->Nr * ncol;
+  k_tc_seed_scan<<<(unsigned)((warps + 7) / 8), 256, 0, c->stream>>>(d, c->Nr, c->Nc, ncol, gs, c->d_xscale);
+  c->launches += 1;
+  DY_CUDA(c, cudaGetLastError());
+  return DYSON_OK;
+}
+
+int tc_set_scale(dyson_ctx* c, int ng) {
+  k_tc_scale<<<(ng + 127) / 128, 128, 0, c->stream>>>(c->d_xscale, ng, tc_jbound(c));
+  c->launches += 1;
+  DY_CUDA(c, cudaGetLastError());
+  return DYSON_OK;
+}
 
 int tc_prepare_sweep(dyson_ctx* c, int ncol) { return tc_prepare(c, ncol, fused_gt(c) == 0); }
 

@@ -181,6 +181,13 @@ __device__ __forceinline__ void mma_pair_tf32(uint32_t tmem_d, uint64_t adesc, u
           tmem_d),
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
 }
+__device__ __forceinline__ void mma_pair_f16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                             uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
+          tmem_d),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
+}
 // arrive once on the barrier at this offset in every CTA of `mask` when the pair's MMAs complete
 __device__ __forceinline__ void mma_commit_pair_mc(uint64_t* bar, uint16_t mask) {
   asm volatile(

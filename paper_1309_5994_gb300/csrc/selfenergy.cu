@@ -975,7 +975,7 @@ extern "C" int dyson_selfenergy_step(dyson_ctx* c, const double* gloc, double mi
   if ((rc = gemm(c, st->g0, st->conn, st->w2))) return rc;
   DY_CUDA(c, cudaMemcpyAsync(c->d_lam, st->w2, n_el * sizeof(double2), cudaMemcpyDeviceToDevice, c->stream));
   DY_CUDA(c, cudaStreamSynchronize(c->stream));
-  c->lam32_built = c->lam_split_built = false;
+  c->lam32_built = c->lam_split_built = c->lam16_built = false;
   oz_invalidate(c);
   oz64_invalidate(c);
   c->se_installed = true;

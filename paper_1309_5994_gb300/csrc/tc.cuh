@@ -32,6 +32,14 @@ struct TcInst {
 };
 
 
+// FP16 scales of the fused sweep: before the first sweep of a chain, seed the bound on |d_in| per
+// column group, with ref (device, [ng]) or one bound for all, or by reading the state; the
+// sweeps after it take the bound from the maxima that the previous one left.  No-ops for the other forms.
+int tc_seed_scale(dyson_ctx* c, int ng, const double* ref, double bound);
+int tc_seed_scale_scan(dyson_ctx* c, int ncol, int gs, const float* d);
+// turn the seeded maxima into scales (tc_sweep does this itself outside a captured series)
+int tc_set_scale(dyson_ctx* c, int ng);
+float tc_jbound(const dyson_ctx* c);              // 4 max|J|, the factor of set_scale
 // true when the 3xTF32 tcgen05 sweep supports this contour length
 bool tc_supported(dyson_ctx* c, int Nc);
 // true when tc_sweep runs the CTA-pair (cta_group::2) kernel for this context

@@ -48,6 +48,7 @@ int time_sweeps(dyson_ctx* c, int nq, int warm, int timed, double* ms_per_sweep)
   DY_CUDA(c, cudaEventCreate(&e0));
   DY_CUDA(c, cudaEventCreate(&e1));
   for (int s = 0; s < warm + timed; ++s) {
+    if (s == 0 && (rc = tc_seed_scale_scan(c, ncol, c->Nc, da))) break;
     if (s == warm) DY_CUDA(c, cudaEventRecord(e0, c->stream));
     if ((rc = tc_sweep(c, ncol, c->Nc, r32, da, db, TC_GATHER | TC_GEMM))) break;
     std::swap(da, db);
@@ -117,7 +118,7 @@ int dyson_autotune(dyson_ctx* c, int32_t max_block_columns, dyson_tuning* out) {
     for (int v : variants) {
       c->tc_variant = v;
       double ms = 0.0;
-      if ((rc = time_sweeps(c, nq, 2, 3, &ms))) {
+      if ((rc = prepare_tables(c, DYSON_PREC_TF32X3_F64REF)) || (rc = time_sweeps(c, nq, 2, 3, &ms))) {
         c->tc_variant = saved_variant;
         return rc;
       }

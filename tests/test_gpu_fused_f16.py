@@ -1,0 +1,51 @@
+"""The fused sweep's FP16 operands: scales per row of Lambda W and per column group of X.
+
+Hoppings that differ by orders of magnitude from bond to bond, and right-hand sides that do from column
+group to column group, must not cost digits or overflow FP16."""
+import numpy as np
+import pytest
+
+import workloads as wl
+from oracle import dyson
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def torch_cuda():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return torch
+
+
+@pytest.mark.parametrize("variant", [2, 3])
+@pytest.mark.parametrize("inner", [0, 1])
+@pytest.mark.parametrize("jscale", [1e-6, 1.0, "mixed"])
+def test_fused_solve_over_hopping_scales(torch_cuda, lib, jscale, inner, variant):
+    """Refined to 1e-12 by the FP64-accurate residual; the number of refinements says what the FP32-accurate
+    inner solves deliver (about three digits or more each)."""
+    from paper_1309_5994_gb300 import binding
+    torch = torch_cuda
+    Nc = 128 if variant == 2 else 256
+    p = wl.small(L=3, Ly=2, Nt=3 * Nc // 8, Nm=Nc // 4, dt=0.02, beta=2.0, trap_c=0.3, U0=20.0)
+    r = np.random.default_rng(11)
+    f = jscale if jscale != "mixed" else 10.0 ** r.uniform(-6.0, 0.0, size=(p.Nb, 1))
+    p = p.with_tables(J=p.J * f)
+    S = dyson.setup(p)
+    sources = [0, 4]
+    ref = dyson.dense_solve(S, dyson.rhs_block_columns(S, sources))
+    s = binding.Solver(p, device=0)
+    s.set_sweep_variant(variant)
+    s.set_inner_solver(inner)
+    s.build_sigma()
+    s.profile(True)
+    g = torch.empty((len(sources), p.Nr, p.Nc, p.Nc), dtype=torch.complex128, device="cuda:0")
+    res = s.solve(sources, precision=binding.PREC_TF32X3_F64REF, tol=1e-12, g_out=g)
+    assert s.profile_query(binding.KERNEL_SWEEP_TC_FUSED)[0] > 0
+    assert res.report["refinements"] <= 4
+    got = g.cpu().numpy()
+    for q in range(len(sources)):
+        want = ref[:, :, q * p.Nc:(q + 1) * p.Nc]
+        assert np.abs(got[q] - want).max() / np.abs(want).max() < 1e-11
+    s.close()
