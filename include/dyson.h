@@ -293,13 +293,15 @@ const char* dyson_last_error(const dyson_ctx* ctx);
 enum {
   DYSON_KERNEL_SWEEP_F64 = 0,     /* FP64 series sweep (gather, slicing and complex GEMM)    */
   DYSON_KERNEL_SWEEP_F32 = 1,     /* FP32 CUDA-core sweep                                    */
-  DYSON_KERNEL_SWEEP_TC = 2,      /* 3xTF32 tcgen05 sweep GEMM (split + MMA + epilogue)      */
+  DYSON_KERNEL_SWEEP_TC = 2,      /* tcgen05 sweep: the single-CTA GEMM (split + MMA +
+                                     epilogue), or the default form of a context that has
+                                     selected none                                          */
   DYSON_KERNEL_RESIDUAL_F64 = 3,  /* FP64 Dyson residual r = Lambda delta + K G - G          */
   DYSON_KERNEL_RESIDUAL_SPLIT = 4,/* the same residual from BF16 slice products on tcgen05   */
   DYSON_KERNEL_SWEEP_TC_PAIR = 5, /* the same GEMM on CTA pairs (tcgen05 cta_group::2, M=256) */
   DYSON_KERNEL_GATHER_TC = 6,     /* neighbour gather X = J d of the tensor-core sweep        */
   DYSON_KERNEL_SELFENERGY = 7,    /* connected cumulant contraction of the self-energy step  */
-  DYSON_KERNEL_SWEEP_TC_FUSED = 8,/* fused gather + 3xTF32 GEMM on CTA pairs (one launch/sweep)*/
+  DYSON_KERNEL_SWEEP_TC_FUSED = 8,/* fused gather + GEMM on CTA pairs, selected (one launch/sweep) */
   DYSON_KERNEL_KINDS = 9
 };
 
@@ -320,17 +322,20 @@ int dyson_set_chunk(dyson_ctx* ctx, int32_t block_columns);
 /* Form of the 3xTF32 tensor-core sweep (App. C's series step; Sec. IV.D's
  * blocked application of the local blocks to many right-hand sides).
  *   SINGLE_CTA  a gather launch writes X = J d to global memory, then one CTA
- *               per 128 x 256 output tile multiplies (the default);
+ *               per 128 x 256 output tile multiplies;
  *   CTA_PAIR    the same gather, then clusters of two CTAs on 256 x 256 tiles
  *               with tcgen05 cta_group::2 MMAs;
  *   FUSED_PAIR  one launch per sweep: CTA pairs whose producer warps gather the
  *               four neighbour rows of d straight into the MMA's shared-memory
- *               operand (X never reaches global memory); tiles of 256 rows x 256
- *               columns, two TMEM accumulators;
- *   FUSED_PAIR_WIDE  the fused form with tiles of 512 rows x 256 columns (X
- *               gathered once per site and column tile, one accumulator set).
- * The pair forms need Nc % 128 == 0 (FUSED_PAIR_WIDE: Nc % 256 == 0) and a
- * device that co-schedules CTA pairs; otherwise the single-CTA form runs.  All
+ *               operand (X never reaches global memory), with FP16 hi + lo
+ *               operands under power-of-two scales (22 bits, as the TF32 pairs
+ *               of the other forms);
+ *   FUSED_PAIR_WIDE  the same kernel (kept as a name of its own; the tuner lists
+ *               it where Nc % 256 == 0).
+ * A context that selects none runs the fused form.  SINGLE_CTA needs Nc % 64 == 0
+ * and CTA_PAIR Nc % 128 == 0 (else the single-CTA form runs); the fused form
+ * serves every contour of at least 24 points, padded to a multiple of 64 with
+ * zeros, and takes the place of the others on contours they do not fill.  All
  * give the same results to FP32 rounding; which is fastest depends on the
  * shape, which is what dyson_autotune measures.  Returns INVALID_ARG for an
  * unknown variant. */
@@ -439,8 +444,8 @@ int dyson_set_support_truncation(dyson_ctx* ctx, int enable);
  * block columns are solved exactly as dyson_solve_columns(precision =
  * DYSON_PREC_TF32X3_F64REF) solves them (the series of App. C refined with
  * FP64-accurate residuals).  What the instances share is the inner FP32
- * series.  Every sweep is ONE gather launch and ONE persistent tensor-core
- * launch over the tiles of all instances still iterating, followed by a check
+ * series.  Every sweep is one fused launch per instance still iterating, on
+ * parallel branches, followed by a check
  * kernel that applies each instance's stopping rule on the device.  Blocks of
  * graph_sweeps sweeps are captured once as a CUDA graph and replayed with no
  * host round trip inside a block.  An instance whose series diverges (spectral
@@ -472,7 +477,7 @@ int dyson_batch_create(dyson_batch** out, dyson_ctx* const* ctxs, int32_t n);
 int dyson_batch_solve(dyson_batch* b, const int32_t* const* src, const int32_t* n_src, double tol,
                       int32_t max_sweeps, int32_t graph_sweeps, double* const* g_out, dyson_report* reports);
 
-/* Kernels launched by the batch's sweep graphs (3 per sweep; -1 for NULL). */
+/* Kernels launched by the batch's sweep graphs (one per instance and one check per sweep; -1 for NULL). */
 int64_t dyson_batch_launch_count(const dyson_batch* b);
 const char* dyson_batch_last_error(const dyson_batch* b);
 void dyson_batch_destroy(dyson_batch* b);

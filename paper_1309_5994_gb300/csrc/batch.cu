@@ -3,9 +3,9 @@
 // Each instance is a context of its own (lattice, contour, trap, drive, Lambda)
 // solving its block columns with the series of App. C refined by FP64 residuals,
 // exactly as dyson_solve_columns(precision = TF32X3_F64REF) does.  What is
-// shared is the inner FP32 series: every sweep is ONE gather launch and ONE
-// persistent tensor-core launch over the tiles of all instances still
-// iterating (an instance table on the device, k_tc.cu), followed by a one-block
+// shared is the inner FP32 series: every sweep is one launch of the fused gather + GEMM
+// kernel per instance, on parallel branches of a graph (a launch whose instance has stopped
+// returns at once), followed by a one-block
 // check kernel that applies the inner stopping rule per instance on the device
 // and clears the instance's activity flag when it stops.  A block of
 // graph_sweeps sweeps is captured once as a CUDA graph and replayed until no
@@ -27,13 +27,16 @@
 
 using namespace dyson_detail;
 
-static_assert(DYSON_BATCH_MAX_INSTANCES == TC_MAX_INSTANCES, "one tensor-core launch serves the whole batch");
-
 namespace {
+
+// Parallel branches of the sweep graph: the tail of one instance's launch overlaps the next ones'.
+constexpr int BATCH_LANES = 4;
 
 struct BatchCheck {                 // what the check kernel reads per instance
   unsigned long long* norm;         // ng update max-norm words (bits of a non-negative double)
   const double* rref;               // ng reference norms of the current inner solve
+  TcScale* xscale;                  // ng scales of the fused sweep's FP16 operand
+  float jbound;
   int ng;
   int max_sweeps;
 };
@@ -63,6 +66,7 @@ __global__ void k_batch_check(const BatchCheck* __restrict__ chk, int n, int* __
       if (!(v == v)) bad = true;
       else upd = fmax(upd, v);
       C.norm[q] = 0ull;
+      set_scale(C.xscale + q, __uint_as_float(C.xscale[q].ymax), C.jbound);
     }
     BatchStop S = st[k];
     S.sweeps += 1;
@@ -130,8 +134,8 @@ struct dyson_batch {
   std::string err;
   int64_t launches = 0;
   // device tables (sized for ctx.size() instances)
-  TcInst* d_tab = nullptr;
-  TcInst* h_tab = nullptr;           // pinned
+  cudaStream_t side[BATCH_LANES] = {};   // capture branches of the sweep graph
+  cudaEvent_t ev_fork = nullptr, ev_join[BATCH_LANES] = {};
   BatchCheck* d_chk = nullptr;
   BatchStop* d_stop = nullptr;
   BatchStop* h_stop = nullptr;       // pinned
@@ -193,8 +197,7 @@ int dyson_batch_create(dyson_batch** out, dyson_ctx* const* ctxs, int32_t n) {
   if ((e = cudaStreamCreateWithFlags(&b->gstream, cudaStreamNonBlocking)) != cudaSuccess ||
       (e = cudaEventCreateWithFlags(&b->ev_in, cudaEventDisableTiming)) != cudaSuccess ||
       (e = cudaEventCreateWithFlags(&b->ev_out, cudaEventDisableTiming)) != cudaSuccess ||
-      (e = cudaMalloc((void**)&b->d_tab, n * sizeof(TcInst))) != cudaSuccess ||
-      (e = cudaMallocHost((void**)&b->h_tab, n * sizeof(TcInst))) != cudaSuccess ||
+      (e = cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming)) != cudaSuccess ||
       (e = cudaMalloc((void**)&b->d_chk, n * sizeof(BatchCheck))) != cudaSuccess ||
       (e = cudaMalloc((void**)&b->d_stop, n * sizeof(BatchStop))) != cudaSuccess ||
       (e = cudaMallocHost((void**)&b->h_stop, n * sizeof(BatchStop))) != cudaSuccess ||
@@ -207,6 +210,13 @@ int dyson_batch_create(dyson_batch** out, dyson_ctx* const* ctxs, int32_t n) {
     return fail_noctx(e == cudaErrorMemoryAllocation ? DYSON_ERR_OOM : DYSON_ERR_CUDA,
                       std::string("batch set-up: ") + cudaGetErrorString(e));
   }
+  for (int l = 0; l < BATCH_LANES; ++l)
+    if ((e = cudaStreamCreateWithFlags(&b->side[l], cudaStreamNonBlocking)) != cudaSuccess ||
+        (e = cudaEventCreateWithFlags(&b->ev_join[l], cudaEventDisableTiming)) != cudaSuccess) {
+      cudaGetLastError();
+      dyson_batch_destroy(b);
+      return fail_noctx(DYSON_ERR_CUDA, std::string("batch set-up: ") + cudaGetErrorString(e));
+    }
   *out = b;
   return DYSON_OK;
 }
@@ -237,7 +247,7 @@ int dyson_batch_solve(dyson_batch* b, const int32_t* const* src, const int32_t* 
     for (int q = 0; q < n_src[k]; ++q)
       if (src[k][q] < 0 || src[k][q] >= c->Nr) return bfail(b, DYSON_ERR_INVALID_ARG, "source site out of range");
     if ((rc = prepare_tables(c, DYSON_PREC_TF32X3_F64REF, true))) return bfail(b, rc, c->err);
-    if (!c->use_tc || !c->use_oz)
+    if (!c->use_tc || !c->use_oz || !tc_fused_runs(c))
       return bfail(b, DYSON_ERR_INVALID_ARG,
                    "instance " + std::to_string(k) + ": batched solves need Nc % 64 == 0 and 2 Nc <= 512");
     X.nq = n_src[k];
@@ -256,16 +266,16 @@ int dyson_batch_solve(dyson_batch* b, const int32_t* const* src, const int32_t* 
         c->h_src_time[q * c->Nc + z] = z;
       }
     if ((rc = upload_sources(c, X.ncol))) return bfail(b, rc, c->err);
-    const size_t n_el = (size_t)c->Nr * X.ncol * c->Nc;
+    const size_t n_el = (size_t)c->Nr * X.ncol * c->Nc, n32 = (size_t)c->Nr * X.ncol * 2 * c->Ns;
     X.G = (double2*)c->work;
     X.r32 = (float*)(X.G + n_el);
-    X.da = X.r32 + 2 * n_el;
-    X.db = X.da + 2 * n_el;
+    X.da = X.r32 + n32;
+    X.db = X.da + n32;
     DYB_CUDA(b, cudaMemsetAsync(X.G, 0, n_el * sizeof(double2), c->stream));
     DYB_CUDA(b, cudaMemsetAsync(c->d_norm, 0, 2 * (size_t)X.ng * sizeof(unsigned long long), c->stream));
     launch_init_rhs(c->d_lam, c->d_src_site, c->d_src_time, c->Nr, c->Nc, X.ncol, c->Nc, X.G, c->d_norm + X.ng,
                     c->stream);
-    launch_to_planar32(X.G, X.r32, n_el, c->Nc, c->stream);
+    launch_to_planar32(X.G, X.r32, (size_t)c->Nr * X.ncol, c->Nc, c->Ns, c->stream);
     c->launches += 2;
     DYB_CUDA(b, cudaMemsetAsync(X.G, 0, n_el * sizeof(double2), c->stream));
     if ((rc = read_norms(c, X.ng, true))) return bfail(b, rc, c->err);
@@ -274,7 +284,7 @@ int dyson_batch_solve(dyson_batch* b, const int32_t* const* src, const int32_t* 
     X.rref = X.scale;
     rref_total += X.ng;
   }
-  // ---- device tables: instances, check entries, reference norms ----
+  // ---- device tables: check entries, reference norms ----
   if (b->rref_cap < rref_total) {
     if (b->d_rref) cudaFree(b->d_rref);
     if (b->h_rref) cudaFreeHost(b->h_rref);
@@ -287,47 +297,49 @@ int dyson_batch_solve(dyson_batch* b, const int32_t* const* src, const int32_t* 
   }
   std::vector<BatchCheck> chk(n);
   std::vector<size_t> rref_off(n);
-  std::vector<CUtensorMap> m_hi(n), m_lo(n), m_x(n);
-  int tiles = 0, gblocks = 0;
   size_t off = 0;
   for (int k = 0; k < n; ++k) {
     Inst& X = I[k];
-    TcInst* e = &b->h_tab[k];
-    if ((rc = tc_fill_instance(X.c, X.ncol, X.c->Nc, X.r32, X.da, X.db, X.c->d_norm, b->d_active + k, e, &m_hi[k],
-                               &m_lo[k], &m_x[k])))
-      return bfail(b, rc, X.c->err);
-    e->tile0 = tiles;
-    e->gblk0 = gblocks;
-    tiles += tc_instance_tiles(*e);
-    gblocks += tc_instance_gather_blocks(*e);
     rref_off[k] = off;
-    chk[k] = BatchCheck{X.c->d_norm, b->d_rref + off, X.ng, max_sweeps};
+    chk[k] = BatchCheck{X.c->d_norm, b->d_rref + off, X.c->d_xscale, tc_jbound(X.c), X.ng, max_sweeps};
     off += X.ng;
   }
   // every context's set-up work precedes the tables and the graph
   DYB_CUDA(b, cudaStreamSynchronize(b->stream));
-  DYB_CUDA(b, cudaMemcpyAsync(b->d_tab, b->h_tab, n * sizeof(TcInst), cudaMemcpyHostToDevice, b->stream));
   DYB_CUDA(b, cudaMemcpyAsync(b->d_chk, chk.data(), n * sizeof(BatchCheck), cudaMemcpyHostToDevice, b->stream));
   DYB_CUDA(b, cudaStreamSynchronize(b->stream));
 
-  // ---- the sweep graph: S x (gather, GEMM, check) over the whole table ----
+  // ---- the sweep graph: S x (one fused launch per instance, on BATCH_LANES parallel branches, check) ----
   free_graph(b);
   {
-    dyson_ctx* c0 = b->ctx[0];
-    const int64_t l0 = c0->launches;
     cudaGraph_t graph = nullptr;
+    for (int k = 0; k < n; ++k)                            // nothing to allocate or encode while capturing
+      if ((rc = tc_prepare_sweep(I[k].c, I[k].ncol, true))) return bfail(b, rc, I[k].c->err);
     DYB_CUDA(b, cudaStreamBeginCapture(b->gstream, cudaStreamCaptureModeThreadLocal));
     int cap_rc = DYSON_OK;
+    dyson_ctx* failed = b->ctx[0];
+    const int lanes = std::min(n, BATCH_LANES);
     for (int s = 0; s < S && cap_rc == DYSON_OK; ++s) {
-      cap_rc = tc_launch_table(c0, b->d_tab, n, tiles, gblocks, s & 1, TC_GATHER | TC_GEMM, b->gstream,
-                               m_hi.data(), m_lo.data(), m_x.data());
+      cudaEventRecord(b->ev_fork, b->gstream);
+      for (int l = 0; l < lanes; ++l) cudaStreamWaitEvent(b->side[l], b->ev_fork, 0);
+      for (int k = 0; k < n && cap_rc == DYSON_OK; ++k) {
+        Inst& X = I[k];
+        const int64_t l0 = X.c->launches;
+        cap_rc = tc_fused_sweep(X.c, X.ncol, X.c->Nc, X.r32, s & 1 ? X.db : X.da, s & 1 ? X.da : X.db, nullptr, 0,
+                                TC_R_DENSE, b->d_active + k, nullptr, b->side[k % lanes]);
+        X.c->launches = l0;
+        if (cap_rc) failed = X.c;
+      }
+      for (int l = 0; l < lanes; ++l) {
+        cudaEventRecord(b->ev_join[l], b->side[l]);
+        cudaStreamWaitEvent(b->gstream, b->ev_join[l], 0);
+      }
       if (cap_rc == DYSON_OK) k_batch_check<<<1, 256, 0, b->gstream>>>(b->d_chk, n, b->d_active, b->d_stop, b->d_nactive);
     }
     cudaError_t ce = cudaStreamEndCapture(b->gstream, &graph);
-    c0->launches = l0;
     if (cap_rc != DYSON_OK) {
       if (graph) cudaGraphDestroy(graph);
-      return bfail(b, cap_rc, c0->err);
+      return bfail(b, cap_rc, failed->err);
     }
     if (ce != cudaSuccess) {
       cudaGetLastError();
@@ -355,7 +367,7 @@ int dyson_batch_solve(dyson_batch* b, const int32_t* const* src, const int32_t* 
       b->h_stop[k].target = inner_target(kInnerTarget, tol, X.prev_res);
       if (X.done) continue;
       ++n_live;
-      const size_t n32 = (size_t)X.c->Nr * X.ncol * 2 * X.c->Nc;
+      const size_t n32 = (size_t)X.c->Nr * X.ncol * 2 * X.c->Ns;
       DYB_CUDA(b, cudaMemcpyAsync(X.da, X.r32, n32 * sizeof(float), cudaMemcpyDeviceToDevice, b->stream));
       DYB_CUDA(b, cudaMemsetAsync(X.c->d_norm, 0, (size_t)X.ng * sizeof(unsigned long long), b->stream));
       std::copy(X.rref.begin(), X.rref.end(), b->h_rref + rref_off[k]);
@@ -365,22 +377,31 @@ int dyson_batch_solve(dyson_batch* b, const int32_t* const* src, const int32_t* 
     DYB_CUDA(b, cudaMemcpyAsync(b->d_stop, b->h_stop, n * sizeof(BatchStop), cudaMemcpyHostToDevice, b->stream));
     DYB_CUDA(b, cudaMemcpyAsync(b->d_rref, b->h_rref, rref_total * sizeof(double), cudaMemcpyHostToDevice,
                                 b->stream));
+    for (int k = 0; k < n; ++k) {                          // the series starts from d = r
+      Inst& X = I[k];
+      if (X.done) continue;
+      if ((rc = tc_seed_scale(X.c, X.ng, b->d_rref + rref_off[k], 0.0)) || (rc = tc_set_scale(X.c, X.ng)))
+        return bfail(b, rc, X.c->err);
+    }
     DYB_CUDA(b, cudaEventRecord(b->ev_in, b->stream));
     DYB_CUDA(b, cudaStreamWaitEvent(b->gstream, b->ev_in, 0));
     // replay until every instance has stopped (the check kernel also stops an
     // instance at max_sweeps, so the bound below is never the one that ends it)
     for (int rep = 0; rep <= max_sweeps / S + 1; ++rep) {
       DYB_CUDA(b, cudaGraphLaunch(b->exec, b->gstream));
-      b->launches += 3 * (int64_t)S;
+      b->launches += (n + 1) * (int64_t)S;
       DYB_CUDA(b, cudaMemcpyAsync(b->h_nactive, b->d_nactive, sizeof(int), cudaMemcpyDeviceToHost, b->gstream));
       DYB_CUDA(b, cudaStreamSynchronize(b->gstream));
-      if ((rc = tc_check_error(c0))) return bfail(b, rc, c0->err);
       if (*b->h_nactive == 0) break;
     }
     DYB_CUDA(b, cudaEventRecord(b->ev_out, b->gstream));
     DYB_CUDA(b, cudaStreamWaitEvent(b->stream, b->ev_out, 0));
     DYB_CUDA(b, cudaMemcpyAsync(b->h_stop, b->d_stop, n * sizeof(BatchStop), cudaMemcpyDeviceToHost, b->stream));
+    for (int k = 0; k < n; ++k)
+      if ((rc = tc_error_enqueue(I[k].c))) return bfail(b, rc, I[k].c->err);
     DYB_CUDA(b, cudaStreamSynchronize(b->stream));
+    for (int k = 0; k < n; ++k)
+      if ((rc = tc_error_status(I[k].c))) return bfail(b, rc, I[k].c->err);
     // G += d, then the FP64-accurate residual, per live instance
     for (int k = 0; k < n; ++k) {
       Inst& X = I[k];
@@ -396,7 +417,7 @@ int dyson_batch_solve(dyson_batch* b, const int32_t* const* src, const int32_t* 
         continue;
       }
       const float* d = (St.sweeps & 1) ? X.db : X.da;     // sweep s writes buf[s & 1]
-      launch_accumulate(X.G, d, c->Nr, c->Nc, X.ncol, c->stream);
+      launch_accumulate(X.G, d, c->Nr, c->Nc, c->Ns, X.ncol, c->stream);
       c->launches += 1;
       DYB_CUDA(b, cudaMemsetAsync(c->d_norm, 0, (size_t)X.ng * sizeof(unsigned long long), c->stream));
       if ((rc = oz_residual(c, X.ncol, c->Nc, X.G, X.r32, tol))) return bfail(b, rc, c->err);
@@ -434,6 +455,7 @@ int dyson_batch_solve(dyson_batch* b, const int32_t* const* src, const int32_t* 
     const int saved = c->inner_solver;
     c->inner_solver = DYSON_INNER_GMRES;
     double2* G = nullptr;
+    if ((rc = prepare_tables(c, DYSON_PREC_TF32X3_F64REF))) return bfail(b, rc, c->err);
     rc = solve_mixed(c, X.ncol, c->Nc, DYSON_PREC_TF32X3_F64REF, tol, max_sweeps, &G, &X.rep);
     c->inner_solver = saved;
     if (rc != DYSON_OK && rc != DYSON_ERR_NOT_CONVERGED && rc != DYSON_ERR_DIVERGED) return bfail(b, rc, c->err);
@@ -477,12 +499,17 @@ void dyson_batch_destroy(dyson_batch* b) {
   if (b->gstream) cudaStreamSynchronize(b->gstream);
   free_graph(b);
   if (b->gstream) cudaStreamDestroy(b->gstream);
+  for (int l = 0; l < BATCH_LANES; ++l) {
+    if (b->side[l]) cudaStreamDestroy(b->side[l]);
+    if (b->ev_join[l]) cudaEventDestroy(b->ev_join[l]);
+  }
+  if (b->ev_fork) cudaEventDestroy(b->ev_fork);
   if (b->ev_in) cudaEventDestroy(b->ev_in);
   if (b->ev_out) cudaEventDestroy(b->ev_out);
-  void* dptrs[] = {b->d_tab, b->d_chk, b->d_stop, b->d_active, b->d_nactive, b->d_rref};
+  void* dptrs[] = {b->d_chk, b->d_stop, b->d_active, b->d_nactive, b->d_rref};
   for (void* p : dptrs)
     if (p) cudaFree(p);
-  void* hptrs[] = {b->h_tab, b->h_stop, b->h_active, b->h_nactive, b->h_rref};
+  void* hptrs[] = {b->h_stop, b->h_active, b->h_nactive, b->h_rref};
   for (void* p : hptrs)
     if (p) cudaFreeHost(p);
   delete b;

@@ -150,7 +150,7 @@ int solve_f64(dyson_ctx* c, int ncol, int gs, double tol, int max_sweeps, double
       if (c->use_oz64) {
         if ((rc = oz64_sweep(c, ncol, gs, Ga, Gb, nullptr, 0))) return rc;
       } else {
-        launch_sweep_f64(c->d_lam, c->d_JW, c->d_nbr, c->d_nbond, Ga, Gb, nullptr, c->d_src_site, c->d_src_time,
+        launch_sweep_f64(c->d_lam, c->d_JW, c->d_nbr, c->d_nbond, Ga, Gb, nullptr, c->Nc, c->d_src_site, c->d_src_time,
                          c->Nr, c->Nc, ncol, gs, 0, c->d_norm, c->stream);
         c->launches += 1;
       }
@@ -247,12 +247,20 @@ __global__ void k_series_check(unsigned long long* __restrict__ norm, const doub
   }
 }
 
-// one 3xTF32 tensor-core sweep dout = r + K din with per-kind event timing: the
+// kind that the fused sweep is timed as: its own where the context selected it, the general
+// tensor-core sweep where it runs as the default
+int fused_kind(const dyson_ctx* c) {
+  return c->tc_variant == DYSON_SWEEP_FUSED_PAIR || c->tc_variant == DYSON_SWEEP_FUSED_PAIR_WIDE
+             ? DYSON_KERNEL_SWEEP_TC_FUSED
+             : DYSON_KERNEL_SWEEP_TC;
+}
+
+// one tensor-core sweep dout = r + K din with per-kind event timing: the
 // fused gather + GEMM launch, or the gather launch and the GEMM launch
 int tc_timed_sweep(dyson_ctx* c, int ncol, int gs, const float* r, const float* din, float* dout, const int* act,
                    int sweep, int rform = TC_R_DENSE) {
   if (tc_uses_fused(c)) {
-    KernelTimer t(c, DYSON_KERNEL_SWEEP_TC_FUSED);
+    KernelTimer t(c, fused_kind(c));
     return tc_sweep(c, ncol, gs, r, din, dout, TC_GATHER | TC_GEMM, act, sweep, rform);
   }
   int rc;
@@ -278,7 +286,7 @@ int inner_solve(dyson_ctx* c, int ncol, int gs, int precision, float* r32, float
                 bool* exhausted = nullptr, double target = kInnerTarget, bool r_on_sources = false) {
   if (exhausted) *exhausted = false;
   const int ng = ncol / gs;
-  const size_t n32 = (size_t)c->Nr * ncol * 2 * c->Nc;
+  const size_t n32 = (size_t)c->Nr * ncol * 2 * c->Ns;
   DY_CUDA(c, cudaMemcpyAsync(da, r32, n32 * sizeof(float), cudaMemcpyDeviceToDevice, c->stream));
   if (act) DY_CUDA(c, cudaMemsetAsync(db, 0, n32 * sizeof(float), c->stream));   // skipped tiles stay 0
   const int rform = r_on_sources ? TC_R_ON_SOURCES : TC_R_DENSE;
@@ -305,7 +313,7 @@ int inner_solve(dyson_ctx* c, int ncol, int gs, int precision, float* r32, float
       if ((rc = tc_timed_sweep(c, ncol, gs, r32, da, db, act, sweep, rform))) return rc;
     } else {
       KernelTimer t(c, DYSON_KERNEL_SWEEP_F32);
-      launch_sweep_f32_simt(c->d_lam32, c->d_Jz, c->d_nbr, c->d_nbond, r32, da, db, c->Nr, c->Nc, ncol, gs,
+      launch_sweep_f32_simt(c->d_lam32, c->d_Jz, contour_stride(c), c->d_nbr, c->d_nbond, r32, da, db, c->Nr, c->Nc, ncol, gs,
                             c->d_norm, c->stream);
       c->launches += 1;
     }
@@ -428,8 +436,8 @@ int inner_solve(dyson_ctx* c, int ncol, int gs, int precision, float* r32, float
       rep->update = hS->last;
       float ms = 0.f;
       if (e0 && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess) {
-        c->prof_ms[DYSON_KERNEL_SWEEP_TC_FUSED] += ms;     // the replay, its checks included
-        c->prof_launches[DYSON_KERNEL_SWEEP_TC_FUSED] += n_run;
+        c->prof_ms[fused_kind(c)] += ms;                   // the replay, its checks included
+        c->prof_launches[fused_kind(c)] += n_run;
       }
       if (!hS->run) {
         if (n_run % 2) std::swap(da, db);                  // the last sweep wrote db
@@ -459,12 +467,13 @@ int matvec_f32(dyson_ctx* c, int ncol, int gs, int precision, const float* zero,
                double bound) {
   int rc;
   if (precision == DYSON_PREC_TF32X3_F64REF && c->use_tc) {
-    if ((rc = bound > 0.0 ? tc_seed_scale(c, ncol / gs, nullptr, bound) : tc_seed_scale_scan(c, ncol, gs, in)))
+    if (tc_uses_fused(c) &&
+        (rc = bound > 0.0 ? tc_seed_scale(c, ncol / gs, nullptr, bound) : tc_seed_scale_scan(c, ncol, gs, in)))
       return rc;
     if ((rc = tc_timed_sweep(c, ncol, gs, zero, in, out, nullptr, 0, TC_R_ZERO))) return rc;
   } else {
     KernelTimer t(c, DYSON_KERNEL_SWEEP_F32);
-    launch_sweep_f32_simt(c->d_lam32, c->d_Jz, c->d_nbr, c->d_nbond, zero, in, out, c->Nr, c->Nc, ncol, gs,
+    launch_sweep_f32_simt(c->d_lam32, c->d_Jz, contour_stride(c), c->d_nbr, c->d_nbond, zero, in, out, c->Nr, c->Nc, ncol, gs,
                           c->d_norm, c->stream);
     c->launches += 1;
   }
@@ -522,17 +531,17 @@ const int* support_table(dyson_ctx* c, int ncol) {
 int solve_mixed(dyson_ctx* c, int ncol, int gs, int precision, double tol, int max_sweeps, double2** result,
                 dyson_report* rep) {
   const int ng = ncol / gs;
-  const size_t n_el = (size_t)c->Nr * ncol * c->Nc;
+  const size_t n_el = (size_t)c->Nr * ncol * c->Nc, n32 = (size_t)c->Nr * ncol * 2 * c->Ns;
   double2* G = (double2*)c->work;
   float* r32 = (float*)(G + n_el);
-  float* da = r32 + 2 * n_el;
-  float* db = da + 2 * n_el;
+  float* da = r32 + n32;
+  float* db = da + n32;
   int rc;
   // r = B (FP32), scale = max |B| per group; G = 0
   DY_CUDA(c, cudaMemsetAsync(G, 0, n_el * sizeof(double2), c->stream));
   DY_CUDA(c, cudaMemsetAsync(c->d_norm, 0, 2 * (size_t)ng * sizeof(unsigned long long), c->stream));
   launch_init_rhs(c->d_lam, c->d_src_site, c->d_src_time, c->Nr, c->Nc, ncol, gs, G, c->d_norm + ng, c->stream);
-  launch_to_planar32(G, r32, n_el, c->Nc, c->stream);
+  launch_to_planar32(G, r32, (size_t)c->Nr * ncol, c->Nc, c->Ns, c->stream);
   c->launches += 2;
   DY_CUDA(c, cudaMemsetAsync(G, 0, n_el * sizeof(double2), c->stream));
   if ((rc = read_norms(c, ng, true))) return rc;
@@ -582,7 +591,7 @@ int solve_mixed(dyson_ctx* c, int ncol, int gs, int precision, double tol, int m
       break;
     }
     if (rc) return rc;
-    launch_accumulate(G, d, c->Nr, c->Nc, ncol, c->stream);
+    launch_accumulate(G, d, c->Nr, c->Nc, c->Ns, ncol, c->stream);
     c->launches += 1;
     DY_CUDA(c, cudaMemsetAsync(c->d_norm, 0, (size_t)ng * sizeof(unsigned long long), c->stream));
     if (c->use_oz) {
@@ -593,7 +602,7 @@ int solve_mixed(dyson_ctx* c, int ncol, int gs, int precision, double tol, int m
       if (c->use_oz64) {
         if ((rc = oz64_sweep(c, ncol, gs, G, nullptr, r32, 1))) return rc;
       } else {
-        launch_sweep_f64(c->d_lam, c->d_JW, c->d_nbr, c->d_nbond, G, nullptr, r32, c->d_src_site, c->d_src_time,
+        launch_sweep_f64(c->d_lam, c->d_JW, c->d_nbr, c->d_nbond, G, nullptr, r32, c->Ns, c->d_src_site, c->d_src_time,
                          c->Nr, c->Nc, ncol, gs, 1, c->d_norm, c->stream);
         c->launches += 1;
       }
@@ -722,7 +731,7 @@ int dyson_init(dyson_ctx** out, const dyson_lattice* L, const dyson_contour* C, 
       (e = dalloc(&c->d_nbr, nbr.size())) || (e = dalloc(&c->d_nbond, nbond.size())) ||
       (e = dalloc(&c->d_eps, (size_t)c->Nr)) || (e = dalloc(&c->d_phase, (size_t)c->Nr * (2 * c->Nc + 2))) ||
       (e = dalloc(&c->d_lam, (size_t)c->Nr * NcNc)) || (e = dalloc(&c->d_JW, (size_t)c->Nb * c->Nc)) ||
-      (e = dalloc(&c->d_Jz, (size_t)c->Nb * c->Nc)) || (e = dalloc(&c->d_obs, 3 * (size_t)c->Nr * c->Nt)))
+      (e = dalloc(&c->d_Jz, (size_t)c->Nb * contour_stride(c))) || (e = dalloc(&c->d_obs, 3 * (size_t)c->Nr * c->Nt)))
     return bail(e, "device allocation");
   std::vector<double> nan_obs(3 * (size_t)c->Nr * c->Nt, std::numeric_limits<double>::quiet_NaN());
   if ((e = cudaMemcpyAsync(c->dU, c->U.data(), c->U.size() * 8, cudaMemcpyHostToDevice, c->stream)) ||
@@ -741,7 +750,8 @@ int dyson_build_sigma(dyson_ctx* c) {
   DeviceGuard g(c->device);
   launch_build_sigma(c->dU, c->Lx, c->Ly, c->Nt, c->Nm, c->dt, c->beta, c->curvature, c->mu, c->d_eps,
                      c->d_phase, c->d_lam, c->stream);
-  launch_hopping_tables(c->dJ, c->Nb, c->Nt, c->Nm, c->dt, c->beta, c->d_JW, c->d_Jz, c->stream);
+  launch_hopping_tables(c->dJ, c->Nb, c->Nt, c->Nm, c->dt, c->beta, c->d_JW, c->d_Jz, contour_stride(c),
+                        c->stream);
   c->launches += c->Nb > 0 ? 3 : 2;
   DY_CUDA(c, cudaGetLastError());
   DY_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -779,27 +789,30 @@ int prepare_oz64(dyson_ctx* c) {
   return rc == DYSON_ERR_OOM ? DYSON_OK : rc;
 }
 
-int prepare_tables(dyson_ctx* c, int precision, bool unfused) {
+int prepare_tables(dyson_ctx* c, int precision, bool batch) {
   c->use_tc = c->use_oz = c->use_oz64 = false;
+  c->Ns = c->Nc;
   if (precision == DYSON_PREC_F64) return prepare_oz64(c);
-  const bool tc = c->tc_enabled && tc_supported(c, c->Nc);
+  const bool tc = c->tc_enabled && tc_supported(c);
+  const bool fused = tc && (batch || tc_uses_fused(c));
+  if (tc) c->Ns = contour_stride(c);
   if (!tc && !c->lam32_built) {
     if (!c->d_lam32) DY_CUDA(c, dalloc(&c->d_lam32, (size_t)c->Nr * c->Nc * c->Nc));
     launch_lam_c64(c->d_lam, c->Nr, c->Nt, c->Nm, c->dt, c->beta, c->d_lam32, c->stream);
     c->launches += 1;
     c->lam32_built = true;
   }
-  if (tc && tc_uses_fused(c) && !c->lam16_built) {
-    const size_t n = (size_t)c->Nr * 4 * c->Nc * c->Nc;
+  if (fused && !c->lam16_built) {
+    const size_t n = (size_t)c->Nr * 4 * c->Ns * c->Ns;
     if (!c->d_lam16_hi) DY_CUDA(c, dalloc(&c->d_lam16_hi, n));
     if (!c->d_lam16_lo) DY_CUDA(c, dalloc(&c->d_lam16_lo, n));
-    if (!c->d_a_down) DY_CUDA(c, dalloc(&c->d_a_down, (size_t)c->Nr * 2 * c->Nc));
-    launch_lam_split16(c->d_lam, c->Nr, c->Nt, c->Nm, c->dt, c->beta, c->d_lam16_hi, c->d_lam16_lo, c->d_a_down,
-                       c->stream);
+    if (!c->d_a_down) DY_CUDA(c, dalloc(&c->d_a_down, (size_t)c->Nr * 2 * c->Ns));
+    launch_lam_split16(c->d_lam, c->Nr, c->Nt, c->Nm, c->Ns, c->dt, c->beta, c->d_lam16_hi, c->d_lam16_lo,
+                       c->d_a_down, c->stream);
     c->launches += 1;
     c->lam16_built = true;
   }
-  if (tc && (unfused || !tc_uses_fused(c)) && !c->lam_split_built) {
+  if (tc && !fused && !c->lam_split_built) {
     size_t n = (size_t)c->Nr * 4 * c->Nc * c->Nc;
     if (!c->d_lam_hi) DY_CUDA(c, dalloc(&c->d_lam_hi, n));
     if (!c->d_lam_lo) DY_CUDA(c, dalloc(&c->d_lam_lo, n));
@@ -819,11 +832,11 @@ int prepare_tables(dyson_ctx* c, int precision, bool unfused) {
 // residual or FP64 sweep (*total_per_col: all).
 int64_t chunk_columns(dyson_ctx* c, int precision, int64_t unit, int64_t want, size_t* bytes_per_col,
                       size_t* total_per_col) {
-  const double state = precision == DYSON_PREC_F64 ? 32.0 : 40.0;
-  const double per_el = state + (c->use_tc ? 8.0 : 0.0) + (c->use_oz ? (double)oz_bytes_per_element() : 0.0) +
+  const double state = precision == DYSON_PREC_F64 ? 32.0 : 16.0 + 24.0 * c->Ns / c->Nc;
+  const double per_el = state + (c->use_tc && !tc_uses_fused(c) ? 8.0 : 0.0) + (c->use_oz ? (double)oz_bytes_per_element() : 0.0) +
                         (c->use_oz64 ? oz64_bytes_per_element(c) : 0.0);
   const double col_bytes = per_el * c->Nr * (double)c->Nc;
-  *bytes_per_col = (size_t)(state * c->Nr * (double)c->Nc);
+  *bytes_per_col = (size_t)std::ceil(state * c->Nr * (double)c->Nc);
   if (total_per_col) *total_per_col = (size_t)col_bytes;
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return 0;

@@ -42,9 +42,10 @@ __device__ __forceinline__ void atomic_max_nonneg(unsigned long long* p, double 
 void launch_build_sigma(const double* U, int Lx, int Ly, int Nt, int Nm, double dt, double beta,
                         double curvature, double mu, double* eps, double2* phase,
                         double2* lam, cudaStream_t s);
-// contour hopping weights JW[b][z] = W(z) J_b(t(z)) (complex128) and Jz[b][z] = J_b(t(z)) (fp32)
+// contour hopping weights JW[b][z] = W(z) J_b(t(z)) (complex128) and Jz[b][z] = J_b(t(z)) (fp32,
+// ldj entries per bond, zeros from Nc on)
 void launch_hopping_tables(const double* J, int Nb, int Nt, int Nm, double dt, double beta,
-                           double2* JW, float* Jz, cudaStream_t s);
+                           double2* JW, float* Jz, int ldj, cudaStream_t s);
 // Lambda' = Lambda * W as complex64 (SIMT FP32 path)
 void launch_lam_c64(const double2* lam, int Nr, int Nt, int Nm, double dt, double beta,
                     float2* lam32, cudaStream_t s);
@@ -53,35 +54,36 @@ void launch_lam_c64(const double2* lam, int Nr, int Nt, int Nm, double dt, doubl
 void launch_lam_emb_split(const double2* lam, int Nr, int Nt, int Nm, double dt, double beta,
                           float* hi, float* lo, cudaStream_t s);
 
-// The same embedding as FP16 hi + lo, each row scaled by a power of two to a largest entry in
-// [2^14, 2^15); down [Nr][2Nc]: the inverse powers.
-void launch_lam_split16(const double2* lam, int Nr, int Nt, int Nm, double dt, double beta, __half* hi, __half* lo,
-                        float* down, cudaStream_t s);
+// The same embedding as FP16 hi + lo over Ns >= Nc contour points (zeros beyond Nc), each row scaled
+// by a power of two to a largest entry in [2^14, 2^15); down [Nr][2 Ns]: the inverse powers.
+void launch_lam_split16(const double2* lam, int Nr, int Nt, int Nm, int Ns, double dt, double beta, __half* hi,
+                        __half* lo, float* down, cudaStream_t s);
 
 // transpose every Nc x Nc block of lam in place
 void launch_transpose_blocks(double2* lam, int Nr, int Nc, cudaStream_t s);
 
-// Chunk state: FP64 [Nr][ncol][Nc] complex128, FP32 [Nr][ncol][2Nc] planar.  Vector
+// Chunk state: FP64 [Nr][ncol][Nc] complex128, FP32 [Nr][ncol][2 Ns] planar (real parts at 0, imaginary
+// ones at Ns, zeros from Nc on in each; Ns = Nc on the CUDA-core sweep).  Vector
 // column n has the source (src_site[n], src_time[n]) (site -1: a zero padding column);
 // norms and scales are kept per group of gs consecutive columns (q = n / gs).
 void launch_init_rhs(const double2* lam, const int* src_site, const int* src_time, int Nr, int Nc, int ncol,
                      int gs, double2* G, unsigned long long* scale, cudaStream_t s);
 // K3: out = B + K Gin (mode 0), or B + K Gin - Gin (mode 1); norm[q] = max |out - Gin| (mode 0)
 // or max |out| (mode 1).  If out32 != nullptr (mode 1 only) the result is written as FP32
-// planar state instead of into out.
+// planar state of stride Ns instead of into out.
 void launch_sweep_f64(const double2* lam, const double2* JW, const int* nbr, const int* nbond,
-                      const double2* Gin, double2* out, float* out32, const int* src_site, const int* src_time,
+                      const double2* Gin, double2* out, float* out32, int Ns, const int* src_site, const int* src_time,
                       int Nr, int Nc, int ncol, int gs, int mode, unsigned long long* norm, cudaStream_t s);
 // SIMT FP32 sweep: dout = r + K din over planar FP32 state; norm[q] = max |dout - din|
-void launch_sweep_f32_simt(const float2* lam32, const float* Jz, const int* nbr, const int* nbond,
+void launch_sweep_f32_simt(const float2* lam32, const float* Jz, int ldj, const int* nbr, const int* nbond,
                            const float* r, const float* din, float* dout, int Nr, int Nc, int ncol, int gs,
                            unsigned long long* norm, cudaStream_t s);
 // out[n][j][z] = G[j][n][z] for the first nv vector columns
 void launch_export_vectors(const double2* G, int Nr, int Nc, int ncol, int nv, double2* out, cudaStream_t s);
 // FP64 interleaved state -> FP32 planar state
-void launch_to_planar32(const double2* G, float* out, size_t n_el, int Nc, cudaStream_t s);
+void launch_to_planar32(const double2* G, float* out, size_t columns, int Nc, int Ns, cudaStream_t s);
 // G64 += d32
-void launch_accumulate(double2* G, const float* d, int Nr, int Nc, int ncol, cudaStream_t s);
+void launch_accumulate(double2* G, const float* d, int Nr, int Nc, int Ns, int ncol, cudaStream_t s);
 // observables of the block columns of a chunk
 void launch_observables(const double2* G, const int* src_site, int nq, const int* nbr,
                         const int* nbond, const double* Jtab, const double* eps, const double* U,
@@ -145,13 +147,14 @@ struct dyson_ctx {
   double2* d_phase = nullptr;        // [Nr][2][Nc]
   double2* d_lam = nullptr;          // [Nr][Nc][Nc]
   double2* d_JW = nullptr;           // [Nb][Nc]
-  float* d_Jz = nullptr;             // [Nb][Nc]
+  float* d_Jz = nullptr;             // [Nb][Nc rounded up to 64], zeros from Nc on
   float2* d_lam32 = nullptr;         // [Nr][Nc][Nc] (lazy)
   float* d_lam_hi = nullptr;         // [Nr][2Nc][2Nc] (lazy)
   float* d_lam_lo = nullptr;
-  __half* d_lam16_hi = nullptr;      // [Nr][2Nc][2Nc] FP16 halves of the scaled embedding (fused sweep; lazy)
+  __half* d_lam16_hi = nullptr;      // [Nr][2Ns][2Ns] FP16 halves of the scaled embedding (fused sweep; lazy)
   __half* d_lam16_lo = nullptr;
-  float* d_a_down = nullptr;         // [Nr][2Nc] powers of two that undo the rows' scales
+  float* d_a_down = nullptr;         // [Nr][2Ns] powers of two that undo the rows' scales
+  int Ns = 0;                        // contour stride of the FP32 states of the current solve (contour_stride, or Nc)
   bool lam16_built = false;
   float j_max = 0.f;                 // max |J_b(t_k)|
   TcScale* d_xscale = nullptr;       // [norm_cap] scales of the FP16 X per column group
@@ -174,7 +177,7 @@ struct dyson_ctx {
   bool lam_split_built = false;
   bool tc_enabled = true;            // 3xTF32 tcgen05 sweep allowed where the contour fits it
   bool use_tc = false;               // chosen for the current solve
-  int tc_variant = 0;                // DYSON_SWEEP_SINGLE_CTA or DYSON_SWEEP_CTA_PAIR
+  int tc_variant = -1;               // DYSON_SWEEP_*; -1: none selected, the fused form
   int max_refinements = 12;
   int chunk_override = 0;
   int64_t launches = 0;              // kernels launched by this context since dyson_init

@@ -411,7 +411,7 @@ int gm_prepare(dyson_ctx* c, size_t vsz, int ncol, int m) {
 }  // namespace
 
 int gmres_restart_length(dyson_ctx* c, int ncol) {
-  const size_t vbytes = (size_t)c->Nr * ncol * 2 * c->Nc * sizeof(float);
+  const size_t vbytes = (size_t)c->Nr * ncol * 2 * c->Ns * sizeof(float);
   GmState* st = static_cast<GmState*>(c->gm);
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return 0;
@@ -426,12 +426,12 @@ int gmres_inner_solve(dyson_ctx* c, int ncol, const float* r, float* x, int max_
   if (ncol > 65535 || c->Nr > 65535) return ctx_fail(c, DYSON_ERR_INVALID_ARG, "GMRES chunks hold <= 65535 columns");
   const int m = gmres_restart_length(c, ncol);
   if (m < 2) return ctx_fail(c, DYSON_ERR_OOM, "GMRES needs room for at least 3 Krylov vectors");
-  const size_t vsz = (size_t)c->Nr * ncol * 2 * c->Nc;
+  const size_t vsz = (size_t)c->Nr * ncol * 2 * c->Ns;
   int rc = gm_prepare(c, vsz, ncol, m);
   if (rc) return rc;
   GmState* st = gstate(c);
   cudaStream_t s = c->stream;
-  const int Nc = c->Nc;
+  const int Nc = c->Ns;                                  // (the padding points are zeros)
   const dim3 grid_el(c->Nr, ncol);
   // dot blocks: enough (basis x column x chunk) blocks without tiny chunks
   const int chunks = (int)std::max<int64_t>(1, std::min<int64_t>(c->Nr, 4096 / std::max(1, ncol)));

@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     k_oz64_gemm(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap xmap,
                 const int* __restrict__ esig, const int* __restrict__ etau, const double* __restrict__ Gin,
                 const double2* __restrict__ lam, const int* __restrict__ src_site, const int* __restrict__ src_time,
-                int Nr, int Nc, int KB, int ncol, int gs, double* __restrict__ out, float* __restrict__ r32,
+                int Nr, int Nc, int KB, int ncol, int gs, double* __restrict__ out, float* __restrict__ r32, int Ns,
                 unsigned long long* __restrict__ norm, int* __restrict__ err) {
   using namespace ptx;
   extern __shared__ uint8_t smem_raw[];
@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         const float a = row_ok ? magnitude(d) : 0.f;
         if (row_ok) {
           if (MODE == 0) out[off0 + (size_t)j * N2] = y;
-          else r32[((size_t)site * ncol + n_first + j) * N2 + (m >> 1) + ((m & 1) ? Nc : 0)] = (float)d;
+          else r32[((size_t)site * ncol + n_first + j) * 2 * Ns + (m >> 1) + ((m & 1) ? Ns : 0)] = (float)d;
         }
         const float a2 = a * a;
         sq = fmaxf(sq, a2 + __shfl_xor_sync(0xffffffffu, a2, 1));
@@ -631,7 +631,7 @@ int oz64_sweep(dyson_ctx* c, int ncol, int gs, const double2* Gin, double2* out,
   auto go = [&](auto kernel) {
     kernel<<<grid, THREADS, SMEM_BYTES, c->stream>>>(
         st->amap, st->xmap, st->esig, st->etau, reinterpret_cast<const double*>(Gin), c->d_lam, c->d_src_site,
-        c->d_src_time, Nr, Nc, Kp / BK, ncol, gs, reinterpret_cast<double*>(out), r32, c->d_norm, st->d_err);
+        c->d_src_time, Nr, Nc, Kp / BK, ncol, gs, reinterpret_cast<double*>(out), r32, c->Ns, c->d_norm, st->d_err);
   };
   if (mode == 0) go(k_oz64_gemm<0>);
   else go(k_oz64_gemm<1>);

@@ -86,15 +86,18 @@ __global__ void k_lambda(const double2* __restrict__ phase, int Nt, int Nm, doub
 }
 
 __global__ void k_hopping(const double* __restrict__ J, int Nb, int Nt, int Nm, double dt, double beta,
-                          double2* __restrict__ JW, float* __restrict__ Jz) {
+                          double2* __restrict__ JW, float* __restrict__ Jz, int ldj) {
   int Nc = 2 * Nt + Nm;
   int z = blockIdx.x * blockDim.x + threadIdx.x;
   int b = blockIdx.y;
-  if (z >= Nc) return;
+  if (z >= Nc) {
+    if (z < ldj) Jz[(size_t)b * ldj + z] = 0.f;
+    return;
+  }
   double j = J[(size_t)b * Nt + time_of(z, Nt)];
   double2 w = weight_of(z, Nt, Nm, dt, beta);
   JW[(size_t)b * Nc + z] = make_double2(w.x * j, w.y * j);
-  Jz[(size_t)b * Nc + z] = (float)j;
+  Jz[(size_t)b * ldj + z] = (float)j;
 }
 
 __global__ void k_lam_c64(const double2* __restrict__ lam, int Nt, int Nm, double dt, double beta,
@@ -132,48 +135,51 @@ __global__ void k_lam_emb_split(const double2* __restrict__ lam, int Nt, int Nm,
   }
 }
 
-// One warp per (site, contour row z): the embedding's rows z (Re, -Im) and z + Nc (Im, Re) share
+// One warp per (site, contour row z): the embedding's rows z (Re, -Im) and z + Ns (Im, Re) share
 // their scale; each lane takes two neighbouring columns, so that the four FP16 planes are written
 // as 128-byte lines.
-__global__ void __launch_bounds__(256) k_lam_split16(const double2* __restrict__ lam, int Nr, int Nt, int Nm, double dt,
-                                                     double beta, __half* __restrict__ hi, __half* __restrict__ lo,
-                                                     float* __restrict__ down) {
-  const int Nc = 2 * Nt + Nm, N2 = 2 * Nc;
+__global__ void __launch_bounds__(256) k_lam_split16(const double2* __restrict__ lam, int Nr, int Nt, int Nm, int Ns,
+                                                     double dt, double beta, __half* __restrict__ hi,
+                                                     __half* __restrict__ lo, float* __restrict__ down) {
+  const int Nc = 2 * Nt + Nm, N2 = 2 * Ns;
   const size_t row = (size_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
   const int lane = threadIdx.x & 31;
-  if (row >= (size_t)Nr * Nc) return;
-  const size_t i = row / Nc;
-  const int z = (int)(row % Nc);
-  const double2* lrow = lam + row * Nc;
+  if (row >= (size_t)Nr * Ns) return;
+  const size_t i = row / Ns;
+  const int z = (int)(row % Ns);
+  const double2* lrow = lam + (i * Nc + (z < Nc ? z : 0)) * Nc;
+  auto value = [&](int k) {
+    return z < Nc && k < Nc ? cmul(lrow[k], weight_of(k, Nt, Nm, dt, beta)) : make_double2(0.0, 0.0);
+  };
   unsigned int mb = 0;                                   // high words of |re|, |im|: their order is the values' order
   for (int k = lane; k < Nc; k += 32) {
-    const double2 v = cmul(lrow[k], weight_of(k, Nt, Nm, dt, beta));
+    const double2 v = value(k);
     mb = max(mb, max((unsigned)__double2hiint(v.x) & 0x7FFFFFFFu, (unsigned)__double2hiint(v.y) & 0x7FFFFFFFu));
   }
   mb = __reduce_max_sync(0xffffffffu, mb);
   // largest entry in [2^e, 2^(e+1)); clamped so that the scale and its inverse are normal FP32 numbers
   const int e = max(-100, min(100, (int)(mb >> 20) - 1023));
   const double up = ldexp(1.0, 14 - e);
-  const size_t r0 = i * N2 + z, r1 = r0 + Nc;
+  const size_t r0 = i * N2 + z, r1 = r0 + Ns;
   if (lane == 0) down[r0] = down[r1] = ldexpf(1.f, e - 14);
   auto split = [](double x, __half* h, __half* l) {
     *h = __float2half_rn((float)x);
     *l = __float2half_rn((float)(x - (double)__half2float(*h)));
   };
-  for (int k = 2 * lane; k < Nc; k += 64) {              // Nc is even here (a multiple of 64)
+  for (int k = 2 * lane; k < Ns; k += 64) {              // Ns is a multiple of 64
     __half h[4], l[4];                                   // re, im of the two columns
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-      const double2 v = cmul(lrow[k + u], weight_of(k + u, Nt, Nm, dt, beta));
+      const double2 v = value(k + u);
       split(v.x * up, &h[2 * u], &l[2 * u]);
       split(v.y * up, &h[2 * u + 1], &l[2 * u + 1]);
     }
     auto put = [&](__half* dst, const __half* p) {
       const __half2 re = __halves2half2(p[0], p[2]), im = __halves2half2(p[1], p[3]);
       *reinterpret_cast<__half2*>(dst + r0 * N2 + k) = re;
-      *reinterpret_cast<__half2*>(dst + r0 * N2 + Nc + k) = __hneg2(im);
+      *reinterpret_cast<__half2*>(dst + r0 * N2 + Ns + k) = __hneg2(im);
       *reinterpret_cast<__half2*>(dst + r1 * N2 + k) = im;
-      *reinterpret_cast<__half2*>(dst + r1 * N2 + Nc + k) = re;
+      *reinterpret_cast<__half2*>(dst + r1 * N2 + Ns + k) = re;
     };
     put(hi, h);
     put(lo, l);
@@ -220,10 +226,9 @@ void launch_build_sigma(const double* U, int Lx, int Ly, int Nt, int Nm, double 
 }
 
 void launch_hopping_tables(const double* J, int Nb, int Nt, int Nm, double dt, double beta, double2* JW,
-                           float* Jz, cudaStream_t s) {
+                           float* Jz, int ldj, cudaStream_t s) {
   if (Nb == 0) return;
-  int Nc = 2 * Nt + Nm;
-  k_hopping<<<dim3((Nc + 127) / 128, Nb), 128, 0, s>>>(J, Nb, Nt, Nm, dt, beta, JW, Jz);
+  k_hopping<<<dim3((ldj + 127) / 128, Nb), 128, 0, s>>>(J, Nb, Nt, Nm, dt, beta, JW, Jz, ldj);
 }
 
 void launch_lam_c64(const double2* lam, int Nr, int Nt, int Nm, double dt, double beta, float2* lam32,
@@ -240,10 +245,10 @@ void launch_lam_emb_split(const double2* lam, int Nr, int Nt, int Nm, double dt,
   k_lam_emb_split<<<grid_for(total, 256), 256, 0, s>>>(lam, Nt, Nm, dt, beta, hi, lo, Nr);
 }
 
-void launch_lam_split16(const double2* lam, int Nr, int Nt, int Nm, double dt, double beta, __half* hi, __half* lo,
-                        float* down, cudaStream_t s) {
-  const size_t rows = (size_t)Nr * (2 * Nt + Nm);
-  k_lam_split16<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(lam, Nr, Nt, Nm, dt, beta, hi, lo, down);
+void launch_lam_split16(const double2* lam, int Nr, int Nt, int Nm, int Ns, double dt, double beta, __half* hi,
+                        __half* lo, float* down, cudaStream_t s) {
+  const size_t rows = (size_t)Nr * Ns;
+  k_lam_split16<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(lam, Nr, Nt, Nm, Ns, dt, beta, hi, lo, down);
 }
 
 void launch_transpose_blocks(double2* lam, int Nr, int Nc, cudaStream_t s) {

@@ -47,7 +47,7 @@ template <int MODE>
 __global__ __launch_bounds__(256) void k_sweep_f64(
     const double2* __restrict__ lam, const double2* __restrict__ JW, const int* __restrict__ nbr,
     const int* __restrict__ nbond, const double2* __restrict__ Gin, double2* __restrict__ out,
-    float* __restrict__ out32, const int* __restrict__ src_site, const int* __restrict__ src_time, int Nc,
+    float* __restrict__ out32, int Ns, const int* __restrict__ src_site, const int* __restrict__ src_time, int Nc,
     int ncol, int gs, unsigned long long* __restrict__ norm) {
   constexpr int KT = 16;
   __shared__ double2 As[TZ][KT + 1];
@@ -139,9 +139,9 @@ __global__ __launch_bounds__(256) void k_sweep_f64(
           if (MODE == 0) {
             out[off] = y;
           } else if (out32) {
-            size_t o2 = ((size_t)i * ncol + n) * (2 * Nc) + z;
+            size_t o2 = ((size_t)i * ncol + n) * (2 * Ns) + z;
             out32[o2] = (float)dx;
-            out32[o2 + Nc] = (float)dy;
+            out32[o2 + Ns] = (float)dy;
           } else {
             out[off] = make_double2(dx, dy);
           }
@@ -163,7 +163,7 @@ __global__ __launch_bounds__(256) void k_sweep_f64(
 // SIMT FP32 sweep over planar state: dout = r + Lambda' X, Lambda' = Lambda * W (complex64),
 // X(n, zb) = sum_j J_ij(zb) din_j(n, zb).  norm[q] = max |dout - din|.
 __global__ __launch_bounds__(256) void k_sweep_f32_simt(
-    const float2* __restrict__ lam32, const float* __restrict__ Jz, const int* __restrict__ nbr,
+    const float2* __restrict__ lam32, const float* __restrict__ Jz, int ldj, const int* __restrict__ nbr,
     const int* __restrict__ nbond, const float* __restrict__ r, const float* __restrict__ din,
     float* __restrict__ dout, int Nc, int ncol, int gs, unsigned long long* __restrict__ norm) {
   constexpr int KT = 32;
@@ -202,7 +202,7 @@ __global__ __launch_bounds__(256) void k_sweep_f32_simt(
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
           if (nb[s] >= 0) {
-            float j = Jz[(size_t)bd[s] * Nc + k];
+            float j = Jz[(size_t)bd[s] * ldj + k];
             const float* g = din + ((size_t)nb[s] * ncol + n) * N2;
             xr = fmaf(j, g[k], xr);
             xi = fmaf(j, g[Nc + k], xi);
@@ -282,25 +282,26 @@ __global__ void k_init_rhs(const double2* __restrict__ lam, const int* __restric
   if (lane == 0) atomicMax(scale + n / gs, nonneg_bits(m));
 }
 
-__global__ void k_accumulate(double2* __restrict__ G, const float* __restrict__ d, int Nc, size_t total) {
+__global__ void k_accumulate(double2* __restrict__ G, const float* __restrict__ d, int Nc, int Ns, size_t total) {
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
     size_t col = e / Nc;
     int z = (int)(e - col * Nc);
-    const float* dc = d + col * 2 * Nc;
+    const float* dc = d + col * 2 * Ns;
     double2 g = G[e];
     g.x += (double)dc[z];
-    g.y += (double)dc[Nc + z];
+    g.y += (double)dc[Ns + z];
     G[e] = g;
   }
 }
 
-__global__ void k_to_planar32(const double2* __restrict__ G, float* __restrict__ out, int Nc, size_t total) {
+// (the padding points Nc .. Ns - 1 of a column are written as zeros)
+__global__ void k_to_planar32(const double2* __restrict__ G, float* __restrict__ out, int Nc, int Ns, size_t total) {
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-    size_t col = e / Nc;
-    int z = (int)(e - col * Nc);
-    double2 g = G[e];
-    out[col * 2 * Nc + z] = (float)g.x;
-    out[col * 2 * Nc + Nc + z] = (float)g.y;
+    size_t col = e / Ns;
+    int z = (int)(e - col * Ns);
+    double2 g = z < Nc ? G[col * Nc + z] : make_double2(0.0, 0.0);
+    out[col * 2 * Ns + z] = (float)g.x;
+    out[col * 2 * Ns + Ns + z] = (float)g.y;
   }
 }
 
@@ -384,22 +385,22 @@ void launch_init_rhs(const double2* lam, const int* src_site, const int* src_tim
 }
 
 void launch_sweep_f64(const double2* lam, const double2* JW, const int* nbr, const int* nbond,
-                      const double2* Gin, double2* out, float* out32, const int* src_site, const int* src_time,
+                      const double2* Gin, double2* out, float* out32, int Ns, const int* src_site, const int* src_time,
                       int Nr, int Nc, int ncol, int gs, int mode, unsigned long long* norm, cudaStream_t s) {
   dim3 grd((ncol + TN - 1) / TN, (Nc + TZ - 1) / TZ, Nr);
   if (mode == 0)
-    k_sweep_f64<0><<<grd, 256, 0, s>>>(lam, JW, nbr, nbond, Gin, out, nullptr, src_site, src_time, Nc, ncol, gs,
-                                       norm);
+    k_sweep_f64<0><<<grd, 256, 0, s>>>(lam, JW, nbr, nbond, Gin, out, nullptr, Nc, src_site, src_time, Nc, ncol,
+                                       gs, norm);
   else
-    k_sweep_f64<1><<<grd, 256, 0, s>>>(lam, JW, nbr, nbond, Gin, out, out32, src_site, src_time, Nc, ncol, gs,
+    k_sweep_f64<1><<<grd, 256, 0, s>>>(lam, JW, nbr, nbond, Gin, out, out32, Ns, src_site, src_time, Nc, ncol, gs,
                                        norm);
 }
 
-void launch_sweep_f32_simt(const float2* lam32, const float* Jz, const int* nbr, const int* nbond,
+void launch_sweep_f32_simt(const float2* lam32, const float* Jz, int ldj, const int* nbr, const int* nbond,
                            const float* r, const float* din, float* dout, int Nr, int Nc, int ncol, int gs,
                            unsigned long long* norm, cudaStream_t s) {
   dim3 grd((ncol + TN - 1) / TN, (Nc + TZ - 1) / TZ, Nr);
-  k_sweep_f32_simt<<<grd, 256, 0, s>>>(lam32, Jz, nbr, nbond, r, din, dout, Nc, ncol, gs, norm);
+  k_sweep_f32_simt<<<grd, 256, 0, s>>>(lam32, Jz, ldj, nbr, nbond, r, din, dout, Nc, ncol, gs, norm);
 }
 
 void launch_export_vectors(const double2* G, int Nr, int Nc, int ncol, int nv, double2* out, cudaStream_t s) {
@@ -407,13 +408,13 @@ void launch_export_vectors(const double2* G, int Nr, int Nc, int ncol, int nv, d
   k_export_vectors<<<grid_for(total, 256), 256, 0, s>>>(G, Nr, Nc, ncol, nv, out);
 }
 
-void launch_accumulate(double2* G, const float* d, int Nr, int Nc, int ncol, cudaStream_t s) {
-  size_t total = (size_t)Nr * ncol * Nc;
-  k_accumulate<<<grid_for(total, 256), 256, 0, s>>>(G, d, Nc, total);
+void launch_accumulate(double2* G, const float* d, int Nr, int Nc, int Ns, int ncol, cudaStream_t s) {
+  const size_t total = (size_t)Nr * ncol * Nc;
+  k_accumulate<<<grid_for(total, 256), 256, 0, s>>>(G, d, Nc, Ns, total);
 }
 
-void launch_to_planar32(const double2* G, float* out, size_t n_el, int Nc, cudaStream_t s) {
-  k_to_planar32<<<grid_for(n_el, 256), 256, 0, s>>>(G, out, Nc, n_el);
+void launch_to_planar32(const double2* G, float* out, size_t columns, int Nc, int Ns, cudaStream_t s) {
+  k_to_planar32<<<grid_for(columns * Ns, 256), 256, 0, s>>>(G, out, Nc, Ns, columns * Ns);
 }
 
 void launch_observables(const double2* G, const int* src_site, int nq, const int* nbr, const int* nbond,

@@ -57,7 +57,6 @@ struct TcState {
   CUtensorMap a_hi, a_lo, x;
   const float* a_hi_ptr = nullptr;
   const float* a_lo_ptr = nullptr;
-  int a_Nr = 0, a_Nc = 0;
   const float* x_ptr = nullptr;
   int x_ncol = -1;
   float* xbuf = nullptr;
@@ -72,15 +71,11 @@ struct TcState {
   const float* xh_ptr = nullptr;
   int pair_clusters = -1;
   // fused gather + GEMM (k_tc_fused<GT>): maps of the FP16 Lambda halves, co-resident clusters
-  // per GT (-1: not yet asked)
+  // (-1: not yet asked)
   CUtensorMap h_hi, h_lo;
   const void* h_hi_ptr = nullptr;
   const void* h_lo_ptr = nullptr;
-  int fused_clusters[2] = {-1, -1};
-  // one-entry instance table of the single-context sweep (pinned host copy and device copy)
-  TcInst* h_inst = nullptr;
-  TcInst* d_inst = nullptr;
-  bool inst_valid = false;
+  int fused_clusters = -1;
 };
 
 // Round to TF32 (10 explicit mantissa bits), to nearest with ties away from zero,
@@ -98,30 +93,13 @@ __device__ __forceinline__ unsigned long long nonneg_bits(float v) {
 
 // ---------------------------------------------------------------------------
 // gather: X[i][n][k] = sum_j J_ij(k mod Nc) d_j[n][k]
-// grid: the instances' blocks back to back; within an instance one CTA per
-// (block of 16 vector columns, site), column block outermost
+// grid: one CTA per (block of 16 vector columns, site), column block outermost
 // ---------------------------------------------------------------------------
 constexpr int GATHER_COLS = 16;
 
-// the instance whose range [key0, next key0) holds t (keys ascending, first key 0)
-template <int FIELD>
-__device__ __forceinline__ int find_inst(const TcInst* __restrict__ tab, int n, int t) {
-  int lo = 0, hi = n - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    const int key = FIELD == 0 ? tab[mid].tile0 : tab[mid].gblk0;
-    if (key <= t) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
-}
-
-__device__ __forceinline__ bool inst_active(const TcInst& I) { return I.active == nullptr || *I.active != 0; }
-
-// single instance: pointers and sizes as kernel parameters (32 registers, 8 blocks per SM)
 // act (optional, [Nr][column tiles of BN]): the first sweep at which the tile can
 // be non-zero; blocks of later tiles are skipped (support truncation)
-__global__ __launch_bounds__(256) void k_tc_gather_one(const float* __restrict__ din, const float* __restrict__ Jz,
+__global__ __launch_bounds__(256) void k_tc_gather(const float* __restrict__ din, const float* __restrict__ Jz,
                                                        const int* __restrict__ nbr, const int* __restrict__ nbond,
                                                        float* __restrict__ X, int Nr, int Nc, int ncol,
                                                        const int* __restrict__ act, int sweep) {
@@ -154,58 +132,6 @@ __global__ __launch_bounds__(256) void k_tc_gather_one(const float* __restrict__
       acc.w = fmaf(j.w, g.w, acc.w);
     }
     *reinterpret_cast<float4*>(X + ((size_t)i * ncol + n) * N2 + k) = acc;
-  }
-}
-
-// batched: the instance table; an instance's blocks follow the previous instance's
-__global__ __launch_bounds__(256) void k_tc_gather(const TcInst* __restrict__ tab, int ninst, int parity) {
-  // the instance's pointers and this site's neighbours, read once per block
-  __shared__ const float* s_din;
-  __shared__ const float* s_Jz;
-  __shared__ float* s_X;
-  __shared__ int s_nb[4], s_bd[4], s_dim[4];
-  if (threadIdx.x == 0) {
-    const TcInst& I = tab[find_inst<1>(tab, ninst, blockIdx.x)];
-    const bool act = inst_active(I);
-    const int b = blockIdx.x - I.gblk0;
-    const int i = b % I.Nr;
-    s_din = I.buf[parity];
-    s_Jz = I.Jz;
-    s_X = I.X;
-    s_dim[0] = act ? I.Nc : 0;
-    s_dim[1] = I.ncol;
-    s_dim[2] = i;
-    s_dim[3] = b / I.Nr;
-    for (int q = 0; q < 4; ++q) {
-      s_nb[q] = I.nbr[i * 4 + q];
-      s_bd[q] = I.nbond[i * 4 + q];
-    }
-  }
-  __syncthreads();
-  const int Nc = s_dim[0];
-  if (Nc == 0) return;                                  // converged instance
-  const int ncol = s_dim[1], i = s_dim[2], nblk = s_dim[3];
-  const int N2 = 2 * Nc;
-  const int per_col4 = N2 / 4;
-  const int total4 = GATHER_COLS * per_col4;
-  for (int e = threadIdx.x; e < total4; e += blockDim.x) {
-    int c = e / per_col4, k = (e - c * per_col4) * 4;
-    int n = nblk * GATHER_COLS + c;
-    if (n >= ncol) break;
-    int kz = k < Nc ? k : k - Nc;
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-      const int nb = s_nb[s];
-      if (nb < 0) continue;
-      float4 j = *reinterpret_cast<const float4*>(s_Jz + (size_t)s_bd[s] * Nc + kz);
-      float4 g = *reinterpret_cast<const float4*>(s_din + ((size_t)nb * ncol + n) * N2 + k);
-      acc.x = fmaf(j.x, g.x, acc.x);
-      acc.y = fmaf(j.y, g.y, acc.y);
-      acc.z = fmaf(j.z, g.z, acc.z);
-      acc.w = fmaf(j.w, g.w, acc.w);
-    }
-    *reinterpret_cast<float4*>(s_X + ((size_t)i * ncol + n) * N2 + k) = acc;
   }
 }
 
@@ -318,38 +244,30 @@ __device__ __forceinline__ void epilogue_rows(uint32_t tacc, int mg, int n_first
 }
 
 // ---------------------------------------------------------------------------
-// persistent GEMM + epilogue over the tiles of every instance of the table
+// persistent GEMM + epilogue of the single-CTA form
 // ---------------------------------------------------------------------------
-// One 128 x 256 output tile of an instance, as every warp role decodes it.
+// One 128 x 256 output tile, as every warp role decodes it.
 struct TileRef {
-  const TcInst* I;
-  int k;                             // instance index (its tensor maps are maps.*[k])
-  int KB, mt, nt, site;
+  int mt, nt, site;
   bool active;
 };
 
-// act/sweep: support truncation of a one-entry table (tiles whose act entry exceeds
-// the sweep hold zeros and are skipped), act == nullptr: none
-__device__ __forceinline__ TileRef decode_tile(const TcInst* __restrict__ tab, int ninst, int tile,
-                                               const int* __restrict__ act, int sweep) {
+// act/sweep: support truncation (tiles whose act entry exceeds the sweep hold zeros and are
+// skipped), act == nullptr: none
+__device__ __forceinline__ TileRef decode_tile(int tile, int MT, int NT, const int* __restrict__ act, int sweep) {
   TileRef T;
-  T.k = find_inst<0>(tab, ninst, tile);
-  T.I = &tab[T.k];
-  const int Nc = T.I->Nc;
-  const int MT = (2 * Nc) / BM, NT = (T.I->ncol + BN - 1) / BN;
-  const int lt = tile - T.I->tile0;
-  T.KB = (2 * Nc) / BK;
-  T.mt = lt % MT;
-  T.nt = (lt / MT) % NT;
-  T.site = lt / (MT * NT);
-  T.active = inst_active(*T.I) && !(act && act[T.site * NT + T.nt] > sweep);
+  T.mt = tile % MT;
+  T.nt = (tile / MT) % NT;
+  T.site = tile / (MT * NT);
+  T.active = !(act && act[T.site * NT + T.nt] > sweep);
   return T;
 }
 
-template <int MAXI>
 __global__ void __launch_bounds__(THREADS, 1)
-    k_tc_gemm(const __grid_constant__ TcMaps<MAXI> maps, const TcInst* __restrict__ tab, int ninst, int tiles,
-              int parity, int* __restrict__ err, const int* __restrict__ act, int sweep) {
+    k_tc_gemm(const __grid_constant__ CUtensorMap map_ahi, const __grid_constant__ CUtensorMap map_alo,
+              const __grid_constant__ CUtensorMap map_x, const float* __restrict__ r, const float* __restrict__ din,
+              float* __restrict__ dout, int Nr, int Nc, int ncol, int gs, unsigned long long* __restrict__ norm,
+              int* __restrict__ err, const int* __restrict__ act, int sweep) {
   using namespace ptx;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -359,6 +277,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   __shared__ WaitCtl wctl;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int KB = (2 * Nc) / BK, MT = (2 * Nc) / BM, NT = (ncol + BN - 1) / BN;
+  const int tiles = MT * NT * Nr;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -388,20 +308,17 @@ __global__ void __launch_bounds__(THREADS, 1)
       int g = 0;                                        // k-blocks issued by this CTA
       bool ok = true;
       for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
-        const TileRef T = decode_tile(tab, ninst, tile, act, sweep);
+        const TileRef T = decode_tile(tile, MT, NT, act, sweep);
         if (!T.active) continue;
-        const CUtensorMap* ma_hi = &maps.a_hi[T.k];
-        const CUtensorMap* ma_lo = &maps.a_lo[T.k];
-        const CUtensorMap* mx = &maps.x[T.k];
         // the next active tile of this CTA, for the L2 prefetch that runs ahead of the loads
         int t2 = tile + (int)gridDim.x;
         TileRef N;
         N.active = false;
         for (; t2 < tiles; t2 += gridDim.x) {
-          N = decode_tile(tab, ninst, t2, act, sweep);
+          N = decode_tile(t2, MT, NT, act, sweep);
           if (N.active) break;
         }
-        for (int kb = 0; kb < T.KB; ++kb, ++g) {
+        for (int kb = 0; kb < KB; ++kb, ++g) {
           const int s = g % STAGES;
           if (g >= STAGES && !mbar_wait(&empty[s], ((g / STAGES) - 1) & 1, abort_p)) {
             ok = false;
@@ -409,21 +326,21 @@ __global__ void __launch_bounds__(THREADS, 1)
           }
           uint8_t* st = stage_ptr(s);
           mbar_expect_tx(&full_tma[s], TMA_BYTES);
-          tma_load_3d(st, ma_hi, &full_tma[s], kb * BK, T.mt * BM, T.site);
-          tma_load_3d(st + A_TILE, ma_lo, &full_tma[s], kb * BK, T.mt * BM, T.site);
-          tma_load_3d(st + 2 * A_TILE, mx, &full_tma[s], kb * BK, T.nt * BN, T.site);
+          tma_load_3d(st, &map_ahi, &full_tma[s], kb * BK, T.mt * BM, T.site);
+          tma_load_3d(st + A_TILE, &map_alo, &full_tma[s], kb * BK, T.mt * BM, T.site);
+          tma_load_3d(st + 2 * A_TILE, &map_x, &full_tma[s], kb * BK, T.nt * BN, T.site);
           // warm L2 with the tiles of the k-block PREFETCH steps ahead: the stage
           // loads then see L2 latency instead of DRAM latency
           const int ahead = kb + PREFETCH;
-          if (ahead < T.KB) {
-            tma_prefetch_3d(ma_hi, ahead * BK, T.mt * BM, T.site);
-            tma_prefetch_3d(ma_lo, ahead * BK, T.mt * BM, T.site);
-            tma_prefetch_3d(mx, ahead * BK, T.nt * BN, T.site);
-          } else if (N.active && ahead - T.KB < N.KB) {
-            const int k2 = ahead - T.KB;
-            tma_prefetch_3d(&maps.a_hi[N.k], k2 * BK, N.mt * BM, N.site);
-            tma_prefetch_3d(&maps.a_lo[N.k], k2 * BK, N.mt * BM, N.site);
-            tma_prefetch_3d(&maps.x[N.k], k2 * BK, N.nt * BN, N.site);
+          if (ahead < KB) {
+            tma_prefetch_3d(&map_ahi, ahead * BK, T.mt * BM, T.site);
+            tma_prefetch_3d(&map_alo, ahead * BK, T.mt * BM, T.site);
+            tma_prefetch_3d(&map_x, ahead * BK, T.nt * BN, T.site);
+          } else if (N.active && ahead - KB < KB) {
+            const int k2 = ahead - KB;
+            tma_prefetch_3d(&map_ahi, k2 * BK, N.mt * BM, N.site);
+            tma_prefetch_3d(&map_alo, k2 * BK, N.mt * BM, N.site);
+            tma_prefetch_3d(&map_x, k2 * BK, N.nt * BN, N.site);
           }
         }
       }
@@ -437,14 +354,14 @@ __global__ void __launch_bounds__(THREADS, 1)
       int g = 0, t = 0;
       bool ok = true, any = false;
       for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
-        const TileRef T = decode_tile(tab, ninst, tile, act, sweep);
+        const TileRef T = decode_tile(tile, MT, NT, act, sweep);
         if (!T.active) continue;
         const int buf = t & 1;
         if (t >= 2 && !mbar_wait(&acc_empty[buf], ((t >> 1) - 1) & 1, abort_p)) break;
         ++t;
         tc_fence_after();
         const uint32_t dacc = tmem + (uint32_t)(buf * ACC_COLS);
-        for (int kb = 0; kb < T.KB; ++kb, ++g) {
+        for (int kb = 0; kb < KB; ++kb, ++g) {
           const int s = g % STAGES;
           if (!mbar_wait(&full_split[s], (g / STAGES) & 1, abort_p)) {
             ok = false;
@@ -480,9 +397,9 @@ __global__ void __launch_bounds__(THREADS, 1)
     int g = 0;
     bool ok = true;
     for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
-      const TileRef T = decode_tile(tab, ninst, tile, act, sweep);
+      const TileRef T = decode_tile(tile, MT, NT, act, sweep);
       if (!T.active) continue;
-      for (int kb = 0; kb < T.KB; ++kb, ++g) {
+      for (int kb = 0; kb < KB; ++kb, ++g) {
         const int s = g % STAGES;
         if (!mbar_wait(&full_tma[s], (g / STAGES) & 1, abort_p)) {
           ok = false;
@@ -498,7 +415,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     const int q4 = warp - 8;                            // TMEM lane quarter (warp % 4)
     int t = 0;
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-      const TileRef T = decode_tile(tab, ninst, tile, act, sweep);
+      const TileRef T = decode_tile(tile, MT, NT, act, sweep);
       if (!T.active) continue;
       const int buf = t & 1;
       bool go = mbar_wait(&acc_full[buf], (t >> 1) & 1, abort_p);
@@ -506,10 +423,8 @@ __global__ void __launch_bounds__(THREADS, 1)
       go = __all_sync(0xffffffffu, go);                 // tcgen05.ld below is warp-collective
       if (!go) break;
       tc_fence_after();
-      const TcInst& I = *T.I;
       epilogue_rows(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(buf * ACC_COLS), T.mt * BM + q4 * 32 + lane,
-                    T.nt * BN, T.site, I.ncol, I.gs, 2 * (size_t)I.Nc, I.r, I.buf[parity], I.buf[parity ^ 1],
-                    I.norm, lane);
+                    T.nt * BN, T.site, ncol, gs, 2 * (size_t)Nc, r, din, dout, norm, lane);
       // this accumulator may be overwritten by the MMAs of tile t + 2
       tc_fence_before();
       mbar_arrive(&acc_empty[buf]);
@@ -809,19 +724,32 @@ __device__ __forceinline__ int band_site(int v, int Lx, int Ly) {
   return (y0 + w % h) * Lx + w / h;
 }
 
+// A tile as every warp role decodes it.
 struct FTile {
   int site, nt, gt;
   bool active;
 };
-// (act has one entry per site and TC_TILE_COLS columns, nact of them a site)
-template <int NB>
-__device__ __forceinline__ FTile fused_tile(int tile, int NGT, int NT, int Lx, int Ly, const int* __restrict__ act,
-                                            int nact, int sweep) {
+
+// 256-row tiles of one accumulator
+template <int GT>
+__host__ __device__ __forceinline__ int fused_row_tiles(int Ns) {
+  return ((GT == 2 ? Ns : 2 * Ns) + PM - 1) / PM;
+}
+
+// (act has one entry per site and TC_TILE_COLS columns)
+template <int GT>
+__device__ __forceinline__ FTile fused_tile(const FusedInst& I, int tile, int sweep) {
+  constexpr int NB = FusedCfg<GT>::NB;
   FTile T;
+  const int NGT = fused_row_tiles<GT>(I.Ns), NT = (I.ncol + NB - 1) / NB;
   T.gt = tile % NGT;
   T.nt = (tile / NGT) % NT;
-  T.site = band_site(tile / (NGT * NT), Lx, Ly);
-  T.active = !(act && act[T.site * nact + T.nt / (TC_TILE_COLS / NB)] > sweep);
+  T.site = band_site(tile / (NGT * NT), I.Lx, I.Ly);
+  T.active = true;
+  if (I.act) {
+    const int nact = (I.ncol + TC_TILE_COLS - 1) / TC_TILE_COLS;
+    T.active = I.act[T.site * nact + T.nt / (TC_TILE_COLS / NB)] <= sweep;
+  }
   return T;
 }
 
@@ -829,8 +757,9 @@ __device__ __forceinline__ FTile fused_tile(int tile, int NGT, int NT, int Lx, i
 // accumulators hold 2^(a + x) times the product, the row's and the column group's powers of two:
 // y = r + acc adown sc[q].down; y is stored, max|y - d_in| folded into norm[] and max|y| into
 // sc[].ymax (for the next sweep's scale) per group of gs columns.  The loads of r and d_in run one
-// chunk ahead, the first ones before the accumulators are complete: a chunk costs no DRAM latency.
-// RZERO: r is zero on this tile.
+// chunk ahead, the first ones before the accumulators are complete.  (Three chunks of 8 columns ahead,
+// or a ring of four 8-column slots in shared memory filled by bulk copies, took 2.5-2.7 ms per sweep
+// where this takes 2.1: 16x16, Nc = 256, 4096 columns.)  RZERO: r is zero on this tile.
 template <int GT, bool RZERO>
 struct FusedEpilogue {
   static constexpr int NB = FusedCfg<GT>::NB, CH = 16, PER = NB / CH, CHUNKS = GT * PER;
@@ -846,16 +775,26 @@ struct FusedEpilogue {
   }
   template <int B>
   __device__ __forceinline__ void load(int e) {
-    if (n_first + (e % PER) * CH >= ncol) return;        // warp-uniform (ncol is a multiple of 32)
+    const int left = ncol - n_first - (e % PER) * CH;    // warp-uniform
+    if (left <= 0) return;
     const size_t o = at(e);
+    if (left >= CH) {
 #pragma unroll
-    for (int j = 0; j < CH; ++j) {
-      if (!RZERO) rv[B][j] = __ldcs(r + o + (size_t)j * N2);
-      dv[B][j] = __ldcs(din + o + (size_t)j * N2);
+      for (int j = 0; j < CH; ++j) {
+        if (!RZERO) rv[B][j] = __ldcs(r + o + (size_t)j * N2);
+        dv[B][j] = __ldcs(din + o + (size_t)j * N2);
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < CH; ++j)
+        if (j < left) {
+          if (!RZERO) rv[B][j] = __ldcs(r + o + (size_t)j * N2);
+          dv[B][j] = __ldcs(din + o + (size_t)j * N2);
+        }
     }
   }
   float runmax = 0.f, ymax = 0.f, down = 0.f;
-  int qcur = -1;
+  int qcur = -1, qbeg = 0, qend = 0;                     // current norm group and its columns
   __device__ __forceinline__ void flush(unsigned long long* norm, TcScale* sc, int lane) {
     const unsigned int m = __reduce_max_sync(0xffffffffu, __float_as_uint(runmax));
     if (lane == 0) atomicMax(norm + qcur, nonneg_bits(__uint_as_float(m)));
@@ -867,37 +806,56 @@ struct FusedEpilogue {
                                         TcScale* sc, int lane) {
     const int n0 = n_first + (e % PER) * CH;
     if (n0 >= ncol) return;
-    const int q = n0 / gs;
-    if (q != qcur) {
+    auto enter = [&](int n) {                            // warp-uniform
+      if (n >= qbeg && n < qend) return;
       if (qcur >= 0) flush(norm, sc, lane);
-      qcur = q;
-      down = adown * sc[q].down;
-    }
+      qcur = n / gs;
+      qbeg = qcur * gs;
+      qend = qbeg + gs;
+      down = adown * sc[qcur].down;
+    };
+    enter(n0);
     uint32_t v[CH];
     ptx::tmem_ld16(tacc + (uint32_t)(e * CH), v);
     ptx::tmem_wait_ld();
     const size_t o = at(e);
-#pragma unroll
-    for (int j = 0; j < CH; ++j) {
+    auto column = [&](int j) {
       const float y = RZERO ? __uint_as_float(v[j]) * down : fmaf(__uint_as_float(v[j]), down, rv[B][j]);
       float d = fabsf(y - dv[B][j]);
       d = (d == d) ? d : __int_as_float(0x7f800000);
       __stcs(dout + o + (size_t)j * N2, y);
       runmax = fmaxf(runmax, d);
       ymax = fmaxf(ymax, fabsf(y));
+    };
+    if (n0 + CH <= ncol && n0 + CH <= qend) {
+#pragma unroll
+      for (int j = 0; j < CH; ++j) column(j);
+    } else {                                             // the last columns, or a group ends inside the chunk
+#pragma unroll
+      for (int j = 0; j < CH; ++j) {
+        if (n0 + j >= ncol) break;
+        enter(n0 + j);
+        column(j);
+      }
     }
   }
 };
 
+// r = 0 (a matvec), or r non-zero only on the rows of each column's source site (the first right-hand
+// side Lambda delta_s) and no column of the tile has its source here
+__device__ __forceinline__ bool r_is_zero(const FusedInst& I, int site, int n_first, int NB, int lane) {
+  if (I.r == nullptr) return true;
+  if (!I.rsrc) return false;
+  bool here = false;
+  for (int n = n_first + lane; n < min(I.ncol, n_first + NB); n += 32) here |= __ldg(I.rsrc + n) == site;
+  return !__any_sync(0xffffffffu, here);
+}
+
 template <int GT>
 __global__ void __launch_bounds__(F_THREADS, 1)
-    k_tc_fused(const __grid_constant__ CUtensorMap map_ahi, const __grid_constant__ CUtensorMap map_alo,
-               const float* __restrict__ r, const float* __restrict__ din, float* __restrict__ dout,
-               const int* __restrict__ rsrc, const float* __restrict__ Jz, const int* __restrict__ nbr,
-               const int* __restrict__ nbond, int Lx,
-               int Ly, int Nc, int ncol, int gs, unsigned long long* __restrict__ norm, int* __restrict__ err,
-               const int* __restrict__ act, int sweep, const int* __restrict__ run,
-               const int* __restrict__ sweeps_done, const float* __restrict__ adown, TcScale* __restrict__ sc) {
+    k_tc_fused(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
+               const __grid_constant__ FusedInst I, int* __restrict__ err, int sweep, const int* __restrict__ run,
+               const int* __restrict__ sweeps_done) {
   using namespace ptx;
   using Cfg = FusedCfg<GT>;
   // a sweep of a captured graph after the series has stopped: nothing to do (every CTA
@@ -905,7 +863,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
   // the sweep number (for the support table) is the device count of sweeps done, plus one
   if (run && *run == 0) return;
   if (sweeps_done) sweep = *sweeps_done + 1;
-  constexpr int STAGES = Cfg::STAGES, NBUF = Cfg::NBUF, STAGE = Cfg::STAGE;
+  constexpr int STAGES = Cfg::STAGES, NBUF = Cfg::NBUF, STAGE = Cfg::STAGE, NB = Cfg::NB, X_TILE = Cfg::X_TILE;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ __align__(8) uint64_t full_a[STAGES], xready[STAGES], full[STAGES], empty[STAGES];
@@ -916,13 +874,9 @@ __global__ void __launch_bounds__(F_THREADS, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
-  constexpr int NB = Cfg::NB, X_TILE = Cfg::X_TILE;
-  const int N2 = 2 * Nc;
-  const int KB = (GT == 2 ? Nc : N2) / F_BK;            // k-blocks of 64 complex points or 64 real values
-  const int NGT = GT == 2 ? (Nc + PM - 1) / PM : N2 / PM;
-  const int row_gap = GT == 2 ? Nc : 0;                 // rows of the two accumulators: z and Nc + z
-  const int NT = (ncol + NB - 1) / NB, nact = (ncol + TC_TILE_COLS - 1) / TC_TILE_COLS;
-  const int tiles = Lx * Ly * NT * NGT;
+  const int KB = (GT == 2 ? I.Ns : 2 * I.Ns) / F_BK;    // k-blocks of 64 complex points, or 64 real values
+  const int row_gap = GT == 2 ? I.Ns : 0;               // rows of the two accumulators: z and Ns + z
+  const int tiles = I.Lx * I.Ly * ((I.ncol + NB - 1) / NB) * fused_row_tiles<GT>(I.Ns);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -958,7 +912,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
         int g = 0;
         bool ok = true;
         for (int tile = pair; tile < tiles && ok; tile += npairs) {
-          const FTile T = fused_tile<NB>(tile, NGT, NT, Lx, Ly, act, nact, sweep);
+          const FTile T = fused_tile<GT>(I, tile, sweep);
           if (!T.active) continue;
           for (int kb = 0; kb < KB; ++kb, ++g) {
             const int s = g % STAGES;
@@ -971,8 +925,8 @@ __global__ void __launch_bounds__(F_THREADS, 1)
 #pragma unroll
             for (int gi = 0; gi < GT; ++gi) {
               const int row0 = T.gt * PM + (int)rank * BM + gi * row_gap;
-              tma_load_3d(st + gi * F_A_GROUP, &map_ahi, &full_a[s], kb * F_BK, row0, T.site);
-              tma_load_3d(st + gi * F_A_GROUP + A_TILE, &map_alo, &full_a[s], kb * F_BK, row0, T.site);
+              tma_load_3d(st + gi * F_A_GROUP, &map_hi, &full_a[s], kb * F_BK, row0, T.site);
+              tma_load_3d(st + gi * F_A_GROUP + A_TILE, &map_lo, &full_a[s], kb * F_BK, row0, T.site);
             }
           }
         }
@@ -985,7 +939,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
         int g = 0, t = 0;
         bool ok = true, any = false;
         for (int tile = pair; tile < tiles && ok; tile += npairs) {
-          const FTile T = fused_tile<NB>(tile, NGT, NT, Lx, Ly, act, nact, sweep);
+          const FTile T = fused_tile<GT>(I, tile, sweep);
           if (!T.active) continue;
           const int buf = t % NBUF;
           if (t >= NBUF && !mbar_wait_cluster(&acc_empty[buf], ((t / NBUF) - 1) & 1, abort_p)) break;
@@ -1037,7 +991,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
         int g = 0;
         bool ok = true;
         for (int tile = pair; tile < tiles && ok; tile += npairs) {
-          const FTile T = fused_tile<NB>(tile, NGT, NT, Lx, Ly, act, nact, sweep);
+          const FTile T = fused_tile<GT>(I, tile, sweep);
           if (!T.active) continue;
           for (int kb = 0; kb < KB; ++kb, ++g) {
             const int s = g % STAGES;
@@ -1063,13 +1017,17 @@ __global__ void __launch_bounds__(F_THREADS, 1)
     int g = 0;
     int ok = 1;
     for (int tile = pair; tile < tiles && ok; tile += npairs) {
-      const FTile T = fused_tile<NB>(tile, NGT, NT, Lx, Ly, act, nact, sweep);
+      const FTile T = fused_tile<GT>(I, tile, sweep);
       if (!T.active) continue;
+      const int Ns = I.Ns, N2 = 2 * Ns, ncol = I.ncol, gs = I.gs;
+      const float* __restrict__ din = I.din;
+      const float* __restrict__ Jz = I.Jz;
+      const TcScale* sc = I.sc;
       int nb[4], bd[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        nb[q] = __ldg(nbr + T.site * 4 + q);
-        bd[q] = nb[q] >= 0 ? __ldg(nbond + T.site * 4 + q) : 0;
+        nb[q] = __ldg(I.nbr + T.site * 4 + q);
+        bd[q] = nb[q] >= 0 ? __ldg(I.nbond + T.site * 4 + q) : 0;
       }
       const int col0 = T.nt * NB + (int)rank * (NB / 2);
       // this thread's columns col0 + c0 + 32 i, i < ni, lie before the end
@@ -1095,7 +1053,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
           for (int i = 0; i < 2; ++i) {
             const int ci = GT == 2 ? i : 2 * h + i;
             const bool ok_qi = nb[q] >= 0 && ci < ni;
-            const float* p = ok_qi ? nbp[q] + ci * cstride + kb * F_BK + (GT == 2 ? h * Nc : 0) : nbp[q];
+            const float* p = ok_qi ? nbp[q] + ci * cstride + kb * F_BK + (GT == 2 ? h * Ns : 0) : nbp[q];
             v[q][i][0] = __ldg(reinterpret_cast<const float4*>(p));
             v[q][i][1] = __ldg(reinterpret_cast<const float4*>(p + 32));
           }
@@ -1104,10 +1062,10 @@ __global__ void __launch_bounds__(F_THREADS, 1)
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
           const int k = kb * F_BK + 32 * u + 4 * j;
-          const int kz = k < Nc ? k : k - Nc;
+          const int kz = k < Ns ? k : k - Ns;
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
-            jv[q][u] = __ldg(reinterpret_cast<const float4*>(Jz + (size_t)bd[q] * Nc + kz));
+            jv[q][u] = __ldg(reinterpret_cast<const float4*>(Jz + (size_t)bd[q] * Ns + kz));
             if (nb[q] < 0) jv[q][u] = make_float4(0.f, 0.f, 0.f, 0.f);
           }
         }
@@ -1170,39 +1128,31 @@ __global__ void __launch_bounds__(F_THREADS, 1)
     }
   } else {
     reg_budget<F_REG_EPI, F_REGS_AT_LAUNCH>();
-    // ---------------- epilogue (both CTAs, own 128 rows of each group) ----------------
+    // ---------------- epilogue (both CTAs, own 128 rows of each accumulator) ----------------
     const int q4 = warp - F_EPI_W0;
     const uint32_t empty_bar0 = mapa(smem_u32(&acc_empty[0]), 0);
     int t = 0;
-    for (int tile = pair; tile < tiles; tile += npairs) {
-      const FTile T = fused_tile<NB>(tile, NGT, NT, Lx, Ly, act, nact, sweep);
+    bool go = true;
+    for (int tile = pair; tile < tiles && go; tile += npairs) {
+      const FTile T = fused_tile<GT>(I, tile, sweep);
       if (!T.active) continue;
       const int buf = t % NBUF;
-      // r = 0 (a matvec), or r non-zero only on the rows of each column's source site
-      // (the first right-hand side Lambda delta_s) and no column of the tile has its
-      // source here: its loads are skipped
-      const int n_first = T.nt * NB;
-      bool rz = r == nullptr;
-      if (!rz && rsrc) {
-        bool here = false;
-        for (int n = n_first + lane; n < min(ncol, n_first + NB); n += 32) here |= __ldg(rsrc + n) == T.site;
-        rz = !__any_sync(0xffffffffu, here);
-      }
-      const int mg = T.gt * PM + (int)rank * BM + q4 * 32 + lane;
-      const bool rows = GT == 1 || T.gt * PM + (int)rank * BM < Nc;   // Nc = 384: the last tile's odd CTA has none
-      const float ad = rows ? __ldg(adown + (size_t)T.site * N2 + mg) : 0.f;   // one scale for rows z and Nc + z
-      const size_t base0 = ((size_t)T.site * ncol + n_first) * N2 + mg;
+      const int N2 = 2 * I.Ns, gs = I.gs, n_first = T.nt * NB;
+      const int m0 = T.gt * PM + (int)rank * BM + q4 * 32;
+      const bool rows = m0 < (GT == 2 ? I.Ns : N2);       // a last row tile may be short (warp-uniform)
+      const float ad = rows ? __ldg(I.adown + (size_t)T.site * N2 + m0 + lane) : 0.f;   // one scale for rows z and Ns + z
+      unsigned long long* norm = I.norm;
+      TcScale* sc = I.sc;
       const uint32_t tacc = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(buf * GT * NB);
-      bool go = true;
       auto body = [&](auto E) {
-        E.r = r;
-        E.din = din;
-        E.dout = dout;
+        E.r = I.r;
+        E.din = I.din;
+        E.dout = I.dout;
         E.n_first = n_first;
-        E.ncol = rows ? ncol : 0;
-        E.row_gap = row_gap;
+        E.ncol = rows ? I.ncol : 0;
         E.N2 = N2;
-        E.base0 = base0;
+        E.row_gap = row_gap;
+        E.base0 = ((size_t)T.site * I.ncol + n_first) * N2 + m0 + lane;
         E.template load<0>(0);
         go = mbar_wait(&acc_full[buf], (t / NBUF) & 1, abort_p);
         go = __all_sync(0xffffffffu, go);                 // tcgen05.ld below is warp-collective
@@ -1217,7 +1167,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
         }
         if (E.qcur >= 0) E.flush(norm, sc, lane);
       };
-      if (rz) body(FusedEpilogue<GT, true>{});
+      if (r_is_zero(I, T.site, n_first, NB, lane)) body(FusedEpilogue<GT, true>{});
       else body(FusedEpilogue<GT, false>{});
       ++t;
       if (!go) break;
@@ -1283,6 +1233,21 @@ TcState* state(dyson_ctx* c) {
   return static_cast<TcState*>(c->tc);
 }
 
+cudaLaunchConfig_t pair_config(cudaLaunchAttribute* at, unsigned pairs, int threads, size_t smem, cudaStream_t stream) {
+  cudaLaunchConfig_t cfg = {};
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 2;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(2 * pairs);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
 // co-resident CTA pairs of k_tc_gemm_pair on this device (0: the pair kernel cannot run)
 int pair_clusters(dyson_ctx* c, TcState* st) {
   if (st->pair_clusters >= 0) return st->pair_clusters;
@@ -1291,18 +1256,8 @@ int pair_clusters(dyson_ctx* c, TcState* st) {
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) sms = 0;
   if (sms >= 2 &&
       cudaFuncSetAttribute(k_tc_gemm_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, P_SMEM_BYTES) == cudaSuccess) {
-    cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(2 * (unsigned)(sms / 2));
-    cfg.blockDim = dim3(THREADS);
-    cfg.dynamicSmemBytes = P_SMEM_BYTES;
-    cfg.stream = c->stream;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cudaLaunchConfig_t cfg = pair_config(at, (unsigned)(sms / 2), THREADS, P_SMEM_BYTES, c->stream);
     int ncl = 0;
     if (cudaOccupancyMaxActiveClusters(&ncl, k_tc_gemm_pair, &cfg) == cudaSuccess) st->pair_clusters = ncl;
   }
@@ -1312,11 +1267,8 @@ int pair_clusters(dyson_ctx* c, TcState* st) {
 
 // co-resident CTA pairs of k_tc_fused<GT> on this device (0: it cannot run)
 template <int GT>
-int fused_clusters(dyson_ctx* c, TcState* st) {
-  int& n = st->fused_clusters[GT - 1];
-  if (n >= 0) return n;
-  n = 0;
-  int sms = 0;
+int fused_clusters_of(dyson_ctx* c) {
+  int sms = 0, n = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) sms = 0;
   // the warpgroups' register shares add up to exactly F_REGS_AT_LAUNCH per thread: with
   // any other count at launch the producers' increase could not be met, so the kernel is
@@ -1325,18 +1277,8 @@ int fused_clusters(dyson_ctx* c, TcState* st) {
   if (cudaFuncGetAttributes(&fa, k_tc_fused<GT>) != cudaSuccess || fa.numRegs != F_REGS_AT_LAUNCH) sms = 0;
   if (sms >= 2 && cudaFuncSetAttribute(k_tc_fused<GT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        FusedCfg<GT>::SMEM) == cudaSuccess) {
-    cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(2 * (unsigned)(sms / 2));
-    cfg.blockDim = dim3(F_THREADS);
-    cfg.dynamicSmemBytes = FusedCfg<GT>::SMEM;
-    cfg.stream = c->stream;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cudaLaunchConfig_t cfg = pair_config(at, (unsigned)(sms / 2), F_THREADS, FusedCfg<GT>::SMEM, c->stream);
     int ncl = 0;
     if (cudaOccupancyMaxActiveClusters(&ncl, k_tc_fused<GT>, &cfg) == cudaSuccess) n = ncl;
   }
@@ -1344,17 +1286,30 @@ int fused_clusters(dyson_ctx* c, TcState* st) {
   return n;
 }
 
-// row groups per fused tile for the context's variant (0: the fused kernel does not serve it)
+// pairs for both forms of the fused kernel (0 where one of them cannot run)
+int fused_clusters(dyson_ctx* c) {
+  TcState* st = state(c);
+  if (st->fused_clusters < 0) st->fused_clusters = std::min(fused_clusters_of<1>(c), fused_clusters_of<2>(c));
+  return st->fused_clusters;
+}
+
+// Complex tiles wherever their 256 points are at least five eighths full: X is then gathered once per
+// (site, column tile) and Lambda read once.  Shorter contours (64, 128) would fill a half at most; their
+// embedding has a single tile of 256 rows.
+int fused_gt_of(const dyson_ctx* c) { return contour_stride(c) >= 192 ? 2 : 1; }
+
+// form of the fused kernel that serves the context's variant (0: none).  The unfused forms serve
+// only contours that fill their tiles; every other contour takes the fused kernel.
 int fused_gt(dyson_ctx* c) {
-  if (c->Nc % 128 != 0 || c->Lx * c->Ly != c->Nr) return 0;
-  if (c->tc_variant != DYSON_SWEEP_FUSED_PAIR && c->tc_variant != DYSON_SWEEP_FUSED_PAIR_WIDE) return 0;
-  if (c->tc_variant == DYSON_SWEEP_FUSED_PAIR_WIDE && c->Nc % 256 != 0) return 0;
-  // tiles of complex points wherever they are at least three quarters full
-  if (c->Nc >= 256 && fused_clusters<2>(c, state(c)) > 0) return 2;
-  return fused_clusters<1>(c, state(c)) > 0 ? 1 : 0;
+  const bool unfused = (c->tc_variant == DYSON_SWEEP_SINGLE_CTA || c->tc_variant == DYSON_SWEEP_CTA_PAIR) &&
+                       c->Nc % 64 == 0;
+  if (unfused || !encode_fn()) return 0;
+  return fused_clusters(c) > 0 ? fused_gt_of(c) : 0;
 }
 
 }  // namespace
+
+int contour_stride(const dyson_ctx* c) { return (c->Nc + 63) / 64 * 64; }
 
 bool tc_uses_fused(dyson_ctx* c) { return fused_gt(c) > 0; }
 
@@ -1362,44 +1317,52 @@ bool tc_uses_pair(dyson_ctx* c) {
   return c->tc_variant == DYSON_SWEEP_CTA_PAIR && c->Nc % 128 == 0 && pair_clusters(c, state(c)) > 0;
 }
 
-bool tc_supported(dyson_ctx* c, int Nc) {
-  (void)c;
-  return Nc % 64 == 0 && encode_fn() != nullptr;
+// (below 24 points more than five eighths of a padded column would be zeros)
+bool tc_supported(dyson_ctx* c) {
+  return c->Nc >= 24 && encode_fn() != nullptr && (c->Nc % 64 == 0 || fused_gt(c) > 0);
 }
 
 namespace {
 
-// tensor maps of Lambda and the gather buffer of context c for ncol columns
-int tc_prepare(dyson_ctx* c, int ncol, bool need_x = true) {
+int tc_prepare_common(dyson_ctx* c) {
   TcState* st = state(c);
-  const int Nc = c->Nc, N2 = 2 * Nc, Nr = c->Nr;
   if (!st->d_err) {
     DY_CUDA(c, cudaMalloc(&st->d_err, sizeof(int)));
     DY_CUDA(c, cudaMemsetAsync(st->d_err, 0, sizeof(int), c->stream));
     DY_CUDA(c, cudaDeviceGetAttribute(&st->num_sms, cudaDevAttrMultiProcessorCount, c->device));
   }
-  if (!need_x) {                                         // the fused sweep gathers in shared memory
-    if (st->h_hi_ptr != c->d_lam16_hi || st->h_lo_ptr != c->d_lam16_lo) {
-      if (!make_map16(&st->h_hi, c->d_lam16_hi, N2, N2, Nr, BM) || !make_map16(&st->h_lo, c->d_lam16_lo, N2, N2, Nr, BM))
-        return ctx_fail(c, DYSON_ERR_CUDA, "cuTensorMapEncodeTiled failed for the FP16 Lambda");
-      st->h_hi_ptr = c->d_lam16_hi;
-      st->h_lo_ptr = c->d_lam16_lo;
-    }
-    return DYSON_OK;
+  return DYSON_OK;
+}
+
+// tensor maps of the FP16 Lambda
+int tc_prepare_fused(dyson_ctx* c) {
+  int rc = tc_prepare_common(c);
+  if (rc) return rc;
+  TcState* st = state(c);
+  const int N2 = 2 * contour_stride(c);
+  if (st->h_hi_ptr != c->d_lam16_hi || st->h_lo_ptr != c->d_lam16_lo) {
+    if (!make_map16(&st->h_hi, c->d_lam16_hi, N2, N2, c->Nr, BM) || !make_map16(&st->h_lo, c->d_lam16_lo, N2, N2, c->Nr, BM))
+      return ctx_fail(c, DYSON_ERR_CUDA, "cuTensorMapEncodeTiled failed for the FP16 Lambda");
+    st->h_hi_ptr = c->d_lam16_hi;
+    st->h_lo_ptr = c->d_lam16_lo;
   }
-  if (st->a_hi_ptr != c->d_lam_hi || st->a_lo_ptr != c->d_lam_lo || st->a_Nr != Nr || st->a_Nc != Nc) {
+  return DYSON_OK;
+}
+
+// tensor maps of the TF32 Lambda and the gather buffer of the unfused forms, for ncol columns
+int tc_prepare(dyson_ctx* c, int ncol) {
+  int rc = tc_prepare_common(c);
+  if (rc) return rc;
+  TcState* st = state(c);
+  const int Nc = c->Nc, N2 = 2 * Nc, Nr = c->Nr;
+  if (st->a_hi_ptr != c->d_lam_hi || st->a_lo_ptr != c->d_lam_lo) {
     if (!make_map(&st->a_hi, c->d_lam_hi, N2, N2, Nr, BM) || !make_map(&st->a_lo, c->d_lam_lo, N2, N2, Nr, BM))
       return ctx_fail(c, DYSON_ERR_CUDA, "cuTensorMapEncodeTiled failed for Lambda");
     st->a_hi_ptr = c->d_lam_hi;
     st->a_lo_ptr = c->d_lam_lo;
-    st->a_Nr = Nr;
-    st->a_Nc = Nc;
-    st->inst_valid = false;
   }
   if (!st->smem_set) {
-    DY_CUDA(c, cudaFuncSetAttribute(k_tc_gemm<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-    DY_CUDA(c, cudaFuncSetAttribute(k_tc_gemm<TC_MAX_INSTANCES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    SMEM_BYTES));
+    DY_CUDA(c, cudaFuncSetAttribute(k_tc_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
     st->smem_set = true;
   }
   size_t xbytes = (size_t)Nr * ncol * N2 * sizeof(float);
@@ -1420,41 +1383,20 @@ int tc_prepare(dyson_ctx* c, int ncol, bool need_x = true) {
       return ctx_fail(c, DYSON_ERR_CUDA, "cuTensorMapEncodeTiled failed for X");
     st->x_ptr = st->xbuf;
     st->x_ncol = ncol;
-    st->inst_valid = false;
   }
   return DYSON_OK;
 }
 
 template <int GT>
-int launch_fused(dyson_ctx* c, int ncol, int gs, const float* r, const float* din, float* dout, const int* act,
-                 int sweep, const int* rsrc) {
+int launch_fused(dyson_ctx* c, const FusedInst& e, int sweep, const int* run, const int* sweeps_done,
+                 cudaStream_t stream) {
   TcState* st = state(c);
   const int NB = FusedCfg<GT>::NB;
-  const int row_tiles = GT == 2 ? (c->Nc + PM - 1) / PM : 2 * c->Nc / PM;
-  const long long tiles = (long long)c->Nr * ((ncol + NB - 1) / NB) * row_tiles;
-  const int pairs = (int)std::min<long long>(tiles, fused_clusters<GT>(c, st));
-  cudaLaunchConfig_t cfg = {};
+  const long long tiles = (long long)e.Lx * e.Ly * ((e.ncol + NB - 1) / NB) * fused_row_tiles<GT>(e.Ns);
   cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = 2;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3(2 * (unsigned)pairs);
-  cfg.blockDim = dim3(F_THREADS);
-  cfg.dynamicSmemBytes = FusedCfg<GT>::SMEM;
-  cfg.stream = c->stream;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  const int ng = ncol / gs;
-  if (!c->sweep_run) {                                   // (in a captured series the check kernel sets the scales)
-    k_tc_scale<<<(ng + 127) / 128, 128, 0, c->stream>>>(c->d_xscale, ng, tc_jbound(c));
-    c->launches += 1;
-  }
-  DY_CUDA(c, cudaLaunchKernelEx(&cfg, k_tc_fused<GT>, st->h_hi, st->h_lo, r, din, dout, rsrc,
-                                (const float*)c->d_Jz,
-                                (const int*)c->d_nbr, (const int*)c->d_nbond, c->Lx, c->Ly, c->Nc, ncol, gs,
-                                c->d_norm, st->d_err, act, sweep, c->sweep_run, c->sweep_count,
-                                (const float*)c->d_a_down, c->d_xscale));
+  cudaLaunchConfig_t cfg = pair_config(at, (unsigned)std::min<long long>(tiles, fused_clusters(c)), F_THREADS,
+                                       FusedCfg<GT>::SMEM, stream);
+  DY_CUDA(c, cudaLaunchKernelEx(&cfg, k_tc_fused<GT>, st->h_hi, st->h_lo, e, st->d_err, sweep, run, sweeps_done));
   DY_CUDA(c, cudaGetLastError());
   c->launches += 1;
   return DYSON_OK;
@@ -1465,7 +1407,6 @@ int launch_fused(dyson_ctx* c, int ncol, int gs, const float* r, const float* di
 float tc_jbound(const dyson_ctx* c) { return 4.f * c->j_max; }
 
 int tc_seed_scale(dyson_ctx* c, int ng, const double* ref, double bound) {
-  if (!tc_uses_fused(c)) return DYSON_OK;
   k_tc_seed<<<(ng + 127) / 128, 128, 0, c->stream>>>(c->d_xscale, ng, ref, (float)bound);
   c->launches += 1;
   DY_CUDA(c, cudaGetLastError());
@@ -1473,11 +1414,11 @@ int tc_seed_scale(dyson_ctx* c, int ng, const double* ref, double bound) {
 }
 
 int tc_seed_scale_scan(dyson_ctx* c, int ncol, int gs, const float* d) {
-  if (!tc_uses_fused(c)) return DYSON_OK;
-  int rc = tc_seed_scale(c, ncol / gs, nullptr, 0.0);
+  int rc = tc_seed_scale(c, (ncol + gs - 1) / gs, nullptr, 0.0);
   if (rc) return rc;
   const size_t warps = (size_t)c->Nr * ncol;
-  k_tc_seed_scan<<<(unsigned)((warps + 7) / 8), 256, 0, c->stream>>>(d, c->Nr, c->Nc, ncol, gs, c->d_xscale);
+  k_tc_seed_scan<<<(unsigned)((warps + 7) / 8), 256, 0, c->stream>>>(d, c->Nr, contour_stride(c), ncol, gs,
+                                                                     c->d_xscale);
   c->launches += 1;
   DY_CUDA(c, cudaGetLastError());
   return DYSON_OK;
@@ -1490,109 +1431,60 @@ int tc_set_scale(dyson_ctx* c, int ng) {
   return DYSON_OK;
 }
 
-int tc_prepare_sweep(dyson_ctx* c, int ncol) { return tc_prepare(c, ncol, fused_gt(c) == 0); }
+int tc_prepare_sweep(dyson_ctx* c, int ncol, bool fused) {
+  return fused || fused_gt(c) > 0 ? tc_prepare_fused(c) : tc_prepare(c, ncol);
+}
 
-int tc_fill_instance(dyson_ctx* c, int ncol, int gs, const float* r, float* buf0, float* buf1,
-                     unsigned long long* norm, const int* active, TcInst* e, CUtensorMap* a_hi, CUtensorMap* a_lo,
-                     CUtensorMap* x) {
-  int rc = tc_prepare(c, ncol);
+bool tc_fused_runs(dyson_ctx* c) { return encode_fn() && fused_clusters(c) > 0; }
+
+int tc_fused_sweep(dyson_ctx* c, int ncol, int gs, const float* r, const float* din, float* dout, const int* act,
+                   int sweep, int rform, const int* run, const int* sweeps_done, cudaStream_t stream) {
+  int rc = tc_prepare_fused(c);
   if (rc) return rc;
-  TcState* st = state(c);
-  std::memset(static_cast<void*>(e), 0, sizeof(TcInst));
-  *a_hi = st->a_hi;
-  *a_lo = st->a_lo;
-  *x = st->x;
-  e->r = r;
-  e->buf[0] = buf0;
-  e->buf[1] = buf1;
-  e->X = st->xbuf;
-  e->Jz = c->d_Jz;
-  e->nbr = c->d_nbr;
-  e->nbond = c->d_nbond;
-  e->norm = norm;
-  e->active = active;
-  e->Nr = c->Nr;
-  e->Nc = c->Nc;
-  e->ncol = ncol;
-  e->gs = gs;
-  return DYSON_OK;
-}
-
-int tc_instance_tiles(const TcInst& e) { return (2 * e.Nc / BM) * ((e.ncol + BN - 1) / BN) * e.Nr; }
-int tc_instance_gather_blocks(const TcInst& e) { return e.Nr * ((e.ncol + GATHER_COLS - 1) / GATHER_COLS); }
-
-namespace {
-
-template <int MAXI>
-int launch_gemm(dyson_ctx* c, const CUtensorMap* a_hi, const CUtensorMap* a_lo, const CUtensorMap* x,
-                const TcInst* d_tab, int ninst, int tiles, int parity, cudaStream_t stream, const int* act,
-                int sweep) {
-  TcState* st = state(c);
-  static_assert(sizeof(TcMaps<MAXI>) <= 30000, "tensor maps exceed the kernel-parameter space");
-  TcMaps<MAXI> maps;
-  for (int k = 0; k < ninst; ++k) {
-    maps.a_hi[k] = a_hi[k];
-    maps.a_lo[k] = a_lo[k];
-    maps.x[k] = x[k];
-  }
-  const int grid = std::min(tiles, st->num_sms > 0 ? st->num_sms : 148);
-  k_tc_gemm<MAXI><<<grid, THREADS, SMEM_BYTES, stream>>>(maps, d_tab, ninst, tiles, parity, st->d_err, act,
-                                                         sweep);
-  return DYSON_OK;
-}
-
-}  // namespace
-
-int tc_launch_table(dyson_ctx* c, const TcInst* d_tab, int ninst, int tiles, int gblocks, int parity, int phases,
-                    cudaStream_t stream, const CUtensorMap* a_hi, const CUtensorMap* a_lo, const CUtensorMap* x,
-                    const TcInst* h_one, const int* act, int sweep) {
-  if (ninst < 1 || ninst > TC_MAX_INSTANCES)
-    return ctx_fail(c, DYSON_ERR_INVALID_ARG, "instance table of 1.." + std::to_string(TC_MAX_INSTANCES) + " entries");
-  if (act && !(ninst == 1 && h_one))
-    return ctx_fail(c, DYSON_ERR_INVALID_ARG, "support truncation needs a one-entry table with its host copy");
-  TcState* st = state(c);
-  if (phases & TC_GATHER) {
-    if (h_one && ninst == 1)
-      k_tc_gather_one<<<gblocks, 256, 0, stream>>>(h_one->buf[parity], h_one->Jz, h_one->nbr, h_one->nbond, h_one->X,
-                                                   h_one->Nr, h_one->Nc, h_one->ncol, act, sweep);
-    else
-      k_tc_gather<<<gblocks, 256, 0, stream>>>(d_tab, ninst, parity);
-    DY_CUDA(c, cudaGetLastError());
-    c->launches += 1;
-  }
-  if (phases & TC_GEMM) {
-    int rc = ninst == 1 ? launch_gemm<1>(c, a_hi, a_lo, x, d_tab, ninst, tiles, parity, stream, act, sweep)
-                        : launch_gemm<TC_MAX_INSTANCES>(c, a_hi, a_lo, x, d_tab, ninst, tiles, parity, stream,
-                                                        nullptr, 0);
-    if (rc) return rc;
-    DY_CUDA(c, cudaGetLastError());
-    c->launches += 1;
-  }
-  return DYSON_OK;
+  FusedInst e = {};
+  e.r = rform == TC_R_ZERO ? nullptr : r;
+  e.din = din;
+  e.dout = dout;
+  e.Jz = c->d_Jz;
+  e.nbr = c->d_nbr;
+  e.nbond = c->d_nbond;
+  e.norm = c->d_norm;
+  e.adown = c->d_a_down;
+  e.sc = c->d_xscale;
+  e.rsrc = rform == TC_R_ON_SOURCES ? c->d_src_site : nullptr;
+  e.act = act;
+  e.Lx = c->Lx;
+  e.Ly = c->Ly;
+  e.Ns = contour_stride(c);
+  e.ncol = ncol;
+  e.gs = gs;
+  return fused_gt_of(c) == 1 ? launch_fused<1>(c, e, sweep, run, sweeps_done, stream)
+                             : launch_fused<2>(c, e, sweep, run, sweeps_done, stream);
 }
 
 int tc_sweep(dyson_ctx* c, int ncol, int gs, const float* r, const float* din, float* dout, int phases,
              const int* act, int sweep, int rform) {
-  const int gt = (phases & TC_TABLE_ONLY) ? 0 : fused_gt(c);
-  int rc = tc_prepare(c, ncol, gt == 0);
-  if (rc) return rc;
+  const int gt = fused_gt(c);
+  int rc;
   if (gt > 0) {
     // one launch gathers and multiplies: the gather phase alone launches nothing
-    if (!(phases & TC_GEMM)) return DYSON_OK;
-    const float* rr = rform == TC_R_ZERO ? nullptr : r;
-    const int* rsrc = rform == TC_R_ON_SOURCES ? c->d_src_site : nullptr;
-    return gt == 1 ? launch_fused<1>(c, ncol, gs, rr, din, dout, act, sweep, rsrc)
-                   : launch_fused<2>(c, ncol, gs, rr, din, dout, act, sweep, rsrc);
+    if (!(phases & TC_GEMM)) return tc_prepare_fused(c);
+    // (in a captured series the check kernel sets the scales)
+    if (!c->sweep_run && (rc = tc_set_scale(c, (ncol + gs - 1) / gs))) return rc;
+    return tc_fused_sweep(c, ncol, gs, r, din, dout, act, sweep, rform, c->sweep_run, c->sweep_count, c->stream);
   }
+  if ((rc = tc_prepare(c, ncol))) return rc;
   TcState* st = state(c);
   const int Nc = c->Nc, N2 = 2 * Nc, Nr = c->Nr;
+  if (phases & TC_GATHER) {
+    k_tc_gather<<<Nr * ((ncol + GATHER_COLS - 1) / GATHER_COLS), 256, 0, c->stream>>>(
+        din, c->d_Jz, c->d_nbr, c->d_nbond, st->xbuf, Nr, Nc, ncol, act, sweep);
+    DY_CUDA(c, cudaGetLastError());
+    c->launches += 1;
+  }
+  if (!(phases & TC_GEMM)) return DYSON_OK;
   // truncated sweeps run on the single-CTA kernel, which skips tiles
-  if (!(phases & TC_TABLE_ONLY) && !act && tc_uses_pair(c)) {
-    if (phases & TC_GATHER) {
-      // the one-entry table serves the gather of the pair form too
-      if ((rc = tc_sweep(c, ncol, gs, r, din, dout, TC_GATHER | TC_TABLE_ONLY))) return rc;
-    }
-    if (!(phases & TC_GEMM)) return DYSON_OK;
+  if (!act && tc_uses_pair(c)) {
     if (st->xh_ptr != st->xbuf || st->xh_ncol != ncol) {
       if (!make_map(&st->xh, st->xbuf, N2, ncol, Nr, BN / 2))
         return ctx_fail(c, DYSON_ERR_CUDA, "cuTensorMapEncodeTiled failed for X halves");
@@ -1600,49 +1492,20 @@ int tc_sweep(dyson_ctx* c, int ncol, int gs, const float* r, const float* din, f
       st->xh_ncol = ncol;
     }
     const long long tiles = (long long)(N2 / PM) * ((ncol + BN - 1) / BN) * Nr;
-    const int pairs = (int)std::min<long long>(tiles, st->pair_clusters);
-    cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(2 * (unsigned)pairs);
-    cfg.blockDim = dim3(THREADS);
-    cfg.dynamicSmemBytes = P_SMEM_BYTES;
-    cfg.stream = c->stream;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cudaLaunchConfig_t cfg = pair_config(at, (unsigned)std::min<long long>(tiles, st->pair_clusters), THREADS,
+                                         P_SMEM_BYTES, c->stream);
     DY_CUDA(c, cudaLaunchKernelEx(&cfg, k_tc_gemm_pair, st->a_hi, st->a_lo, st->xh, r, din, dout, Nr, Nc, ncol, gs,
                                   c->d_norm, st->d_err));
-    DY_CUDA(c, cudaGetLastError());
-    c->launches += 1;
-    return DYSON_OK;
+  } else {
+    const long long tiles = (long long)(N2 / BM) * ((ncol + BN - 1) / BN) * Nr;
+    const int grid = (int)std::min<long long>(tiles, st->num_sms);
+    k_tc_gemm<<<grid, THREADS, SMEM_BYTES, c->stream>>>(st->a_hi, st->a_lo, st->x, r, din, dout, Nr, Nc, ncol, gs,
+                                                        c->d_norm, st->d_err, act, sweep);
   }
-  // one-entry table; the two states keep their slots, the parity says which is d_in
-  if (!st->h_inst) {
-    DY_CUDA(c, cudaMallocHost((void**)&st->h_inst, sizeof(TcInst)));
-    DY_CUDA(c, cudaMalloc((void**)&st->d_inst, sizeof(TcInst)));
-    st->inst_valid = false;
-  }
-  TcInst* h = st->h_inst;
-  int parity = -1;
-  if (st->inst_valid && h->r == r && h->ncol == ncol && h->gs == gs && h->norm == c->d_norm) {
-    if (h->buf[0] == din && h->buf[1] == dout) parity = 0;
-    else if (h->buf[1] == din && h->buf[0] == dout) parity = 1;
-  }
-  if (parity < 0) {
-    // the previous launches may still read the table: refill it behind them on the stream
-    DY_CUDA(c, cudaStreamSynchronize(c->stream));
-    CUtensorMap m0, m1, m2;
-    if ((rc = tc_fill_instance(c, ncol, gs, r, const_cast<float*>(din), dout, c->d_norm, nullptr, h, &m0, &m1, &m2)))
-      return rc;
-    DY_CUDA(c, cudaMemcpyAsync(st->d_inst, h, sizeof(TcInst), cudaMemcpyHostToDevice, c->stream));
-    st->inst_valid = true;
-    parity = 0;
-  }
-  return tc_launch_table(c, st->d_inst, 1, tc_instance_tiles(*h), tc_instance_gather_blocks(*h), parity,
-                         phases & (TC_GATHER | TC_GEMM), c->stream, &st->a_hi, &st->a_lo, &st->x, h, act, sweep);
+  DY_CUDA(c, cudaGetLastError());
+  c->launches += 1;
+  return DYSON_OK;
 }
 
 int tc_set_wait_limit(dyson_ctx* c, unsigned long long ns) {
@@ -1683,8 +1546,6 @@ void tc_release(dyson_ctx* c) {
   if (st->xbuf) cudaFree(st->xbuf);
   if (st->d_err) cudaFree(st->d_err);
   if (st->h_err) cudaFreeHost(st->h_err);
-  if (st->h_inst) cudaFreeHost(st->h_inst);
-  if (st->d_inst) cudaFree(st->d_inst);
   delete st;
   c->tc = nullptr;
 }

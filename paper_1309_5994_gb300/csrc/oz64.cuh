@@ -12,7 +12,7 @@ void oz64_invalidate(dyson_ctx* c);
 // build the Lambda slices now (so that the free memory a caller sizes its chunk by is what is left)
 int oz64_prepare(dyson_ctx* c);
 // mode 0: out = B + K Gin, c->d_norm[q] = max |out - Gin| (complex modulus);
-// mode 1: r32 = B + K Gin - Gin (FP32 planar), c->d_norm[q] = max |r|.
+// mode 1: r32 = B + K Gin - Gin (FP32 planar of stride c->Ns; only the Nc points are written), c->d_norm[q] = max |r|.
 // Groups of gs columns as launch_sweep_f64; two kernel launches, counted on the context.
 int oz64_sweep(dyson_ctx* c, int ncol, int gs, const double2* Gin, double2* out, float* r32, int mode);
 // DYSON_ERR_TIMEOUT if a bounded pipeline wait of an earlier sweep expired (clears the flag);

@@ -4,54 +4,47 @@
 
 #include "common.cuh"
 
-// Most instances one tensor-core launch serves.  Their TMA maps travel as
-// __grid_constant__ kernel parameters (3 x 128 bytes each, 24 KB for 64), not in
-// global memory, where a map written at a recycled address could meet a stale
-// descriptor in the TMA unit's cache.
-constexpr int TC_MAX_INSTANCES = 64;
-template <int MAXI>
-struct TcMaps {
-  CUtensorMap a_hi[MAXI], a_lo[MAXI], x[MAXI];
-};
-
-// One problem instance of a (batched) tensor-core sweep: a device table entry.
-// The state of the series alternates between buf[0] and buf[1]: a sweep of
-// parity p reads d_in = buf[p] and writes d_out = buf[p ^ 1].
-struct TcInst {
-  const float* r;                    // right-hand side of the series [Nr][ncol][2Nc]
-  float* buf[2];                     // the two FP32 states
-  float* X;                          // gather output, the GEMM's B operand
-  const float* Jz;                   // [Nb][Nc] hopping on the contour
+// Arguments of a fused sweep (a kernel parameter).
+struct FusedInst {
+  const float* r;                    // right-hand side of the series [Nr][ncol][2 Ns] (nullptr: 0)
+  const float* din;                  // the two FP32 states
+  float* dout;
+  const float* Jz;                   // [Nb][Ns] hopping on the contour
   const int* nbr;                    // [Nr][4] neighbour sites (-1: none)
   const int* nbond;                  // [Nr][4] bond of each neighbour slot
   unsigned long long* norm;          // update max-norm per group of gs columns
-  const int* active;                 // nullptr, or a device flag: 0 skips the instance
-  int Nr, Nc, ncol, gs;
-  int tile0;                         // first global GEMM tile of this instance
-  int gblk0;                         // first global gather block of this instance
+  const float* adown;                // [Nr][2 Ns] inverse row scales of the FP16 Lambda
+  TcScale* sc;                       // scales per group of gs columns
+  const int* rsrc;                   // r is non-zero only where column n has its source (site rsrc[n]); or nullptr
+  const int* act;                    // support truncation table; or nullptr
+  int Lx, Ly, Ns, ncol, gs;
 };
 
+// Contour points a column of the FP32 planar state holds, Ns: Nc rounded up to 64 (the rest are
+// zeros) on the tensor-core sweeps
+int contour_stride(const dyson_ctx* c);
 
 // FP16 scales of the fused sweep: before the first sweep of a chain, seed the bound on |d_in| per
 // column group, with ref (device, [ng]) or one bound for all, or by reading the state; the
-// sweeps after it take the bound from the maxima that the previous one left.  No-ops for the other forms.
+// sweeps after it take the bound from the maxima that the previous one left.
 int tc_seed_scale(dyson_ctx* c, int ng, const double* ref, double bound);
 int tc_seed_scale_scan(dyson_ctx* c, int ncol, int gs, const float* d);
 // turn the seeded maxima into scales (tc_sweep does this itself outside a captured series)
 int tc_set_scale(dyson_ctx* c, int ng);
 float tc_jbound(const dyson_ctx* c);              // 4 max|J|, the factor of set_scale
-// true when the 3xTF32 tcgen05 sweep supports this contour length
-bool tc_supported(dyson_ctx* c, int Nc);
+// true when a tcgen05 sweep serves this context
+bool tc_supported(dyson_ctx* c);
 // true when tc_sweep runs the CTA-pair (cta_group::2) kernel for this context
 bool tc_uses_pair(dyson_ctx* c);
-// true when tc_sweep runs the fused gather + GEMM kernel (k_tc_fused) for this context:
-// the context's variant is DYSON_SWEEP_FUSED_PAIR (Nc % 128 == 0) or
-// DYSON_SWEEP_FUSED_PAIR_WIDE (Nc % 256 == 0); TC_GATHER alone then launches nothing
+// true when tc_sweep runs the fused gather + GEMM kernel (k_tc_fused) for this context: unless
+// its variant is DYSON_SWEEP_SINGLE_CTA or DYSON_SWEEP_CTA_PAIR and Nc a multiple of 64;
+// TC_GATHER alone then launches nothing
 bool tc_uses_fused(dyson_ctx* c);
-// tensor maps and buffers of tc_sweep for ncol columns, set up ahead of a stream capture
-int tc_prepare_sweep(dyson_ctx* c, int ncol);
+// tensor maps and buffers of tc_sweep (fused: of tc_fused_sweep) for ncol columns, set up ahead of
+// a stream capture
+int tc_prepare_sweep(dyson_ctx* c, int ncol, bool fused = false);
 // one sweep d_out = r + K d_in over the FP32 planar chunk state of ncol vector columns;
-// writes c->d_norm[q] for groups of gs columns (gs a multiple of 32, Nc a multiple of 64).
+// writes c->d_norm[q] for groups of gs columns (unfused forms: gs a multiple of 32).
 // phases: TC_GATHER launches X = J d_in, TC_GEMM launches the tensor-core product and
 // epilogue (in that order; both = one whole sweep).
 // act (optional, device [Nr][ceil(ncol / 256)]): support truncation (App. C, Sec. IV.D):
@@ -60,7 +53,7 @@ int tc_prepare_sweep(dyson_ctx* c, int ncol);
 // rform: what the caller knows of r, for the fused kernel to skip loads of zeros:
 // TC_R_DENSE (general), TC_R_ZERO (r = 0: a matvec), TC_R_ON_SOURCES (r non-zero only
 // on the rows of each column's source site, c->d_src_site: the first right-hand side)
-enum { TC_GATHER = 1, TC_GEMM = 2, TC_TABLE_ONLY = 4 };
+enum { TC_GATHER = 1, TC_GEMM = 2 };
 enum { TC_R_DENSE = 0, TC_R_ZERO = 1, TC_R_ON_SOURCES = 2 };
 constexpr int TC_TILE_COLS = 256;
 int tc_sweep(dyson_ctx* c, int ncol, int gs, const float* r, const float* d_in, float* d_out, int phases,
@@ -77,19 +70,10 @@ int tc_error_status(dyson_ctx* c);
 // free tensor-core module state
 void tc_release(dyson_ctx* c);
 
-// Fill one instance-table entry for context c (gather buffer, the state buffers
-// buf0/buf1, norm words and an optional device activity flag) and return its
-// three TMA maps; tile0 and gblk0 are left 0 for the caller to set.
-int tc_fill_instance(dyson_ctx* c, int ncol, int gs, const float* r, float* buf0, float* buf1,
-                     unsigned long long* norm, const int* active, TcInst* e, CUtensorMap* a_hi, CUtensorMap* a_lo,
-                     CUtensorMap* x);
-int tc_instance_tiles(const TcInst& e);           // 128 x 256 GEMM tiles of the entry
-int tc_instance_gather_blocks(const TcInst& e);   // gather blocks of the entry
-// Launch the gather and/or the GEMM of one sweep of parity `parity` over a device
-// table of ninst entries (tiles, gblocks: totals); errors and the launch count
-// are recorded on context c.  a_hi, a_lo, x: the entries' maps (host arrays of
-// ninst <= TC_MAX_INSTANCES).  h_one: for a one-entry table, its host copy (the
-// gather then takes the entry's pointers as kernel parameters), else nullptr.
-int tc_launch_table(dyson_ctx* c, const TcInst* d_tab, int ninst, int tiles, int gblocks, int parity, int phases,
-                    cudaStream_t stream, const CUtensorMap* a_hi, const CUtensorMap* a_lo, const CUtensorMap* x,
-                    const TcInst* h_one = nullptr, const int* act = nullptr, int sweep = 0);
+// true when the fused sweep can run on this context's device
+bool tc_fused_runs(dyson_ctx* c);
+// The fused sweep of tc_sweep on a stream of the caller's, with scales set (tc_set_scale, or by a
+// captured check kernel): run (or nullptr): device flag, 0 skips the sweep; sweeps_done (or nullptr):
+// device count that gives the sweep number
+int tc_fused_sweep(dyson_ctx* c, int ncol, int gs, const float* r, const float* din, float* dout, const int* act,
+                   int sweep, int rform, const int* run, const int* sweeps_done, cudaStream_t stream);

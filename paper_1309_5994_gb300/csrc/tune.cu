@@ -34,21 +34,21 @@ int time_sweeps(dyson_ctx* c, int nq, int warm, int timed, double* ms_per_sweep)
     }
   int rc;
   if ((rc = ensure_cols(c, ncol, nq)) || (rc = upload_sources(c, ncol))) return rc;
-  const size_t n_el = (size_t)c->Nr * ncol * c->Nc;
+  const size_t n_el = (size_t)c->Nr * ncol * c->Nc, n32 = (size_t)c->Nr * ncol * 2 * c->Ns;
   double2* G = (double2*)c->work;
   float* r32 = (float*)(G + n_el);
-  float* da = r32 + 2 * n_el;
-  float* db = da + 2 * n_el;
+  float* da = r32 + n32;
+  float* db = da + n32;
   DY_CUDA(c, cudaMemsetAsync(G, 0, n_el * sizeof(double2), c->stream));
   launch_init_rhs(c->d_lam, c->d_src_site, c->d_src_time, c->Nr, c->Nc, ncol, c->Nc, G, c->d_norm + nq, c->stream);
-  launch_to_planar32(G, r32, n_el, c->Nc, c->stream);
-  DY_CUDA(c, cudaMemcpyAsync(da, r32, 2 * n_el * sizeof(float), cudaMemcpyDeviceToDevice, c->stream));
+  launch_to_planar32(G, r32, (size_t)c->Nr * ncol, c->Nc, c->Ns, c->stream);
+  DY_CUDA(c, cudaMemcpyAsync(da, r32, n32 * sizeof(float), cudaMemcpyDeviceToDevice, c->stream));
   c->launches += 2;
   cudaEvent_t e0, e1;
   DY_CUDA(c, cudaEventCreate(&e0));
   DY_CUDA(c, cudaEventCreate(&e1));
   for (int s = 0; s < warm + timed; ++s) {
-    if (s == 0 && (rc = tc_seed_scale_scan(c, ncol, c->Nc, da))) break;
+    if (s == 0 && tc_uses_fused(c) && (rc = tc_seed_scale_scan(c, ncol, c->Nc, da))) break;
     if (s == warm) DY_CUDA(c, cudaEventRecord(e0, c->stream));
     if ((rc = tc_sweep(c, ncol, c->Nc, r32, da, db, TC_GATHER | TC_GEMM))) break;
     std::swap(da, db);
@@ -76,6 +76,7 @@ int dyson_autotune(dyson_ctx* c, int32_t max_block_columns, dyson_tuning* out) {
   if (!c->sigma_built || c->sigma_transposed) return ctx_fail(c, DYSON_ERR_STATE, "Lambda not built or transposed");
   DeviceGuard g(c->device);
   int rc;
+  if (c->Nc % 64 != 0) return ctx_fail(c, DYSON_ERR_INVALID_ARG, "the tuner needs Nc % 64 == 0");
   if ((rc = prepare_tables(c, DYSON_PREC_TF32X3_F64REF))) return rc;
   if (!c->use_tc) return ctx_fail(c, DYSON_ERR_INVALID_ARG, "the tensor-core sweep needs Nc % 64 == 0");
   size_t col_bytes = 0, col_total = 0;
@@ -107,7 +108,7 @@ int dyson_autotune(dyson_ctx* c, int32_t max_block_columns, dyson_tuning* out) {
   if (tc_uses_pair(c)) variants.push_back(DYSON_SWEEP_CTA_PAIR);
   for (int v : {DYSON_SWEEP_FUSED_PAIR, DYSON_SWEEP_FUSED_PAIR_WIDE}) {
     c->tc_variant = v;
-    if (tc_uses_fused(c)) variants.push_back(v);
+    if (tc_uses_fused(c) && (v != DYSON_SWEEP_FUSED_PAIR_WIDE || c->Nc % 256 == 0)) variants.push_back(v);
   }
   c->tc_variant = saved_variant;
 

@@ -49,3 +49,33 @@ def test_fused_solve_over_hopping_scales(torch_cuda, lib, jscale, inner, variant
         want = ref[:, :, q * p.Nc:(q + 1) * p.Nc]
         assert np.abs(got[q] - want).max() / np.abs(want).max() < 1e-11
     s.close()
+
+
+@pytest.mark.parametrize("inner", [0, 1])
+@pytest.mark.parametrize("Nt,Nm", [(9, 6), (12, 9), (24, 17), (38, 24), (48, 34), (70, 50), (72, 48), (96, 65), (120, 80)])
+def test_fused_sweep_serves_every_contour(torch_cuda, lib, Nt, Nm, inner):
+    """Contours that are no multiple of 64 (padded with zeros inside), of every tile form, with column counts and
+    norm groups that end inside a 16-column chunk; no variant selected."""
+    from paper_1309_5994_gb300 import binding
+    torch = torch_cuda
+    p = wl.random_tables(wl.small(L=3, Ly=2, Nt=Nt, Nm=Nm, dt=0.02, beta=1.0, trap_c=0.3, U0=14.0), seed=7, rel=0.1)
+    S = dyson.setup(p)
+    sources = [0, 4, 5]
+    ref = dyson.dense_solve(S, dyson.rhs_block_columns(S, sources))
+    s = binding.Solver(p, device=0)
+    s.set_inner_solver(inner)
+    s.build_sigma()
+    s.profile(True)
+    g = torch.empty((len(sources), p.Nr, p.Nc, p.Nc), dtype=torch.complex128, device="cuda:0")
+    s.solve(sources, precision=binding.PREC_TF32X3_F64REF, tol=1e-12, g_out=g)
+    assert s.profile_query(binding.KERNEL_SWEEP_TC)[0] > 0 and s.profile_query(binding.KERNEL_GATHER_TC)[0] == 0
+    got = g.cpu().numpy()
+    for q in range(len(sources)):
+        want = ref[:, :, q * p.Nc:(q + 1) * p.Nc]
+        assert np.abs(got[q] - want).max() / np.abs(want).max() < 1e-11
+    sites, times = [k % p.Nr for k in range(40)], [(7 * k) % p.Nc for k in range(40)]
+    v = torch.empty((40, p.Nr, p.Nc), dtype=torch.complex128, device="cuda:0")
+    s.solve_vectors(sites, times, precision=binding.PREC_TF32X3_F64REF, tol=1e-12, g_out=v)
+    want = dyson.dense_solve(S, dyson.rhs_vector_columns(S, list(zip(sites, times))))
+    assert np.abs(v.cpu().numpy() - want.transpose(2, 0, 1)).max() / np.abs(want).max() < 1e-11
+    s.close()
