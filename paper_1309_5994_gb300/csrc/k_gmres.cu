@@ -65,107 +65,192 @@ __device__ __forceinline__ double2 gm_mul(double2 a, double2 b) {
 }
 __device__ __forceinline__ double2 gm_conj(double2 a) { return make_double2(a.x, -a.y); }
 
-__device__ __forceinline__ double block_sum(double v, double* sh) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) sh[wid] = v;
-  __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x < 32) {
-    t = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  }
-  __syncthreads();
-  return t;   // valid in thread 0
-}
-
 // Second Gram-Schmidt pass only where the first lost most of the vector: the
 // test of Daniel, Gragg, Kaufman and Stewart, |w| < 0.7 |(I - K) q_j|.
 __device__ __forceinline__ bool reorth_needed(const double* after, const double* before, int n) {
   return after[n] < 0.49 * before[n];
 }
 
-// h[n][i] += <Q_i[n], a[n] - b[n]>  (b may be null) over a chunk of sites;
-// blocks with i = 0 also add |a - b|^2 to nrm0[n] when nrm0 is given.  With a
-// gate (after, before), columns that need no second pass are skipped.
-// grid: (basis vectors, ncol, site chunks) - the basis index runs fastest, so the
-// blocks of one (column, chunk) follow each other and re-read a, b from L2.
-__global__ void __launch_bounds__(GM_THREADS) k_gm_dots(const float* __restrict__ Q, size_t vsz,
+// The vector kernels work on items: one warp, one column n, VEC 32 T contour points of one site, real
+// and imaginary parts in registers (VEC = 4 where the stride allows float4 loads).  Items of a column
+// are numbered site-major; a block takes a range of one column's items, its warps every eighth of them.
+// They are bound by HBM: per Arnoldi step the basis is read once for the projections and once for
+// the update.  12x12, Nc = 384, 384 columns (170 MB a vector): see the rates at k_gm_dots.
+template <int VEC, int T>
+struct Slab {
+  float re[T][VEC], im[T][VEC];
+};
+struct ItemPos {
+  size_t base;                                          // first element of (site, column)
+  int z0;                                               // first contour point of this lane
+};
+template <int VEC, int T>
+__device__ __forceinline__ ItemPos item_pos(int item, int nz, int n, int ncol, int Ns, int lane) {
+  const int s = item / nz, zc = item - s * nz;
+  return {((size_t)s * ncol + n) * 2 * Ns, (zc * 32 * T + lane) * VEC};
+}
+template <int VEC, int T>
+__device__ __forceinline__ void load_slab(Slab<VEC, T>& x, const float* __restrict__ p, ItemPos at, int Ns) {
+#pragma unroll
+  for (int t = 0; t < T; ++t) {
+    const int z = at.z0 + 32 * VEC * t;
+    const bool in = z < Ns;
+    if (VEC == 4) {
+      const float4 r = in ? *reinterpret_cast<const float4*>(p + at.base + z) : make_float4(0.f, 0.f, 0.f, 0.f);
+      const float4 i = in ? *reinterpret_cast<const float4*>(p + at.base + Ns + z) : make_float4(0.f, 0.f, 0.f, 0.f);
+      x.re[t][0] = r.x; x.re[t][1 % VEC] = r.y; x.re[t][2 % VEC] = r.z; x.re[t][3 % VEC] = r.w;
+      x.im[t][0] = i.x; x.im[t][1 % VEC] = i.y; x.im[t][2 % VEC] = i.z; x.im[t][3 % VEC] = i.w;
+    } else {
+      x.re[t][0] = in ? p[at.base + z] : 0.f;
+      x.im[t][0] = in ? p[at.base + Ns + z] : 0.f;
+    }
+  }
+}
+template <int VEC, int T>
+__device__ __forceinline__ void store_slab(const Slab<VEC, T>& x, float* __restrict__ p, ItemPos at, int Ns) {
+#pragma unroll
+  for (int t = 0; t < T; ++t) {
+    const int z = at.z0 + 32 * VEC * t;
+    if (z >= Ns) continue;
+    if (VEC == 4) {
+      *reinterpret_cast<float4*>(p + at.base + z) =
+          make_float4(x.re[t][0], x.re[t][1 % VEC], x.re[t][2 % VEC], x.re[t][3 % VEC]);
+      *reinterpret_cast<float4*>(p + at.base + Ns + z) =
+          make_float4(x.im[t][0], x.im[t][1 % VEC], x.im[t][2 % VEC], x.im[t][3 % VEC]);
+    } else {
+      p[at.base + z] = x.re[t][0];
+      p[at.base + Ns + z] = x.im[t][0];
+    }
+  }
+}
+template <int VEC, int T>
+__device__ __forceinline__ float slab_norm2(const Slab<VEC, T>& x) {
+  float q = 0.f;
+#pragma unroll
+  for (int t = 0; t < T; ++t)
+#pragma unroll
+    for (int v = 0; v < VEC; ++v) q = fmaf(x.re[t][v], x.re[t][v], fmaf(x.im[t][v], x.im[t][v], q));
+  return q;
+}
+
+// h[n][i] += <Q_i[n], a[n] - b[n]>  (b may be null) over a range of items; nrm0 (given): += |a - b|^2.
+// With a gate (after, before), columns that need no second pass are skipped.  Grid (ncol, ranges).
+// w = a - b of an item stays in registers while GROUP basis vectors pass by it; FP32 products are
+// summed in FP32 within an item and in FP64 across items (GB300's FP64 pipe is too slow for a product
+// per element).  As one block per (basis vector, column, range), which read a and b again for
+// every basis vector in 4-byte loads, the projections ran at 1.4 TB/s.
+constexpr int GM_GROUP = 4;
+template <int VEC, int T>
+__global__ void __launch_bounds__(GM_THREADS) k_gm_dots(const float* __restrict__ Q, size_t vsz, int nvec,
                                                         const float* __restrict__ a, const float* __restrict__ b,
-                                                        int Nr, int Nc, int ncol, int sites_per_blk,
+                                                        int items, int nz, int Ns, int ncol, int items_per_blk,
                                                         double2* __restrict__ h, int hstride,
                                                         double* __restrict__ nrm0, const double* __restrict__ after,
                                                         const double* __restrict__ before) {
-  __shared__ double sh[GM_THREADS / 32];
-  const int i = blockIdx.x, n = blockIdx.y;
+  __shared__ double sh[GM_THREADS / 32][2 * GM_GROUP + 1];
+  const int n = blockIdx.x;
   if (after && !reorth_needed(after, before, n)) return;
-  const int s0 = blockIdx.z * sites_per_blk, s1 = min(Nr, s0 + sites_per_blk);
-  const float* __restrict__ q = Q + (size_t)i * vsz;
-  const bool self = nrm0 && i == 0;
-  // Each warp walks the block's sites (stride: warps per block), its lanes the
-  // contour index, four elements per lane at a time (independent loads in
-  // flight).  FP32 products are summed in FP32 within a site and in FP64 across
-  // sites - GB300's FP64 pipe is too slow for a product per element.
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-  double re = 0.0, im = 0.0, sq = 0.0;
-  for (int s = s0 + warp; s < s1; s += nwarps) {
-    const size_t base = ((size_t)s * ncol + n) * 2 * Nc;
-    const float* __restrict__ ar = a + base;
-    const float* __restrict__ br = b ? b + base : nullptr;
-    const float* __restrict__ qr_ = q + base;
-    float sre = 0.f, sim = 0.f, ssq = 0.f;
-    for (int z0 = lane; z0 < Nc; z0 += 128) {
+  const int i0 = blockIdx.y * items_per_blk, i1 = min(items, i0 + items_per_blk);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int g0 = 0; g0 < nvec; g0 += GM_GROUP) {
+    const bool self = nrm0 && g0 == 0;
+    double re[GM_GROUP] = {}, im[GM_GROUP] = {}, sq = 0.0;
+    for (int item = i0 + warp; item < i1; item += GM_THREADS / 32) {
+      const ItemPos at = item_pos<VEC, T>(item, nz, n, ncol, Ns, lane);
+      Slab<VEC, T> w, x;
+      load_slab(w, a, at, Ns);
+      if (b) {
+        load_slab(x, b, at, Ns);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int z = z0 + 32 * k;
-        if (z < Nc) {
-          float wr = ar[z], wi = ar[Nc + z];
-          if (br) {
-            wr -= br[z];
-            wi -= br[Nc + z];
+        for (int t = 0; t < T; ++t)
+#pragma unroll
+          for (int v = 0; v < VEC; ++v) {
+            w.re[t][v] -= x.re[t][v];
+            w.im[t][v] -= x.im[t][v];
           }
-          const float qre = qr_[z], qim = qr_[Nc + z];
-          sre = fmaf(qre, wr, fmaf(qim, wi, sre));    // conj(q) w
-          sim = fmaf(qre, wi, fmaf(-qim, wr, sim));
-          if (self) ssq = fmaf(wr, wr, fmaf(wi, wi, ssq));
-        }
+      }
+      if (self) sq += (double)slab_norm2(w);
+#pragma unroll
+      for (int k = 0; k < GM_GROUP; ++k) {
+        if (g0 + k >= nvec) break;
+        load_slab(x, Q + (size_t)(g0 + k) * vsz, at, Ns);
+        float sr = 0.f, si = 0.f;
+#pragma unroll
+        for (int t = 0; t < T; ++t)
+#pragma unroll
+          for (int v = 0; v < VEC; ++v) {                // conj(q) w
+            sr = fmaf(x.re[t][v], w.re[t][v], fmaf(x.im[t][v], w.im[t][v], sr));
+            si = fmaf(x.re[t][v], w.im[t][v], fmaf(-x.im[t][v], w.re[t][v], si));
+          }
+        re[k] += (double)sr;
+        im[k] += (double)si;
       }
     }
-    re += sre;
-    im += sim;
-    sq += ssq;
-  }
-  re = block_sum(re, sh);
-  im = block_sum(im, sh);
-  if (self) sq = block_sum(sq, sh);
-  if (threadIdx.x == 0) {
-    atomicAdd(&h[(size_t)n * hstride + i].x, re);
-    atomicAdd(&h[(size_t)n * hstride + i].y, im);
-    if (self) atomicAdd(&nrm0[n], sq);
+#pragma unroll
+    for (int k = 0; k < GM_GROUP; ++k) {
+      for (int o = 16; o > 0; o >>= 1) {
+        re[k] += __shfl_xor_sync(0xffffffffu, re[k], o);
+        im[k] += __shfl_xor_sync(0xffffffffu, im[k], o);
+      }
+    }
+    if (self)
+      for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    if (lane == 0) {
+#pragma unroll
+      for (int k = 0; k < GM_GROUP; ++k) {
+        sh[warp][2 * k] = re[k];
+        sh[warp][2 * k + 1] = im[k];
+      }
+      sh[warp][2 * GM_GROUP] = sq;
+    }
+    __syncthreads();
+    const int e = threadIdx.x;
+    if (e < 2 * GM_GROUP + 1) {
+      double v = 0.0;
+      for (int q = 0; q < GM_THREADS / 32; ++q) v += sh[q][e];
+      if (e == 2 * GM_GROUP) {
+        if (self) atomicAdd(&nrm0[n], v);
+      } else if (g0 + e / 2 < nvec) {
+        double2* hp = &h[(size_t)n * hstride + g0 + e / 2];
+        atomicAdd(e & 1 ? &hp->y : &hp->x, v);
+      }
+    }
+    __syncthreads();
   }
 }
 
-// nrm[n] += |a[n]|^2; grid (Nr, ncol)
-__global__ void __launch_bounds__(GM_THREADS) k_gm_norm2(const float* __restrict__ a, int Nc, int ncol,
-                                                         double* __restrict__ nrm) {
+// sum over the block's warps of one FP64 value per lane, added to *out by one thread
+__device__ __forceinline__ void block_add(double v, double* out) {
   __shared__ double sh[GM_THREADS / 32];
-  const int s = blockIdx.x, n = blockIdx.y;
-  const size_t base = ((size_t)s * ncol + n) * 2 * Nc;
-  float part = 0.f;
-  for (int z = threadIdx.x; z < 2 * Nc; z += blockDim.x) part = fmaf(a[base + z], a[base + z], part);
-  const double acc = block_sum((double)part, sh);
-  if (threadIdx.x == 0) atomicAdd(&nrm[n], acc);
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int q = 0; q < GM_THREADS / 32; ++q) t += sh[q];
+    atomicAdd(out, t);
+  }
+}
+
+// nrm[n] += |a[n]|^2; grid (ncol, ranges)
+template <int VEC, int T>
+__global__ void __launch_bounds__(GM_THREADS) k_gm_norm2(const float* __restrict__ a, int items, int nz, int Ns,
+                                                         int ncol, int items_per_blk, double* __restrict__ nrm) {
+  const int n = blockIdx.x, i0 = blockIdx.y * items_per_blk, i1 = min(items, i0 + items_per_blk);
+  double acc = 0.0;
+  for (int item = i0 + (int)(threadIdx.x >> 5); item < i1; item += GM_THREADS / 32) {
+    Slab<VEC, T> x;
+    load_slab(x, a, item_pos<VEC, T>(item, nz, n, ncol, Ns, threadIdx.x & 31), Ns);
+    acc += (double)slab_norm2(x);
+  }
+  block_add(acc, &nrm[n]);
 }
 
 // out = a - b + c elementwise over the whole chunk state
 __global__ void k_gm_lin3(const float* __restrict__ a, const float* __restrict__ b, const float* __restrict__ c,
-                          float* __restrict__ out, size_t n4) {
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n4; e += (size_t)gridDim.x * blockDim.x) {
-    const float4 x = reinterpret_cast<const float4*>(a)[e];
-    const float4 y = reinterpret_cast<const float4*>(b)[e];
-    const float4 z = reinterpret_cast<const float4*>(c)[e];
-    reinterpret_cast<float4*>(out)[e] = make_float4(x.x - y.x + z.x, x.y - y.y + z.y, x.z - y.z + z.z, x.w - y.w + z.w);
-  }
+                          float* __restrict__ out, size_t n) {
+  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x)
+    out[e] = a[e] - b[e] + c[e];
 }
 
 // v <- sqrt(v)
@@ -174,115 +259,92 @@ __global__ void k_gm_sqrt(double* __restrict__ v, int n) {
   if (i < n) v[i] = sqrt(fmax(v[i], 0.0));
 }
 
-// w[n] = (a[n] - b[n]) - sum_{i < nvec} h[n][i] Q_i[n]  (b may be null), nrm[n] += |w[n]|^2.
+// w[n] = (a[n] - b[n]) + sign sum_{i < nvec} h[n][i] Q_i[n]  (b may be null), nrm[n] (given) += |w[n]|^2.
 // With a gate (after, before): columns that need no second pass keep w and
-// take nrm[n] = after[n].  grid: (Nr, ncol)
+// take nrm[n] = after[n].  Grid (ncol, ranges).
 // (a and w may be the same array: each element is read, then written, by one thread)
+template <int VEC, int T>
 __global__ void __launch_bounds__(GM_THREADS) k_gm_update(const float* __restrict__ Q, size_t vsz, int nvec,
-                                                          const double2* __restrict__ h, int hstride,
+                                                          const double2* __restrict__ h, int hstride, float sign,
                                                           const float* a, const float* __restrict__ b, float* w,
-                                                          int Nc, int ncol, double* __restrict__ nrm,
-                                                          const double* __restrict__ after,
+                                                          int items, int nz, int Ns, int ncol, int items_per_blk,
+                                                          double* __restrict__ nrm, const double* __restrict__ after,
                                                           const double* __restrict__ before) {
-  __shared__ double sh[GM_THREADS / 32];
   __shared__ float2 hs[64];
-  const int s = blockIdx.x, n = blockIdx.y;
+  const int n = blockIdx.x;
   if (after && !reorth_needed(after, before, n)) {
-    if (s == 0 && threadIdx.x == 0) atomicAdd(&nrm[n], after[n]);
+    if (blockIdx.y == 0 && threadIdx.x == 0) atomicAdd(&nrm[n], after[n]);
     return;
   }
   for (int i = threadIdx.x; i < nvec; i += blockDim.x) {
     const double2 v = h[(size_t)n * hstride + i];
-    hs[i] = make_float2((float)v.x, (float)v.y);
+    hs[i] = make_float2(sign * (float)v.x, sign * (float)v.y);
   }
   __syncthreads();
-  const size_t base = ((size_t)s * ncol + n) * 2 * Nc;
+  const int i0 = blockIdx.y * items_per_blk, i1 = min(items, i0 + items_per_blk);
   double acc = 0.0;
-  for (int z = threadIdx.x; z < Nc; z += blockDim.x) {
-    float wr = a[base + z], wi = a[base + Nc + z];
+  for (int item = i0 + (int)(threadIdx.x >> 5); item < i1; item += GM_THREADS / 32) {
+    const ItemPos at = item_pos<VEC, T>(item, nz, n, ncol, Ns, threadIdx.x & 31);
+    Slab<VEC, T> x, q[2];
+    load_slab(x, a, at, Ns);
     if (b) {
-      wr -= b[base + z];
-      wi -= b[base + Nc + z];
+      load_slab(q[0], b, at, Ns);
+#pragma unroll
+      for (int t = 0; t < T; ++t)
+#pragma unroll
+        for (int v = 0; v < VEC; ++v) {
+          x.re[t][v] -= q[0].re[t][v];
+          x.im[t][v] -= q[0].im[t][v];
+        }
     }
-    const float* qz = Q + base + z;
+    auto fold = [&](const Slab<VEC, T>& y, float2 c) {
+#pragma unroll
+      for (int t = 0; t < T; ++t)
+#pragma unroll
+        for (int v = 0; v < VEC; ++v) {
+          x.re[t][v] += c.x * y.re[t][v] - c.y * y.im[t][v];
+          x.im[t][v] += c.x * y.im[t][v] + c.y * y.re[t][v];
+        }
+    };
     int i = 0;
-    for (; i + 4 <= nvec; i += 4) {                      // four independent loads in flight
-      float qr[4], qi[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        qr[k] = qz[(size_t)(i + k) * vsz];
-        qi[k] = qz[(size_t)(i + k) * vsz + Nc];
-      }
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const float2 c = hs[i + k];
-        wr -= c.x * qr[k] - c.y * qi[k];
-        wi -= c.x * qi[k] + c.y * qr[k];
-      }
+    for (; i + 2 <= nvec; i += 2) {                      // two vectors' loads in flight
+      load_slab(q[0], Q + (size_t)i * vsz, at, Ns);
+      load_slab(q[1], Q + (size_t)(i + 1) * vsz, at, Ns);
+      fold(q[0], hs[i]);
+      fold(q[1], hs[i + 1]);
     }
-    for (; i < nvec; ++i) {
-      const float qr = qz[(size_t)i * vsz], qi = qz[(size_t)i * vsz + Nc];
-      const float2 c = hs[i];
-      wr -= c.x * qr - c.y * qi;
-      wi -= c.x * qi + c.y * qr;
+    if (i < nvec) {
+      load_slab(q[0], Q + (size_t)i * vsz, at, Ns);
+      fold(q[0], hs[i]);
     }
-    w[base + z] = wr;
-    w[base + Nc + z] = wi;
-    acc += fmaf(wr, wr, wi * wi);
+    store_slab(x, w, at, Ns);
+    acc += (double)slab_norm2(x);
   }
-  acc = block_sum(acc, sh);
-  if (threadIdx.x == 0 && nrm) atomicAdd(&nrm[n], acc);
+  if (nrm) block_add(acc, &nrm[n]);
 }
 
-// out[n] = scale[n] * x[n] with scale = 1 / sqrt(nrm[n]) (0 where nrm = 0); grid (Nr, ncol)
+// out[n] = x[n] / sqrt(nrm[n]) (0 where nrm = 0); grid (ncol, ranges)
+template <int VEC, int T>
 __global__ void __launch_bounds__(GM_THREADS) k_gm_scale(const float* __restrict__ x, const double* __restrict__ nrm,
-                                                         float* __restrict__ out, int Nc, int ncol) {
-  const int s = blockIdx.x, n = blockIdx.y;
-  const double v = nrm[n];
-  const float f = v > 0.0 ? (float)(1.0 / sqrt(v)) : 0.f;
-  const size_t base = ((size_t)s * ncol + n) * 2 * Nc;
-  for (int z = threadIdx.x; z < 2 * Nc; z += blockDim.x) out[base + z] = f * x[base + z];
-}
-
-// out[n] = x0[n] + sum_{i < nvec} y[n][i] Q_i[n]; grid (Nr, ncol)
-// (x0 and out may be the same array)
-__global__ void __launch_bounds__(GM_THREADS) k_gm_combine(const float* __restrict__ Q, size_t vsz, int nvec,
-                                                           const double2* __restrict__ y, int ystride,
-                                                           const float* x0, float* out, int Nc, int ncol) {
-  __shared__ float2 ys[64];
-  const int s = blockIdx.x, n = blockIdx.y;
-  for (int i = threadIdx.x; i < nvec; i += blockDim.x) {
-    const double2 v = y[(size_t)n * ystride + i];
-    ys[i] = make_float2((float)v.x, (float)v.y);
-  }
+                                                         float* __restrict__ out, int items, int nz, int Ns, int ncol,
+                                                         int items_per_blk) {
+  const int n = blockIdx.x, i0 = blockIdx.y * items_per_blk, i1 = min(items, i0 + items_per_blk);
+  __shared__ float f_sh;
+  if (threadIdx.x == 0) f_sh = nrm[n] > 0.0 ? (float)(1.0 / sqrt(nrm[n])) : 0.f;
   __syncthreads();
-  const size_t base = ((size_t)s * ncol + n) * 2 * Nc;
-  for (int z = threadIdx.x; z < Nc; z += blockDim.x) {
-    float xr = x0[base + z], xi = x0[base + Nc + z];
-    const float* qz = Q + base + z;
-    int i = 0;
-    for (; i + 4 <= nvec; i += 4) {
-      float qr[4], qi[4];
+  const float f = f_sh;
+  for (int item = i0 + (int)(threadIdx.x >> 5); item < i1; item += GM_THREADS / 32) {
+    const ItemPos at = item_pos<VEC, T>(item, nz, n, ncol, Ns, threadIdx.x & 31);
+    Slab<VEC, T> v;
+    load_slab(v, x, at, Ns);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        qr[k] = qz[(size_t)(i + k) * vsz];
-        qi[k] = qz[(size_t)(i + k) * vsz + Nc];
-      }
+    for (int t = 0; t < T; ++t)
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const float2 c = ys[i + k];
-        xr += c.x * qr[k] - c.y * qi[k];
-        xi += c.x * qi[k] + c.y * qr[k];
+      for (int k = 0; k < VEC; ++k) {
+        v.re[t][k] *= f;
+        v.im[t][k] *= f;
       }
-    }
-    for (; i < nvec; ++i) {
-      const float qr = qz[(size_t)i * vsz], qi = qz[(size_t)i * vsz + Nc];
-      const float2 c = ys[i];
-      xr += c.x * qr - c.y * qi;
-      xi += c.x * qi + c.y * qr;
-    }
-    out[base + z] = xr;
-    out[base + Nc + z] = xi;
+    store_slab(v, out, at, Ns);
   }
 }
 
@@ -421,30 +483,29 @@ int gmres_restart_length(dyson_ctx* c, int ncol) {
   return std::max(0, std::min(c->gmres_restart > 0 ? c->gmres_restart : 40, std::min(fit, 60)));
 }
 
-int gmres_inner_solve(dyson_ctx* c, int ncol, const float* r, float* x, int max_iters, double tol,
-                      dyson_report* rep, const MatvecFn& matvec) {
-  if (ncol > 65535 || c->Nr > 65535) return ctx_fail(c, DYSON_ERR_INVALID_ARG, "GMRES chunks hold <= 65535 columns");
-  const int m = gmres_restart_length(c, ncol);
-  if (m < 2) return ctx_fail(c, DYSON_ERR_OOM, "GMRES needs room for at least 3 Krylov vectors");
-  const size_t vsz = (size_t)c->Nr * ncol * 2 * c->Ns;
-  int rc = gm_prepare(c, vsz, ncol, m);
-  if (rc) return rc;
+namespace {
+
+// the vector kernels for one item shape
+template <int VEC, int T>
+int gmres_run(dyson_ctx* c, int ncol, const float* r, float* x, int max_iters, double tol, dyson_report* rep,
+              const MatvecFn& matvec, int m) {
   GmState* st = gstate(c);
   cudaStream_t s = c->stream;
-  const int Nc = c->Ns;                                  // (the padding points are zeros)
-  const dim3 grid_el(c->Nr, ncol);
-  // dot blocks: enough (basis x column x chunk) blocks without tiny chunks
-  const int chunks = (int)std::max<int64_t>(1, std::min<int64_t>(c->Nr, 4096 / std::max(1, ncol)));
-  const int sites_per_blk = (c->Nr + chunks - 1) / chunks;
-  const int nchunk = (c->Nr + sites_per_blk - 1) / sites_per_blk;
+  const int Ns = c->Ns;                                  // (padding points are zeros)
+  const size_t vsz = (size_t)c->Nr * ncol * 2 * Ns;
+  int rc;
+  // ranges of items per column: enough blocks for every SM, and at least two items per warp
+  const int nz = (Ns + 32 * VEC * T - 1) / (32 * VEC * T), items = c->Nr * nz;
+  const int want = std::max(1, std::min((items + 15) / 16, (152 * 16 + ncol - 1) / ncol));
+  const int per = (items + want - 1) / want;
+  const dim3 grid(ncol, (items + per - 1) / per);
   const int cb = (ncol + 127) / 128;
-  const size_t n4 = vsz / 4;
-  const int lin_grid = (int)std::min<size_t>((n4 + 255) / 256, 152 * 16);
+  const int lin_grid = (int)std::min<size_t>((vsz + 255) / 256, 152 * 16);
   const size_t hbytes = (size_t)ncol * (m + 1) * sizeof(double2);
 
   // |r| per column, and the iterate starts at u0 = r
   DY_CUDA(c, cudaMemsetAsync(st->bnorm, 0, ncol * sizeof(double), s));
-  k_gm_norm2<<<grid_el, GM_THREADS, 0, s>>>(r, Nc, ncol, st->bnorm);
+  k_gm_norm2<VEC, T><<<grid, GM_THREADS, 0, s>>>(r, items, nz, Ns, ncol, per, st->bnorm);
   k_gm_sqrt<<<cb, 128, 0, s>>>(st->bnorm, ncol);
   DY_CUDA(c, cudaMemcpyAsync(x, r, vsz * sizeof(float), cudaMemcpyDeviceToDevice, s));
   c->launches += 2;
@@ -455,11 +516,11 @@ int gmres_inner_solve(dyson_ctx* c, int ncol, const float* r, float* x, int max_
     if ((rc = matvec(st->zero, x, st->u, 0.0))) return rc;
     rep->sweeps += 1;
     rep->gemm_flops += sweep_flops(c, ncol);
-    k_gm_lin3<<<lin_grid, 256, 0, s>>>(r, x, st->u, st->w, n4);
+    k_gm_lin3<<<lin_grid, 256, 0, s>>>(r, x, st->u, st->w, vsz);
     DY_CUDA(c, cudaMemsetAsync(st->nrm, 0, ncol * sizeof(double), s));
-    k_gm_norm2<<<grid_el, GM_THREADS, 0, s>>>(st->w, Nc, ncol, st->nrm);
+    k_gm_norm2<VEC, T><<<grid, GM_THREADS, 0, s>>>(st->w, items, nz, Ns, ncol, per, st->nrm);
     k_gm_start<<<cb, 128, 0, s>>>(ncol, m, st->nrm, st->beta, st->g);
-    k_gm_scale<<<grid_el, GM_THREADS, 0, s>>>(st->w, st->nrm, st->Q, Nc, ncol);
+    k_gm_scale<VEC, T><<<grid, GM_THREADS, 0, s>>>(st->w, st->nrm, st->Q, items, nz, Ns, ncol, per);
     c->launches += 4;
     int d = 0;
     for (int j = 0; j < m && its < max_iters; ++j) {
@@ -476,17 +537,16 @@ int gmres_inner_solve(dyson_ctx* c, int ncol, const float* r, float* x, int max_
       DY_CUDA(c, cudaMemsetAsync(st->nrm0, 0, ncol * sizeof(double), s));
       DY_CUDA(c, cudaMemsetAsync(st->nrm1, 0, ncol * sizeof(double), s));
       DY_CUDA(c, cudaMemsetAsync(st->nrm, 0, ncol * sizeof(double), s));
-      k_gm_dots<<<dim3(j + 1, ncol, nchunk), GM_THREADS, 0, s>>>(st->Q, vsz, qj, st->u, c->Nr, Nc, ncol,
-                                                                 sites_per_blk, st->h, m + 1, st->nrm0, nullptr,
-                                                                 nullptr);
-      k_gm_update<<<grid_el, GM_THREADS, 0, s>>>(st->Q, vsz, j + 1, st->h, m + 1, qj, st->u, st->w, Nc, ncol,
-                                                  st->nrm1, nullptr, nullptr);
-      k_gm_dots<<<dim3(j + 1, ncol, nchunk), GM_THREADS, 0, s>>>(st->Q, vsz, st->w, nullptr, c->Nr, Nc, ncol,
-                                                                 sites_per_blk, st->h2, m + 1, nullptr, st->nrm1,
-                                                                 st->nrm0);
-      k_gm_update<<<grid_el, GM_THREADS, 0, s>>>(st->Q, vsz, j + 1, st->h2, m + 1, st->w, nullptr, st->w, Nc, ncol,
-                                                  st->nrm, st->nrm1, st->nrm0);
-      k_gm_scale<<<grid_el, GM_THREADS, 0, s>>>(st->w, st->nrm, st->Q + (size_t)(j + 1) * vsz, Nc, ncol);
+      k_gm_dots<VEC, T><<<grid, GM_THREADS, 0, s>>>(st->Q, vsz, j + 1, qj, st->u, items, nz, Ns, ncol, per, st->h,
+                                                    m + 1, st->nrm0, nullptr, nullptr);
+      k_gm_update<VEC, T><<<grid, GM_THREADS, 0, s>>>(st->Q, vsz, j + 1, st->h, m + 1, -1.f, qj, st->u, st->w, items,
+                                                      nz, Ns, ncol, per, st->nrm1, nullptr, nullptr);
+      k_gm_dots<VEC, T><<<grid, GM_THREADS, 0, s>>>(st->Q, vsz, j + 1, st->w, nullptr, items, nz, Ns, ncol, per,
+                                                    st->h2, m + 1, nullptr, st->nrm1, st->nrm0);
+      k_gm_update<VEC, T><<<grid, GM_THREADS, 0, s>>>(st->Q, vsz, j + 1, st->h2, m + 1, -1.f, st->w, nullptr, st->w,
+                                                      items, nz, Ns, ncol, per, st->nrm, st->nrm1, st->nrm0);
+      k_gm_scale<VEC, T><<<grid, GM_THREADS, 0, s>>>(st->w, st->nrm, st->Q + (size_t)(j + 1) * vsz, items, nz, Ns,
+                                                     ncol, per);
       DY_CUDA(c, cudaMemsetAsync(st->res, 0, sizeof(unsigned long long), s));
       k_gm_givens<<<cb, 128, 0, s>>>(j, ncol, m, st->h, st->h2, st->nrm, st->bnorm, st->cs, st->sn, st->g, st->R,
                                      st->res);
@@ -504,12 +564,32 @@ int gmres_inner_solve(dyson_ctx* c, int ncol, const float* r, float* x, int max_
     }
     // x += Q_d y,  y = R^{-1} g
     k_gm_backsolve<<<cb, 128, 0, s>>>(d, ncol, m, st->R, st->g, st->y);
-    k_gm_combine<<<grid_el, GM_THREADS, 0, s>>>(st->Q, vsz, d, st->y, m, x, x, Nc, ncol);
+    k_gm_update<VEC, T><<<grid, GM_THREADS, 0, s>>>(st->Q, vsz, d, st->y, m, 1.f, x, nullptr, x, items, nz, Ns, ncol,
+                                                    per, nullptr, nullptr, nullptr);
     c->launches += 2;
     DY_CUDA(c, cudaGetLastError());
     if (rel <= tol) break;
   }
   return DYSON_OK;
+}
+
+}  // namespace
+
+int gmres_inner_solve(dyson_ctx* c, int ncol, const float* r, float* x, int max_iters, double tol,
+                      dyson_report* rep, const MatvecFn& matvec) {
+  if (ncol > 65535 || c->Nr > 65535) return ctx_fail(c, DYSON_ERR_INVALID_ARG, "GMRES chunks hold <= 65535 columns");
+  const int m = gmres_restart_length(c, ncol);
+  if (m < 2) return ctx_fail(c, DYSON_ERR_OOM, "GMRES needs room for at least 3 Krylov vectors");
+  const size_t vsz = (size_t)c->Nr * ncol * 2 * c->Ns;
+  int rc = gm_prepare(c, vsz, ncol, m);
+  if (rc) return rc;
+  // float4 items where every column's halves are 16-byte aligned (the tensor-core sweeps' stride is a
+  // multiple of 64; the CUDA-core sweep's is Nc)
+  if (c->Ns % 4 != 0) return gmres_run<1, 1>(c, ncol, r, x, max_iters, tol, rep, matvec, m);
+  const int t = (c->Ns + 127) / 128;                     // float4 per lane and part that cover a column
+  if (t == 1) return gmres_run<4, 1>(c, ncol, r, x, max_iters, tol, rep, matvec, m);
+  if (t % 3 == 0) return gmres_run<4, 3>(c, ncol, r, x, max_iters, tol, rep, matvec, m);
+  return gmres_run<4, 2>(c, ncol, r, x, max_iters, tol, rep, matvec, m);
 }
 
 void gmres_release(dyson_ctx* c) {

@@ -79,3 +79,25 @@ def test_fused_sweep_serves_every_contour(torch_cuda, lib, Nt, Nm, inner):
     want = dyson.dense_solve(S, dyson.rhs_vector_columns(S, list(zip(sites, times))))
     assert np.abs(v.cpu().numpy() - want.transpose(2, 0, 1)).max() / np.abs(want).max() < 1e-11
     s.close()
+
+
+@pytest.mark.parametrize("Nt,Nm", [(7, 5), (8, 4), (200, 112)])
+def test_gmres_item_shapes(torch_cuda, lib, Nt, Nm):
+    """The GMRES vector kernels on strides they cannot load as float4 (19), on the CUDA-core stride (20) and on a
+    contour of several items per column (512)."""
+    from paper_1309_5994_gb300 import binding
+    torch = torch_cuda
+    p = wl.random_tables(wl.small(L=2, Ly=2, Nt=Nt, Nm=Nm, dt=0.01, beta=1.0, trap_c=0.3, U0=14.0), seed=9, rel=0.1)
+    S = dyson.setup(p)
+    ref = dyson.dense_solve(S, dyson.rhs_block_columns(S, [1, 2]))
+    s = binding.Solver(p, device=0)
+    s.set_inner_solver(1)
+    s.build_sigma()
+    g = torch.empty((2, p.Nr, p.Nc, p.Nc), dtype=torch.complex128, device="cuda:0")
+    res = s.solve([1, 2], precision=binding.PREC_TF32X3_F64REF, tol=1e-12, g_out=g)
+    assert res.report["inner_gmres"] == 1
+    got = g.cpu().numpy()
+    for q in range(2):
+        want = ref[:, :, q * p.Nc:(q + 1) * p.Nc]
+        assert np.abs(got[q] - want).max() / np.abs(want).max() < 1e-11
+    s.close()
