@@ -157,9 +157,10 @@ __global__ void __launch_bounds__(GM_THREADS) k_gm_dots(const float* __restrict_
     double re[GM_GROUP] = {}, im[GM_GROUP] = {}, sq = 0.0;
     for (int item = i0 + warp; item < i1; item += GM_THREADS / 32) {
       const ItemPos at = item_pos<VEC, T>(item, nz, n, ncol, Ns, lane);
-      Slab<VEC, T> w, x;
+      Slab<VEC, T> w;
       load_slab(w, a, at, Ns);
       if (b) {
+        Slab<VEC, T> x;
         load_slab(x, b, at, Ns);
 #pragma unroll
         for (int t = 0; t < T; ++t)
@@ -170,17 +171,22 @@ __global__ void __launch_bounds__(GM_THREADS) k_gm_dots(const float* __restrict_
           }
       }
       if (self) sq += (double)slab_norm2(w);
+      // the next basis vector's loads are in flight while one is multiplied (a vector past the last
+      // reads the last one again; its sums are dropped)
+      Slab<VEC, T> q[2];
+      auto fetch = [&](int k) { load_slab(q[k & 1], Q + (size_t)min(g0 + k, nvec - 1) * vsz, at, Ns); };
+      fetch(0);
 #pragma unroll
       for (int k = 0; k < GM_GROUP; ++k) {
-        if (g0 + k >= nvec) break;
-        load_slab(x, Q + (size_t)(g0 + k) * vsz, at, Ns);
+        if (k + 1 < GM_GROUP) fetch(k + 1);
+        const Slab<VEC, T>& y = q[k & 1];
         float sr = 0.f, si = 0.f;
 #pragma unroll
         for (int t = 0; t < T; ++t)
 #pragma unroll
           for (int v = 0; v < VEC; ++v) {                // conj(q) w
-            sr = fmaf(x.re[t][v], w.re[t][v], fmaf(x.im[t][v], w.im[t][v], sr));
-            si = fmaf(x.re[t][v], w.im[t][v], fmaf(-x.im[t][v], w.re[t][v], si));
+            sr = fmaf(y.re[t][v], w.re[t][v], fmaf(y.im[t][v], w.im[t][v], sr));
+            si = fmaf(y.re[t][v], w.im[t][v], fmaf(-y.im[t][v], w.re[t][v], si));
           }
         re[k] += (double)sr;
         im[k] += (double)si;
@@ -285,7 +291,7 @@ __global__ void __launch_bounds__(GM_THREADS) k_gm_update(const float* __restric
   double acc = 0.0;
   for (int item = i0 + (int)(threadIdx.x >> 5); item < i1; item += GM_THREADS / 32) {
     const ItemPos at = item_pos<VEC, T>(item, nz, n, ncol, Ns, threadIdx.x & 31);
-    Slab<VEC, T> x, q[2];
+    Slab<VEC, T> x, q[3];
     load_slab(x, a, at, Ns);
     if (b) {
       load_slab(q[0], b, at, Ns);
@@ -306,16 +312,21 @@ __global__ void __launch_bounds__(GM_THREADS) k_gm_update(const float* __restric
           x.im[t][v] += c.x * y.im[t][v] + c.y * y.re[t][v];
         }
     };
-    int i = 0;
-    for (; i + 2 <= nvec; i += 2) {                      // two vectors' loads in flight
-      load_slab(q[0], Q + (size_t)i * vsz, at, Ns);
-      load_slab(q[1], Q + (size_t)(i + 1) * vsz, at, Ns);
+    // three vectors' loads in flight: two ahead of the one that is added
+    auto fetch = [&](Slab<VEC, T>& y, int i) {
+      if (i < nvec) load_slab(y, Q + (size_t)i * vsz, at, Ns);
+    };
+    fetch(q[0], 0);
+    fetch(q[1], 1);
+    for (int i = 0; i < nvec; i += 3) {
+      fetch(q[2], i + 2);
       fold(q[0], hs[i]);
+      if (i + 1 >= nvec) break;
+      fetch(q[0], i + 3);
       fold(q[1], hs[i + 1]);
-    }
-    if (i < nvec) {
-      load_slab(q[0], Q + (size_t)i * vsz, at, Ns);
-      fold(q[0], hs[i]);
+      if (i + 2 >= nvec) break;
+      fetch(q[1], i + 4);
+      fold(q[2], hs[i + 2]);
     }
     store_slab(x, w, at, Ns);
     acc += (double)slab_norm2(x);
