@@ -15,7 +15,7 @@
 // energy eps + U), and the trace is a sum over the four initial states.  For
 // fixed (a, b, d) the contour order of the four operators changes only where the
 // creator's point c passes a, b or d, so c runs through at most four intervals,
-// each with one operator order.  A host-built table gives, for each order, spin
+// each with one operator order.  A constexpr function gives, for each order, spin
 // case and initial state, the fermionic sign and the four channels; the kernel
 // adds per interval the coefficient of exp(i Phi_p(c)) F(c, b) for p = 1, 2.  The
 // interval sums over the real branches come from prefix sums over c (unit-modulus
@@ -54,16 +54,17 @@ void oz64_invalidate(dyson_ctx* c);
 namespace {
 
 // ---------------------------------------------------------------------------
-// operator-path table
+// operator paths
 // ---------------------------------------------------------------------------
 // operators of G2_{up s1}(a, b; c, d) in product order: kind 0 = c_up(a), 1 = c_s1(b),
-// 2 = c+_s1(c), 3 = c+_up(d).  An order is four kinds, latest first, coded
-// o0*64 + o1*16 + o2*4 + o3.  Entry [code][spin case * 4 + initial state]:
+// 2 = c+_s1(c), 3 = c+_up(d).  An order is four kinds, latest first.  Its path of one spin case and
+// initial state:
 //   bit 0 valid, bit 1 sign negative, bits 2..5 channel - 1 of kinds 0..3, bits 6..7 state class
 //   (0: |0>, 1: one particle, 2: doubly occupied).  The sign includes (-i)^2 = -1.
 constexpr int PATHS = 8;
 
-uint32_t path_entry(const int o[4], int spin_case, int nu) {
+constexpr uint32_t path_entry(int o0, int o1, int o2, int o3, int spin_case, int nu) {
+  const int o[4] = {o0, o1, o2, o3};
   // permutation parity of the order against the product order 0 1 2 3
   int inv = 0;
   for (int x = 0; x < 4; ++x)
@@ -88,21 +89,6 @@ uint32_t path_entry(const int o[4], int spin_case, int nu) {
   uint32_t e = 1u | (sign < 0 ? 2u : 0u);
   for (int k = 0; k < 4; ++k) e |= (uint32_t)ch[k] << (2 + k);
   return e | ((uint32_t)cls << 6);
-}
-
-std::vector<uint32_t> path_table() {
-  std::vector<uint32_t> t(256 * PATHS, 0);
-  int o[4];
-  for (o[0] = 0; o[0] < 4; ++o[0])
-    for (o[1] = 0; o[1] < 4; ++o[1])
-      for (o[2] = 0; o[2] < 4; ++o[2])
-        for (o[3] = 0; o[3] < 4; ++o[3]) {
-          if (o[0] == o[1] || o[0] == o[2] || o[0] == o[3] || o[1] == o[2] || o[1] == o[3] || o[2] == o[3]) continue;
-          const int code = o[0] * 64 + o[1] * 16 + o[2] * 4 + o[3];
-          for (int sc = 0; sc < 2; ++sc)
-            for (int nu = 0; nu < 4; ++nu) t[code * PATHS + sc * 4 + nu] = path_entry(o, sc, nu);
-        }
-  return t;
 }
 
 // ---------------------------------------------------------------------------
@@ -131,6 +117,30 @@ __device__ __forceinline__ double2 cexp_phase(double2 phi, double sgn) {
 __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ double2 cfma(double2 a, double2 b, double2 c) {
   return make_double2(fma(a.x, b.x, fma(-a.y, b.y, c.x)), fma(a.x, b.y, fma(a.y, b.x, c.y)));
+}
+
+// One path (spin case and initial state Q) of an operator order, added to its channel's coefficient: the
+// entry is a compile-time constant, so this is two FMAs with known registers, or nothing.
+// f[pad + 4 pb]: products of the factors at a, d (channels pa, pd: pad = 2 pa + pd) and b.
+template <int O0, int O1, int O2, int O3, int Q = 0>
+__device__ __forceinline__ void add_paths(const double2 (&f)[8], const double (&rho)[3], double2 (&A)[2]) {
+  constexpr uint32_t t = path_entry(O0, O1, O2, O3, Q / 4, Q % 4);
+  if constexpr (t & 1u) {
+    constexpr int x = ((t & 4u) ? 2 : 0) + ((t & 32u) ? 1 : 0) + ((t & 8u) ? 4 : 0), pc = (t & 16u) ? 1 : 0;
+    const double w = (t & 2u) ? -rho[(t >> 6) & 3u] : rho[(t >> 6) & 3u];
+    A[pc].x = fma(w, f[x].x, A[pc].x);
+    A[pc].y = fma(w, f[x].y, A[pc].y);
+  }
+  if constexpr (Q + 1 < PATHS) add_paths<O0, O1, O2, O3, Q + 1>(f, rho, A);
+}
+// coefficients of P_1(c), P_2(c) on the four c intervals for the fixed operators K0, K1, K2 (latest first);
+// interval iv: iv fixed operators are earlier than c
+template <int K0, int K1, int K2>
+__device__ __forceinline__ void interval_coefs(const double2 (&f)[8], const double (&rho)[3], double2 (&A)[4][2]) {
+  add_paths<K0, K1, K2, 2>(f, rho, A[0]);
+  add_paths<K0, K1, 2, K2>(f, rho, A[1]);
+  add_paths<K0, 2, K1, K2>(f, rho, A[2]);
+  add_paths<2, K0, K1, K2>(f, rho, A[3]);
 }
 
 // ---------------------------------------------------------------------------
@@ -189,13 +199,15 @@ __global__ void k_se_prefix(const double2* __restrict__ phase, const double2* __
 // grid (ceil(Nc^2 / 256), sites), 256 threads, one (a, d) per thread; blockIdx.y indexes `sites`
 // (all sites in order when NULL).  Per b the creator point c
 // runs through four intervals of fixed operator order: their real-branch parts come from the
-// prefix sums Q, their imaginary-branch parts are summed directly.
+// prefix sums Q, their imaginary-branch parts from sums over that branch's start or end, or directly.
+// Bound by the FP64 pipe (2 FMA per SM and clock).  64 sites, Nc = 64, Nm = 16: with eight FP64 operations
+// per operator path and a product per imaginary point 9.2 ms; with the factors' products shared by the
+// paths (two operations each) and the branch sums 5.5 ms.
 constexpr int CONN_THREADS = 256;
-__global__ void __launch_bounds__(CONN_THREADS) k_se_conn(const uint32_t* __restrict__ paths,
-                                                           const double2* __restrict__ phase,
+__global__ void __launch_bounds__(CONN_THREADS) k_se_conn(const double2* __restrict__ phase,
                                                            const double2* __restrict__ FT,
                                                            const double2* __restrict__ Q, int Nt, int Nm,
-                                                           const int* __restrict__ sites,
+                                                           const int* __restrict__ sites, int use_sums,
                                                            double2* __restrict__ conn) {
   extern __shared__ double2 sm[];
   const int Nc = 2 * Nt + Nm, R = 2 * Nt;
@@ -204,20 +216,16 @@ __global__ void __launch_bounds__(CONN_THREADS) k_se_conn(const uint32_t* __rest
   double2* ep = em + 2 * Nc;         // [2][Nc] exp(+i Phi_p(z)): creator factors
   double2* Qs = ep + 2 * Nc;         // [2][R + 1] prefix sums of the current b
   double2* Pi = Qs + 2 * (R + 1);    // [2][Nm] exp(+i Phi_p(c)) F(c, b) on the imaginary branch
-  uint32_t* tab = reinterpret_cast<uint32_t*>(Pi + 2 * Nm);   // [256][PATHS]
-  __shared__ double rho[3];
+  const int sums = use_sums ? 2 * (Nm + 1) : 0;
+  double2* Pb = Pi + 2 * Nm;         // [2][Nm + 1] its sums from the branch's start up to each point
+  double2* Pe = Pb + sums;           // [2][Nm + 1] its sums from each point to the branch's end
   const double2* ph = phase + (size_t)i * (2 * Nc + 2);
   for (int e = threadIdx.x; e < 2 * Nc; e += blockDim.x) {
     em[e] = cexp_phase(ph[e], 1.0);
     ep[e] = cexp_phase(ph[e], -1.0);
   }
-  for (int e = threadIdx.x; e < 256 * PATHS; e += blockDim.x) tab[e] = paths[e];
-  if (threadIdx.x == 0) {
-    const double2 l1 = ph[2 * Nc], l2 = ph[2 * Nc + 1];  // (log rho_0, log rho_s), (log rho_s, log rho_d)
-    rho[0] = exp(l1.x);
-    rho[1] = exp(l1.y);
-    rho[2] = exp(l2.y);
-  }
+  // Boltzmann weights from (log rho_0, log rho_s), (log rho_s, log rho_d)
+  const double rho[3] = {exp(ph[2 * Nc].x), exp(ph[2 * Nc].y), exp(ph[2 * Nc + 1].y)};
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   const bool live = e < Nc * Nc;
   const int a = live ? e / Nc : 0, d = live ? e % Nc : 0;
@@ -244,6 +252,18 @@ __global__ void __launch_bounds__(CONN_THREADS) k_se_conn(const uint32_t* __rest
       Pi[Nm + x] = cmul(ep[Nc + R + x], f);
     }
     __syncthreads();
+    if (use_sums && threadIdx.x < 4) {                 // one warp each would not be faster: Nm additions in a row
+      const int p = threadIdx.x & 1;
+      double2 sum = make_double2(0.0, 0.0);
+      if (threadIdx.x < 2) {
+        Pb[p * (Nm + 1)] = sum;
+        for (int x = 0; x < Nm; ++x) Pb[p * (Nm + 1) + x + 1] = sum = cadd(sum, Pi[p * Nm + x]);
+      } else {
+        Pe[p * (Nm + 1) + Nm] = sum;
+        for (int x = Nm - 1; x >= 0; --x) Pe[p * (Nm + 1) + x] = sum = cadd(Pi[p * Nm + x], sum);
+      }
+    }
+    __syncthreads();
     const int Kb = key_ann(b, Nt, 1);
     // the three fixed operators, latest first
     int k0 = 0, k1 = 1, k2 = 3;                          // kinds
@@ -252,32 +272,24 @@ __global__ void __launch_bounds__(CONN_THREADS) k_se_conn(const uint32_t* __rest
     if (K2 > K1) { int t = K1; K1 = K2; K2 = t; t = k1; k1 = k2; k2 = t; }
     if (K1 > K0) { int t = K0; K0 = K1; K1 = t; t = k0; k0 = k1; k1 = t; }
     const int n0 = first_c_above(K0, Nt), n1 = first_c_above(K1, Nt), n2 = first_c_above(K2, Nt);
-    const double2 fb0 = em[b], fb1 = em[Nc + b];
-    // coefficients of P_1(c), P_2(c) on the four c intervals
+    // products of the factors at a, d and b for the eight channel triples, shared by the four intervals
+    double2 fabd[8];
+#pragma unroll
+    for (int x = 0; x < 8; ++x) fabd[x] = cmul(fad[x & 3], em[(x >> 2) * Nc + b]);
+    // coefficients of P_1(c), P_2(c) on the four c intervals, one branch per order of a, b, d (a warp's
+    // threads share a and b, so it takes two or three of them at most)
     double2 A[4][2];
 #pragma unroll
-    for (int iv = 0; iv < 4; ++iv) {
-      // iv = number of fixed operators earlier than c
-      const int code = iv == 0 ? (k0 * 64 + k1 * 16 + k2 * 4 + 2)
-                     : iv == 1 ? (k0 * 64 + k1 * 16 + 2 * 4 + k2)
-                     : iv == 2 ? (k0 * 64 + 2 * 16 + k1 * 4 + k2)
-                               : (2 * 64 + k0 * 16 + k1 * 4 + k2);
-      double2 s1 = make_double2(0.0, 0.0), s2 = make_double2(0.0, 0.0);
-#pragma unroll
-      for (int q = 0; q < PATHS; ++q) {
-        const uint32_t t = tab[code * PATHS + q];
-        if (!(t & 1u)) continue;
-        const double w = ((t & 2u) ? -1.0 : 1.0) * rho[(t >> 6) & 3u];
-        const int pad = ((t & 4u) ? 2 : 0) + ((t & 32u) ? 1 : 0);
-        const double2 f1 = pad == 0 ? fad[0] : pad == 1 ? fad[1] : pad == 2 ? fad[2] : fad[3];
-        double2 v = cmul(f1, (t & 8u) ? fb1 : fb0);
-        v.x *= w;
-        v.y *= w;
-        if (t & 16u) s2 = cadd(s2, v);
-        else s1 = cadd(s1, v);
-      }
-      A[iv][0] = s1;
-      A[iv][1] = s2;
+    for (int iv = 0; iv < 4; ++iv) A[iv][0] = A[iv][1] = make_double2(0.0, 0.0);
+    if (k0 == 0) {
+      if (k1 == 1) interval_coefs<0, 1, 3>(fabd, rho, A);
+      else interval_coefs<0, 3, 1>(fabd, rho, A);
+    } else if (k0 == 1) {
+      if (k1 == 0) interval_coefs<1, 0, 3>(fabd, rho, A);
+      else interval_coefs<1, 3, 0>(fabd, rho, A);
+    } else {
+      if (k1 == 0) interval_coefs<3, 0, 1>(fabd, rho, A);
+      else interval_coefs<3, 1, 0>(fabd, rho, A);
     }
     // real branches: interval iv covers [lo, hi) with lo/hi from (0, n2, n1, n0, Nc), clipped to R
     {
@@ -290,13 +302,28 @@ __global__ void __launch_bounds__(CONN_THREADS) k_se_conn(const uint32_t* __rest
         acc = cfma(A[iv][0], q1, cfma(A[iv][1], q2, acc));
       }
     }
-    // imaginary branch: direct
-    for (int x = 0; x < Nm; ++x) {
-      const int c = R + x;
-      const bool g0 = c >= n0, g1 = c >= n1, g2 = c >= n2;
-      const double2 x0 = g0 ? A[3][0] : g1 ? A[2][0] : g2 ? A[1][0] : A[0][0];
-      const double2 x1 = g0 ? A[3][1] : g1 ? A[2][1] : g2 ? A[1][1] : A[0][1];
-      acc = cfma(x0, Pi[x], cfma(x1, Pi[Nm + x], acc));
+    // imaginary branch: the interval that contains its start takes the sum from there, the last one the
+    // sum to its end (sums of the summands themselves: nothing cancels that did not before); what
+    // lies between, only where two of a, b, d are on this branch, is summed directly
+    {
+      const int x2 = max(n2 - R, 0), x1 = max(n1 - R, 0), x0 = max(n0 - R, 0);   // interval bounds 0 | x2 | x1 | x0 | Nm
+      auto add = [&](int iv, double2 p1, double2 p2) { acc = cfma(A[iv][0], p1, cfma(A[iv][1], p2, acc)); };
+      auto direct = [&](int iv, int from, int to) {
+        for (int x = from; x < to; ++x) add(iv, Pi[x], Pi[Nm + x]);
+      };
+      if (!use_sums) {
+        direct(0, 0, x2);
+        direct(1, x2, x1);
+        direct(2, x1, x0);
+        direct(3, x0, Nm);
+        continue;
+      }
+      if (x2 > 0) add(0, Pb[x2], Pb[Nm + 1 + x2]);
+      else if (x1 > 0) add(1, Pb[x1], Pb[Nm + 1 + x1]);
+      else if (x0 > 0) add(2, Pb[x0], Pb[Nm + 1 + x0]);
+      if (x2 > 0) direct(1, x2, x1);
+      if (x1 > 0) direct(2, x1, x0);
+      if (x0 < Nm) add(3, Pe[x0], Pe[Nm + 1 + x0]);
     }
   }
   if (live) conn[((size_t)i * Nc + a) * Nc + d] = acc;
@@ -647,7 +674,6 @@ struct SeState {
   int Nr = 0, Nc = 0;
   double2 *g0 = nullptr, *Sm = nullptr, *FT = nullptr, *conn = nullptr, *w1 = nullptr, *w2 = nullptr,
           *St = nullptr, *tr = nullptr, *Q = nullptr;
-  uint32_t* paths = nullptr;
   double* part = nullptr;
   int* err = nullptr;
   int* reps = nullptr;               // [Nr] orbit representatives, when the context has C4v set
@@ -676,7 +702,7 @@ void free_aa(SeState* st) {
 }
 
 void free_state(SeState* st) {
-  void* ptrs[] = {st->g0, st->Sm, st->FT, st->conn, st->w1, st->w2, st->St, st->tr, st->Q, st->paths, st->part,
+  void* ptrs[] = {st->g0, st->Sm, st->FT, st->conn, st->w1, st->w2, st->St, st->tr, st->Q, st->part,
                   st->err, st->reps};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -770,12 +796,9 @@ int ensure_state(dyson_ctx* c) {
   for (double2** b : bufs) ok = ok && cudaMalloc(b, blk) == cudaSuccess;
   ok = ok && cudaMalloc(&st->Q, (size_t)c->Nr * 2 * c->Nc * (2 * c->Nt + 1) * sizeof(double2)) == cudaSuccess &&
        cudaMalloc(&st->tr, (size_t)c->Nr * sizeof(double2)) == cudaSuccess &&
-       cudaMalloc(&st->paths, 256 * PATHS * sizeof(uint32_t)) == cudaSuccess &&
        cudaMalloc(&st->part, 2 * MIX_BLOCKS * sizeof(double)) == cudaSuccess &&
        cudaMalloc(&st->err, (size_t)c->Nr * sizeof(int)) == cudaSuccess &&
        cudaMalloc(&st->reps, (size_t)c->Nr * sizeof(int)) == cudaSuccess;
-  const std::vector<uint32_t> tab = path_table();
-  ok = ok && cudaMemcpy(st->paths, tab.data(), tab.size() * sizeof(uint32_t), cudaMemcpyHostToDevice) == cudaSuccess;
   if (!ok) {                                             // nothing half-built stays behind
     cudaGetLastError();
     free_state(st);
@@ -917,8 +940,11 @@ extern "C" int dyson_selfenergy_step(dyson_ctx* c, const double* gloc, double mi
   // F (transposed), the connected contraction, the disconnected terms
   k_se_hyb<<<tiles32(Nc, Nr), dim3(32, 8), 0, c->stream>>>(G, c->d_JW, c->d_nbr, c->d_nbond, Nc, st->FT);
   const int R = 2 * c->Nt;
-  const size_t smem = (4 * (size_t)Nc + 2 * (R + 1) + 2 * (size_t)c->Nm) * sizeof(double2) +
-                      256 * PATHS * sizeof(uint32_t);
+  size_t smem = (4 * (size_t)Nc + 2 * (R + 1) + 2 * (size_t)c->Nm) * sizeof(double2);
+  // the imaginary branch's partial sums where shared memory holds them too
+  const size_t sums = 4 * ((size_t)c->Nm + 1) * sizeof(double2);
+  const int use_sums = smem + sums <= 220 * 1024;
+  if (use_sums) smem += sums;
   if (smem > 48 * 1024)
     DY_CUDA(c, cudaFuncSetAttribute(k_se_conn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   // with C4v the contraction runs for one site per orbit; a site s = g(r) has F_s = F_r and
@@ -938,7 +964,7 @@ extern "C" int dyson_selfenergy_step(dyson_ctx* c, const double* gloc, double mi
     k_se_prefix<<<dim3((unsigned)((2 * Nc + 127) / 128), n_conn), 128, 0, c->stream>>>(c->d_phase, st->FT, c->Nt,
                                                                                       c->Nm, d_sites, st->Q);
     k_se_conn<<<dim3((unsigned)((Nc * Nc + CONN_THREADS - 1) / CONN_THREADS), n_conn), CONN_THREADS, smem,
-                c->stream>>>(st->paths, c->d_phase, st->FT, st->Q, c->Nt, c->Nm, d_sites, st->conn);
+                c->stream>>>(c->d_phase, st->FT, st->Q, c->Nt, c->Nm, d_sites, use_sums, st->conn);
   }
   if (!reps.empty()) {
     const size_t blk = (size_t)Nc * Nc;
