@@ -20,13 +20,12 @@
 // complex modulus).
 //
 // Kernels: k_oz64_aprep (once per Lambda), k_oz64_xprep (gather, scale, digits of X),
-// k_oz64_gemm (persistent: TMA + tcgen05.mma kind::f16, 128 x 64 tiles); k_oz64_tslice slices the
+// k_oz64_gemm (persistent: bulk copies + tcgen05.mma kind::f16, 128 x 64 tiles); k_oz64_tslice slices the
 // operands of a batched complex product (the adjoint's site contraction) for the same kernel.
 #include <algorithm>
 #include <type_traits>
 
 #include <cuda_bf16.h>
-#include <cudaTypedefs.h>
 
 #include "common.cuh"
 #include "oz64.cuh"
@@ -37,10 +36,12 @@ namespace {
 constexpr int S = 8;                                      // digits of 7 bits
 constexpr int FIX = 7 * S;
 constexpr int BM = 128, BN = 64, BK = 32;                 // 32 bf16 = 64-byte rows (64-byte swizzle)
+constexpr int ROW_BYTES = BK * 2;
 constexpr int A_TILE = BM * BK * 2;                       // 8 KB per A slice
 constexpr int X_TILE = BN * BK * 2;                       // 4 KB per X slice
 constexpr int STAGE_BYTES = S * (A_TILE + X_TILE);        // 96 KB
 constexpr int STAGES = 2;
+constexpr int HALF = S / 2;                               // accumulator blocks of a group
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024;
 constexpr int SEG_KB = 512 / BK;                          // k-blocks of one exact K segment
 constexpr int THREADS = 640;                              // warp 0 TMA, warp 1 MMA, warps 4-19 epilogue
@@ -51,17 +52,35 @@ constexpr int E_BAD = 1 << 20;                            // scale exponent of a
 // kind::f16, D = F32, A = B = BF16, K-major, M = 128 (N set per MMA)
 constexpr uint32_t IDESC0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BM >> 4) << 24);
 
+// The slices are stored as the GEMM's shared memory holds them, so that a stage arrives in one or a few bulk
+// copies: per site, tile of BT rows (the last one with the R rows that are left) and k-block the S slice
+// tiles, R rows of 64 bytes each, 16-byte pieces swizzled as SWIZZLE_64B does.  (Tensor-map copies of
+// 64-byte rows delivered 96 KB in 3000 to 6000 cycles, the MMAs on it take 2600.)
+struct SliceRow {
+  __nv_bfloat162* p;
+  size_t block;                                            // pairs of a k-block's S slice tiles
+  int slice, sw;                                           // pairs of a slice tile; the row's swizzle
+  __device__ __forceinline__ SliceRow(__nv_bfloat16* base, size_t site, int rows, int BT, int row, int Kp) {
+    const int t = row / BT, R = min(BT, rows - t * BT), in = row - t * BT;
+    slice = R * (BK / 2);
+    block = (size_t)S * slice;
+    sw = (in >> 1) & 3;
+    p = reinterpret_cast<__nv_bfloat162*>(base) + (site * rows + (size_t)t * BT) * ((size_t)Kp / 2 * S) + in * (BK / 2);
+  }
+  // pair k (elements 2 k, 2 k + 1) of slice 1; slice s lies (s - 1) * slice further
+  __device__ __forceinline__ __nv_bfloat162* at(int k) const {
+    return p + (size_t)(k / (BK / 2)) * block + ((((k >> 2) & 3) ^ sw) << 2) + (k & 3);
+  }
+};
+
 struct Oz64State {
-  CUtensorMap amap, xmap;
-  __nv_bfloat16* as = nullptr;        // [S][Nr][2Nc][Kp]
+  __nv_bfloat16* as = nullptr;        // tiles of the 2 Nc rows of every site (SliceRow)
   int* esig = nullptr;                // [Nr][2Nc] row scale exponents
   size_t a_bytes = 0;
   bool a_ready = false;
-  __nv_bfloat16* xs = nullptr;        // [S][Nr][ncol][Kp]
+  __nv_bfloat16* xs = nullptr;        // tiles of the ncol columns of every site
   int* etau = nullptr;                // [Nr][ncol] column scale exponents
   size_t x_bytes = 0, tau_bytes = 0;
-  const void* xmap_ptr = nullptr;
-  int xmap_ncol = -1;
   int* d_err = nullptr;
   int num_sms = 1;
   bool smem_set = false;
@@ -151,7 +170,7 @@ __global__ void __launch_bounds__(256) k_oz64_aprep(const double2* __restrict__ 
   const int e = scale_exponent(mb);
   const size_t r0 = 2 * row;                               // = i N2 + 2 z
   if (lane < 2) esig[r0 + lane] = e;
-  const size_t stride = (size_t)Nr * N2 * Kp;
+  const SliceRow dst(as, row / Nc, N2, BM, 2 * (int)(row % Nc), Kp);
   for (int k = lane; 2 * k < Kp; k += 32) {
     const double2 v = k < Nc ? value(k) : make_double2(0.0, 0.0);
     const unsigned long long Ar = biased_digits(v.x, e), Ai = biased_digits(v.y, e);
@@ -159,9 +178,9 @@ __global__ void __launch_bounds__(256) k_oz64_aprep(const double2* __restrict__ 
     const PairSigns top = pair_signs(nr, !ni), bot = pair_signs(ni, nr);
     each_digit([&](auto sc) {
       constexpr int s = decltype(sc)::value;
-      __nv_bfloat162* d = reinterpret_cast<__nv_bfloat162*>(as + (s - 1) * stride + r0 * Kp) + k;
+      __nv_bfloat162* d = dst.at(k) + (s - 1) * dst.slice;
       d[0] = digit_pair<s>(Ar, Ai, top);
-      d[Kp / 2] = digit_pair<s>(Ai, Ar, bot);
+      d[BK / 2] = digit_pair<s>(Ai, Ar, bot);              // the next row: the same swizzle
     });
   }
 }
@@ -169,6 +188,8 @@ __global__ void __launch_bounds__(256) k_oz64_aprep(const double2* __restrict__ 
 // One warp per (site i, vector column n), sites fastest (the four reads of a neighbour's column
 // meet in L2): X = sum_j J_ij G_j in FP64, column scale, digits.  UNIFORM: J sits in the Lambda
 // slices.  PER_LANE contour points per lane in registers; PER_LANE = 0: any Nc, X summed twice.
+// Bound by the FP64 pipe (83 % busy): 8x8, Nc = 64, 4096 columns 0.259 ms with four additions per part,
+// 0.197 with the three it needs (floor of its bytes 0.118).
 template <bool UNIFORM, int PER_LANE>
 __global__ void __launch_bounds__(256) k_oz64_xprep(const double2* __restrict__ G, const double* __restrict__ Jtab,
                                                     const int* __restrict__ nbr, const int* __restrict__ nbond, int Nr,
@@ -197,12 +218,16 @@ __global__ void __launch_bounds__(256) k_oz64_xprep(const double2* __restrict__ 
       if (!has[q]) continue;
       const double2 g = col[q][z];
       if (UNIFORM) {
-        x.x += g.x;
-        x.y += g.y;
+        if (q == 0) {                                      // (x is still zero: one FP64 addition less)
+          x = g;
+        } else {
+          x.x += g.x;
+          x.y += g.y;
+        }
       } else {
         const double j = jrow[q][tk];
-        x.x = fma(j, g.x, x.x);
-        x.y = fma(j, g.y, x.y);
+        x.x = q == 0 ? j * g.x : fma(j, g.x, x.x);
+        x.y = q == 0 ? j * g.y : fma(j, g.y, x.y);
       }
     }
     return x;
@@ -226,14 +251,13 @@ __global__ void __launch_bounds__(256) k_oz64_xprep(const double2* __restrict__ 
   for (int o = 16; o > 0; o >>= 1) mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, o));
   const int e = scale_exponent(mb);
   if (lane == 0) etau[w] = e;
-  const size_t stride = (size_t)Nr * ncol * Kp;
-  __nv_bfloat162* dst = reinterpret_cast<__nv_bfloat162*>(xs + w * Kp);
+  const SliceRow dst(xs, i, ncol, BN, n, Kp);
   auto put = [&](int z, double2 v) {
     const unsigned long long Ar = biased_digits(v.x, e), Ai = biased_digits(v.y, e);
     const PairSigns g = pair_signs(sign_of(v.x), sign_of(v.y));
     each_digit([&](auto sc) {
       constexpr int s = decltype(sc)::value;
-      dst[(s - 1) * (stride / 2) + z] = digit_pair<s>(Ar, Ai, g);
+      dst.at(z)[(s - 1) * dst.slice] = digit_pair<s>(Ar, Ai, g);
     });
   };
   if (PER_LANE > 0) {
@@ -278,7 +302,6 @@ __global__ void __launch_bounds__(256) k_oz64_tslice(const double2* __restrict__
     if (AROWS) ex[(size_t)b * rows + 2 * (t0 + lane)] = ex[(size_t)b * rows + 2 * (t0 + lane) + 1] = e;
     else ex[(size_t)b * rows + t0 + lane] = e;
   }
-  const size_t stride = (size_t)batch * rows * Kp;
   for (int i0 = 0; 2 * i0 < Kp; i0 += 32) {
     for (int r = warp; r < 32; r += 8)
       tile[r][lane] = i0 + r < nk && t0 + lane < Nc ? Vb[(size_t)(i0 + r) * Nc + t0 + lane] : make_double2(0.0, 0.0);
@@ -289,13 +312,13 @@ __global__ void __launch_bounds__(256) k_oz64_tslice(const double2* __restrict__
         const int e = (int)smax[0][r];
         const unsigned long long Ar = biased_digits(v.x, e), Ai = biased_digits(v.y, e);
         const bool nr = sign_of(v.x), ni = sign_of(v.y);
-        const size_t row = (size_t)b * rows + (AROWS ? 2 : 1) * (t0 + r);
+        const SliceRow dst(sl, b, rows, AROWS ? BM : BN, (AROWS ? 2 : 1) * (t0 + r), Kp);
         const PairSigns top = pair_signs(nr, AROWS ? !ni : ni), bot = pair_signs(ni, nr);
         each_digit([&](auto sc) {
           constexpr int s = decltype(sc)::value;
-          __nv_bfloat162* d = reinterpret_cast<__nv_bfloat162*>(sl + (s - 1) * stride + row * Kp) + i0 + lane;
+          __nv_bfloat162* d = dst.at(i0 + lane) + (s - 1) * dst.slice;
           d[0] = digit_pair<s>(Ar, Ai, top);
-          if (AROWS) d[Kp / 2] = digit_pair<s>(Ai, Ar, bot);
+          if (AROWS) d[BK / 2] = digit_pair<s>(Ai, Ar, bot);
         });
       }
     __syncthreads();
@@ -316,6 +339,19 @@ __device__ __forceinline__ double fixed_to_double(long long V, int e) {
   return __longlong_as_double((long long)(bits | ((unsigned long long)V & 0x8000000000000000ull)));
 }
 
+// The same where every nonzero result is in the normal range (|e| < 900), in two thirds of the instructions
+__device__ __forceinline__ double fixed_to_double_normal(long long V, int e) {
+  const unsigned long long a = (unsigned long long)(V < 0 ? -V : V);
+  const unsigned int ah = (unsigned int)(a >> 32), al = (unsigned int)a;
+  const unsigned int hi = ah ? ah : al, lo = ah ? al : 0u;
+  const int lz = __clz((int)hi);
+  const unsigned int mh = __funnelshift_l(lo, hi, lz), ml = lo << (lz & 31);
+  const unsigned long long q = (((unsigned long long)(mh >> 11) << 32) | __funnelshift_r(ml, mh, 11)) + ((ml >> 10) & 1);
+  const unsigned int top = (unsigned int)((ah ? 1085 : 1053) - lz + e) << 20;
+  const unsigned int h = (unsigned int)(q >> 32) + top;
+  return __hiloint2double((int)(((a == 0 ? 0u : h)) | ((unsigned int)(V >> 32) & 0x80000000u)), (int)(unsigned int)q);
+}
+
 // |d| as FP32 from its bits (truncated; no conversion on the FP64 pipe): 0 below 2^-126, inf from 2^127
 // and for NaN
 __device__ __forceinline__ float magnitude(double d) {
@@ -326,24 +362,29 @@ __device__ __forceinline__ float magnitude(double d) {
 // sqrt of a running maximum of squares (inf stays inf)
 __device__ __forceinline__ void flush_norm(float sq, unsigned long long* norm, int lane) {
   for (int o = 16; o > 0; o >>= 1) sq = fmaxf(sq, __shfl_xor_sync(0xffffffffu, sq, o));
-  if (lane == 0) atomicMax(norm, (unsigned long long)__double_as_longlong(sqrt((double)sq)));
+  // (an FP64 square root, even of one lane, holds the SM's FP64 pipe for hundreds of cycles a warp)
+  if (lane == 0) atomicMax(norm, (unsigned long long)__double_as_longlong((double)sqrtf(sq)));
 }
 
 // Persistent: one CTA per SM walks 128 x 64 output tiles (row tile fastest, then column tile, then
 // site).  A stage is a 32-deep k-block of all eight slices of both operands.  Per k16 step,
 // slice s of A times slices 1..9-s of X (back to back in the stage) lands in the TMEM blocks of
 // diagonals s+1..9: twelve MMAs of N <= 256 for the 36 products.
-// The eight accumulators fill TMEM, so the MMAs of a tile wait until the epilogue has read the
-// previous tile's into int64 registers; the rest of the epilogue overlaps them.  64 columns per
-// tile, because at 32 (two sets) each A slice would be read from L2 twice as often.
-// Measured on 10x10, Nc = 128, 512 columns (6.7 GFLOP of FP64): 0.19 ms, against 6.33 ms of the FP64-pipe
-// kernel.  A k-block's 24 MMAs take about 2600 cycles; reading the accumulators out takes
-// 4400 of a tile's 31000 cycles, and loads of the slices from DRAM another 6000 that two stages do
-// not hide.  Sixteen epilogue warps, their G loaded ahead and integer forms of the FP64
-// conversions: with eight warps that loaded G as they went the epilogue alone took 0.39 ms.
+// The eight accumulators fill TMEM, in two groups with barriers of their own: a segment's last k-block
+// finishes diagonals 2..5 first, which the epilogue reads into int64 registers under the products of
+// diagonals 6..9, and the next tile's first k-block starts on each group as soon as it is read.  The
+// rest of the epilogue overlaps the MMAs.  64 columns per tile, because at 32 (two sets) each A slice
+// would be read from L2 twice as often.
+// Measured per launch: 10x10, Nc = 128, 512 columns (6.7 GFLOP of FP64) 0.160 ms, 8x8, Nc = 64, 4096
+// columns 0.244 ms; the FP64-pipe kernel took 6.33 and 8.04 ms.  On the way there (10x10 / 8x8, ms): one
+// accumulator group and tensor-map copies 0.190 / 0.298; the epilogue's loop without branches - / 0.285;
+// two groups 0.176 / 0.252; slices in tile order 0.160 / 0.244.  k-blocks of 16 in four stages: 0.173 /
+// 0.256 (a k-block of 16 takes 1560 cycles, one of 32 2680; the tensor rate alone would be 2304).
+// Nc = 128 is bound by the MMAs, Nc = 64 by the epilogue (about 13000 of a tile's 16500 cycles) and the
+// 1.1 GB of DRAM traffic.
 template <int MODE>
 __global__ void __launch_bounds__(THREADS, 1)
-    k_oz64_gemm(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap xmap,
+    k_oz64_gemm(const __nv_bfloat16* __restrict__ as, const __nv_bfloat16* __restrict__ xs,
                 const int* __restrict__ esig, const int* __restrict__ etau, const double* __restrict__ Gin,
                 const double2* __restrict__ lam, const int* __restrict__ src_site, const int* __restrict__ src_time,
                 int Nr, int Nc, int KB, int ncol, int gs, double* __restrict__ out, float* __restrict__ r32, int Ns,
@@ -351,7 +392,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   using namespace ptx;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], acc_full, acc_empty, drain;
+  __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], acc_full[2], acc_empty[2], drain;
   __shared__ uint32_t tmem_holder;
   __shared__ WaitCtl wctl;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -365,8 +406,10 @@ __global__ void __launch_bounds__(THREADS, 1)
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
-    mbar_init(&acc_full, 1);
-    mbar_init(&acc_empty, 512);
+    for (int h = 0; h < 2; ++h) {
+      mbar_init(&acc_full[h], 1);
+      mbar_init(&acc_empty[h], 512);
+    }
     mbar_init(&drain, 1);
     wait_ctl_init(&wctl);
     fence_barrier_init();
@@ -386,6 +429,9 @@ __global__ void __launch_bounds__(THREADS, 1)
       bool ok = true;
       for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
         const int mt = tile % MT, nt = (tile / MT) % NT, site = tile / (MT * NT);
+        const uint32_t ra = min(BM, N2 - mt * BM) * ROW_BYTES, rx = min(BN, ncol - nt * BN) * ROW_BYTES;
+        const uint8_t* pa = reinterpret_cast<const uint8_t*>(as) + ((size_t)site * N2 + mt * BM) * KB * (S * ROW_BYTES);
+        const uint8_t* px = reinterpret_cast<const uint8_t*>(xs) + ((size_t)site * ncol + nt * BN) * KB * (S * ROW_BYTES);
         for (int kb = 0; kb < KB; ++kb, ++g) {
           const int s = g % STAGES;
           if (g >= STAGES && !mbar_wait(&empty[s], ((g / STAGES) - 1) & 1, abort_p)) {
@@ -393,11 +439,15 @@ __global__ void __launch_bounds__(THREADS, 1)
             break;
           }
           uint8_t* st = stage_ptr(s);
-          mbar_expect_tx(&full[s], STAGE_BYTES);
-          for (int q = 0; q < S; ++q) {
-            tma_load_4d(st + q * A_TILE, &amap, &full[s], kb * BK, mt * BM, site, q);
-            tma_load_4d(st + S * A_TILE + q * X_TILE, &xmap, &full[s], kb * BK, nt * BN, site, q);
-          }
+          mbar_expect_tx(&full[s], S * (ra + rx));
+          // (rows of a tile's end that no copy writes hold what was there: only unused results see them)
+          auto load = [&](uint8_t* to, uint32_t tile_bytes, const uint8_t* from, uint32_t bytes) {
+            if (bytes == tile_bytes) bulk_load(to, from, S * tile_bytes, &full[s]);
+            else
+              for (int q = 0; q < S; ++q) bulk_load(to + q * tile_bytes, from + q * bytes, bytes, &full[s]);
+          };
+          load(st, A_TILE, pa + (size_t)kb * S * ra, ra);
+          load(st + S * A_TILE, X_TILE, px + (size_t)kb * S * rx, rx);
         }
       }
       for (int q = g > STAGES ? g - STAGES : 0; q < g; ++q)
@@ -409,40 +459,40 @@ __global__ void __launch_bounds__(THREADS, 1)
       int g = 0, t = 0;
       bool ok = true, any = false;
       for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
-        for (int kb = 0; kb < KB; ++kb, ++g) {
-          const bool first = kb % SEG_KB == 0;
-          if (first) {                                      // a new segment overwrites the accumulators
-            if (t >= 1 && !mbar_wait(&acc_empty, (t - 1) & 1, abort_p)) {
-              ok = false;
-              break;
-            }
-            ++t;
-            tc_fence_after();
-          }
+        for (int kb = 0; kb < KB && ok; ++kb, ++g) {
+          const bool first = kb % SEG_KB == 0;              // a new segment overwrites the accumulators
+          const bool last = kb + 1 == KB || (kb + 1) % SEG_KB == 0;
           const int s = g % STAGES;
           if (!mbar_wait(&full[s], (g / STAGES) & 1, abort_p)) {
             ok = false;
             break;
           }
-          tc_fence_after();
           const uint32_t base = smem_u32(stage_ptr(s));
+          // blocks 0..3 first, so that the epilogue empties them under the other blocks' products
 #pragma unroll
-          for (int k16 = 0; k16 < BK / 16; ++k16) {
+          for (int h = 0; h < 2; ++h) {
+            if (first && t >= 1 && !mbar_wait(&acc_empty[h], (t - 1) & 1, abort_p)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
 #pragma unroll
-            for (int sl = 0; sl < S; ++sl) {
-              const uint64_t ad = sdesc_sw64(base + sl * A_TILE + k16 * 32);
+            for (int k16 = 0; k16 < BK / 16; ++k16) {
 #pragma unroll
-              for (int t0 = 0; t0 < S - sl; t0 += 256 / BN) {
-                const int nblk = (S - sl - t0) < 256 / BN ? (S - sl - t0) : 256 / BN;
+              for (int sl = 0; sl < (h ? S : HALF); ++sl) {
+                const int t0 = h && sl < HALF ? HALF - sl : 0;            // first X slice
+                const int nblk = (h ? S : HALF) - (h && sl < HALF ? HALF : sl);   // <= 4: N <= 256
                 const uint32_t idesc = IDESC0 | ((uint32_t)(nblk * BN >> 3) << 17);
-                const uint64_t xd = sdesc_sw64(base + S * A_TILE + t0 * X_TILE + k16 * 32);
-                mma<0>(tmem + (uint32_t)((sl + t0) * BN), ad, xd, idesc, (first && k16 == 0 && sl == 0) ? 0u : 1u);
+                mma<0>(tmem + (uint32_t)((sl + t0) * BN), sdesc_sw64(base + sl * A_TILE + k16 * 32),
+                       sdesc_sw64(base + S * A_TILE + t0 * X_TILE + k16 * 32), idesc,
+                       (first && k16 == 0 && sl == 0) ? 0u : 1u);
               }
             }
+            any = true;
+            if (h) mma_commit(&empty[s]);
+            if (last) mma_commit(&acc_full[h]);
           }
-          mma_commit(&empty[s]);
-          any = true;
-          if (kb + 1 == KB || (kb + 1) % SEG_KB == 0) mma_commit(&acc_full);
+          if (last) ++t;
         }
       }
       if (any) {
@@ -473,47 +523,79 @@ __global__ void __launch_bounds__(THREADS, 1)
           __ballot_sync(0xffffffffu, MODE != 2 && lane < cols && __ldg(src_site + n_first + lane) == site);
       const size_t off0 = ((size_t)site * ncol + n_first) * N2 + (row_ok ? m : 0);
       // G of this lane's row, eight columns at a time (the first ones before the wait)
-      double gin[8];
-      auto load_g = [&](int c) {
+      double gin[2][8];
+      auto load_g = [&](int h) {
+        const int c = 8 * h;
 #pragma unroll
         for (int j = 0; j < 8; ++j)
-          gin[j] = MODE != 2 && c + j < cols ? __ldg(Gin + off0 + (size_t)(c + j) * N2) : 0.0;
+          gin[h][j] = MODE != 2 && c + j < cols ? __ldg(Gin + off0 + (size_t)(c + j) * N2) : 0.0;
       };
       load_g(0);
       long long V[COLS_PER_WARP];
       for (int seg = 0; seg < nseg; ++seg, ++t) {
-        go = mbar_wait(&acc_full, t & 1, abort_p);
-        go = __all_sync(0xffffffffu, go);                   // tcgen05.ld below is warp-collective
-        if (!go) break;
-        tc_fence_after();
 #pragma unroll
-        for (int c = 0; c < COLS_PER_WARP / 4; ++c) {
-          uint32_t r[S][4];
+        for (int h = 0; h < 2 && go; ++h) {
+          go = mbar_wait(&acc_full[h], t & 1, abort_p);
+          go = __all_sync(0xffffffffu, go);                 // tcgen05.ld below is warp-collective
+          if (!go) break;
+          tc_fence_after();
 #pragma unroll
-          for (int d = 0; d < S; ++d) tmem_ld4(tacc + (uint32_t)(d * BN + c * 4), r[d]);
-          tmem_wait_ld();
+          for (int c = 0; c < COLS_PER_WARP / 4; ++c) {
+            uint32_t r[HALF][4];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            auto f = [&](int d) { return __uint_as_float(r[d][j]); };
-            // diagonals 2..7 are integers; 8 and 9 are below the unit's last bits
-            long long v = (long long)__float2int_rn(fmaf(f(7), 0x1p-10f, f(6) * 0x1p-3f));
-            v += (long long)__float2int_rn(f(5)) * (1ll << 4) + (long long)__float2int_rn(f(4)) * (1ll << 11);
-            v += (long long)__float2int_rn(f(3)) * (1ll << 18) + (long long)__float2int_rn(f(2)) * (1ll << 25);
-            v += ((long long)__float2int_rn(f(1)) + (long long)__float2int_rn(f(0)) * (1ll << 7)) * (1ll << 32);
-            if (extra) v = (v + (1ll << (extra - 1))) >> extra;
-            V[c * 4 + j] = seg ? V[c * 4 + j] + v : v;
+            for (int d = 0; d < HALF; ++d) tmem_ld4(tacc + (uint32_t)((h * HALF + d) * BN + c * 4), r[d]);
+            tmem_wait_ld();
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              auto f = [&](int d) { return __uint_as_float(r[d][j]); };
+              auto n = [&](int d) { return (long long)__float2int_rn(f(d)); };
+              long long v;
+              if (h == 0) {                                 // diagonals 2..5: a multiple of 2^18
+                v = n(3) * (1ll << 18) + n(2) * (1ll << 25) + (n(1) + n(0) * (1ll << 7)) * (1ll << 32);
+                if (extra) v >>= extra;
+                V[c * 4 + j] = seg ? V[c * 4 + j] + v : v;
+              } else {                                      // 6 and 7; 8 and 9 are below the unit's last bits
+                v = (long long)__float2int_rn(fmaf(f(3), 0x1p-10f, f(2) * 0x1p-3f));
+                v += n(1) * (1ll << 4) + n(0) * (1ll << 11);
+                if (extra) v = (v + (1ll << (extra - 1))) >> extra;
+                V[c * 4 + j] += v;
+              }
+            }
           }
+          tc_fence_before();
+          mbar_arrive(&acc_empty[h]);                       // the next segment's MMAs may start
         }
-        tc_fence_before();
-        mbar_arrive(&acc_empty);                            // the next segment's MMAs may start
+        if (!go) break;
       }
       if (!go) break;
+      load_g(1);
       int qcur = n_first / gs;
       int left = min(COLS_PER_WARP, (qcur + 1) * gs - n_first);   // columns to the next norm group
       float sq = 0.f;                                       // running max |d|^2 of the group
+      // A whole tile without sources, in one norm group and far from the ends of the exponent range takes
+      // a loop without branches, whose columns overlap; two columns share a shuffle for their norms.
+      if (MODE == 0 && cols == COLS_PER_WARP && left == COLS_PER_WARP && src_here == 0 &&
+          __all_sync(0xffffffffu, row_ok && abs(es) < 400 && abs(et_l) < 400)) {
+        const bool odd = lane & 1;
+#pragma unroll
+        for (int j = 0; j < COLS_PER_WARP; j += 2) {
+          float a2[2];
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const int et = __shfl_sync(0xffffffffu, et_l, j + u);
+            const double y = fixed_to_double_normal(V[j + u], es + et - 53 + extra);
+            out[off0 + (size_t)(j + u) * N2] = y;
+            const float a = magnitude(y - gin[j / 8][(j + u) % 8]);
+            a2[u] = a * a;
+          }
+          const float other = __shfl_xor_sync(0xffffffffu, odd ? a2[0] : a2[1], 1);
+          sq = fmaxf(sq, (odd ? a2[1] : a2[0]) + other);
+        }
+        flush_norm(sq, norm + qcur, lane);
+        continue;
+      }
 #pragma unroll
       for (int j = 0; j < COLS_PER_WARP; ++j) {
-        if (j == 8) load_g(8);
         const int et = __shfl_sync(0xffffffffu, et_l, j);
         double y = fixed_to_double(V[j], es + et - 53 + extra);
         if (j >= cols) continue;                            // warp-uniform
@@ -531,7 +613,7 @@ __global__ void __launch_bounds__(THREADS, 1)
           const double2 b = lam[((size_t)site * Nc + (m >> 1)) * Nc + src_time[n_first + j]];
           y += (m & 1) ? b.y : b.x;
         }
-        const double d = y - gin[j % 8];
+        const double d = y - gin[j / 8][j % 8];
         const float a = row_ok ? magnitude(d) : 0.f;
         if (row_ok) {
           if (MODE == 0) out[off0 + (size_t)j * N2] = y;
@@ -557,31 +639,6 @@ __global__ void __launch_bounds__(THREADS, 1)
     atomicExch(err, 1);
     if (MODE != 2) atomicMax(norm, 0x7FF0000000000000ull);
   }
-}
-
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-    return static_cast<PFN_cuTensorMapEncodeTiled_v12000>(nullptr);
-  }();
-  return fn;
-}
-
-// 4D bf16 map [d3][d2][d1][d0] with a (32 x rows x 1 x 1) box and 64-byte swizzle
-bool make_map4(CUtensorMap* m, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t d3, uint32_t rows) {
-  auto fn = encode_fn();
-  if (!fn) return false;
-  cuuint64_t dims[4] = {d0, d1, d2, d3};
-  cuuint64_t strides[3] = {d0 * 2, d0 * d1 * 2, d0 * d1 * d2 * 2};
-  cuuint32_t box[4] = {(cuuint32_t)BK, rows, 1, 1};
-  cuuint32_t es[4] = {1, 1, 1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, es,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 Oz64State* state(dyson_ctx* c) {
@@ -627,7 +684,7 @@ void launch_xprep(dyson_ctx* c, int ncol, const double2* G, Oz64State* st) {
 }  // namespace
 
 bool oz64_usable(dyson_ctx* c) {
-  if (!c->oz64_enabled || !encode_fn()) return false;
+  if (!c->oz64_enabled) return false;
   Oz64State* st = static_cast<Oz64State*>(c->oz64);
   if (st && st->a_bytes >= a_slice_bytes(c)) return true;
   size_t free_b = 0, total_b = 0;
@@ -674,8 +731,6 @@ int oz64_prepare(dyson_ctx* c) {
                                                                    c->dt, c->beta, Kp, st->as, st->esig);
     DY_CUDA(c, cudaGetLastError());
     c->launches += 1;
-    if (!make_map4(&st->amap, st->as, Kp, N2, Nr, S, BM))
-      return ctx_fail(c, DYSON_ERR_CUDA, "cuTensorMapEncodeTiled failed for the FP64 Lambda slices");
     st->a_ready = true;
   }
   return DYSON_OK;
@@ -688,12 +743,6 @@ int oz64_sweep(dyson_ctx* c, int ncol, int gs, const double2* Gin, double2* out,
   const int Nr = c->Nr, Nc = c->Nc, N2 = 2 * Nc, Kp = k_pad(Nc);
   if ((rc = grow(c, &st->xs, &st->x_bytes, (size_t)S * Nr * ncol * Kp * 2, "FP64 slices of X"))) return rc;
   if ((rc = grow(c, &st->etau, &st->tau_bytes, (size_t)Nr * ncol * sizeof(int), "FP64 column scales"))) return rc;
-  if (st->xmap_ptr != st->xs || st->xmap_ncol != ncol) {
-    if (!make_map4(&st->xmap, st->xs, Kp, ncol, Nr, S, BN))
-      return ctx_fail(c, DYSON_ERR_CUDA, "cuTensorMapEncodeTiled failed for the FP64 X slices");
-    st->xmap_ptr = st->xs;
-    st->xmap_ncol = ncol;
-  }
   if (uniform_hopping(c)) launch_xprep<true>(c, ncol, Gin, st);
   else launch_xprep<false>(c, ncol, Gin, st);
   DY_CUDA(c, cudaGetLastError());
@@ -701,7 +750,7 @@ int oz64_sweep(dyson_ctx* c, int ncol, int gs, const double2* Gin, double2* out,
   const int grid = (int)std::min<long long>(tiles, st->num_sms);
   auto go = [&](auto kernel) {
     kernel<<<grid, THREADS, SMEM_BYTES, c->stream>>>(
-        st->amap, st->xmap, st->esig, st->etau, reinterpret_cast<const double*>(Gin), c->d_lam, c->d_src_site,
+        st->as, st->xs, st->esig, st->etau, reinterpret_cast<const double*>(Gin), c->d_lam, c->d_src_site,
         c->d_src_time, Nr, Nc, Kp / BK, ncol, gs, reinterpret_cast<double*>(out), r32, c->Ns, c->d_norm, st->d_err);
   };
   if (mode == 0) go(k_oz64_gemm<0>);
@@ -712,7 +761,7 @@ int oz64_sweep(dyson_ctx* c, int ncol, int gs, const double2* Gin, double2* out,
 }
 
 int oz64_batched_product(dyson_ctx* c, int batch, int nk, int Nc, const double2* A, const double2* X, double2* out) {
-  if (!c->oz64_enabled || !encode_fn()) return DYSON_ERR_OOM;
+  if (!c->oz64_enabled) return DYSON_ERR_OOM;
   int rc = prepare_common(c);
   if (rc) return rc;
   Oz64State* st = state(c);
@@ -737,18 +786,13 @@ int oz64_batched_product(dyson_ctx* c, int batch, int nk, int Nc, const double2*
   cudaError_t e = cudaSuccess;
   for (int b0 = 0; b0 < batch && rc == DYSON_OK && e == cudaSuccess; b0 += step) {
     const int nb = std::min(step, batch - b0);
-    CUtensorMap amap, xmap;
-    if (!make_map4(&amap, as, Kp, N2, nb, S, BM) || !make_map4(&xmap, xs, Kp, Nc, nb, S, BN)) {
-      rc = ctx_fail(c, DYSON_ERR_CUDA, "cuTensorMapEncodeTiled failed for a batched product");
-      break;
-    }
     const dim3 grid((Nc + 31) / 32, nb);
     const size_t o = (size_t)b0 * nk * Nc;
     k_oz64_tslice<true><<<grid, 256, 0, c->stream>>>(A + o, nk, Nc, Kp, nb, as, esig);
     k_oz64_tslice<false><<<grid, 256, 0, c->stream>>>(X + o, nk, Nc, Kp, nb, xs, etau);
     const long long tiles = (long long)((N2 + BM - 1) / BM) * ((Nc + BN - 1) / BN) * nb;
     k_oz64_gemm<2><<<(int)std::min<long long>(tiles, st->num_sms), THREADS, SMEM_BYTES, c->stream>>>(
-        amap, xmap, esig, etau, nullptr, nullptr, nullptr, nullptr, nb, Nc, Kp / BK, Nc, Nc,
+        as, xs, esig, etau, nullptr, nullptr, nullptr, nullptr, nb, Nc, Kp / BK, Nc, Nc,
         reinterpret_cast<double*>(out + (size_t)b0 * Nc * Nc), nullptr, Nc, nullptr, st->d_err);
     c->launches += 3;
     e = cudaGetLastError();

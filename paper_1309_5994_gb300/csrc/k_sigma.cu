@@ -74,7 +74,7 @@ __global__ void k_phase_trig(const double2* __restrict__ phase, int Nc, size_t t
 }
 
 // Lambda_i(z, z') = -i sum_p exp(-i (Phi_p(z) - Phi_p(z'))) * (a_p if z later than z', else -b_p)
-// 16x16, Nc = 256: 2.9 ms with exp and sincos per entry and channel (FP64 pipe), 0.2 ms from the table.
+// 16x16, Nc = 256: 2.9 ms with exp and sincos per entry and channel (FP64 pipe), 0.86 ms from the table.
 __global__ void k_lambda(const double2* __restrict__ phase, const double2* __restrict__ trig, int Nt, int Nm,
                          double2* __restrict__ lam) {
   int Nc = 2 * Nt + Nm;

@@ -1,8 +1,8 @@
 """The FP64 sweep and residual from BF16 slice products (k_oz64) against the oracle's dense solve.
 
 Contour lengths at the edges of its tiles: shorter than one k-block, no multiple of 16, one point past a
-row tile (2 Nc = 130), past one exact K segment (2 Nc = 514, 600), and column counts that leave a
-remainder; hopping equal on every bond (J folded into the Lambda slices) and per bond."""
+row tile (2 Nc = 130), norm groups that end inside a warp's 16 columns (Nc = 40, 33), past one exact K
+segment (2 Nc = 514, 600), and column counts that leave a remainder; hopping equal on every bond (J folded into the Lambda slices) and per bond."""
 import numpy as np
 import pytest
 
@@ -21,8 +21,8 @@ def torch_cuda():
 
 
 @pytest.mark.parametrize("uniform", [True, False])
-@pytest.mark.parametrize("Lx,Ly,Nt,Nm", [(1, 1, 2, 3), (2, 1, 1, 1), (3, 2, 8, 3), (2, 2, 15, 3), (2, 2, 24, 16),
-                                         (3, 1, 25, 15), (2, 1, 96, 65), (2, 1, 120, 60)])
+@pytest.mark.parametrize("Lx,Ly,Nt,Nm", [(1, 1, 2, 3), (2, 1, 1, 1), (3, 2, 8, 3), (4, 1, 16, 8),
+                                         (2, 2, 15, 3), (2, 2, 24, 16), (3, 1, 25, 15), (2, 1, 96, 65), (2, 1, 120, 60)])
 def test_fp64_sweep_and_residual_match_dense(torch_cuda, lib, Lx, Ly, Nt, Nm, uniform):
     """1e-12 of the largest entry, the FP64 path's tolerance (the slices keep 56 bits below each row's and
     column's largest value, so the sums are as exact as FP64 ones)."""
