@@ -133,52 +133,73 @@ __device__ __forceinline__ float slab_norm2(const Slab<VEC, T>& x) {
   return q;
 }
 
+// Sum of eight FP64 values over a warp: halving exchanges (nine additions; the FP64 pipe takes 16 cycles
+// for each); lanes 4 i .. 4 i + 3 return value i.
+__device__ __forceinline__ double reduce8(double (&v)[8], int lane) {
+#pragma unroll
+  for (int o = 16, half = 4; o >= 4; o >>= 1, half >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < half; ++i) {
+      const double send = up ? v[i] : v[i + half], keep = up ? v[i + half] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
 // h[n][i] += <Q_i[n], a[n] - b[n]>  (b may be null) over a range of items; nrm0 (given): += |a - b|^2.
 // With a gate (after, before), columns that need no second pass are skipped.  Grid (ncol, ranges).
-// w = a - b of an item stays in registers while GROUP basis vectors pass by it; FP32 products are
-// summed in FP32 within an item and in FP64 across items (GB300's FP64 pipe is too slow for a product
-// per element).  As one block per (basis vector, column, range), which read a and b again for
-// every basis vector in 4-byte loads, the projections ran at 1.4 TB/s.
+// w = a - b of an item stays in registers while the whole basis passes by it; FP32 products are summed in
+// FP32 within a lane's part of an item and in FP64 across lanes and items (GB300's FP64 pipe is too slow
+// for a product per element); a warp adds up its items in shared memory.  12x12, Nc = 384, 384 columns
+// (170 MB a vector), 20 basis vectors on average: 0.78 ms with groups of four basis vectors per pass over
+// the items, which read a and b again for every group (not from L2: 60 MB of them are in use at a time),
+// 0.44 ms with the whole basis (both Gram-Schmidt passes averaged; 6.9 TB/s).
 constexpr int GM_GROUP = 4;
+constexpr int GM_MAX_VEC = 64;                          // basis vectors (the restart length is at most 60)
 template <int VEC, int T>
-__global__ void __launch_bounds__(GM_THREADS) k_gm_dots(const float* __restrict__ Q, size_t vsz, int nvec,
-                                                        const float* __restrict__ a, const float* __restrict__ b,
-                                                        int items, int nz, int Ns, int ncol, int items_per_blk,
-                                                        double2* __restrict__ h, int hstride,
-                                                        double* __restrict__ nrm0, const double* __restrict__ after,
-                                                        const double* __restrict__ before) {
-  __shared__ double sh[GM_THREADS / 32][2 * GM_GROUP + 1];
+__global__ void __launch_bounds__(GM_THREADS, 2) k_gm_dots(const float* __restrict__ Q, size_t vsz, int nvec,
+                                                           const float* __restrict__ a, const float* __restrict__ b,
+                                                           int items, int nz, int Ns, int ncol, int items_per_blk,
+                                                           double2* __restrict__ h, int hstride,
+                                                           double* __restrict__ nrm0, const double* __restrict__ after,
+                                                           const double* __restrict__ before) {
+  __shared__ double sh[GM_THREADS / 32][2 * GM_MAX_VEC];
+  __shared__ double sh_sq[GM_THREADS / 32];
   const int n = blockIdx.x;
   if (after && !reorth_needed(after, before, n)) return;
   const int i0 = blockIdx.y * items_per_blk, i1 = min(items, i0 + items_per_blk);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int g0 = 0; g0 < nvec; g0 += GM_GROUP) {
-    const bool self = nrm0 && g0 == 0;
-    double re[GM_GROUP] = {}, im[GM_GROUP] = {}, sq = 0.0;
-    for (int item = i0 + warp; item < i1; item += GM_THREADS / 32) {
-      const ItemPos at = item_pos<VEC, T>(item, nz, n, ncol, Ns, lane);
-      Slab<VEC, T> w;
-      load_slab(w, a, at, Ns);
-      if (b) {
-        Slab<VEC, T> x;
-        load_slab(x, b, at, Ns);
+  double* mine = sh[warp];
+  for (int e = lane; e < 2 * GM_MAX_VEC; e += 32) mine[e] = 0.0;
+  __syncwarp();
+  double sq = 0.0;
+  for (int item = i0 + warp; item < i1; item += GM_THREADS / 32) {
+    const ItemPos at = item_pos<VEC, T>(item, nz, n, ncol, Ns, lane);
+    Slab<VEC, T> w, q[2];
+    // the next basis vector's loads are in flight while one is multiplied (a vector past the last
+    // reads the last one again; its sums are dropped)
+    auto fetch = [&](int k, Slab<VEC, T>& y) { load_slab(y, Q + (size_t)min(k, nvec - 1) * vsz, at, Ns); };
+    fetch(0, q[0]);
+    load_slab(w, a, at, Ns);
+    if (b) {
+      load_slab(q[1], b, at, Ns);
 #pragma unroll
-        for (int t = 0; t < T; ++t)
+      for (int t = 0; t < T; ++t)
 #pragma unroll
-          for (int v = 0; v < VEC; ++v) {
-            w.re[t][v] -= x.re[t][v];
-            w.im[t][v] -= x.im[t][v];
-          }
-      }
-      if (self) sq += (double)slab_norm2(w);
-      // the next basis vector's loads are in flight while one is multiplied (a vector past the last
-      // reads the last one again; its sums are dropped)
-      Slab<VEC, T> q[2];
-      auto fetch = [&](int k) { load_slab(q[k & 1], Q + (size_t)min(g0 + k, nvec - 1) * vsz, at, Ns); };
-      fetch(0);
+        for (int v = 0; v < VEC; ++v) {
+          w.re[t][v] -= q[1].re[t][v];
+          w.im[t][v] -= q[1].im[t][v];
+        }
+    }
+    if (nrm0) sq += (double)slab_norm2(w);
+    for (int g0 = 0; g0 < nvec; g0 += GM_GROUP) {
+      double v8[2 * GM_GROUP];
 #pragma unroll
       for (int k = 0; k < GM_GROUP; ++k) {
-        if (k + 1 < GM_GROUP) fetch(k + 1);
+        fetch(g0 + k + 1, q[(k + 1) & 1]);
         const Slab<VEC, T>& y = q[k & 1];
         float sr = 0.f, si = 0.f;
 #pragma unroll
@@ -188,40 +209,23 @@ __global__ void __launch_bounds__(GM_THREADS) k_gm_dots(const float* __restrict_
             sr = fmaf(y.re[t][v], w.re[t][v], fmaf(y.im[t][v], w.im[t][v], sr));
             si = fmaf(y.re[t][v], w.im[t][v], fmaf(-y.im[t][v], w.re[t][v], si));
           }
-        re[k] += (double)sr;
-        im[k] += (double)si;
+        v8[2 * k] = (double)sr;
+        v8[2 * k + 1] = (double)si;
       }
+      const double sum = reduce8(v8, lane);
+      if ((lane & 3) == 0) mine[2 * g0 + (lane >> 2)] += sum;
     }
-#pragma unroll
-    for (int k = 0; k < GM_GROUP; ++k) {
-      for (int o = 16; o > 0; o >>= 1) {
-        re[k] += __shfl_xor_sync(0xffffffffu, re[k], o);
-        im[k] += __shfl_xor_sync(0xffffffffu, im[k], o);
-      }
-    }
-    if (self)
-      for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-    if (lane == 0) {
-#pragma unroll
-      for (int k = 0; k < GM_GROUP; ++k) {
-        sh[warp][2 * k] = re[k];
-        sh[warp][2 * k + 1] = im[k];
-      }
-      sh[warp][2 * GM_GROUP] = sq;
-    }
-    __syncthreads();
-    const int e = threadIdx.x;
-    if (e < 2 * GM_GROUP + 1) {
-      double v = 0.0;
-      for (int q = 0; q < GM_THREADS / 32; ++q) v += sh[q][e];
-      if (e == 2 * GM_GROUP) {
-        if (self) atomicAdd(&nrm0[n], v);
-      } else if (g0 + e / 2 < nvec) {
-        double2* hp = &h[(size_t)n * hstride + g0 + e / 2];
-        atomicAdd(e & 1 ? &hp->y : &hp->x, v);
-      }
-    }
-    __syncthreads();
+  }
+  if (nrm0) {
+    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    if (lane == 0) sh_sq[warp] = sq;
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < 2 * nvec + (nrm0 ? 1 : 0); e += blockDim.x) {
+    double v = 0.0;
+    for (int q = 0; q < GM_THREADS / 32; ++q) v += e < 2 * nvec ? sh[q][e] : sh_sq[q];
+    double2* hp = &h[(size_t)n * hstride + e / 2];
+    atomicAdd(e == 2 * nvec ? &nrm0[n] : (e & 1 ? &hp->y : &hp->x), v);
   }
 }
 
@@ -508,7 +512,7 @@ int gmres_run(dyson_ctx* c, int ncol, const float* r, float* x, int max_iters, d
   // ranges of items per column: enough blocks for every SM, and at least two items per warp
   const int nz = (Ns + 32 * VEC * T - 1) / (32 * VEC * T), items = c->Nr * nz;
   const int want = std::max(1, std::min((items + 15) / 16, (152 * 16 + ncol - 1) / ncol));
-  const int per = (items + want - 1) / want;
+  const int per = ((items + want - 1) / want + 7) / 8 * 8;   // (a block's eight warps take equally many)
   const dim3 grid(ncol, (items + per - 1) / per);
   const int cb = (ncol + 127) / 128;
   const int lin_grid = (int)std::min<size_t>((vsz + 255) / 256, 152 * 16);
