@@ -135,6 +135,9 @@ __device__ __forceinline__ void set_scale(TcScale* s, float dmax, float jbound) 
   s->ymax = 0u;
 }
 
+// FP64 series sweeps enqueued ahead of the update that the host waits for
+constexpr int kF64Ahead = 4;
+
 struct dyson_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
@@ -227,6 +230,9 @@ struct dyson_ctx {
   bool oz_enabled = true;            // split-product residual allowed where 2 Nc <= 512
   bool use_oz = false;               // chosen for the current solve
   void* oz64 = nullptr;              // split-product FP64 sweep state (slices, scales, maps)
+  double* h_f64_upd = nullptr;       // pinned: update of each enqueued FP64 sweep (ring)
+  int* d_f64_run = nullptr;          // 1 while the FP64 series goes on
+  cudaEvent_t f64_ev[kF64Ahead] = {};
   bool oz64_enabled = true;          // split-product FP64 sweeps allowed (memory permitting)
   bool use_oz64 = false;             // chosen for the current solve: FP64 sweeps and residuals on the tensor cores
 

@@ -194,7 +194,8 @@ template <bool UNIFORM, int PER_LANE>
 __global__ void __launch_bounds__(256) k_oz64_xprep(const double2* __restrict__ G, const double* __restrict__ Jtab,
                                                     const int* __restrict__ nbr, const int* __restrict__ nbond, int Nr,
                                                     int Nt, int Nc, int ncol, int Kp, __nv_bfloat16* __restrict__ xs,
-                                                    int* __restrict__ etau) {
+                                                    int* __restrict__ etau, const int* __restrict__ run) {
+  if (run && !*run) return;                                // the series has stopped
   const size_t wi = (size_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
   const int lane = threadIdx.x & 31;
   if (wi >= (size_t)Nr * ncol) return;
@@ -388,8 +389,9 @@ __global__ void __launch_bounds__(THREADS, 1)
                 const int* __restrict__ esig, const int* __restrict__ etau, const double* __restrict__ Gin,
                 const double2* __restrict__ lam, const int* __restrict__ src_site, const int* __restrict__ src_time,
                 int Nr, int Nc, int KB, int ncol, int gs, double* __restrict__ out, float* __restrict__ r32, int Ns,
-                unsigned long long* __restrict__ norm, int* __restrict__ err) {
+                unsigned long long* __restrict__ norm, int* __restrict__ err, const int* __restrict__ run) {
   using namespace ptx;
+  if (run && !*run) return;                                // the series has stopped
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], acc_full[2], acc_empty[2], drain;
@@ -666,13 +668,13 @@ size_t a_slice_bytes(const dyson_ctx* c) { return (size_t)S * c->Nr * 2 * c->Nc 
 const double* uniform_hopping(const dyson_ctx* c) { return c->j_uniform && c->Nb > 0 ? c->dJ : nullptr; }
 
 template <bool UNIFORM>
-void launch_xprep(dyson_ctx* c, int ncol, const double2* G, Oz64State* st) {
+void launch_xprep(dyson_ctx* c, int ncol, const double2* G, Oz64State* st, const int* run) {
   const size_t warps = (size_t)c->Nr * ncol;
   const unsigned blocks = (unsigned)((warps + 7) / 8);
   const int Kp = k_pad(c->Nc), pts = Kp / 2;               // padded points per column
   auto go = [&](auto kernel) {
     kernel<<<blocks, 256, 0, c->stream>>>(G, c->dJ, c->d_nbr, c->d_nbond, c->Nr, c->Nt, c->Nc, ncol, Kp, st->xs,
-                                          st->etau);
+                                          st->etau, run);
   };
   if (pts <= 32) go(k_oz64_xprep<UNIFORM, 1>);
   else if (pts <= 64) go(k_oz64_xprep<UNIFORM, 2>);
@@ -736,22 +738,24 @@ int oz64_prepare(dyson_ctx* c) {
   return DYSON_OK;
 }
 
-int oz64_sweep(dyson_ctx* c, int ncol, int gs, const double2* Gin, double2* out, float* r32, int mode) {
+int oz64_sweep(dyson_ctx* c, int ncol, int gs, const double2* Gin, double2* out, float* r32, int mode,
+               const int* run) {
   int rc = oz64_prepare(c);
   if (rc) return rc;
   Oz64State* st = state(c);
   const int Nr = c->Nr, Nc = c->Nc, N2 = 2 * Nc, Kp = k_pad(Nc);
   if ((rc = grow(c, &st->xs, &st->x_bytes, (size_t)S * Nr * ncol * Kp * 2, "FP64 slices of X"))) return rc;
   if ((rc = grow(c, &st->etau, &st->tau_bytes, (size_t)Nr * ncol * sizeof(int), "FP64 column scales"))) return rc;
-  if (uniform_hopping(c)) launch_xprep<true>(c, ncol, Gin, st);
-  else launch_xprep<false>(c, ncol, Gin, st);
+  if (uniform_hopping(c)) launch_xprep<true>(c, ncol, Gin, st, run);
+  else launch_xprep<false>(c, ncol, Gin, st, run);
   DY_CUDA(c, cudaGetLastError());
   const long long tiles = (long long)((N2 + BM - 1) / BM) * ((ncol + BN - 1) / BN) * Nr;
   const int grid = (int)std::min<long long>(tiles, st->num_sms);
   auto go = [&](auto kernel) {
     kernel<<<grid, THREADS, SMEM_BYTES, c->stream>>>(
         st->as, st->xs, st->esig, st->etau, reinterpret_cast<const double*>(Gin), c->d_lam, c->d_src_site,
-        c->d_src_time, Nr, Nc, Kp / BK, ncol, gs, reinterpret_cast<double*>(out), r32, c->Ns, c->d_norm, st->d_err);
+        c->d_src_time, Nr, Nc, Kp / BK, ncol, gs, reinterpret_cast<double*>(out), r32, c->Ns, c->d_norm, st->d_err,
+        run);
   };
   if (mode == 0) go(k_oz64_gemm<0>);
   else go(k_oz64_gemm<1>);
@@ -793,7 +797,7 @@ int oz64_batched_product(dyson_ctx* c, int batch, int nk, int Nc, const double2*
     const long long tiles = (long long)((N2 + BM - 1) / BM) * ((Nc + BN - 1) / BN) * nb;
     k_oz64_gemm<2><<<(int)std::min<long long>(tiles, st->num_sms), THREADS, SMEM_BYTES, c->stream>>>(
         as, xs, esig, etau, nullptr, nullptr, nullptr, nullptr, nb, Nc, Kp / BK, Nc, Nc,
-        reinterpret_cast<double*>(out + (size_t)b0 * Nc * Nc), nullptr, Nc, nullptr, st->d_err);
+        reinterpret_cast<double*>(out + (size_t)b0 * Nc * Nc), nullptr, Nc, nullptr, st->d_err, nullptr);
     c->launches += 3;
     e = cudaGetLastError();
   }

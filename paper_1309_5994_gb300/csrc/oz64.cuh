@@ -14,7 +14,8 @@ int oz64_prepare(dyson_ctx* c);
 // mode 0: out = B + K Gin, c->d_norm[q] = max |out - Gin| (complex modulus);
 // mode 1: r32 = B + K Gin - Gin (FP32 planar of stride c->Ns; only the Nc points are written), c->d_norm[q] = max |r|.
 // Groups of gs columns as launch_sweep_f64; two kernel launches, counted on the context.
-int oz64_sweep(dyson_ctx* c, int ncol, int gs, const double2* Gin, double2* out, float* r32, int mode);
+int oz64_sweep(dyson_ctx* c, int ncol, int gs, const double2* Gin, double2* out, float* r32, int mode,
+               const int* run = nullptr);
 // DYSON_ERR_TIMEOUT if a bounded pipeline wait of an earlier sweep expired (clears the flag);
 // synchronises.  Such a sweep also leaves norm word 0 infinite: to be asked where a norm is.
 int oz64_check_error(dyson_ctx* c);
