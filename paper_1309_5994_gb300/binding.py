@@ -377,7 +377,7 @@ class Solver:
         self._check(self.lib.dyson_set_wait_limit(self.h, float(seconds)))
 
     def set_graph_sweeps(self, sweeps: int):
-        """Sweeps per captured graph of the inner series (0: one synchronisation per sweep)."""
+        """Sweeps of the inner series per host synchronisation (0: one synchronisation per sweep)."""
         self._check(self.lib.dyson_set_graph_sweeps(self.h, int(sweeps)))
 
     def set_sweep_variant(self, variant: int):

@@ -11,6 +11,7 @@
 #include "gmres.cuh"
 #include "oz.cuh"
 #include "oz64.cuh"
+#include "ptx.cuh"
 #include "symmetry.cuh"
 #include "tc.cuh"
 
@@ -130,7 +131,9 @@ double sweep_flops(const dyson_ctx* c, int ncol) { return 8.0 * c->Nc * (double)
 // the host loop's rule; norm words cleared for the next sweep.  One warp.
 __global__ void k_f64_check(unsigned long long* __restrict__ norm, const unsigned long long* __restrict__ scale, int ng,
                             double tol, double* __restrict__ upd, int* __restrict__ run) {
-  if (!*run) return;
+  ptx::grid_launch_next();
+  ptx::grid_wait();
+  if (!*(volatile int*)run) return;
   double m = 0.0;
   int bad = 0;
   for (int q = threadIdx.x; q < ng; q += 32) {
@@ -160,10 +163,10 @@ int prepare_f64_series(dyson_ctx* c) {
 // Plain FP64 series over the chunk (ncol vector columns, norm groups of gs columns):
 // G <- B + K G until the relative update <= tol.
 // Up to kF64Ahead sweeps are enqueued before the first one's update has reached the host; those behind
-// the last one find the series stopped and return at once (its result is in the other buffer).  With a
-// synchronisation after each sweep the GPU stood idle for 20 us a sweep: 4x4, Nc = 64, 29 sweeps of 49 us,
-// 1.75 ms in place of 2.07.  A profiled series and the FP64-pipe sweep, which does not read the flag, wait
-// for each sweep.
+// the last one find the series stopped and return at once (its result is in the other buffer).  Their
+// launches overlap (launch_overlapped).  4x4, Nc = 64, 29 sweeps of 49 us: 2.07 ms with a synchronisation after
+// each sweep (20 us of idle GPU), 1.79 enqueued ahead, 1.60 overlapped; 3x3, Nc = 26: 1.33, 1.04, 0.85.
+// A profiled series and the FP64-pipe sweep, which does not read the flag, wait for each sweep.
 int solve_f64(dyson_ctx* c, int ncol, int gs, double tol, int max_sweeps, double2** result, dyson_report* r) {
   const int ng = ncol / gs;
   const size_t n_el = (size_t)c->Nr * ncol * c->Nc;
@@ -190,10 +193,9 @@ int solve_f64(dyson_ctx* c, int ncol, int gs, double tol, int max_sweeps, double
         c->launches += 1;
       }
     }
-    k_f64_check<<<1, 32, 0, c->stream>>>(c->d_norm, c->d_norm + ng, ng, tol, c->h_f64_upd + enqueued % kF64Ahead,
-                                         c->d_f64_run);
+    DY_CUDA(c, launch_overlapped(true, k_f64_check, 1, 32, 0, c->stream, c->d_norm, c->d_norm + ng, ng, tol,
+                                 c->h_f64_upd + enqueued % kF64Ahead, c->d_f64_run));
     c->launches += 1;
-    DY_CUDA(c, cudaGetLastError());
     DY_CUDA(c, cudaEventRecord(c->f64_ev[enqueued % kF64Ahead], c->stream));
     std::swap(Ga, Gb);
     ++enqueued;
@@ -225,7 +227,7 @@ int solve_f64(dyson_ctx* c, int ncol, int gs, double tol, int max_sweeps, double
 }
 
 // Stopping state of the inner series, the same fields the host loop of inner_solve keeps;
-// on the device for sweeps replayed from a captured graph.
+// on the device for sweeps enqueued in batches.
 struct SeriesState {
   double best, peak, last;
   double hist[kStallSweeps];           // the last kStallSweeps updates (ring)
@@ -235,13 +237,15 @@ struct SeriesState {
 };
 enum { SERIES_RUNNING = 0, SERIES_STOPPED, SERIES_EXHAUSTED, SERIES_ABORTED, SERIES_NOT_FINITE };
 
-// After one sweep of a captured series: the update max_q norm_q / rref_q (norm words
+// After one sweep of a batch: the update max_q norm_q / rref_q (norm words
 // cleared for the next sweep), the next sweep's FP16 scales, and the stopping rule of
 // inner_solve's host loop, in the same order.  One warp; returns at once once the series has stopped.
 __global__ void k_series_check(unsigned long long* __restrict__ norm, const double* __restrict__ rref, int ng,
                                int max_sweeps, double target, double abort_peak, SeriesState* __restrict__ S,
                                TcScale* __restrict__ xscale, float jbound) {
-  if (!S->run) return;
+  ptx::grid_launch_next();
+  ptx::grid_wait();
+  if (!*(volatile int*)&S->run) return;
   for (int q = threadIdx.x; q < ng; q += 32) set_scale(xscale + q, __uint_as_float(xscale[q].ymax), jbound);
   double m = 0.0;
   int bad = 0;
@@ -324,10 +328,12 @@ int tc_timed_sweep(dyson_ctx* c, int ncol, int gs, const float* r, const float* 
 // act (optional): support truncation of the tensor-core sweeps (tc_sweep), valid
 // while every column of r32 is zero off its source site
 // r_on_sources: r32 is non-zero only on each column's source site (the first right-hand side)
-// With the fused sweep the series runs from replays of a captured graph of
-// c->graph_sweeps sweeps, each followed by k_series_check: one host synchronisation per
-// replay instead of one per sweep.  The replayed sweeps take their sweep number (for the
-// support table) from the device count of sweeps done.
+// With the fused sweep, c->graph_sweeps sweeps at a time are enqueued, each followed by k_series_check: one
+// host synchronisation per batch instead of one per sweep.  These sweeps take their sweep number (for the
+// support table) from the device count of sweeps done.  The launches overlap (launch_overlapped): a
+// sweep's CTAs set up under the check before it.  As replays of a captured graph, whose capture and
+// instantiation every inner solve paid for: 8x8, Nc = 128, 6.58 ms a solve, 9x7, Nc = 100, 4.46; so 6.52 and
+// 4.33 (enqueued without the overlap 6.88 and 4.56).
 int inner_solve(dyson_ctx* c, int ncol, int gs, int precision, float* r32, float* da, float* db, int max_sweeps,
                 const std::vector<double>& rref, float** dres, dyson_report* rep, double* peak_out,
                 double abort_peak = std::numeric_limits<double>::infinity(), const int* act = nullptr,
@@ -340,10 +346,10 @@ int inner_solve(dyson_ctx* c, int ncol, int gs, int precision, float* r32, float
   const int rform = r_on_sources ? TC_R_ON_SOURCES : TC_R_DENSE;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   // (not inside a caller's own capture of the stream)
-  const bool graph = c->graph_sweeps > 0 && precision == DYSON_PREC_TF32X3_F64REF && c->use_tc &&
+  const bool batches = c->graph_sweeps > 0 && precision == DYSON_PREC_TF32X3_F64REF && c->use_tc &&
                      tc_uses_fused(c) && cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess &&
                      cap == cudaStreamCaptureStatusNone;
-  const int eager_until = graph ? 0 : max_sweeps;
+  const int eager_until = batches ? 0 : max_sweeps;
   SeriesState S = {};
   S.best = std::numeric_limits<double>::infinity();
   S.run = 1;
@@ -411,9 +417,8 @@ int inner_solve(dyson_ctx* c, int ncol, int gs, int precision, float* r32, float
       S.outcome = SERIES_EXHAUSTED;
     }
   }
-  if (S.run && graph) {
-    // the rest of the series from a captured graph of S_g sweeps (even, so that every
-    // replay starts from da), each followed by its check
+  if (S.run && batches) {
+    // batches of S_g sweeps (even, so that every batch starts from da), each followed by its check
     const int Sg = c->graph_sweeps;
     if (!c->d_series) {
       DY_CUDA(c, cudaMalloc(&c->d_series, sizeof(SeriesState)));
@@ -422,40 +427,28 @@ int inner_solve(dyson_ctx* c, int ncol, int gs, int precision, float* r32, float
     SeriesState* hS = static_cast<SeriesState*>(c->h_series);
     SeriesState* dS = static_cast<SeriesState*>(c->d_series);
     *hS = S;
-    if ((rc = tc_prepare_sweep(c, ncol))) return rc;     // nothing to allocate or encode while capturing
+    if ((rc = tc_prepare_sweep(c, ncol))) return rc;     // (buffers and tensor maps)
     if ((rc = tc_set_scale(c, ng))) return rc;
     DY_CUDA(c, cudaMemcpyAsync(dS, hS, sizeof(SeriesState), cudaMemcpyHostToDevice, c->stream));
     DY_CUDA(c, cudaMemsetAsync(c->d_norm, 0, (size_t)ng * sizeof(unsigned long long), c->stream));
-    const int64_t launches0 = c->launches;
-    cudaGraph_t g = nullptr;
-    cudaGraphExec_t ge = nullptr;
-    // captured on a private stream (any stream of the caller's, the default one included,
-    // can then launch it); the context's launches go there while capturing
-    if (!c->cap_stream) DY_CUDA(c, cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
-    cudaStream_t user = c->stream;
-    DY_CUDA(c, cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
-    c->stream = c->cap_stream;
-    c->sweep_run = &dS->run;
-    c->sweep_count = &dS->sweeps;
-    int cap_rc = DYSON_OK;
-    for (int k = 0; k < Sg && cap_rc == DYSON_OK; ++k) {
-      cap_rc = tc_sweep(c, ncol, gs, r32, k % 2 ? db : da, k % 2 ? da : db, TC_GATHER | TC_GEMM, act, 0, rform);
-      if (cap_rc == DYSON_OK)
-        k_series_check<<<1, 32, 0, c->stream>>>(c->d_norm, c->d_rref, ng, max_sweeps, target, abort_peak, dS,
-                                                   c->d_xscale, tc_jbound(c));
-    }
-    c->sweep_run = nullptr;
-    c->sweep_count = nullptr;
-    c->stream = user;
-    cudaError_t ce = cudaStreamEndCapture(c->cap_stream, &g);
-    if (cap_rc) {
-      if (g) cudaGraphDestroy(g);
-      return cap_rc;
-    }
-    if (ce == cudaSuccess) ce = cudaGraphInstantiate(&ge, g, 0);
-    if (g) cudaGraphDestroy(g);
-    if (ce != cudaSuccess) return ctx_fail(c, DYSON_ERR_CUDA, std::string("inner series graph: ") + cudaGetErrorString(ce));
-    c->launches = launches0;
+    auto enqueue = [&]() -> int {
+      const int64_t launches0 = c->launches;
+      int rc1 = DYSON_OK;
+      c->sweep_run = &dS->run;
+      c->sweep_count = &dS->sweeps;
+      for (int k = 0; k < Sg && rc1 == DYSON_OK; ++k) {
+        rc1 = tc_sweep(c, ncol, gs, r32, k % 2 ? db : da, k % 2 ? da : db, TC_GATHER | TC_GEMM, act, 0, rform);
+        if (rc1 == DYSON_OK)
+          launch_overlapped(true, k_series_check, 1, 32, 0, c->stream, c->d_norm, c->d_rref, ng, max_sweeps, target,
+                            abort_peak, dS, c->d_xscale, tc_jbound(c));
+        c->overlap = true;
+      }
+      c->overlap = false;
+      c->sweep_run = nullptr;
+      c->sweep_count = nullptr;
+      c->launches = launches0 + 2 * Sg;
+      return rc1;
+    };
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (c->profiling) {
       cudaEventCreate(&e0);
@@ -465,26 +458,26 @@ int inner_solve(dyson_ctx* c, int ncol, int gs, int precision, float* r32, float
     while (rc == DYSON_OK) {
       const int before = hS->sweeps;
       if (e0) cudaEventRecord(e0, c->stream);
-      cudaError_t le = cudaGraphLaunch(ge, c->stream);
+      if ((rc = enqueue())) break;
+      cudaError_t le = cudaGetLastError();
       if (e1) cudaEventRecord(e1, c->stream);
       if (le == cudaSuccess && c->use_tc) rc = tc_error_enqueue(c);
       if (le == cudaSuccess && rc == DYSON_OK)
         le = cudaMemcpyAsync(hS, dS, sizeof(SeriesState), cudaMemcpyDeviceToHost, c->stream);
       if (le == cudaSuccess && rc == DYSON_OK) le = cudaStreamSynchronize(c->stream);
       if (le != cudaSuccess) {
-        rc = ctx_fail(c, DYSON_ERR_CUDA, std::string("inner series graph: ") + cudaGetErrorString(le));
+        rc = ctx_fail(c, DYSON_ERR_CUDA, std::string("inner series: ") + cudaGetErrorString(le));
         break;
       }
       c->host_syncs += 1;
       if (rc || (c->use_tc && (rc = tc_error_status(c)))) break;
       const int n_run = hS->sweeps - before;
-      c->launches += 2 * Sg;
       rep->sweeps += n_run;
       rep->gemm_flops += n_run * sweep_flops(c, ncol);
       rep->update = hS->last;
       float ms = 0.f;
       if (e0 && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess) {
-        c->prof_ms[fused_kind(c)] += ms;                   // the replay, its checks included
+        c->prof_ms[fused_kind(c)] += ms;                   // the batch, its checks included
         c->prof_launches[fused_kind(c)] += n_run;
       }
       if (!hS->run) {
@@ -494,7 +487,6 @@ int inner_solve(dyson_ctx* c, int ncol, int gs, int precision, float* r32, float
     }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
-    cudaGraphExecDestroy(ge);
     if (rc) return rc;
     S = *hS;
     if (S.outcome == SERIES_NOT_FINITE) return ctx_fail(c, DYSON_ERR_DIVERGED, "FP32 series update not finite");
@@ -1302,7 +1294,6 @@ void dyson_destroy(dyson_ctx* c) {
   for (cudaEvent_t e : c->f64_ev)
     if (e) cudaEventDestroy(e);
   if (c->h_series) cudaFreeHost(c->h_series);
-  if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   delete c;
 }
 

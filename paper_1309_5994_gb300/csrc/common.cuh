@@ -135,6 +135,25 @@ __device__ __forceinline__ void set_scale(TcScale* s, float dmax, float jbound) 
   s->ymax = 0u;
 }
 
+// Launch that may be scheduled while the stream's previous kernel runs (overlap), for kernels that
+// call ptx::grid_wait before their first read of anything an earlier kernel wrote, and before their first
+// write.
+template <class... Params, class... Args>
+inline cudaError_t launch_overlapped(bool overlap, void (*kernel)(Params...), unsigned grid, unsigned threads, size_t smem,
+                                     cudaStream_t stream, Args... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = at;
+  cfg.numAttrs = overlap ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
 // FP64 series sweeps enqueued ahead of the update that the host waits for
 constexpr int kF64Ahead = 4;
 
@@ -145,13 +164,12 @@ struct dyson_ctx {
   double dt = 0, beta = 0, curvature = 0, mu = 0;
   std::vector<double> U, J;          // host copies of the drive tables
   bool j_uniform = false;            // every bond carries the same J(t) row
-  // inner series under captured graphs: sweeps per graph (0: one host synchronisation per
-  // sweep); while a graph is captured, the flag its fused sweeps read (0: the series stopped)
+  // inner series in batches: sweeps per batch (0: one host synchronisation per sweep); while a batch
+  // is enqueued, the flag its fused sweeps read (0: the series stopped) and the count of sweeps done
   int graph_sweeps = 16;
   const int* sweep_run = nullptr;
   const int* sweep_count = nullptr;  // while capturing: the device count of sweeps done
-  cudaStream_t cap_stream = nullptr; // private stream the series graph is captured on (lazy)
-  void* d_series = nullptr;          // device stopping state of the captured series
+  void* d_series = nullptr;          // device stopping state of the series
   void* h_series = nullptr;          // pinned mirror
   double* d_rref = nullptr;          // [norm_cap] reference norms of the current inner solve
 
@@ -230,6 +248,7 @@ struct dyson_ctx {
   bool oz_enabled = true;            // split-product residual allowed where 2 Nc <= 512
   bool use_oz = false;               // chosen for the current solve
   void* oz64 = nullptr;              // split-product FP64 sweep state (slices, scales, maps)
+  bool overlap = false;              // series sweeps and checks are launched overlapped
   double* h_f64_upd = nullptr;       // pinned: update of each enqueued FP64 sweep (ring)
   int* d_f64_run = nullptr;          // 1 while the FP64 series goes on
   cudaEvent_t f64_ev[kF64Ahead] = {};

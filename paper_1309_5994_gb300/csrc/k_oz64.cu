@@ -195,7 +195,9 @@ __global__ void __launch_bounds__(256) k_oz64_xprep(const double2* __restrict__ 
                                                     const int* __restrict__ nbr, const int* __restrict__ nbond, int Nr,
                                                     int Nt, int Nc, int ncol, int Kp, __nv_bfloat16* __restrict__ xs,
                                                     int* __restrict__ etau, const int* __restrict__ run) {
-  if (run && !*run) return;                                // the series has stopped
+  ptx::grid_launch_next();
+  ptx::grid_wait();
+  if (run && !*(volatile const int*)run) return;           // the series has stopped
   const size_t wi = (size_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
   const int lane = threadIdx.x & 31;
   if (wi >= (size_t)Nr * ncol) return;
@@ -391,7 +393,6 @@ __global__ void __launch_bounds__(THREADS, 1)
                 int Nr, int Nc, int KB, int ncol, int gs, double* __restrict__ out, float* __restrict__ r32, int Ns,
                 unsigned long long* __restrict__ norm, int* __restrict__ err, const int* __restrict__ run) {
   using namespace ptx;
-  if (run && !*run) return;                                // the series has stopped
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], acc_full[2], acc_empty[2], drain;
@@ -400,7 +401,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int N2 = 2 * Nc;
   const int MT = (N2 + BM - 1) / BM, NT = (ncol + BN - 1) / BN;
-  const int tiles = MT * NT * Nr;
+  int tiles = MT * NT * Nr;
   const int nseg = (KB + SEG_KB - 1) / SEG_KB;
 
   if (threadIdx.x == 0) {
@@ -421,6 +422,9 @@ __global__ void __launch_bounds__(THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_holder;
+  grid_launch_next();
+  grid_wait();
+  if (run && !*(volatile const int*)run) tiles = 0;        // the series has stopped
   volatile WaitCtl* abort_p = &wctl;
   auto stage_ptr = [&](int s) { return smem + (size_t)s * STAGE_BYTES; };
 
@@ -673,8 +677,8 @@ void launch_xprep(dyson_ctx* c, int ncol, const double2* G, Oz64State* st, const
   const unsigned blocks = (unsigned)((warps + 7) / 8);
   const int Kp = k_pad(c->Nc), pts = Kp / 2;               // padded points per column
   auto go = [&](auto kernel) {
-    kernel<<<blocks, 256, 0, c->stream>>>(G, c->dJ, c->d_nbr, c->d_nbond, c->Nr, c->Nt, c->Nc, ncol, Kp, st->xs,
-                                          st->etau, run);
+    launch_overlapped(run != nullptr, kernel, blocks, 256, 0, c->stream, G, c->dJ, c->d_nbr, c->d_nbond, c->Nr, c->Nt,
+                      c->Nc, ncol, Kp, st->xs, st->etau, run);
   };
   if (pts <= 32) go(k_oz64_xprep<UNIFORM, 1>);
   else if (pts <= 64) go(k_oz64_xprep<UNIFORM, 2>);
@@ -752,10 +756,9 @@ int oz64_sweep(dyson_ctx* c, int ncol, int gs, const double2* Gin, double2* out,
   const long long tiles = (long long)((N2 + BM - 1) / BM) * ((ncol + BN - 1) / BN) * Nr;
   const int grid = (int)std::min<long long>(tiles, st->num_sms);
   auto go = [&](auto kernel) {
-    kernel<<<grid, THREADS, SMEM_BYTES, c->stream>>>(
-        st->as, st->xs, st->esig, st->etau, reinterpret_cast<const double*>(Gin), c->d_lam, c->d_src_site,
-        c->d_src_time, Nr, Nc, Kp / BK, ncol, gs, reinterpret_cast<double*>(out), r32, c->Ns, c->d_norm, st->d_err,
-        run);
+    launch_overlapped(run != nullptr, kernel, (unsigned)grid, THREADS, SMEM_BYTES, c->stream, st->as, st->xs, st->esig,
+                      st->etau, reinterpret_cast<const double*>(Gin), c->d_lam, c->d_src_site, c->d_src_time, Nr, Nc,
+                      Kp / BK, ncol, gs, reinterpret_cast<double*>(out), r32, c->Ns, c->d_norm, st->d_err, run);
   };
   if (mode == 0) go(k_oz64_gemm<0>);
   else go(k_oz64_gemm<1>);

@@ -858,11 +858,6 @@ __global__ void __launch_bounds__(F_THREADS, 1)
                const int* __restrict__ sweeps_done) {
   using namespace ptx;
   using Cfg = FusedCfg<GT>;
-  // a sweep of a captured graph after the series has stopped: nothing to do (every CTA
-  // reads the same flag, before any barrier, cluster or TMEM step); in a captured graph
-  // the sweep number (for the support table) is the device count of sweeps done, plus one
-  if (run && *run == 0) return;
-  if (sweeps_done) sweep = *sweeps_done + 1;
   constexpr int STAGES = Cfg::STAGES, NBUF = Cfg::NBUF, STAGE = Cfg::STAGE, NB = Cfg::NB, X_TILE = Cfg::X_TILE;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -876,7 +871,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
   const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
   const int KB = (GT == 2 ? I.Ns : 2 * I.Ns) / F_BK;    // k-blocks of 64 complex points, or 64 real values
   const int row_gap = GT == 2 ? I.Ns : 0;               // rows of the two accumulators: z and Ns + z
-  const int tiles = I.Lx * I.Ly * ((I.ncol + NB - 1) / NB) * fused_row_tiles<GT>(I.Ns);
+  int tiles = I.Lx * I.Ly * ((I.ncol + NB - 1) / NB) * fused_row_tiles<GT>(I.Ns);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -901,6 +896,13 @@ __global__ void __launch_bounds__(F_THREADS, 1)
   const uint32_t tmem = tmem_holder;
   volatile WaitCtl* abort_p = &wctl;
   auto stage_ptr = [&](int s) { return smem + (size_t)s * STAGE; };
+  // Everything above runs under the end of the kernel before (launch_overlapped).  A sweep enqueued behind
+  // the end of its series has no tiles (every CTA reads the same flag); in a batch the sweep number (for the
+  // support table) is the device count of sweeps done, plus one.
+  grid_launch_next();
+  grid_wait();
+  if (run && *(volatile const int*)run == 0) tiles = 0;
+  if (sweeps_done) sweep = *(volatile const int*)sweeps_done + 1;
 
   // each warpgroup sets its register budget first, in its own branch, so that the code of
   // each role is compiled against that budget
@@ -1393,9 +1395,12 @@ int launch_fused(dyson_ctx* c, const FusedInst& e, int sweep, const int* run, co
   TcState* st = state(c);
   const int NB = FusedCfg<GT>::NB;
   const long long tiles = (long long)e.Lx * e.Ly * ((e.ncol + NB - 1) / NB) * fused_row_tiles<GT>(e.Ns);
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   cudaLaunchConfig_t cfg = pair_config(at, (unsigned)std::min<long long>(tiles, fused_clusters(c)), F_THREADS,
                                        FusedCfg<GT>::SMEM, stream);
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  if (c->overlap) cfg.numAttrs = 2;
   DY_CUDA(c, cudaLaunchKernelEx(&cfg, k_tc_fused<GT>, st->h_hi, st->h_lo, e, st->d_err, sweep, run, sweeps_done));
   DY_CUDA(c, cudaGetLastError());
   c->launches += 1;
@@ -1469,7 +1474,7 @@ int tc_sweep(dyson_ctx* c, int ncol, int gs, const float* r, const float* din, f
   if (gt > 0) {
     // one launch gathers and multiplies: the gather phase alone launches nothing
     if (!(phases & TC_GEMM)) return tc_prepare_fused(c);
-    // (in a captured series the check kernel sets the scales)
+    // (in a batch of sweeps the check kernel sets the scales)
     if (!c->sweep_run && (rc = tc_set_scale(c, (ncol + gs - 1) / gs))) return rc;
     return tc_fused_sweep(c, ncol, gs, r, din, dout, act, sweep, rform, c->sweep_run, c->sweep_count, c->stream);
   }

@@ -29,7 +29,7 @@ int contour_stride(const dyson_ctx* c);
 // sweeps after it take the bound from the maxima that the previous one left.
 int tc_seed_scale(dyson_ctx* c, int ng, const double* ref, double bound);
 int tc_seed_scale_scan(dyson_ctx* c, int ncol, int gs, const float* d);
-// turn the seeded maxima into scales (tc_sweep does this itself outside a captured series)
+// turn the seeded maxima into scales (tc_sweep does this itself outside a batch of sweeps)
 int tc_set_scale(dyson_ctx* c, int ng);
 float tc_jbound(const dyson_ctx* c);              // 4 max|J|, the factor of set_scale
 // true when a tcgen05 sweep serves this context
@@ -73,7 +73,7 @@ void tc_release(dyson_ctx* c);
 // true when the fused sweep can run on this context's device
 bool tc_fused_runs(dyson_ctx* c);
 // The fused sweep of tc_sweep on a stream of the caller's, with scales set (tc_set_scale, or by a
-// captured check kernel): run (or nullptr): device flag, 0 skips the sweep; sweeps_done (or nullptr):
+// check kernel): run (or nullptr): device flag, 0 skips the sweep; sweeps_done (or nullptr):
 // device count that gives the sweep number
 int tc_fused_sweep(dyson_ctx* c, int ncol, int gs, const float* r, const float* din, float* dout, const int* act,
                    int sweep, int rform, const int* run, const int* sweeps_done, cudaStream_t stream);
