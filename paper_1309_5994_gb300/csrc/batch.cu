@@ -23,6 +23,7 @@
 #include "common.cuh"
 #include "detail.cuh"
 #include "oz.cuh"
+#include "oz64.cuh"
 #include "tc.cuh"
 
 using namespace dyson_detail;
@@ -246,8 +247,8 @@ int dyson_batch_solve(dyson_batch* b, const int32_t* const* src, const int32_t* 
     if (n_src[k] < 1 || !src[k]) return bfail(b, DYSON_ERR_INVALID_ARG, "every instance needs a source site");
     for (int q = 0; q < n_src[k]; ++q)
       if (src[k][q] < 0 || src[k][q] >= c->Nr) return bfail(b, DYSON_ERR_INVALID_ARG, "source site out of range");
-    if ((rc = prepare_tables(c, DYSON_PREC_TF32X3_F64REF, true))) return bfail(b, rc, c->err);
-    if (!c->use_tc || !c->use_oz || !tc_fused_runs(c))
+    if ((rc = prepare_tables(c, DYSON_PREC_TF32X3_F64REF, tol, true))) return bfail(b, rc, c->err);
+    if (!c->use_tc || !oz_supported(c) || !tc_fused_runs(c))
       return bfail(b, DYSON_ERR_INVALID_ARG,
                    "instance " + std::to_string(k) + ": batched solves need Nc % 64 == 0 and 2 Nc <= 512");
     X.nq = n_src[k];
@@ -420,7 +421,7 @@ int dyson_batch_solve(dyson_batch* b, const int32_t* const* src, const int32_t* 
       launch_accumulate(X.G, d, c->Nr, c->Nc, c->Ns, X.ncol, c->stream);
       c->launches += 1;
       DYB_CUDA(b, cudaMemsetAsync(c->d_norm, 0, (size_t)X.ng * sizeof(unsigned long long), c->stream));
-      if ((rc = oz_residual(c, X.ncol, c->Nc, X.G, X.r32, tol))) return bfail(b, rc, c->err);
+      if ((rc = enqueue_residual(c, X.ncol, c->Nc, X.G, X.r32))) return bfail(b, rc, c->err);
     }
     for (int k = 0; k < n; ++k) {
       Inst& X = I[k];
@@ -434,6 +435,7 @@ int dyson_batch_solve(dyson_batch* b, const int32_t* const* src, const int32_t* 
       X.rep.residual = res;
       for (int q = 0; q < X.ng; ++q) X.rref[q] = std::max(bits_to_double(c->h_norm[q]), 1e-300);
       if (!(res < kDivergedGrowth)) {
+        if (c->use_oz64 && (rc = oz64_check_error(c))) return bfail(b, rc, c->err);
         X.status = DYSON_ERR_DIVERGED;
         X.done = true;
       } else if (res <= tol) {
@@ -455,7 +457,7 @@ int dyson_batch_solve(dyson_batch* b, const int32_t* const* src, const int32_t* 
     const int saved = c->inner_solver;
     c->inner_solver = DYSON_INNER_GMRES;
     double2* G = nullptr;
-    if ((rc = prepare_tables(c, DYSON_PREC_TF32X3_F64REF))) return bfail(b, rc, c->err);
+    if ((rc = prepare_tables(c, DYSON_PREC_TF32X3_F64REF, tol))) return bfail(b, rc, c->err);
     rc = solve_mixed(c, X.ncol, c->Nc, DYSON_PREC_TF32X3_F64REF, tol, max_sweeps, &G, &X.rep);
     c->inner_solver = saved;
     if (rc != DYSON_OK && rc != DYSON_ERR_NOT_CONVERGED && rc != DYSON_ERR_DIVERGED) return bfail(b, rc, c->err);

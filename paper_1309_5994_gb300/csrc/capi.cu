@@ -634,20 +634,7 @@ int solve_mixed(dyson_ctx* c, int ncol, int gs, int precision, double tol, int m
     launch_accumulate(G, d, c->Nr, c->Nc, c->Ns, ncol, c->stream);
     c->launches += 1;
     DY_CUDA(c, cudaMemsetAsync(c->d_norm, 0, (size_t)ng * sizeof(unsigned long long), c->stream));
-    if (c->use_oz) {
-      KernelTimer t(c, DYSON_KERNEL_RESIDUAL_SPLIT);
-      if ((rc = oz_residual(c, ncol, gs, G, r32, tol))) return rc;
-    } else {
-      KernelTimer t(c, DYSON_KERNEL_RESIDUAL_F64);
-      if (c->use_oz64) {
-        if ((rc = oz64_sweep(c, ncol, gs, G, nullptr, r32, 1))) return rc;
-      } else {
-        launch_sweep_f64(c->d_lam, c->d_JW, c->d_nbr, c->d_nbond, G, nullptr, r32, c->Ns, c->d_src_site, c->d_src_time,
-                         c->Nr, c->Nc, ncol, gs, 1, c->d_norm, c->stream);
-        c->launches += 1;
-      }
-    }
-    DY_CUDA(c, cudaGetLastError());
+    if ((rc = enqueue_residual(c, ncol, gs, G, r32))) return rc;
     if (c->use_oz && (rc = oz_error_enqueue(c))) return rc;   // read with the norms: one synchronisation
     if ((rc = read_norms(c, ng, false))) return rc;
     if (c->use_oz && (rc = oz_error_status(c))) return rc;
@@ -817,8 +804,6 @@ int dyson_copy_sigma(dyson_ctx* c, double* dst, int on_device) {
 
 namespace dyson_detail {
 
-// Build the reduced-precision copies of Lambda a solve needs and pick the sweep
-// and residual kernels (sets c->use_tc, c->use_oz).
 // FP64 sweeps and residuals on the tensor cores where the slices of Lambda fit (sets c->use_oz64);
 // the FP64-pipe kernel otherwise
 int prepare_oz64(dyson_ctx* c) {
@@ -829,7 +814,11 @@ int prepare_oz64(dyson_ctx* c) {
   return rc == DYSON_ERR_OOM ? DYSON_OK : rc;
 }
 
-int prepare_tables(dyson_ctx* c, int precision, bool batch) {
+// Build the reduced-precision copies of Lambda a solve needs and pick the sweep
+// and residual kernels (sets c->use_tc, c->use_oz, c->use_oz64).
+// The residual of a mixed solve: five slices (15 products) for tolerances down to 1e-8, where they run at
+// 85 TFLOP/s of the contraction (16x16, Nc = 256, 4096 columns: 6.5 ms); eight (36 products, 53 TFLOP/s) below.
+int prepare_tables(dyson_ctx* c, int precision, double tol, bool batch) {
   c->use_tc = c->use_oz = c->use_oz64 = false;
   c->Ns = c->Nc;
   if (precision == DYSON_PREC_F64) return prepare_oz64(c);
@@ -861,8 +850,26 @@ int prepare_tables(dyson_ctx* c, int precision, bool batch) {
     c->lam_split_built = true;
   }
   c->use_tc = tc;
-  c->use_oz = tc && c->oz_enabled && oz_supported(c);
+  c->use_oz = tc && tol >= kOzTol && c->oz_enabled && oz_supported(c);
   return c->use_oz ? DYSON_OK : prepare_oz64(c);
+}
+
+// r32 = B + K G - G with the residual kernel that prepare_tables picked; c->d_norm[q] = max |r|
+int enqueue_residual(dyson_ctx* c, int ncol, int gs, const double2* G, float* r32) {
+  int rc = DYSON_OK;
+  KernelTimer t(c, c->use_oz || c->use_oz64 ? DYSON_KERNEL_RESIDUAL_SPLIT : DYSON_KERNEL_RESIDUAL_F64);
+  if (c->use_oz) {
+    rc = oz_residual(c, ncol, gs, G, r32);
+  } else if (c->use_oz64) {
+    rc = oz64_sweep(c, ncol, gs, G, nullptr, r32, 1);
+  } else {
+    launch_sweep_f64(c->d_lam, c->d_JW, c->d_nbr, c->d_nbond, G, nullptr, r32, c->Ns, c->d_src_site, c->d_src_time,
+                     c->Nr, c->Nc, ncol, gs, 1, c->d_norm, c->stream);
+    c->launches += 1;
+  }
+  if (rc) return rc;
+  DY_CUDA(c, cudaGetLastError());
+  return DYSON_OK;
 }
 
 // Largest number of vector columns, a multiple of `unit` and at most `want`, whose
@@ -947,7 +954,7 @@ int solve_columns_impl(dyson_ctx* c, const int32_t* src, int64_t n_src, int prec
   for (int64_t q = 0; q < n_src; ++q)
     if (src[q] < 0 || src[q] >= c->Nr) return R.finish(ctx_fail(c, DYSON_ERR_INVALID_ARG, "source site out of range"));
   DeviceGuard g(c->device);
-  if ((rc = prepare_tables(c, precision))) return R.finish(rc);
+  if ((rc = prepare_tables(c, precision, tol))) return R.finish(rc);
   size_t col_bytes = 0;
   const int64_t cols = chunk_columns(c, precision, c->Nc, n_src * (int64_t)c->Nc, &col_bytes);
   if (cols < c->Nc) return R.finish(ctx_fail(c, DYSON_ERR_OOM, "one block column does not fit in device memory"));
@@ -1022,7 +1029,7 @@ int dyson_solve_vector_columns(dyson_ctx* c, const int32_t* sites, const int32_t
     if (sites[q] < 0 || sites[q] >= c->Nr || times[q] < 0 || times[q] >= c->Nc)
       return R.finish(ctx_fail(c, DYSON_ERR_INVALID_ARG, "column source out of range"));
   DeviceGuard g(c->device);
-  if ((rc = prepare_tables(c, precision))) return R.finish(rc);
+  if ((rc = prepare_tables(c, precision, tol))) return R.finish(rc);
   constexpr int GS = 32;                                   // norm group; columns padded to a multiple
   const int64_t padded = (n + GS - 1) / GS * GS;
   size_t col_bytes = 0;

@@ -5,19 +5,17 @@
 // The real GEMM A X (A = [[Re,-Im],[Im,Re]] of Lambda W, per site 2Nc x 2Nc) is
 // evaluated exactly enough in FP32 tensor-core arithmetic by splitting both
 // operands into integer slices (the Ozaki scheme): every row of A and every
-// column of X is scaled by a power of two into [-1, 1] and cut into S = 7 slices
-// of 7 bits, v = sum_s q_s 2^{-7 s} with integers |q_s| <= 128.  A slice product
-// sum_k A_s X_t is then an integer multiple of 2^{-7(s+t)} below 2^24 in
-// magnitude for every diagonal s + t <= 5 when K = 2Nc <= 512, so BF16 inputs
-// with FP32 accumulation are exact there.
-// The 28 products with s + t <= 8 (truncation ~2^-50 of |A||X|) accumulate per
-// diagonal in five TMEM accumulators, {2}, {3}, {4}, {5} exact and {6, 7, 8}
-// rounded at 2^-24 of its own size (about 2^-48 of the result).  The epilogue
-// adds them in FP64, rescales, and forms r = B + A X - G in FP64.  Solves whose
-// tolerance is 1e-8 or looser use the first five slices of each operand and the
-// 15 products with s + t <= 6 (X is split into five digits rounded at 2^-35 of its
-// column scale, the Lambda slices are the first five of seven; truncation ~2^-35 of
-// |A||X|, two orders below such a tolerance).
+// column of X is scaled by a power of two into [-1, 1] and cut into S = 5 slices
+// of 7 bits, v = sum_s q_s 2^{-7 s} with integers |q_s| <= 128, rounded at 2^-35 of
+// the scale.  A slice product sum_k A_s X_t is then an integer multiple of 2^{-7(s+t)}
+// below 2^24 in magnitude for every diagonal s + t <= 5 when K = 2Nc <= 512, so BF16
+// inputs with FP32 accumulation are exact there.
+// The 15 products with s + t <= 6 (truncation ~2^-35 of |A||X|) accumulate per
+// diagonal in five TMEM accumulators, 2..5 exact and 6 rounded at 2^-24 of its own
+// size.  The epilogue adds them in FP64, rescales, and forms r = B + A X - G in FP64.
+// This serves solves whose tolerance is 1e-8 or looser, two orders above the truncation; tighter
+// ones take the residual of k_oz64 (eight slices, any contour).  A seven-slice form of this
+// kernel took 1.4 to 1.5 times as long as that one (24x24, Nc = 256, 576 columns: 4.87 ms against 3.28).
 //
 // Kernels: k_oz_aprep (once per Lambda), k_oz_xprep, or k_oz_xprep_sum where every
 // bond carries the same J(t) (gather + scale + slice of X per residual), k_oz_gemm
@@ -37,24 +35,17 @@
 
 namespace {
 
-constexpr int S = 7;                                      // slices stored
-constexpr int S_SHORT = 5;                                 // slices used for tolerances >= 1e-8
-constexpr double SHORT_TOL = 1e-8;
+constexpr int S = 5;                                      // slices
 constexpr int BM = 128, BN = 48, BK = 32;                 // BK bf16 = 64-byte rows (64-byte swizzle)
 constexpr int A_TILE = BM * BK * 2;                       // 8 KB per A slice tile
 constexpr int X_TILE = BN * BK * 2;                       // 3 KB per X slice tile
-// pipeline of one slice count: a stage holds SE A slices and SE X slices (55 KB for
-// five, 77 KB for seven); as many stages as fit, at most four
-template <int SE>
-struct OzPipe {
-  static constexpr int STAGE_BYTES = SE * (A_TILE + X_TILE);
-  static constexpr int FIT = (227 * 1024 - 1024) / STAGE_BYTES;
-  static constexpr int STAGES = FIT > 4 ? 4 : FIT;
-  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024;
-};
+constexpr int STAGE_BYTES = S * (A_TILE + X_TILE);        // 55 KB
+constexpr int STAGES = 4;
+constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024;
+static_assert(SMEM_BYTES <= 227 * 1024, "shared memory of one CTA");
 constexpr int THREADS = 384;                               // warps 4-11: epilogue, two per TMEM lane quarter
 constexpr int EPI_CHUNK = 8;                               // accumulator columns per tcgen05.ld
-constexpr int NACC = 5;                                    // diagonals {2}, {3}, {4}, {5}, {6, 7, 8}
+constexpr int NACC = S;                                   // diagonals 2..6
 constexpr uint32_t ACC_COLS = NACC * BN;                   // one tile's accumulators: 240 columns
 constexpr uint32_t TMEM_COLS = 512;                        // two tiles' accumulators (double-buffered)
 
@@ -110,23 +101,20 @@ __device__ __forceinline__ long long fixed_right(double x, int k) {
   return (b >> 63) ? -v : v;
 }
 
-// The first NS signed 7-bit digits of V (|V| <= 2^FIX) in one pass: for A = |V| plus 64 in
-// every digit position below the top (and half a unit of the last kept digit when NS < S),
-// digit s of A in base 128, less 64, is the balanced digit q_s in [-64, 63]; the top digit
-// is A >> 7 (S - 1) <= 128.  Then sum_s q_s 2^{7 (S - s)} = |V| rounded to the last kept
-// digit, and the digits of V are those of |V| with its sign.  Slice s holds q_s 2^{-7 s}.
-template <int NS>
-__device__ __forceinline__ void write_digits_fast(long long V, __nv_bfloat16* dst, size_t slice_stride) {
-  static_assert(NS >= 1 && NS <= S, "digits kept");
+// The S signed 7-bit digits of V (|V| <= 2^FIX) in one pass: for A = |V| plus 64 in
+// every digit position below the top, digit s of A in base 128, less 64, is the balanced digit q_s in
+// [-64, 63]; the top digit is A >> 7 (S - 1) <= 128.  Then sum_s q_s 2^{7 (S - s)} = |V|,
+// and the digits of V are those of |V| with its sign.  Slice s holds q_s 2^{-7 s}.
+__device__ __forceinline__ void write_digits(long long V, __nv_bfloat16* dst, size_t slice_stride) {
   constexpr unsigned long long BIAS = [] {
-    unsigned long long b = NS < S ? 1ull << (7 * (S - NS) - 1) : 0ull;
-    for (int s = 2; s <= NS; ++s) b += 64ull << (7 * (S - s));
+    unsigned long long b = 0ull;
+    for (int s = 2; s <= S; ++s) b += 64ull << (7 * (S - s));
     return b;
   }();
   const bool neg = V < 0;
   const unsigned long long A = (unsigned long long)(neg ? -V : V) + BIAS;
 #pragma unroll
-  for (int s = 1; s <= NS; ++s) {
+  for (int s = 1; s <= S; ++s) {
     const int sh = 7 * (S - s);
     const int q = s == 1 ? (int)(A >> sh) : (int)((A >> sh) & 127u) - 64;
     const float unit = __int_as_float((127 - 7 * s) << 23);                    // 2^{-7 s}
@@ -182,13 +170,12 @@ __global__ void k_oz_aprep(const double2* __restrict__ lam, const double* __rest
   if (lane == 0) sigma[row] = sc;
   const double fix_over_sc = ldexp(1.0, FIX) / sc;
   const size_t stride = (size_t)Nr * N2 * N2;
-  for (int k = lane; k < N2; k += 32) write_digits_fast<S>(lambda_fixed(value(k), fix_over_sc), as + row * N2 + k, stride);
+  for (int k = lane; k < N2; k += 32) write_digits(lambda_fixed(value(k), fix_over_sc), as + row * N2 + k, stride);
 }
 
 // one warp per (site i, vector column n): X = sum_j J_ij G_j (FP64), column scale, slices.
 // Warps walk the sites fastest for one column, so that the four reads of a neighbour's
 // column meet in L1 or L2 instead of coming from HBM four times.
-template <int NS>
 __global__ void k_oz_xprep(const double2* __restrict__ G, const double* __restrict__ Jtab, const int* __restrict__ nbr,
                            const int* __restrict__ nbond, int Nr, int Nt, int Nc, int ncol,
                            __nv_bfloat16* __restrict__ xs, double* __restrict__ tau) {
@@ -241,8 +228,8 @@ __global__ void k_oz_xprep(const double2* __restrict__ G, const double* __restri
   for (int u = 0; u < PER_LANE; ++u) {
     const int z = lane + 32 * u;
     if (z < Nc) {
-      write_digits_fast<NS>(fixed_right(x[u].x, FIX - e), dst + z, stride);
-      write_digits_fast<NS>(fixed_right(x[u].y, FIX - e), dst + Nc + z, stride);
+      write_digits(fixed_right(x[u].x, FIX - e), dst + z, stride);
+      write_digits(fixed_right(x[u].y, FIX - e), dst + Nc + z, stride);
     }
   }
 }
@@ -250,7 +237,6 @@ __global__ void k_oz_xprep(const double2* __restrict__ G, const double* __restri
 // The same where every bond carries the same J(t): the factor sits in the Lambda slices
 // (k_oz_aprep with Jrow), and X = sum_j G_j needs only additions, done on the FP64 pipe
 // (which this kernel leaves otherwise idle) while the integer pipe cuts the digits.
-template <int NS>
 __global__ void k_oz_xprep_sum(const double2* __restrict__ G, const int* __restrict__ nbr, int Nr, int Nc, int ncol,
                                __nv_bfloat16* __restrict__ xs, double* __restrict__ tau) {
   const size_t wi = (size_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
@@ -279,8 +265,13 @@ __global__ void k_oz_xprep_sum(const double2* __restrict__ G, const int* __restr
       for (int q = 0; q < 4; ++q) {
         if (!has[q]) continue;
         const double2 g = col[q][z];
-        xr += g.x;
-        xi += g.y;
+        if (q == 0) {                                      // (nothing to add to yet)
+          xr = g.x;
+          xi = g.y;
+        } else {
+          xr += g.x;
+          xi += g.y;
+        }
       }
     }
     x[u] = make_double2(xr, xi);
@@ -296,34 +287,16 @@ __global__ void k_oz_xprep_sum(const double2* __restrict__ G, const int* __restr
   for (int u = 0; u < PER_LANE; ++u) {
     const int z = lane + 32 * u;
     if (z >= Nc) continue;
-    write_digits_fast<NS>(fixed_right(x[u].x, FIX - e), dst + z, stride);
-    write_digits_fast<NS>(fixed_right(x[u].y, FIX - e), dst + Nc + z, stride);
+    write_digits(fixed_right(x[u].x, FIX - e), dst + z, stride);
+    write_digits(fixed_right(x[u].y, FIX - e), dst + Nc + z, stride);
   }
 }
 
-struct Prod {
-  int s, t, acc;
-};
-template <int SE>
-__host__ __device__ constexpr Prod prod_of(int p) {
-  // products of the first SE slices with s + t <= SE + 1, ordered by diagonal; accumulator min(d - 2, 4)
-  int idx = 0;
-  for (int d = 2; d <= SE + 1; ++d)
-    for (int s = 1; s < d; ++s) {
-      int t = d - s;
-      if (s > SE || t > SE) continue;
-      if (idx == p) return Prod{s, t, d - 2 < NACC - 1 ? d - 2 : NACC - 1};
-      ++idx;
-    }
-  return Prod{0, 0, 0};
-}
-
 // Persistent: one CTA per SM walks the 128 x 48 output tiles (row tile fastest, then
-// column tile, then site).  Warp roles: warp 0 TMA loads (SE A slices and SE X slices
+// column tile, then site).  Warp roles: warp 0 TMA loads (S A slices and S X slices
 // per k-block), warp 1 one thread issuing the slice products into one of two
 // accumulator sets in TMEM, warps 4-7 the epilogue of the previous tile.  Every
 // mbarrier wait is bounded; on expiry the CTA raises the error flag and drains.
-template <int SE>
 __global__ void __launch_bounds__(THREADS, 1)
     k_oz_gemm(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap xmap,
               const double* __restrict__ sigma, const double* __restrict__ tau, const double2* __restrict__ G,
@@ -333,7 +306,6 @@ __global__ void __launch_bounds__(THREADS, 1)
   using namespace ptx;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  constexpr int STAGES = OzPipe<SE>::STAGES, STAGE_BYTES = OzPipe<SE>::STAGE_BYTES;
   __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], acc_full[2], acc_empty[2], drain;
   __shared__ uint32_t tmem_holder;
   __shared__ WaitCtl wctl;
@@ -377,10 +349,10 @@ __global__ void __launch_bounds__(THREADS, 1)
             break;
           }
           uint8_t* st = stage_ptr(s);
-          mbar_expect_tx(&full[s], SE * (A_TILE + X_TILE));
-          for (int q = 0; q < SE; ++q) {
+          mbar_expect_tx(&full[s], S * (A_TILE + X_TILE));
+          for (int q = 0; q < S; ++q) {
             tma_load_4d(st + q * A_TILE, &amap, &full[s], kb * BK, mt * BM, site, q);
-            tma_load_4d(st + SE * A_TILE + q * X_TILE, &xmap, &full[s], kb * BK, nt * BN, site, q);
+            tma_load_4d(st + S * A_TILE + q * X_TILE, &xmap, &full[s], kb * BK, nt * BN, site, q);
           }
         }
       }
@@ -409,30 +381,18 @@ __global__ void __launch_bounds__(THREADS, 1)
           const uint32_t base = smem_u32(stage_ptr(s));
 #pragma unroll
           for (int k16 = 0; k16 < BK / 16; ++k16) {
-            if constexpr (SE + 1 == NACC + 1) {
-              // the X slices lie back to back in the stage, so A_s times X_1 .. X_{SE+1-s} is one
-              // MMA of N = (SE + 1 - s) BN whose column block t lands at accumulator s + t - 2:
-              // D starts at accumulator s - 1.  SE MMAs per k step instead of SE (SE + 1) / 2,
-              // each A slice read once from shared memory.
+            // the X slices lie back to back in the stage, so A_s times X_1 .. X_{S+1-s} is one
+            // MMA of N = (S + 1 - s) BN whose column block t lands at accumulator s + t - 2:
+            // D starts at accumulator s - 1.  S MMAs per k step instead of S (S + 1) / 2,
+            // each A slice read once from shared memory.
 #pragma unroll
-              for (int sl = 1; sl <= SE; ++sl) {
-                const uint32_t n = (uint32_t)((SE + 1 - sl) * BN);
-                const uint32_t idesc = (IDESC & ~(0x3Fu << 17)) | ((n >> 3) << 17);
-                const uint64_t ad = sdesc_sw64(base + (sl - 1) * A_TILE + k16 * 32);
-                const uint64_t xd = sdesc_sw64(base + SE * A_TILE + k16 * 32);
-                // the first MMA of the tile (sl = 1 covers every accumulator) overwrites
-                mma<0>(dacc + (uint32_t)((sl - 1) * BN), ad, xd, idesc, (kb == 0 && k16 == 0 && sl == 1) ? 0u : 1u);
-              }
-            } else {
-#pragma unroll
-              for (int p = 0; p < SE * (SE + 1) / 2; ++p) {
-                const Prod pr = prod_of<SE>(p);
-                const uint64_t ad = sdesc_sw64(base + (pr.s - 1) * A_TILE + k16 * 32);
-                const uint64_t xd = sdesc_sw64(base + SE * A_TILE + (pr.t - 1) * X_TILE + k16 * 32);
-                // the first product of each accumulator at the first k step overwrites it
-                const bool first = (kb == 0 && k16 == 0 && (p == 0 || prod_of<SE>(p - 1).acc != pr.acc));
-                mma<0>(dacc + (uint32_t)(pr.acc * BN), ad, xd, IDESC, first ? 0u : 1u);
-              }
+            for (int sl = 1; sl <= S; ++sl) {
+              const uint32_t n = (uint32_t)((S + 1 - sl) * BN);
+              const uint32_t idesc = (IDESC & ~(0x3Fu << 17)) | ((n >> 3) << 17);
+              const uint64_t ad = sdesc_sw64(base + (sl - 1) * A_TILE + k16 * 32);
+              const uint64_t xd = sdesc_sw64(base + S * A_TILE + k16 * 32);
+              // the first MMA of the tile (sl = 1 covers every accumulator) overwrites
+              mma<0>(dacc + (uint32_t)((sl - 1) * BN), ad, xd, idesc, (kb == 0 && k16 == 0 && sl == 1) ? 0u : 1u);
             }
           }
           mma_commit(&empty[s]);
@@ -588,8 +548,7 @@ void oz_invalidate(dyson_ctx* c) {
   if (c->oz) static_cast<OzState*>(c->oz)->a_ready = false;
 }
 
-int oz_residual(dyson_ctx* c, int ncol, int gs, const double2* G, float* r32, double tol) {
-  const bool short_split = tol >= SHORT_TOL;
+int oz_residual(dyson_ctx* c, int ncol, int gs, const double2* G, float* r32) {
   OzState* st = state(c);
   const int Nr = c->Nr, Nc = c->Nc, N2 = 2 * Nc;
   int rc;
@@ -621,37 +580,21 @@ int oz_residual(dyson_ctx* c, int ncol, int gs, const double2* G, float* r32, do
     st->xmap_ncol = ncol;
   }
   if (!st->smem_set) {
-    DY_CUDA(c, cudaFuncSetAttribute(k_oz_gemm<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    OzPipe<S>::SMEM_BYTES));
-    DY_CUDA(c, cudaFuncSetAttribute(k_oz_gemm<S_SHORT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    OzPipe<S_SHORT>::SMEM_BYTES));
+    DY_CUDA(c, cudaFuncSetAttribute(k_oz_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
     st->smem_set = true;
   }
   size_t warps = (size_t)Nr * ncol;
   const unsigned xblocks = (unsigned)((warps + 7) / 8);
-  if (c->j_uniform && c->Nb > 0) {
-    if (short_split)
-      k_oz_xprep_sum<S_SHORT><<<xblocks, 256, 0, c->stream>>>(G, c->d_nbr, Nr, Nc, ncol, st->xslices, st->tau);
-    else
-      k_oz_xprep_sum<S><<<xblocks, 256, 0, c->stream>>>(G, c->d_nbr, Nr, Nc, ncol, st->xslices, st->tau);
-  } else {
-    if (short_split)
-      k_oz_xprep<S_SHORT><<<xblocks, 256, 0, c->stream>>>(G, c->dJ, c->d_nbr, c->d_nbond, Nr, c->Nt, Nc, ncol,
-                                                           st->xslices, st->tau);
-    else
-      k_oz_xprep<S><<<xblocks, 256, 0, c->stream>>>(G, c->dJ, c->d_nbr, c->d_nbond, Nr, c->Nt, Nc, ncol,
-                                                     st->xslices, st->tau);
-  }
+  if (c->j_uniform && c->Nb > 0)
+    k_oz_xprep_sum<<<xblocks, 256, 0, c->stream>>>(G, c->d_nbr, Nr, Nc, ncol, st->xslices, st->tau);
+  else
+    k_oz_xprep<<<xblocks, 256, 0, c->stream>>>(G, c->dJ, c->d_nbr, c->d_nbond, Nr, c->Nt, Nc, ncol, st->xslices,
+                                               st->tau);
   const long long tiles = (long long)(N2 / BM) * ((ncol + BN - 1) / BN) * Nr;
   const int grid = (int)std::min<long long>(tiles, st->num_sms);
-  if (short_split)
-    k_oz_gemm<S_SHORT><<<grid, THREADS, OzPipe<S_SHORT>::SMEM_BYTES, c->stream>>>(
-        st->amap, st->xmap, st->sigma, st->tau, G, c->d_lam, c->d_src_site, c->d_src_time, Nr, Nc, ncol, gs, r32,
-        c->d_norm, st->d_err);
-  else
-    k_oz_gemm<S><<<grid, THREADS, OzPipe<S>::SMEM_BYTES, c->stream>>>(
-        st->amap, st->xmap, st->sigma, st->tau, G, c->d_lam, c->d_src_site, c->d_src_time, Nr, Nc, ncol, gs, r32,
-        c->d_norm, st->d_err);
+  k_oz_gemm<<<grid, THREADS, SMEM_BYTES, c->stream>>>(st->amap, st->xmap, st->sigma, st->tau, G, c->d_lam,
+                                                      c->d_src_site, c->d_src_time, Nr, Nc, ncol, gs, r32, c->d_norm,
+                                                      st->d_err);
   c->launches += 2;
   DY_CUDA(c, cudaGetLastError());
   return DYSON_OK;

@@ -16,6 +16,7 @@
 
 #include "common.cuh"
 #include "detail.cuh"
+#include "oz.cuh"
 #include "tc.cuh"
 
 using namespace dyson_detail;
@@ -77,7 +78,7 @@ int dyson_autotune(dyson_ctx* c, int32_t max_block_columns, dyson_tuning* out) {
   DeviceGuard g(c->device);
   int rc;
   if (c->Nc % 64 != 0) return ctx_fail(c, DYSON_ERR_INVALID_ARG, "the tuner needs Nc % 64 == 0");
-  if ((rc = prepare_tables(c, DYSON_PREC_TF32X3_F64REF))) return rc;
+  if ((rc = prepare_tables(c, DYSON_PREC_TF32X3_F64REF, kOzTol))) return rc;
   if (!c->use_tc) return ctx_fail(c, DYSON_ERR_INVALID_ARG, "the tensor-core sweep needs Nc % 64 == 0");
   size_t col_bytes = 0, col_total = 0;
   const int64_t cap = chunk_columns(c, DYSON_PREC_TF32X3_F64REF, c->Nc, (int64_t)max_block_columns * c->Nc,
@@ -119,7 +120,7 @@ int dyson_autotune(dyson_ctx* c, int32_t max_block_columns, dyson_tuning* out) {
     for (int v : variants) {
       c->tc_variant = v;
       double ms = 0.0;
-      if ((rc = prepare_tables(c, DYSON_PREC_TF32X3_F64REF)) || (rc = time_sweeps(c, nq, 2, 3, &ms))) {
+      if ((rc = prepare_tables(c, DYSON_PREC_TF32X3_F64REF, kOzTol)) || (rc = time_sweeps(c, nq, 2, 3, &ms))) {
         c->tc_variant = saved_variant;
         return rc;
       }
