@@ -1,13 +1,16 @@
 // K2: one series sweep of App. C on the 5th-generation tensor cores,
 //     d_out = r + (Lambda W) X,   X_i(n, k) = sum_{j in NN(i)} J_ij(k) d_in_j(n, k),
-// over the FP32 planar chunk state (per vector column: Nc real parts, then Nc
-// imaginary parts).  The complex product is the real GEMM of the embedding
-// [[Re, -Im], [Im, Re]] (M = K = 2Nc) with the planar column vectors (N = vector
-// columns), and FP32 accuracy comes from three TF32 products
-//     A_hi X_hi + A_hi X_lo + A_lo X_hi
-// accumulated in FP32 in tensor memory.
+// over the FP32 planar chunk state (per vector column: Ns real parts, then Ns
+// imaginary parts; Ns is Nc rounded up to a multiple of 64, the padding zeros).
 //
-// Two launches per sweep:
+//   k_tc_fused   the general form: one persistent launch per sweep on CTA pairs
+//                (tcgen05 cta_group::2), the gather X = sum_j J_ij d_j computed by the
+//                GEMM's own producer warps, Lambda W and X as FP16 hi + lo halves under
+//                power-of-two scales, three products
+//                A_hi X_hi + A_hi X_lo + A_lo X_hi accumulated in FP32 in tensor
+//                memory (its own comment below has the tiles and the measurements).
+// The explicitly selected unfused forms (dyson_set_sweep_variant; Nc % 64 == 0) run 3xTF32 products of
+// the real embedding [[Re, -Im], [Im, Re]] (M = K = 2Nc) in two launches per sweep:
 //   k_tc_gather  X = sum_j J_ij d_j (FP32, coalesced float4, columns of all
 //                sites visited block by block so neighbour rows hit in L2);
 //   k_tc_gemm    persistent: one CTA per SM walks 128 x 256 output tiles (row
@@ -19,9 +22,8 @@
 //                               256-column TMEM accumulators
 //                  warps 8-11   epilogue: tcgen05.ld, + r, store d_out, update norm
 //                so the epilogue of one tile overlaps the MMAs of the next.
-//   k_tc_gemm_pair  the same sweep on clusters of two CTAs (tcgen05 cta_group::2,
-//                256 x 256 tiles, three 64 KB stages); selected per context with
-//                dyson_set_sweep_variant.
+//   k_tc_gemm_pair  the same GEMM on clusters of two CTAs (256 x 256 tiles, three 64 KB
+//                stages).
 // Every mbarrier wait is bounded (2 s of %globaltimer); on expiry the CTA
 // raises an error flag, lets in-flight copies and MMAs land, frees TMEM and
 // exits, and the host returns DYSON_ERR_TIMEOUT.
@@ -658,9 +660,9 @@ __global__ void __launch_bounds__(THREADS, 1)
 //        real and the imaginary rows of those points.  A k-block is 64 complex points; the tiles
 //        Re and Im of Lambda are loaded once and serve both halves of the embedding
 //        [[Re, -Im], [Im, Re]] (the minus sign is the MMA's negate bit), and X is gathered once
-//        per ceil(Nc / 256) tiles.  Two stages of 96 KB.  Nc >= 256.
+//        per ceil(Ns / 256) tiles.  Two stages of 96 KB.  Ns >= 192.
 //   <1>  a tile is (site, 256 vector columns, 256 rows of the embedding); a k-block is 64 real
-//        values, three stages of 64 KB.  Nc = 128, where <2> would fill half of its rows.
+//        values, three stages of 64 KB.  Ns = 64 and 128, where <2> would fill half of its rows at most.
 // Bytes from L2 per sweep at 16x16, Nc = 256, 4096 columns: X 8.6 GB, Lambda 4.3, epilogue 4.3
 // and 2.1 written (<1>: X 17.2, Lambda 4.3; with the embedding in 512-row tiles: X 8.6, Lambda 8.6).
 // Measured there: 2.10 ms per sweep, 9.1 TB/s from L2; 2.67 ms as <1> and 2.37 with the embedding in
@@ -956,24 +958,33 @@ __global__ void __launch_bounds__(F_THREADS, 1)
             tc_fence_after();
             const uint32_t st = smem_u32(stage_ptr(s));
             const uint32_t xb = st + GT * F_A_GROUP;
+            // The small products first, since the accumulators round relative to what they hold: the residual after
+            // an inner solve fell by 20 to 40 % on 26 of 30 drawn problems; 16x16, Nc = 256, 2.10 -> 2.05 ms a sweep,
+            // 8x8, Nc = 128, 1.2 % slower.
 #pragma unroll
-            for (int k16 = 0; k16 < F_BK / 16; ++k16) {
-              const uint32_t off = k16 * 32;
-              const uint32_t first = (kb | k16) ? 1u : 0u;
-              auto three = [&](uint32_t dacc, uint32_t a, uint32_t x, uint32_t idesc, uint32_t accumulate) {
-                const uint64_t ah = sdesc_sw128(a + off), al = sdesc_sw128(a + A_TILE + off);
-                const uint64_t xh = sdesc_sw128(x + off), xl = sdesc_sw128(x + X_TILE + off);
-                mma_pair_f16(dacc, ah, xh, idesc, accumulate);
-                mma_pair_f16(dacc, ah, xl, idesc, 1u);
-                mma_pair_f16(dacc, al, xh, idesc, 1u);
-              };
-              const uint32_t d0 = tmem + (uint32_t)(buf * GT * NB);
-              three(d0, st, xb, Cfg::IDESC, first);                                       // Re Xr (or A X)
-              if constexpr (GT == 2) {
-                const uint32_t im = st + F_A_GROUP, xi = xb + 2 * X_TILE, d1 = d0 + NB;
-                three(d0, im, xi, Cfg::IDESC | F_NEGATE_A, 1u);                             // - Im Xi
-                three(d1, im, xb, Cfg::IDESC, first);                                     // Im Xr
-                three(d1, st, xi, Cfg::IDESC, 1u);                                        // Re Xi
+            for (int hi = 0; hi < 2; ++hi) {
+#pragma unroll
+              for (int k16 = 0; k16 < F_BK / 16; ++k16) {
+                const uint32_t off = k16 * 32;
+                const uint32_t first = (kb | k16 | hi) ? 1u : 0u;
+                auto products = [&](uint32_t dacc, uint32_t a, uint32_t x, uint32_t idesc, uint32_t accumulate) {
+                  const uint64_t ah = sdesc_sw128(a + off), al = sdesc_sw128(a + A_TILE + off);
+                  const uint64_t xh = sdesc_sw128(x + off), xl = sdesc_sw128(x + X_TILE + off);
+                  if (hi) {
+                    mma_pair_f16(dacc, ah, xh, idesc, 1u);
+                  } else {
+                    mma_pair_f16(dacc, ah, xl, idesc, accumulate);
+                    mma_pair_f16(dacc, al, xh, idesc, 1u);
+                  }
+                };
+                const uint32_t d0 = tmem + (uint32_t)(buf * GT * NB);
+                products(d0, st, xb, Cfg::IDESC, first);                                  // Re Xr (or A X)
+                if constexpr (GT == 2) {
+                  const uint32_t im = st + F_A_GROUP, xi = xb + 2 * X_TILE, d1 = d0 + NB;
+                  products(d0, im, xi, Cfg::IDESC | F_NEGATE_A, 1u);                        // - Im Xi
+                  products(d1, im, xb, Cfg::IDESC, first);                                // Im Xr
+                  products(d1, st, xi, Cfg::IDESC, 1u);                                   // Re Xi
+                }
               }
             }
             mma_commit_pair_mc(&empty[s], 0x3);
