@@ -11,7 +11,7 @@
 // graph_sweeps sweeps is captured once as a CUDA graph and replayed until no
 // instance is active, so the host reads one word per replay instead of
 // synchronising after every sweep.  The FP64 residual refinement (split-product
-// residual, k_oz.cu) runs per instance between inner solves.  An instance whose
+// residual, k_oz.cu or k_oz64.cu) runs per instance between inner solves.  An instance whose
 // series diverges (spectral radius of K above 1) is then solved alone with the
 // GMRES of App. C (k_gmres.cu).
 #include <algorithm>
@@ -413,7 +413,7 @@ int dyson_batch_solve(dyson_batch* b, const int32_t* const* src, const int32_t* 
       X.rep.update = St.last;
       X.rep.gemm_flops += St.sweeps * sweep_flops(c, X.ncol);
       if (St.diverged) {
-        X.status = DYSON_ERR_DIVERGED;
+        X.status = X.prev_res <= tol ? DYSON_OK : DYSON_ERR_DIVERGED;
         X.done = true;
         continue;
       }
@@ -439,8 +439,10 @@ int dyson_batch_solve(dyson_batch* b, const int32_t* const* src, const int32_t* 
         X.status = DYSON_ERR_DIVERGED;
         X.done = true;
       } else if (res <= tol) {
-        X.status = DYSON_OK;
-        X.done = true;
+        if (!refine_once_more(res, tol, X.prev_res, ref + 1 == max_ref)) {
+          X.status = DYSON_OK;
+          X.done = true;
+        }
       } else if (res > kRefineContract * X.prev_res && ++X.strikes >= kRefineStrikes) {
         X.status = DYSON_ERR_DIVERGED;
         X.done = true;

@@ -617,7 +617,7 @@ int solve_mixed(dyson_ctx* c, int ncol, int gs, int precision, double tol, int m
       rc = inner_solve(c, ncol, gs, precision, r32, da, db, max_sweeps, rref, &d, rep, &peak,
                        may_switch ? kSeriesPeakMax : std::numeric_limits<double>::infinity(), act, &exhausted,
                        inner_target(kInnerTarget, tol, prev_res), ref == 0);
-      if (rc == DYSON_ERR_DIVERGED && may_switch) {
+      if (rc == DYSON_ERR_DIVERGED && may_switch && !(prev_res <= tol)) {
         gmres = true;                                    // redo this refinement with GMRES
         --ref;
         continue;
@@ -627,7 +627,7 @@ int solve_mixed(dyson_ctx* c, int ncol, int gs, int precision, double tol, int m
       if (rc == DYSON_OK && exhausted && may_switch) gmres = true;
     }
     if (rc == DYSON_ERR_DIVERGED) {
-      status = rc;
+      status = prev_res <= tol ? DYSON_OK : rc;            // (the refinement beyond the tolerance adds nothing)
       break;
     }
     if (rc) return rc;
@@ -648,11 +648,11 @@ int solve_mixed(dyson_ctx* c, int ncol, int gs, int precision, double tol, int m
       status = DYSON_ERR_DIVERGED;
       break;
     }
-    if (res <= tol) {
+    if (res <= tol && !refine_once_more(res, tol, prev_res, ref + 1 == c->max_refinements)) {
       status = DYSON_OK;
       break;
     }
-    if (res > kRefineContract * prev_res) {
+    if (res > tol && res > kRefineContract * prev_res) {
       if (may_switch && !gmres) {
         gmres = true;                                    // the series does not contract: use GMRES
       } else if (++strikes >= kRefineStrikes) {

@@ -39,10 +39,22 @@ constexpr double kInnerTarget = 4e-7;
 // below the tolerance.
 constexpr double kInnerSlack = 0.1;
 constexpr double kInnerCap = 1e-2;
+constexpr double kOnceMoreTarget = 0.1;                  // of a refinement below the tolerance (refine_once_more)
 inline double inner_target(double floor_target, double tol, double prev_res) {
   if (!(prev_res < 1e300)) return floor_target;
+  if (prev_res <= tol) return kOnceMoreTarget;
   const double t = kInnerSlack * tol / prev_res;
   return t > kInnerCap ? kInnerCap : (t > floor_target ? t : floor_target);
+}
+// A first refinement that ends just below a loose tolerance leaves errors of a few tolerances in quantities
+// that amplify the residual (the double occupancy's difference quotient, up to 4 times), where 3xTF32
+// inner solves, whose residuals are about twice as large, went on to a second refinement and 1e-9.  So at
+// tolerances of kLooseTol and above one more refinement follows unless the residual is below
+// kAcceptShare of the tolerance (0.43 was the least residual, in units of 1e-6, for which they did).
+constexpr double kLooseTol = 1e-8;
+constexpr double kAcceptShare = 0.4;
+inline bool refine_once_more(double res, double tol, double prev_res, bool last) {
+  return res <= tol && tol >= kLooseTol && res > kAcceptShare * tol && prev_res > tol && !last;
 }
 constexpr double kStallDrop = 1e-4;
 constexpr int kStallSweeps = 4;
