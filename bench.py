@@ -4,7 +4,7 @@
 Workload: the 16x16 trapped lattice on the Nc = 256 contour (112 + 112 real-time
 points, dt = 0.05, 32 imaginary points, beta = 2, U = 20, J = 1, trap
 0.02 |r|^2, mu = 0): every block column G(:, s) solved to a relative FP64 Dyson
-residual <= tol with the mixed-precision path (3xTF32 tcgen05 series sweeps,
+residual <= tol with the mixed-precision path (tcgen05 series sweeps on FP16 hi + lo operands,
 FP64 residual refinement).  A step builds Lambda, solves one batch of
 `--batch` block columns (disjoint per rank and per step, cycling through the
 256 sources) and computes the observables of those sources; the metric is
@@ -61,7 +61,7 @@ def parse():
     ap.add_argument("--no-adjoint", action="store_true", help="skip the 24x24 adjoint leg")
     ap.add_argument("--no-selfenergy", action="store_true", help="skip the self-consistency loop leg")
     ap.add_argument("--graph-sweeps", type=int, default=16,
-                    help="sweeps per captured graph of the inner series (0: one host synchronisation per sweep)")
+                    help="sweeps of the inner series per host synchronisation (0: one per sweep)")
     ap.add_argument("--sweep-variant", default="auto",
                     choices=["auto", "single_cta", "cta_pair", "fused_pair", "fused_pair_wide"],
                     help="override the autotuner's sweep variant (profiling runs: kernel timings under a "
@@ -623,11 +623,12 @@ def run_gb300(args, rank, world, local):
     peaks, peak_src = load_peaks()
     traffic = load_traffic() if args.lattice == 16 else {}
     Nc, Nr = p.Nc, p.Nr
-    ncol = args.batch * Nc
+    chunks = -(-args.batch // min(args.batch, tuning["chunk_block_columns"]))
+    ncol = args.batch * Nc / chunks                         # vector columns per launch, on average
     alg_flops = 8.0 * Nc * Nc * Nr * ncol                   # contour-GEMM flops of one sweep / residual
     state_bytes = 2.0 * Nc * 4 * Nr * ncol                  # one FP32 planar chunk state
     note = "achieved counts algorithmic complex-GEMM flops (8 Nc^2 per site and vector column)"
-    slices = 15 if args.tol >= 1e-8 else 28
+    slices = 15 if args.tol >= 1e-8 else 36                 # BF16 products of a split residual
     rooflines = {}
     for name, (n, ms) in kstats.items():
         if not n or name == "selfenergy_conn":
@@ -638,16 +639,21 @@ def run_gb300(args, rank, world, local):
             peak = peaks["hbm_gbs"]
             r = {"bound": "hbm", "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,
                  "peak_source": f"{peak_src} copy bandwidth; bytes = read d + write X (FP32 planar state)"}
-        elif name in ("sweep_f64", "residual_f64"):
-            ach = alg_flops / dur / 1e12
-            r = {"bound": "alu", "achieved": ach, "peak": mm["fp64_tflops"], "unit": "TFLOP/s",
-                 "frac": ach / mm["fp64_tflops"], "peak_source": "FP64 matmul rate measured in this run"}
-        elif name == "residual_split_bf16":
+        elif name in ("sweep_f64", "residual_f64", "residual_split_bf16"):
+            if name != "residual_split_bf16":
+                slices = 36
             ach = alg_flops / dur / 1e12
             peak = peaks["bf16_tflops"]
             r = {"bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
                  "executed_tflops": slices * ach, "executed_frac": slices * ach / peak,
                  "peak_source": f"{peak_src} bf16 burst; {note}; the slice split executes {slices} BF16 products"}
+        elif name == "sweep_tc_fused":
+            ach = alg_flops / dur / 1e12
+            peak = peaks["bf16_tflops"]
+            r = {"bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
+                 "executed_tflops": 3 * ach, "executed_frac": 3 * ach / peak,
+                 "peak_source": f"{peak_src} bf16 burst (FP16 runs at the same rate); {note}; the FP16 hi + lo split "
+                                "executes 3x"}
         else:
             ach = alg_flops / dur / 1e12
             peak = mm["tf32_tflops"]
@@ -715,11 +721,13 @@ def run_gb300(args, rank, world, local):
 
     if rank != 0:
         return
+    fused = binding.SWEEP_NAMES[tuning["sweep_variant"]].startswith("fused")
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": max_ms / args.steps, "higher_is_better": True,
-            "scaling": "weak", "vs_baseline": None, "dtype": "tf32x3+f64", "data": "synthetic",
+            "scaling": "weak", "vs_baseline": None, "dtype": "fp16x3+f64" if fused else "tf32x3+f64", "data": "synthetic",
             "config": bench_config(args, p, world),
-            "precision": "3xTF32 tcgen05 series sweeps + FP64 Dyson residual refinement",
+            "precision": ("FP16 hi + lo (three products, FP32 accumulation)" if fused else "3xTF32") +
+                         " tcgen05 series sweeps + FP64 Dyson residual refinement",
             "measured_peaks": mm, "rooflines": rooflines, "kernels": kernels,
             "autotune": {"sweep_variant": binding.SWEEP_NAMES[tuning["sweep_variant"]],
                          "variant_pinned": args.sweep_variant != "auto",

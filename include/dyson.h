@@ -71,8 +71,9 @@ enum {
   DYSON_PREC_F64 = 0,           /* complex128 sweeps, FP64-accurate: BF16 slice products
                                    on the tensor cores, or the FP64 pipes where the
                                    slices of Lambda do not fit in device memory          */
-  DYSON_PREC_TF32X3_F64REF = 1  /* complex FP32 sweeps as 3xTF32 tcgen05 products with
-                                   FP32 accumulation, refined by FP64 Dyson residuals     */
+  DYSON_PREC_TF32X3_F64REF = 1  /* complex FP32 sweeps as three tcgen05 products of FP16
+                                   hi + lo (or, where selected, TF32 hi + lo) operands
+                                   with FP32 accumulation, refined by FP64 Dyson residuals */
 };
 
 typedef struct dyson_ctx dyson_ctx;
@@ -383,8 +384,8 @@ int dyson_set_symmetry(dyson_ctx* ctx, int mode);
 
 /* Autotuner of the tensor-core sweep.  On this context's Lambda it times two
  * warm-up and three timed sweeps for each candidate: every sweep variant the
- * contour allows (DYSON_SWEEP_SINGLE_CTA; DYSON_SWEEP_CTA_PAIR and
- * DYSON_SWEEP_FUSED_PAIR where Nc is a multiple of 128; DYSON_SWEEP_FUSED_PAIR_WIDE
+ * contour allows (DYSON_SWEEP_SINGLE_CTA and DYSON_SWEEP_FUSED_PAIR;
+ * DYSON_SWEEP_CTA_PAIR where Nc is a multiple of 128; DYSON_SWEEP_FUSED_PAIR_WIDE
  * where it is a multiple of 256) times every chunk of 1, 2, 4, ... block columns up to
  * max_block_columns and to what fits in 85 % of free device memory; unless the inner
  * solver is DYSON_INNER_SERIES, also only chunks that leave room for the GMRES basis
@@ -432,7 +433,8 @@ int dyson_set_inner_solver(dyson_ctx* ctx, int solver, int32_t restart);
  * on the tensor cores skips every (site, 256-column) tile that is still zero:
  * the results are bit-identical, the work of the early sweeps shrinks.  Later
  * refinements (whose residuals are dense), GMRES, the FP64 and the CUDA-core FP32
- * sweeps are not truncated.  Truncated sweeps use the single-CTA kernel. */
+ * sweeps are not truncated.  Where DYSON_SWEEP_CTA_PAIR is selected, truncated sweeps
+ * use the single-CTA kernel. */
 int dyson_set_support_truncation(dyson_ctx* ctx, int enable);
 
 /* ---------------------------------------------------------------------------

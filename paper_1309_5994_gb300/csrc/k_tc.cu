@@ -958,9 +958,9 @@ __global__ void __launch_bounds__(F_THREADS, 1)
             tc_fence_after();
             const uint32_t st = smem_u32(stage_ptr(s));
             const uint32_t xb = st + GT * F_A_GROUP;
-            // The small products first, since the accumulators round relative to what they hold: the residual after
-            // an inner solve fell by 20 to 40 % on 26 of 30 drawn problems; 16x16, Nc = 256, 2.10 -> 2.05 ms a sweep,
-            // 8x8, Nc = 128, 1.2 % slower.
+            // The small products first, since the accumulators round relative to what they hold: the final residual fell
+            // on 28 of 30 drawn problems, by 19 % in the median; 16x16, Nc = 256, 1.8 % faster, 8x8, Nc = 128, 1.2 %
+            // slower.
 #pragma unroll
             for (int hi = 0; hi < 2; ++hi) {
 #pragma unroll
