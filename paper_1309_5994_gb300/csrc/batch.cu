@@ -247,7 +247,7 @@ int dyson_batch_solve(dyson_batch* b, const int32_t* const* src, const int32_t* 
     if (n_src[k] < 1 || !src[k]) return bfail(b, DYSON_ERR_INVALID_ARG, "every instance needs a source site");
     for (int q = 0; q < n_src[k]; ++q)
       if (src[k][q] < 0 || src[k][q] >= c->Nr) return bfail(b, DYSON_ERR_INVALID_ARG, "source site out of range");
-    if ((rc = prepare_tables(c, DYSON_PREC_TF32X3_F64REF, tol, true))) return bfail(b, rc, c->err);
+    if ((rc = prepare_tables(c, DYSON_PREC_TF32X3_F64REF, tol, 0, true))) return bfail(b, rc, c->err);
     if (!c->use_tc || !oz_supported(c) || !tc_fused_runs(c))
       return bfail(b, DYSON_ERR_INVALID_ARG,
                    "instance " + std::to_string(k) + ": batched solves need Nc % 64 == 0 and 2 Nc <= 512");

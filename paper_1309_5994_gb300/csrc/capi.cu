@@ -648,7 +648,8 @@ int solve_mixed(dyson_ctx* c, int ncol, int gs, int precision, double tol, int m
       status = DYSON_ERR_DIVERGED;
       break;
     }
-    if (res <= tol && !refine_once_more(res, tol, prev_res, ref + 1 == c->max_refinements)) {
+    if (res <= tol && !(c->use_tc && tc_uses_fused(c) &&
+                        refine_once_more(res, tol, prev_res, ref + 1 == c->max_refinements))) {
       status = DYSON_OK;
       break;
     }
@@ -818,7 +819,13 @@ int prepare_oz64(dyson_ctx* c) {
 // and residual kernels (sets c->use_tc, c->use_oz, c->use_oz64).
 // The residual of a mixed solve: five slices (15 products) for tolerances down to 1e-8, where they run at
 // 85 TFLOP/s of the contraction (16x16, Nc = 256, 4096 columns: 6.5 ms); eight (36 products, 53 TFLOP/s) below.
-int prepare_tables(dyson_ctx* c, int precision, double tol, bool batch) {
+int prepare_tables(dyson_ctx* c, int precision, double tol, int64_t columns, bool batch) {
+  // A fused tile of 256 rows is half empty at 64 contour points (128 rows of the embedding), so from
+  // kManySiteColumns on the unfused form is the faster one although its series waits for every sweep:
+  // single CTA / fused, us a sweep: 8x8 sites, 512 columns 34 / 46, 1024 57 / 83; 12x12, 512 62 / 85;
+  // 16x16, 128 36 / 52; 5x5, 1024 33 / 43.
+  constexpr int64_t kManySiteColumns = 32768;
+  c->many_of_64 = c->Nc == 64 && c->Nr * columns >= kManySiteColumns;
   c->use_tc = c->use_oz = c->use_oz64 = false;
   c->Ns = c->Nc;
   if (precision == DYSON_PREC_F64) return prepare_oz64(c);
@@ -954,7 +961,8 @@ int solve_columns_impl(dyson_ctx* c, const int32_t* src, int64_t n_src, int prec
   for (int64_t q = 0; q < n_src; ++q)
     if (src[q] < 0 || src[q] >= c->Nr) return R.finish(ctx_fail(c, DYSON_ERR_INVALID_ARG, "source site out of range"));
   DeviceGuard g(c->device);
-  if ((rc = prepare_tables(c, precision, tol))) return R.finish(rc);
+  const int64_t at_once = c->chunk_override > 0 ? std::min<int64_t>(n_src, c->chunk_override) : n_src;
+  if ((rc = prepare_tables(c, precision, tol, at_once * c->Nc))) return R.finish(rc);
   size_t col_bytes = 0;
   const int64_t cols = chunk_columns(c, precision, c->Nc, n_src * (int64_t)c->Nc, &col_bytes);
   if (cols < c->Nc) return R.finish(ctx_fail(c, DYSON_ERR_OOM, "one block column does not fit in device memory"));
@@ -1029,7 +1037,7 @@ int dyson_solve_vector_columns(dyson_ctx* c, const int32_t* sites, const int32_t
     if (sites[q] < 0 || sites[q] >= c->Nr || times[q] < 0 || times[q] >= c->Nc)
       return R.finish(ctx_fail(c, DYSON_ERR_INVALID_ARG, "column source out of range"));
   DeviceGuard g(c->device);
-  if ((rc = prepare_tables(c, precision, tol))) return R.finish(rc);
+  if ((rc = prepare_tables(c, precision, tol, n))) return R.finish(rc);
   constexpr int GS = 32;                                   // norm group; columns padded to a multiple
   const int64_t padded = (n + GS - 1) / GS * GS;
   size_t col_bytes = 0;

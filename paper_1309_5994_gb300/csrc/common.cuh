@@ -214,6 +214,7 @@ struct dyson_ctx {
   bool tc_enabled = true;            // 3xTF32 tcgen05 sweep allowed where the contour fits it
   bool use_tc = false;               // chosen for the current solve
   int tc_variant = -1;               // DYSON_SWEEP_*; -1: none selected, the fused form
+  bool many_of_64 = false;           // this solve is large and of 64 contour points (prepare_tables)
   int max_refinements = 12;
   int chunk_override = 0;
   int64_t launches = 0;              // kernels launched by this context since dyson_init

@@ -1314,7 +1314,8 @@ int fused_gt_of(const dyson_ctx* c) { return contour_stride(c) >= 192 ? 2 : 1; }
 // form of the fused kernel that serves the context's variant (0: none).  The unfused forms serve
 // only contours that fill their tiles; every other contour takes the fused kernel.
 int fused_gt(dyson_ctx* c) {
-  const bool unfused = (c->tc_variant == DYSON_SWEEP_SINGLE_CTA || c->tc_variant == DYSON_SWEEP_CTA_PAIR) &&
+  const bool unfused = (c->tc_variant == DYSON_SWEEP_SINGLE_CTA || c->tc_variant == DYSON_SWEEP_CTA_PAIR ||
+                        c->many_of_64) &&
                        c->Nc % 64 == 0;
   if (unfused || !encode_fn()) return 0;
   return fused_clusters(c) > 0 ? fused_gt_of(c) : 0;

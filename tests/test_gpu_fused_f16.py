@@ -101,3 +101,25 @@ def test_gmres_item_shapes(torch_cuda, lib, Nt, Nm):
         want = ref[:, :, q * p.Nc:(q + 1) * p.Nc]
         assert np.abs(got[q] - want).max() / np.abs(want).max() < 1e-11
     s.close()
+
+
+@pytest.mark.parametrize("n,unfused", [(5440, False), (5472, True)])
+def test_large_solves_of_64_points_take_the_unfused_form(torch_cuda, lib, n, unfused):
+    """6 sites times n vector columns on either side of 32768, the rule's line at Nc = 64."""
+    from paper_1309_5994_gb300 import binding
+    torch = torch_cuda
+    p = wl.random_tables(wl.small(L=3, Ly=2, Nt=24, Nm=16, dt=0.02, beta=1.0, trap_c=0.3, U0=14.0), seed=7, rel=0.1)
+    S = dyson.setup(p)
+    sites, times = [k % p.Nr for k in range(n)], [(7 * k) % p.Nc for k in range(n)]
+    distinct = sorted(set(zip(sites, times)))
+    ref = dict(zip(distinct, dyson.dense_solve(S, dyson.rhs_vector_columns(S, distinct)).transpose(2, 0, 1)))
+    s = binding.Solver(p, device=0)
+    s.build_sigma()
+    s.profile(True)
+    v = torch.empty((n, p.Nr, p.Nc), dtype=torch.complex128, device="cuda:0")
+    s.solve_vectors(sites, times, precision=binding.PREC_TF32X3_F64REF, tol=1e-12, g_out=v)
+    assert (s.profile_query(binding.KERNEL_GATHER_TC)[0] > 0) == unfused
+    got, big = v.cpu().numpy(), max(np.abs(w).max() for w in ref.values())
+    for k in list(range(0, n, 97)) + [n - 1]:
+        assert np.abs(got[k] - ref[sites[k], times[k]]).max() / big < 1e-11
+    s.close()
