@@ -660,7 +660,8 @@ def run_gb300(args, rank, world, local):
             r = {"bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
                  "executed_tflops": 3 * ach, "executed_frac": 3 * ach / peak,
                  "peak_source": f"TF32 matmul rate measured in this run; {note}; the 3xTF32 split executes 3x"}
-        r["traffic"] = traffic.get(name)
+        # the record is for 16 block columns per launch
+        r["traffic"] = traffic[name] * ncol / (16 * Nc) if traffic.get(name) else None
         r["kernel"] = name
         r["avg_ms"] = ms / n
         rooflines[name] = r

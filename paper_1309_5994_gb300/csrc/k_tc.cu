@@ -653,8 +653,8 @@ __global__ void __launch_bounds__(THREADS, 1)
 // and one per column group of X (set_scale), taken out again in the epilogue.  hi + lo keeps
 // 22 bits of every entry down to 2^-16 of the row's (group's) largest and 2^-39 of the
 // largest below that, under the FP32 accumulation's own rounding.
-// The kernel is bound by the traffic between L2 and the SMs (10 to 12 TB/s were the most seen), so
-// the two forms differ in what they read there.  Both have two accumulator sets of 256 TMEM
+// The kernel is bound by the latency of the loads through L2 at what an SM keeps in flight (10.4 TB/s of
+// L2 traffic; tensor pipe 29 %, L2 33 %, DRAM 50 % busy), so the two forms differ in what they read.  Both have two accumulator sets of 256 TMEM
 // columns, so that a tile's epilogue overlaps the next tile's MMAs:
 //   <2>  a tile is (site, 128 vector columns, 256 contour points z): its two accumulators are the
 //        real and the imaginary rows of those points.  A k-block is 64 complex points; the tiles
@@ -665,7 +665,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 //        values, three stages of 64 KB.  Ns = 64 and 128, where <2> would fill half of its rows at most.
 // Bytes from L2 per sweep at 16x16, Nc = 256, 4096 columns: X 8.6 GB, Lambda 4.3, epilogue 4.3
 // and 2.1 written (<1>: X 17.2, Lambda 4.3; with the embedding in 512-row tiles: X 8.6, Lambda 8.6).
-// Measured there: 2.10 ms per sweep, 9.1 TB/s from L2; 2.67 ms as <1> and 2.37 with the embedding in
+// Measured there: 2.05 ms per sweep; 2.67 ms as <1> and 2.37 with the embedding in
 // 512-row tiles; 2.66 ms in 3xTF32 with the traffic of <1>.  Each gather step waits for one loaded
 // memory latency (about 2.3 us, 64 KB in flight per SM); fetching the next tile's neighbour rows
 // into L2 ahead adds requests and cost 25 %.
