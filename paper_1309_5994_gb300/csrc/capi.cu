@@ -649,7 +649,7 @@ int solve_mixed(dyson_ctx* c, int ncol, int gs, int precision, double tol, int m
       break;
     }
     if (res <= tol && !(c->use_tc && tc_uses_fused(c) &&
-                        refine_once_more(res, tol, prev_res, ref + 1 == c->max_refinements))) {
+                        refine_once_more(res, tol, prev_res, c->Nc, ref + 1 == c->max_refinements))) {
       status = DYSON_OK;
       break;
     }
