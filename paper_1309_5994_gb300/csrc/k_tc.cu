@@ -671,6 +671,15 @@ __global__ void __launch_bounds__(THREADS, 1)
 // into L2 ahead adds requests and cost 25 %.
 // Error of one inner solve against the FP64 residual, 8x8 to 24x24, six contours: 0.45 to 0.95 of the
 // 3xTF32 form's in every case (fewer roundings: twice the products per MMA).
+// SPLIT: contours that are no multiple of 64, whose other form is the FP32 CUDA-core sweep (every product and
+// sum rounded to nearest).  The tensor memory accumulation truncates once per MMA, and with all three products in
+// one accumulator the residual of an inner solve was 1.1 to 2.8 times that sweep's (Nc 33 to 151; 0.4 to 1.2 from
+// 160 on).  So the small products get an accumulator of their own, and in <1> the large ones two that they take in
+// turn: 0.26 to 1.02 times, 0.6 in the mean of 92 problems, Nc 26 to 250.  That fills the tensor memory with one set of
+// accumulators and <1> takes 128 columns a tile (four stages of 48 KB).  A solve at 1e-10, one accumulator and
+// SPLIT: 9x7, Nc = 100, 6 block columns 4.4 and 4.2 ms; 10x9, Nc = 105, 8 columns 7.1 and 6.8; 7x7, Nc = 151, 3
+// columns 6.0 and 7.3; 9x8, Nc = 223, 6 columns 32.4 and 29.5 (with fewer sweeps); the CUDA-core sweep 21, 39, 27, 305.
+// (13x15, Nc = 180, one column, 1e-6: 14.0 and 18.8; the CUDA-core sweep 70.)
 // Sites are visited in bands of two lattice rows, column by column, so that
 // a site's neighbours are read while they are still in L2.
 // Warp roles (512 threads per CTA, both CTAs of the pair):
@@ -702,18 +711,25 @@ static_assert(F_REG_CTRL + 2 * F_REG_PROD + F_REG_EPI <= 4 * F_REGS_AT_LAUNCH,
               "the warpgroups' register shares exceed the block's registers at launch");
 static_assert(F_PROD_W0 == 4 && F_PROD_WARPS == 8 && F_EPI_W0 == 12 && F_THREADS == 512,
               "the register split assumes warpgroups {0-3: control, 4-11: producers, 12-15: epilogue}");
-template <int GT>
+template <int GT_, bool SPLIT>
 struct FusedCfg {
-  static constexpr int NB = 256 / GT;                   // vector columns of a tile
+  static constexpr int GT = GT_;
+  static constexpr int NB = GT == 1 && !SPLIT ? 256 : 128;   // vector columns of a tile
+  static constexpr int STEPS = GT * NB / 128;           // gather steps of a k-block
   static constexpr int X_TILE = (NB / 2) * F_BK * 2;    // one CTA's half of X hi (or lo)
   // GT = 2: Re hi, Re lo, Im hi, Im lo | Xr hi, Xr lo, Xi hi, Xi lo;  GT = 1: hi, lo | X hi, X lo
   static constexpr int STAGE = GT * F_A_GROUP + GT * 2 * X_TILE;
-  static constexpr int STAGES = GT == 1 ? 3 : 2;
+  static constexpr int STAGES = GT == 2 ? 2 : SPLIT ? 4 : 3;
   static constexpr int SMEM = STAGES * STAGE + 1024;
-  static constexpr int NBUF = 2;                        // accumulator sets of GT x NB columns
+  // accumulators of one output (the first LARGE take hi x hi in turn, the last the small products) and
+  // sets of them
+  static constexpr int ACCS = !SPLIT ? 1 : GT == 1 ? 3 : 2, LARGE = ACCS == 3 ? 2 : 1;
+  static constexpr int NBUF = SPLIT ? 1 : 2;
+  static constexpr uint32_t ACC_STRIDE = GT * NB;       // TMEM columns from one accumulator to the next
   // kind::f16, D = F32, A = B = F16, K-major, M = 256, N = NB
   static constexpr uint32_t IDESC = (1u << 4) | ((uint32_t)(NB >> 3) << 17) | ((uint32_t)(PM >> 4) << 24);
-  static_assert(NBUF * GT * NB <= 512, "TMEM holds 512 columns");
+  static_assert(NBUF * ACCS * GT * NB <= 512, "TMEM holds 512 columns");
+  static_assert(SMEM <= 227 * 1024, "shared memory of one CTA");
   static_assert(TC_TILE_COLS % NB == 0, "a tile lies in one column tile of the support table");
 };
 
@@ -739,11 +755,11 @@ __host__ __device__ __forceinline__ int fused_row_tiles(int Ns) {
 }
 
 // (act has one entry per site and TC_TILE_COLS columns)
-template <int GT>
+template <class Cfg>
 __device__ __forceinline__ FTile fused_tile(const FusedInst& I, int tile, int sweep) {
-  constexpr int NB = FusedCfg<GT>::NB;
+  constexpr int NB = Cfg::NB;
   FTile T;
-  const int NGT = fused_row_tiles<GT>(I.Ns), NT = (I.ncol + NB - 1) / NB;
+  const int NGT = fused_row_tiles<Cfg::GT>(I.Ns), NT = (I.ncol + NB - 1) / NB;
   T.gt = tile % NGT;
   T.nt = (tile / NGT) % NT;
   T.site = band_site(tile / (NGT * NT), I.Lx, I.Ly);
@@ -762,9 +778,9 @@ __device__ __forceinline__ FTile fused_tile(const FusedInst& I, int tile, int sw
 // chunk ahead, the first ones before the accumulators are complete.  (Three chunks of 8 columns ahead,
 // or a ring of four 8-column slots in shared memory filled by bulk copies, took 2.5-2.7 ms per sweep
 // where this takes 2.1: 16x16, Nc = 256, 4096 columns.)  RZERO: r is zero on this tile.
-template <int GT, bool RZERO>
+template <class Cfg, bool RZERO>
 struct FusedEpilogue {
-  static constexpr int NB = FusedCfg<GT>::NB, CH = 16, PER = NB / CH, CHUNKS = GT * PER;
+  static constexpr int NB = Cfg::NB, CH = 16, PER = NB / CH, CHUNKS = Cfg::GT * PER;
   const float* __restrict__ r;
   const float* __restrict__ din;
   float* __restrict__ dout;
@@ -820,6 +836,14 @@ struct FusedEpilogue {
     uint32_t v[CH];
     ptx::tmem_ld16(tacc + (uint32_t)(e * CH), v);
     ptx::tmem_wait_ld();
+#pragma unroll
+    for (int a = 1; a < Cfg::ACCS; ++a) {
+      uint32_t w[CH];
+      ptx::tmem_ld16(tacc + a * Cfg::ACC_STRIDE + (uint32_t)(e * CH), w);
+      ptx::tmem_wait_ld();
+#pragma unroll
+      for (int j = 0; j < CH; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + __uint_as_float(w[j]));
+    }
     const size_t o = at(e);
     auto column = [&](int j) {
       const float y = RZERO ? __uint_as_float(v[j]) * down : fmaf(__uint_as_float(v[j]), down, rv[B][j]);
@@ -853,13 +877,13 @@ __device__ __forceinline__ bool r_is_zero(const FusedInst& I, int site, int n_fi
   return !__any_sync(0xffffffffu, here);
 }
 
-template <int GT>
+template <int GT, bool SPLIT>
 __global__ void __launch_bounds__(F_THREADS, 1)
     k_tc_fused(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
                const __grid_constant__ FusedInst I, int* __restrict__ err, int sweep, const int* __restrict__ run,
                const int* __restrict__ sweeps_done) {
   using namespace ptx;
-  using Cfg = FusedCfg<GT>;
+  using Cfg = FusedCfg<GT, SPLIT>;
   constexpr int STAGES = Cfg::STAGES, NBUF = Cfg::NBUF, STAGE = Cfg::STAGE, NB = Cfg::NB, X_TILE = Cfg::X_TILE;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -916,7 +940,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
         int g = 0;
         bool ok = true;
         for (int tile = pair; tile < tiles && ok; tile += npairs) {
-          const FTile T = fused_tile<GT>(I, tile, sweep);
+          const FTile T = fused_tile<Cfg>(I, tile, sweep);
           if (!T.active) continue;
           for (int kb = 0; kb < KB; ++kb, ++g) {
             const int s = g % STAGES;
@@ -943,7 +967,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
         int g = 0, t = 0;
         bool ok = true, any = false;
         for (int tile = pair; tile < tiles && ok; tile += npairs) {
-          const FTile T = fused_tile<GT>(I, tile, sweep);
+          const FTile T = fused_tile<Cfg>(I, tile, sweep);
           if (!T.active) continue;
           const int buf = t % NBUF;
           if (t >= NBUF && !mbar_wait_cluster(&acc_empty[buf], ((t / NBUF) - 1) & 1, abort_p)) break;
@@ -966,24 +990,26 @@ __global__ void __launch_bounds__(F_THREADS, 1)
 #pragma unroll
               for (int k16 = 0; k16 < F_BK / 16; ++k16) {
                 const uint32_t off = k16 * 32;
-                const uint32_t first = (kb | k16 | hi) ? 1u : 0u;
-                auto products = [&](uint32_t dacc, uint32_t a, uint32_t x, uint32_t idesc, uint32_t accumulate) {
+                // (fresh: the first products of an output overwrite what its accumulators held)
+                auto products = [&](uint32_t dacc, uint32_t a, uint32_t x, uint32_t idesc, bool fresh) {
                   const uint64_t ah = sdesc_sw128(a + off), al = sdesc_sw128(a + A_TILE + off);
                   const uint64_t xh = sdesc_sw128(x + off), xl = sdesc_sw128(x + X_TILE + off);
                   if (hi) {
-                    mma_pair_f16(dacc, ah, xh, idesc, 1u);
+                    mma_pair_f16(dacc + (uint32_t)(k16 % Cfg::LARGE) * Cfg::ACC_STRIDE, ah, xh, idesc,
+                                 SPLIT && fresh && kb == 0 && k16 < Cfg::LARGE ? 0u : 1u);
                   } else {
-                    mma_pair_f16(dacc, ah, xl, idesc, accumulate);
-                    mma_pair_f16(dacc, al, xh, idesc, 1u);
+                    const uint32_t small = dacc + (uint32_t)(Cfg::ACCS - 1) * Cfg::ACC_STRIDE;
+                    mma_pair_f16(small, ah, xl, idesc, fresh && (kb | k16) == 0 ? 0u : 1u);
+                    mma_pair_f16(small, al, xh, idesc, 1u);
                   }
                 };
                 const uint32_t d0 = tmem + (uint32_t)(buf * GT * NB);
-                products(d0, st, xb, Cfg::IDESC, first);                                  // Re Xr (or A X)
+                products(d0, st, xb, Cfg::IDESC, true);                                   // Re Xr (or A X)
                 if constexpr (GT == 2) {
                   const uint32_t im = st + F_A_GROUP, xi = xb + 2 * X_TILE, d1 = d0 + NB;
-                  products(d0, im, xi, Cfg::IDESC | F_NEGATE_A, 1u);                        // - Im Xi
-                  products(d1, im, xb, Cfg::IDESC, first);                                // Im Xr
-                  products(d1, st, xi, Cfg::IDESC, 1u);                                   // Re Xi
+                  products(d0, im, xi, Cfg::IDESC | F_NEGATE_A, false);                     // - Im Xi
+                  products(d1, im, xb, Cfg::IDESC, true);                                 // Im Xr
+                  products(d1, st, xi, Cfg::IDESC, false);                                // Re Xi
                 }
               }
             }
@@ -1004,7 +1030,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
         int g = 0;
         bool ok = true;
         for (int tile = pair; tile < tiles && ok; tile += npairs) {
-          const FTile T = fused_tile<GT>(I, tile, sweep);
+          const FTile T = fused_tile<Cfg>(I, tile, sweep);
           if (!T.active) continue;
           for (int kb = 0; kb < KB; ++kb, ++g) {
             const int s = g % STAGES;
@@ -1030,7 +1056,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
     int g = 0;
     int ok = 1;
     for (int tile = pair; tile < tiles && ok; tile += npairs) {
-      const FTile T = fused_tile<GT>(I, tile, sweep);
+      const FTile T = fused_tile<Cfg>(I, tile, sweep);
       if (!T.active) continue;
       const int Ns = I.Ns, N2 = 2 * Ns, ncol = I.ncol, gs = I.gs;
       const float* __restrict__ din = I.din;
@@ -1089,7 +1115,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
         const int s = g % STAGES;
         uint8_t* xs = stage_ptr(s) + GT * F_A_GROUP;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < Cfg::STEPS; ++h) {
           float4 acc[2][2];
 #pragma unroll
           for (int i = 0; i < 2; ++i)
@@ -1107,7 +1133,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
               }
               acc[i][u] = a;
             }
-          if (h == 0) issue(kb, 1);
+          if (h + 1 < Cfg::STEPS) issue(kb, h + 1);
           else if (kb + 1 < KB) {
             issue(kb + 1, 0);
             issue_j(kb + 1);
@@ -1147,7 +1173,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
     int t = 0;
     bool go = true;
     for (int tile = pair; tile < tiles && go; tile += npairs) {
-      const FTile T = fused_tile<GT>(I, tile, sweep);
+      const FTile T = fused_tile<Cfg>(I, tile, sweep);
       if (!T.active) continue;
       const int buf = t % NBUF;
       const int N2 = 2 * I.Ns, gs = I.gs, n_first = T.nt * NB;
@@ -1180,8 +1206,8 @@ __global__ void __launch_bounds__(F_THREADS, 1)
         }
         if (E.qcur >= 0) E.flush(norm, sc, lane);
       };
-      if (r_is_zero(I, T.site, n_first, NB, lane)) body(FusedEpilogue<GT, true>{});
-      else body(FusedEpilogue<GT, false>{});
+      if (r_is_zero(I, T.site, n_first, NB, lane)) body(FusedEpilogue<Cfg, true>{});
+      else body(FusedEpilogue<Cfg, false>{});
       ++t;
       if (!go) break;
       tc_fence_before();
@@ -1278,38 +1304,44 @@ int pair_clusters(dyson_ctx* c, TcState* st) {
   return st->pair_clusters;
 }
 
-// co-resident CTA pairs of k_tc_fused<GT> on this device (0: it cannot run)
-template <int GT>
+// co-resident CTA pairs of k_tc_fused<GT, SPLIT> on this device (0: it cannot run)
+template <int GT, bool SPLIT>
 int fused_clusters_of(dyson_ctx* c) {
+  const auto kernel = k_tc_fused<GT, SPLIT>;
+  constexpr int smem = FusedCfg<GT, SPLIT>::SMEM;
   int sms = 0, n = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) sms = 0;
   // the warpgroups' register shares add up to exactly F_REGS_AT_LAUNCH per thread: with
   // any other count at launch the producers' increase could not be met, so the kernel is
   // not offered
   cudaFuncAttributes fa = {};
-  if (cudaFuncGetAttributes(&fa, k_tc_fused<GT>) != cudaSuccess || fa.numRegs != F_REGS_AT_LAUNCH) sms = 0;
-  if (sms >= 2 && cudaFuncSetAttribute(k_tc_fused<GT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       FusedCfg<GT>::SMEM) == cudaSuccess) {
+  if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess || fa.numRegs != F_REGS_AT_LAUNCH) sms = 0;
+  if (sms >= 2 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess) {
     cudaLaunchAttribute at[1];
-    cudaLaunchConfig_t cfg = pair_config(at, (unsigned)(sms / 2), F_THREADS, FusedCfg<GT>::SMEM, c->stream);
+    cudaLaunchConfig_t cfg = pair_config(at, (unsigned)(sms / 2), F_THREADS, smem, c->stream);
     int ncl = 0;
-    if (cudaOccupancyMaxActiveClusters(&ncl, k_tc_fused<GT>, &cfg) == cudaSuccess) n = ncl;
+    if (cudaOccupancyMaxActiveClusters(&ncl, kernel, &cfg) == cudaSuccess) n = ncl;
   }
   cudaGetLastError();
   return n;
 }
 
-// pairs for both forms of the fused kernel (0 where one of them cannot run)
+// pairs for every form of the fused kernel (0 where one of them cannot run)
 int fused_clusters(dyson_ctx* c) {
   TcState* st = state(c);
-  if (st->fused_clusters < 0) st->fused_clusters = std::min(fused_clusters_of<1>(c), fused_clusters_of<2>(c));
+  if (st->fused_clusters < 0)
+    st->fused_clusters = std::min({fused_clusters_of<1, false>(c), fused_clusters_of<2, false>(c),
+                                   fused_clusters_of<1, true>(c), fused_clusters_of<2, true>(c)});
   return st->fused_clusters;
 }
 
+// Several accumulators per output where the sweep takes the place of full FP32 products (k_tc_fused's comment).
+bool fused_split(const dyson_ctx* c) { return c->Nc % 64 != 0; }
 // Complex tiles wherever their 256 points are at least five eighths full: X is then gathered once per
-// (site, column tile) and Lambda read once.  Shorter contours (64, 128) would fill a half at most; their
+// (site, column tile) and Lambda read once.  Shorter contours would fill a half at most; up to 128 points their
 // embedding has a single tile of 256 rows.
-int fused_gt_of(const dyson_ctx* c) { return contour_stride(c) >= 192 ? 2 : 1; }
+// (SPLIT <2> has no room for two large accumulators: up to 191 points its residual is as large as the FP32 sweep's.)
+int fused_gt_of(const dyson_ctx* c) { return contour_stride(c) >= (fused_split(c) ? 256 : 192) ? 2 : 1; }
 
 // form of the fused kernel that serves the context's variant (0: none).  The unfused forms serve
 // only contours that fill their tiles; every other contour takes the fused kernel.
@@ -1401,19 +1433,19 @@ int tc_prepare(dyson_ctx* c, int ncol) {
   return DYSON_OK;
 }
 
-template <int GT>
+template <int GT, bool SPLIT>
 int launch_fused(dyson_ctx* c, const FusedInst& e, int sweep, const int* run, const int* sweeps_done,
                  cudaStream_t stream) {
   TcState* st = state(c);
-  const int NB = FusedCfg<GT>::NB;
+  const int NB = FusedCfg<GT, SPLIT>::NB;
   const long long tiles = (long long)e.Lx * e.Ly * ((e.ncol + NB - 1) / NB) * fused_row_tiles<GT>(e.Ns);
   cudaLaunchAttribute at[2];
   cudaLaunchConfig_t cfg = pair_config(at, (unsigned)std::min<long long>(tiles, fused_clusters(c)), F_THREADS,
-                                       FusedCfg<GT>::SMEM, stream);
+                                       FusedCfg<GT, SPLIT>::SMEM, stream);
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
   if (c->overlap) cfg.numAttrs = 2;
-  DY_CUDA(c, cudaLaunchKernelEx(&cfg, k_tc_fused<GT>, st->h_hi, st->h_lo, e, st->d_err, sweep, run, sweeps_done));
+  DY_CUDA(c, cudaLaunchKernelEx(&cfg, k_tc_fused<GT, SPLIT>, st->h_hi, st->h_lo, e, st->d_err, sweep, run, sweeps_done));
   DY_CUDA(c, cudaGetLastError());
   c->launches += 1;
   return DYSON_OK;
@@ -1475,8 +1507,9 @@ int tc_fused_sweep(dyson_ctx* c, int ncol, int gs, const float* r, const float* 
   e.Ns = contour_stride(c);
   e.ncol = ncol;
   e.gs = gs;
-  return fused_gt_of(c) == 1 ? launch_fused<1>(c, e, sweep, run, sweeps_done, stream)
-                             : launch_fused<2>(c, e, sweep, run, sweeps_done, stream);
+  const auto launch = fused_gt_of(c) == 1 ? (fused_split(c) ? launch_fused<1, true> : launch_fused<1, false>)
+                                          : (fused_split(c) ? launch_fused<2, true> : launch_fused<2, false>);
+  return launch(c, e, sweep, run, sweeps_done, stream);
 }
 
 int tc_sweep(dyson_ctx* c, int ncol, int gs, const float* r, const float* din, float* dout, int phases,
