@@ -43,15 +43,13 @@ struct BatchCheck {                 // what the check kernel reads per instance
 };
 
 struct BatchStop {                  // inner-series stopping state per instance
-  double best, peak, last;
+  SeriesState s;
   double target;                     // update at which this refinement's series stops
-  double hist[kStallSweeps];         // the last kStallSweeps updates (ring)
-  int since_best, sweeps, diverged, since_peak;
 };
 
-// Stopping rule of the inner series (the refinement's target, kStallDrop, kStallSweeps, kFlatRatio) per
-// active instance; clears the norm words for the next sweep and counts the
-// instances still active.  One block.
+// Stopping rule of the inner series (series_step) per active instance; clears the norm words for the next
+// sweep and counts the instances still active.  One block.  A transient above kSeriesPeakMax, which the FP32
+// series cannot carry, hands the instance to the GMRES of App. C after the batch.
 __global__ void k_batch_check(const BatchCheck* __restrict__ chk, int n, int* __restrict__ active,
                               BatchStop* __restrict__ st, int* __restrict__ n_active) {
   __shared__ int cnt;
@@ -70,39 +68,9 @@ __global__ void k_batch_check(const BatchCheck* __restrict__ chk, int n, int* __
       set_scale(C.xscale + q, __uint_as_float(C.xscale[q].ymax), C.jbound);
     }
     BatchStop S = st[k];
-    S.sweeps += 1;
-    S.last = upd;
-    bool stop = false;
-    if (bad || !(upd < kDivergedGrowth) || upd > kSeriesPeakMax) {
-      // not finite, or a transient the FP32 series cannot carry: hand the
-      // instance to the GMRES of App. C after the batch
-      S.diverged = 1;
-      stop = true;
-    } else {
-      if (upd > S.peak) {                              // the stall is judged on the decay after the peak
-        S.peak = upd;
-        S.best = upd;
-        S.since_best = 0;
-        S.since_peak = 0;
-      } else {
-        S.since_peak += 1;
-        if (upd < S.best) {
-          S.best = upd;
-          S.since_best = 0;
-        } else {
-          S.since_best += 1;
-        }
-      }
-      const double ago = S.hist[S.sweeps % kStallSweeps];
-      S.hist[S.sweeps % kStallSweeps] = upd;
-      stop = (upd <= S.target && (upd < S.peak || upd == 0.0)) ||
-             (S.since_best >= kStallSweeps && S.best < kStallDrop * S.peak) ||
-             (S.since_best >= kPlateauSweeps && S.best < kPlateauDrop * S.peak) ||
-             (S.since_peak >= kStallSweeps && upd < kStallDrop * S.peak && upd > kFlatRatio * ago) ||
-             S.sweeps >= C.max_sweeps;
-    }
+    series_step(S.s, bad ? __longlong_as_double(0x7ff0000000000000ll) : upd, C.max_sweeps, S.target, kSeriesPeakMax);
     st[k] = S;
-    if (stop) active[k] = 0;
+    if (!S.s.run) active[k] = 0;
     else atomicAdd(&cnt, 1);
   }
   __syncthreads();
@@ -118,6 +86,7 @@ struct Inst {
   std::vector<double> scale, rref;
   double prev_res = std::numeric_limits<double>::infinity();
   int strikes = 0;
+  bool plateau = true;               // the series may end on a plateau
   int status = DYSON_ERR_NOT_CONVERGED;
   bool done = false;
   int64_t launches0 = 0;
@@ -363,8 +332,7 @@ int dyson_batch_solve(dyson_batch* b, const int32_t* const* src, const int32_t* 
     for (int k = 0; k < n; ++k) {
       Inst& X = I[k];
       b->h_active[k] = X.done ? 0 : 1;
-      std::memset(&b->h_stop[k], 0, sizeof(BatchStop));
-      b->h_stop[k].best = std::numeric_limits<double>::infinity();
+      b->h_stop[k].s = series_start(X.plateau);
       b->h_stop[k].target = inner_target(kInnerTarget, tol, X.prev_res);
       if (X.done) continue;
       ++n_live;
@@ -408,11 +376,11 @@ int dyson_batch_solve(dyson_batch* b, const int32_t* const* src, const int32_t* 
       Inst& X = I[k];
       if (X.done) continue;
       dyson_ctx* c = X.c;
-      const BatchStop& St = b->h_stop[k];
+      const SeriesState& St = b->h_stop[k].s;
       X.rep.sweeps += St.sweeps;
       X.rep.update = St.last;
       X.rep.gemm_flops += St.sweeps * sweep_flops(c, X.ncol);
-      if (St.diverged) {
+      if (St.outcome == SERIES_ABORTED || St.outcome == SERIES_NOT_FINITE) {
         X.status = X.prev_res <= tol ? DYSON_OK : DYSON_ERR_DIVERGED;
         X.done = true;
         continue;
@@ -447,6 +415,7 @@ int dyson_batch_solve(dyson_batch* b, const int32_t* const* src, const int32_t* 
         X.status = DYSON_ERR_DIVERGED;
         X.done = true;
       }
+      if (b->h_stop[k].s.outcome == SERIES_PLATEAU && !plateau_served(res, X.prev_res)) X.plateau = false;
       X.prev_res = res;
     }
   }

@@ -226,20 +226,9 @@ int solve_f64(dyson_ctx* c, int ncol, int gs, double tol, int max_sweeps, double
   return status;
 }
 
-// Stopping state of the inner series, the same fields the host loop of inner_solve keeps;
-// on the device for sweeps enqueued in batches.
-struct SeriesState {
-  double best, peak, last;
-  double hist[kStallSweeps];           // the last kStallSweeps updates (ring)
-  int since_best, since_peak, sweeps;
-  int run;                             // 1 while the series goes on (read by the fused sweep)
-  int outcome;
-};
-enum { SERIES_RUNNING = 0, SERIES_STOPPED, SERIES_EXHAUSTED, SERIES_ABORTED, SERIES_NOT_FINITE };
-
 // After one sweep of a batch: the update max_q norm_q / rref_q (norm words
-// cleared for the next sweep), the next sweep's FP16 scales, and the stopping rule of
-// inner_solve's host loop, in the same order.  One warp; returns at once once the series has stopped.
+// cleared for the next sweep), the next sweep's FP16 scales, and the stopping rule (series_step).
+// One warp; returns at once once the series has stopped.
 __global__ void k_series_check(unsigned long long* __restrict__ norm, const double* __restrict__ rref, int ng,
                                int max_sweeps, double target, double abort_peak, SeriesState* __restrict__ S,
                                TcScale* __restrict__ xscale, float jbound) {
@@ -260,43 +249,7 @@ __global__ void k_series_check(unsigned long long* __restrict__ norm, const doub
     bad |= __shfl_xor_sync(0xffffffffu, bad, o);
   }
   if (threadIdx.x != 0) return;
-  const double upd = bad ? __longlong_as_double(0x7ff0000000000000ll) : m;
-  const int sweep = ++S->sweeps;
-  S->last = upd;
-  if (!(upd < kDivergedGrowth)) {
-    S->outcome = SERIES_NOT_FINITE;
-    S->run = 0;
-    return;
-  }
-  if (upd > S->peak) {
-    S->peak = upd;
-    S->best = upd;
-    S->since_best = 0;
-    S->since_peak = 0;
-  } else {
-    ++S->since_peak;
-    if (upd < S->best) {
-      S->best = upd;
-      S->since_best = 0;
-    } else {
-      ++S->since_best;
-    }
-  }
-  const double ago = S->hist[sweep % kStallSweeps];
-  S->hist[sweep % kStallSweeps] = upd;
-  int out = SERIES_RUNNING;
-  if (S->peak > abort_peak) out = SERIES_ABORTED;
-  else if ((upd <= target && (upd < S->peak || upd == 0.0)) ||
-           (S->since_best >= kStallSweeps && S->best < kStallDrop * S->peak) ||
-           (S->since_best >= kPlateauSweeps && S->best < kPlateauDrop * S->peak) ||
-           (S->since_peak >= kStallSweeps && upd < kStallDrop * S->peak && upd > kFlatRatio * ago))
-    out = SERIES_STOPPED;
-  else if (sweep >= max_sweeps)
-    out = SERIES_EXHAUSTED;
-  if (out != SERIES_RUNNING) {
-    S->outcome = out;
-    S->run = 0;
-  }
+  series_step(*S, bad ? __longlong_as_double(0x7ff0000000000000ll) : m, max_sweeps, target, abort_peak);
 }
 
 // kind that the fused sweep is timed as: its own where the context selected it, the general
@@ -335,10 +288,8 @@ int tc_timed_sweep(dyson_ctx* c, int ncol, int gs, const float* r, const float* 
 // instantiation every inner solve paid for: 8x8, Nc = 128, 6.58 ms a solve, 9x7, Nc = 100, 4.46; so 6.52 and
 // 4.33 (enqueued without the overlap 6.88 and 4.56).
 int inner_solve(dyson_ctx* c, int ncol, int gs, int precision, float* r32, float* da, float* db, int max_sweeps,
-                const std::vector<double>& rref, float** dres, dyson_report* rep, double* peak_out,
-                double abort_peak = std::numeric_limits<double>::infinity(), const int* act = nullptr,
-                bool* exhausted = nullptr, double target = kInnerTarget, bool r_on_sources = false) {
-  if (exhausted) *exhausted = false;
+                const std::vector<double>& rref, float** dres, dyson_report* rep, double abort_peak, const int* act,
+                int* outcome, double target, bool r_on_sources, bool plateau) {
   const int ng = ncol / gs;
   const size_t n32 = (size_t)c->Nr * ncol * 2 * c->Ns;
   DY_CUDA(c, cudaMemcpyAsync(da, r32, n32 * sizeof(float), cudaMemcpyDeviceToDevice, c->stream));
@@ -350,9 +301,7 @@ int inner_solve(dyson_ctx* c, int ncol, int gs, int precision, float* r32, float
                      tc_uses_fused(c) && cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess &&
                      cap == cudaStreamCaptureStatusNone;
   const int eager_until = batches ? 0 : max_sweeps;
-  SeriesState S = {};
-  S.best = std::numeric_limits<double>::infinity();
-  S.run = 1;
+  SeriesState S = series_start(plateau);
   int rc;
   if (precision == DYSON_PREC_TF32X3_F64REF && c->use_tc && tc_uses_fused(c)) {
     // the series starts from d = r: its scales come from the reference norms max|r|
@@ -378,44 +327,10 @@ int inner_solve(dyson_ctx* c, int ncol, int gs, int precision, float* r32, float
     if (c->use_tc && (rc = tc_error_status(c))) return rc;
     std::swap(da, db);
     const double upd = rel_max(c->h_norm, rref.data(), ng);
-    S.sweeps = sweep;
-    S.last = upd;
     rep->sweeps += 1;
     rep->gemm_flops += sweep_flops(c, ncol);
     rep->update = upd;
-    if (!(upd < kDivergedGrowth)) return ctx_fail(c, DYSON_ERR_DIVERGED, "FP32 series update not finite");
-    // stopping rule of the inner series (detail.cuh); the stall is judged only on
-    // the decay after the latest peak (k_series_check applies the same, in this order)
-    if (upd > S.peak) {
-      S.peak = upd;
-      S.best = upd;
-      S.since_best = 0;
-      S.since_peak = 0;
-    } else {
-      ++S.since_peak;
-      if (upd < S.best) {
-        S.best = upd;
-        S.since_best = 0;
-      } else {
-        ++S.since_best;
-      }
-    }
-    const double ago = S.hist[sweep % kStallSweeps];     // the update kStallSweeps sweeps ago
-    S.hist[sweep % kStallSweeps] = upd;
-    if (S.peak > abort_peak) {
-      if (peak_out) *peak_out = S.peak;
-      return DYSON_ERR_DIVERGED;                           // the caller switches to GMRES
-    }
-    if ((upd <= target && (upd < S.peak || upd == 0.0)) ||  // on the decay, not before the peak
-        (S.since_best >= kStallSweeps && S.best < kStallDrop * S.peak) ||
-        (S.since_best >= kPlateauSweeps && S.best < kPlateauDrop * S.peak) ||
-        (S.since_peak >= kStallSweeps && upd < kStallDrop * S.peak && upd > kFlatRatio * ago)) {
-      S.run = 0;
-      S.outcome = SERIES_STOPPED;
-    } else if (sweep == max_sweeps) {
-      S.run = 0;
-      S.outcome = SERIES_EXHAUSTED;
-    }
+    series_step(S, upd, max_sweeps, target, abort_peak);
   }
   if (S.run && batches) {
     // batches of S_g sweeps (even, so that every batch starts from da), each followed by its check
@@ -489,15 +404,11 @@ int inner_solve(dyson_ctx* c, int ncol, int gs, int precision, float* r32, float
     if (e1) cudaEventDestroy(e1);
     if (rc) return rc;
     S = *hS;
-    if (S.outcome == SERIES_NOT_FINITE) return ctx_fail(c, DYSON_ERR_DIVERGED, "FP32 series update not finite");
-    if (S.outcome == SERIES_ABORTED) {
-      if (peak_out) *peak_out = S.peak;
-      return DYSON_ERR_DIVERGED;
-    }
   }
-  if (S.outcome == SERIES_EXHAUSTED && exhausted) *exhausted = true;
+  if (outcome) *outcome = S.outcome;
+  if (S.outcome == SERIES_NOT_FINITE) return ctx_fail(c, DYSON_ERR_DIVERGED, "FP32 series update not finite");
+  if (S.outcome == SERIES_ABORTED) return DYSON_ERR_DIVERGED;   // the caller switches to GMRES
   *dres = da;
-  if (peak_out) *peak_out = S.peak;
   return DYSON_OK;
 }
 
@@ -595,28 +506,28 @@ int solve_mixed(dyson_ctx* c, int ncol, int gs, int precision, double tol, int m
   // inner solver: the series of App. C, or its GMRES.  AUTO starts with the series
   // and switches to GMRES for the rest of the chunk when the series cannot serve:
   // it diverges, its transient peak times the FP32 rounding leaves no correct
-  // digit, it uses its whole sweep budget, or the refined residual grows.
-  bool gmres = c->inner_solver == DYSON_INNER_GMRES;
+  // digit, it uses its whole sweep budget, it ends on a plateau without gaining a digit, or the refined
+  // residual grows.
+  bool gmres = c->inner_solver == DYSON_INNER_GMRES, plateau = true;
   const bool may_switch = c->inner_solver == DYSON_INNER_AUTO;
   const MatvecFn mv = [&](const float* zero, const float* in, float* out, double bound) {
     return matvec_f32(c, ncol, gs, precision, zero, in, out, bound);
   };
   for (int ref = 0; ref < c->max_refinements; ++ref) {
     float* d = nullptr;
+    int outcome = SERIES_RUNNING;
     if (gmres) {
       rc = gmres_inner_solve(c, ncol, r32, da, max_sweeps, inner_target(kGmresTarget, tol, prev_res), rep, mv);
       d = da;
       rep->inner_gmres = 1;
     } else {
-      double peak = 0.0;
       // the first right-hand side lives on the source sites: truncate its sweeps
       const int* act = ref == 0 && c->support_trunc && c->use_tc && precision == DYSON_PREC_TF32X3_F64REF
                            ? support_table(c, ncol)
                            : nullptr;
-      bool exhausted = false;
-      rc = inner_solve(c, ncol, gs, precision, r32, da, db, max_sweeps, rref, &d, rep, &peak,
-                       may_switch ? kSeriesPeakMax : std::numeric_limits<double>::infinity(), act, &exhausted,
-                       inner_target(kInnerTarget, tol, prev_res), ref == 0);
+      rc = inner_solve(c, ncol, gs, precision, r32, da, db, max_sweeps, rref, &d, rep,
+                       may_switch ? kSeriesPeakMax : std::numeric_limits<double>::infinity(), act, &outcome,
+                       inner_target(kInnerTarget, tol, prev_res), ref == 0, plateau);
       if (rc == DYSON_ERR_DIVERGED && may_switch && !(prev_res <= tol)) {
         gmres = true;                                    // redo this refinement with GMRES
         --ref;
@@ -624,7 +535,7 @@ int solve_mixed(dyson_ctx* c, int ncol, int gs, int precision, double tol, int m
       }
       // a series that used its whole sweep budget converges too slowly (spectral radius
       // near 1): its correction is kept, the following refinements use GMRES
-      if (rc == DYSON_OK && exhausted && may_switch) gmres = true;
+      if (rc == DYSON_OK && outcome == SERIES_EXHAUSTED && may_switch) gmres = true;
     }
     if (rc == DYSON_ERR_DIVERGED) {
       status = prev_res <= tol ? DYSON_OK : rc;            // (the refinement beyond the tolerance adds nothing)
@@ -652,6 +563,10 @@ int solve_mixed(dyson_ctx* c, int ncol, int gs, int precision, double tol, int m
                         refine_once_more(res, tol, prev_res, c->Nc, ref + 1 == c->max_refinements))) {
       status = DYSON_OK;
       break;
+    }
+    if (outcome == SERIES_PLATEAU && !plateau_served(res, prev_res)) {
+      plateau = false;
+      if (may_switch) gmres = true;
     }
     if (res > tol && res > kRefineContract * prev_res) {
       if (may_switch && !gmres) {

@@ -3,6 +3,7 @@
 #include <string>
 
 #include "common.cuh"
+#include "series.cuh"
 
 namespace dyson_detail {
 
@@ -18,19 +19,13 @@ struct DeviceGuard {
   }
 };
 
-// a relative update above this (or not finite) counts as divergence
-constexpr double kDivergedGrowth = 1e200;
 // An FP64 series whose relative update passes 2^52 has partial sums whose
 // rounding alone exceeds the result: it cannot converge to anything, and a
 // transient of the real-time series never comes near (about 2e7 on the longest
 // contours).  The FP64 series stops there with DYSON_ERR_DIVERGED.
 constexpr double kDivergedF64 = 4503599627370496.0;
 
-// Stopping rule of the FP32 inner series.  Its update first grows (the transient
-// of the real-time series), falls factorially after its peak, then settles at
-// the FP32 rounding level of the partial sums: stop at kInnerTarget, or once it
-// sits kStallDrop below its peak and has not improved for kStallSweeps sweeps
-// (improvement counted from the latest peak, never during the growth).
+// Relative update at which an FP32 inner series stops (series.cuh has the other rules).
 constexpr double kInnerTarget = 4e-7;
 // A refinement only has to take the residual from its previous value r_prev to the
 // tolerance: its inner solve stops at an update of kInnerSlack * tol / r_prev (at
@@ -59,21 +54,6 @@ inline bool refine_once_more(double res, double tol, double prev_res, int Nc, bo
   const double share = Nc % 64 ? kAcceptShareOdd : kAcceptShare;
   return res <= tol && tol >= kLooseTol && res > share * tol && prev_res > tol && !last;
 }
-constexpr double kStallDrop = 1e-4;
-constexpr int kStallSweeps = 4;
-// The same floor seen earlier: on its FP32 floor the update fluctuates, so new minima
-// keep resetting the count above, while the decay itself has stopped.  The series also
-// stops once the update, kStallDrop below its peak, fell by less than a factor
-// kFlatRatio over the last kStallSweeps sweeps (the decay after the peak is factorial:
-// a factor 3 to 10 over four sweeps until the floor).
-constexpr double kFlatRatio = 0.8;
-// Where the transient amplifies the rounding, the floor can lie above kStallDrop of the peak,
-// and both rules above would let the series run through its whole budget on it.  It also stops
-// after kPlateauSweeps sweeps without a new minimum once it has come below kPlateauDrop of the
-// peak: a series that still converges, however slowly, keeps making new minima.
-constexpr int kPlateauSweeps = 10;
-constexpr double kPlateauDrop = 1e-2;
-
 // Refinement that grows the residual: a residual above kRefineContract times the
 // previous one, kRefineStrikes times, means the series of App. C does not
 // converge for this problem (spectral radius of K above 1); the solve ends with
