@@ -226,8 +226,7 @@ int dyson_batch_solve(dyson_batch* b, const int32_t* const* src, const int32_t* 
     size_t col_bytes = 0;
     if (chunk_columns(c, DYSON_PREC_TF32X3_F64REF, c->Nc, X.ncol, &col_bytes) < X.ncol)
       return bfail(b, DYSON_ERR_OOM, "instance " + std::to_string(k) + ": its block columns do not fit at once");
-    if ((rc = ensure_work(c, (size_t)X.ncol * col_bytes)) || (rc = ensure_cols(c, X.ncol, X.ng)))
-      return bfail(b, rc, c->err);
+    if ((rc = reserve_chunk(c, X.ncol, c->Nc, col_bytes, true))) return bfail(b, rc, c->err);
     c->h_src_site.resize(X.ncol);
     c->h_src_time.resize(X.ncol);
     for (int q = 0; q < X.nq; ++q)
@@ -428,7 +427,7 @@ int dyson_batch_solve(dyson_batch* b, const int32_t* const* src, const int32_t* 
     const int saved = c->inner_solver;
     c->inner_solver = DYSON_INNER_GMRES;
     double2* G = nullptr;
-    if ((rc = prepare_tables(c, DYSON_PREC_TF32X3_F64REF, tol))) return bfail(b, rc, c->err);
+    if ((rc = prepare_tables(c, DYSON_PREC_TF32X3_F64REF, tol, 0, false, true))) return bfail(b, rc, c->err);
     rc = solve_mixed(c, X.ncol, c->Nc, DYSON_PREC_TF32X3_F64REF, tol, max_sweeps, &G, &X.rep);
     c->inner_solver = saved;
     if (rc != DYSON_OK && rc != DYSON_ERR_NOT_CONVERGED && rc != DYSON_ERR_DIVERGED) return bfail(b, rc, c->err);

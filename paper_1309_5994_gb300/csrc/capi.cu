@@ -720,10 +720,35 @@ int dyson_copy_sigma(dyson_ctx* c, double* dst, int on_device) {
 
 namespace dyson_detail {
 
+// Scratch that a solve sizes for itself and leaves with the context.  What one precision holds is free memory to
+// another (release_scratch), so that a solve gets the same chunks whatever ran before it.
+size_t scratch_bytes(const dyson_ctx* c) {
+  return c->work_bytes + oz_x_bytes(c) + oz64_x_bytes(c) + tc_x_bytes(c) + gmres_bytes(c);
+}
+
+void release_scratch(dyson_ctx* c) {
+  cudaFree(c->work);
+  c->work = nullptr;
+  c->work_bytes = 0;
+  oz_release_x(c);
+  oz64_release_x(c);
+  tc_release_x(c);
+  gmres_release(c);
+}
+
+// share of the free memory that cudaMalloc is taken to deliver in a few blocks
+constexpr double kFreeShare = 0.95;
+
 // FP64 sweeps and residuals on the tensor cores where the slices of Lambda fit (sets c->use_oz64);
-// the FP64-pipe kernel otherwise
-int prepare_oz64(dyson_ctx* c) {
-  c->use_oz64 = oz64_usable(c);
+// the FP64-pipe kernel otherwise.  hold: the scratch is in use and stays.
+int prepare_oz64(dyson_ctx* c, bool hold) {
+  size_t more = 0, free_b = 0, total_b = 0;
+  c->use_oz64 = oz64_usable(c, &more);
+  if (!c->use_oz64) return DYSON_OK;
+  if (more > 0 && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && more > kFreeShare * free_b) {
+    if (hold) c->use_oz64 = false;
+    else release_scratch(c);
+  }
   if (!c->use_oz64) return DYSON_OK;
   const int rc = oz64_prepare(c);
   if (rc == DYSON_ERR_OOM) c->use_oz64 = false;
@@ -734,7 +759,7 @@ int prepare_oz64(dyson_ctx* c) {
 // and residual kernels (sets c->use_tc, c->use_oz, c->use_oz64).
 // The residual of a mixed solve: five slices (15 products) for tolerances down to 1e-8, where they run at
 // 85 TFLOP/s of the contraction (16x16, Nc = 256, 4096 columns: 6.5 ms); eight (36 products, 53 TFLOP/s) below.
-int prepare_tables(dyson_ctx* c, int precision, double tol, int64_t columns, bool batch) {
+int prepare_tables(dyson_ctx* c, int precision, double tol, int64_t columns, bool batch, bool hold) {
   // A fused tile of 256 rows is half empty at 64 contour points (128 rows of the embedding), so from
   // kManySiteColumns on the unfused form is the faster one although its series waits for every sweep:
   // single CTA / fused, us a sweep: 8x8 sites, 512 columns 34 / 46, 1024 57 / 83; 12x12, 512 62 / 85;
@@ -743,7 +768,7 @@ int prepare_tables(dyson_ctx* c, int precision, double tol, int64_t columns, boo
   c->many_of_64 = c->Nc == 64 && c->Nr * columns >= kManySiteColumns;
   c->use_tc = c->use_oz = c->use_oz64 = false;
   c->Ns = c->Nc;
-  if (precision == DYSON_PREC_F64) return prepare_oz64(c);
+  if (precision == DYSON_PREC_F64) return prepare_oz64(c, hold);
   const bool tc = c->tc_enabled && tc_supported(c);
   const bool fused = tc && (batch || tc_uses_fused(c));
   if (tc) c->Ns = contour_stride(c);
@@ -773,7 +798,7 @@ int prepare_tables(dyson_ctx* c, int precision, double tol, int64_t columns, boo
   }
   c->use_tc = tc;
   c->use_oz = tc && tol >= kOzTol && c->oz_enabled && oz_supported(c);
-  return c->use_oz ? DYSON_OK : prepare_oz64(c);
+  return c->use_oz ? DYSON_OK : prepare_oz64(c, hold);
 }
 
 // r32 = B + K G - G with the residual kernel that prepare_tables picked; c->d_norm[q] = max |r|
@@ -795,26 +820,49 @@ int enqueue_residual(dyson_ctx* c, int ncol, int gs, const double2* G, float* r3
 }
 
 // Largest number of vector columns, a multiple of `unit` and at most `want`, whose
-// work state fits in 85 % of the free device memory.  F64: two complex128 states;
-// mixed: complex128 G + three FP32 states (*bytes_per_col: these, the work buffer); besides it
+// work state fits in 85 % of the device memory that is free or scratch of the context.  F64: two complex128
+// states; mixed: complex128 G + three FP32 states (*bytes_per_col: these, the work buffer); besides it
 // the FP32 gather buffer of the tensor-core sweep and the BF16 slices of the split-product
-// residual or FP64 sweep (*total_per_col: all).
+// residual or FP64 sweep (*total_per_col: all).  Frees the scratch where the buffers for these columns would not
+// fit beside what it holds.
 int64_t chunk_columns(dyson_ctx* c, int precision, int64_t unit, int64_t want, size_t* bytes_per_col,
                       size_t* total_per_col) {
-  const double state = precision == DYSON_PREC_F64 ? 32.0 : 16.0 + 24.0 * c->Ns / c->Nc;
-  const double per_el = state + (c->use_tc && !tc_uses_fused(c) ? 8.0 : 0.0) + (c->use_oz ? (double)oz_bytes_per_element() : 0.0) +
-                        (c->use_oz64 ? oz64_bytes_per_element(c) : 0.0);
-  const double col_bytes = per_el * c->Nr * (double)c->Nc;
-  *bytes_per_col = (size_t)std::ceil(state * c->Nr * (double)c->Nc);
+  const double col_el = c->Nr * (double)c->Nc;
+  const struct { double per_col; size_t held; } buf[4] = {
+      {col_el * (precision == DYSON_PREC_F64 ? 32.0 : 16.0 + 24.0 * c->Ns / c->Nc), c->work_bytes},
+      {col_el * (c->use_tc && !tc_uses_fused(c) ? 8.0 : 0.0), tc_x_bytes(c)},
+      {col_el * (c->use_oz ? (double)oz_bytes_per_element() : 0.0), oz_x_bytes(c)},
+      {col_el * (c->use_oz64 ? oz64_bytes_per_element(c) : 0.0), oz64_x_bytes(c)}};
+  double col_bytes = 0.0;
+  for (const auto& b : buf) col_bytes += b.per_col;
+  *bytes_per_col = (size_t)std::ceil(buf[0].per_col);
   if (total_per_col) *total_per_col = (size_t)col_bytes;
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return 0;
-  const double budget = 0.85 * (double)(free_b + c->work_bytes);
+  const double budget = 0.85 * (double)(free_b + scratch_bytes(c));
   int64_t cols = (int64_t)(budget / col_bytes);
   if (c->chunk_override > 0) cols = std::min<int64_t>(cols, (int64_t)c->chunk_override * unit);
   cols = std::min<int64_t>(cols, want);
   cols = std::min<int64_t>(cols, (int64_t)1 << 24);
-  return (cols / unit) * unit;
+  cols = (cols / unit) * unit;
+  double more = 0.0;                                       // (a buffer that grows is freed first)
+  for (const auto& b : buf) more += std::max(0.0, cols * b.per_col - (double)b.held);
+  if (more > kFreeShare * free_b) release_scratch(c);
+  return cols;
+}
+
+// Buffers of a chunk of ncol columns in groups of gs: work state, sources and norms, and what the sweeps and the
+// residual need besides, ahead of the GMRES basis, which takes most of what is left.  Where the residual's or the
+// FP64 sweep's slices cannot be had, the FP64-pipe kernel runs.
+int reserve_chunk(dyson_ctx* c, int ncol, int gs, size_t bytes_per_col, bool batch) {
+  int rc;
+  if ((rc = ensure_work(c, (size_t)ncol * bytes_per_col)) || (rc = ensure_cols(c, ncol, ncol / gs))) return rc;
+  if (c->use_tc && (rc = tc_prepare_sweep(c, ncol, batch))) return rc;
+  if (c->use_oz && (rc = oz_reserve(c, ncol)) == DYSON_ERR_OOM) c->use_oz = false;
+  else if (c->use_oz && rc) return rc;
+  if (c->use_oz64 && (rc = oz64_reserve(c, ncol)) == DYSON_ERR_OOM) c->use_oz64 = false;
+  else if (c->use_oz64 && rc) return rc;
+  return DYSON_OK;
 }
 
 int solve_chunk(dyson_ctx* c, int ncol, int gs, int precision, double tol, int max_sweeps, double2** G,
@@ -882,8 +930,7 @@ int solve_columns_impl(dyson_ctx* c, const int32_t* src, int64_t n_src, int prec
   const int64_t cols = chunk_columns(c, precision, c->Nc, n_src * (int64_t)c->Nc, &col_bytes);
   if (cols < c->Nc) return R.finish(ctx_fail(c, DYSON_ERR_OOM, "one block column does not fit in device memory"));
   const int64_t chunk = cols / c->Nc;
-  if ((rc = ensure_work(c, (size_t)cols * col_bytes))) return R.finish(rc);
-  if ((rc = ensure_cols(c, (int)cols, (int)chunk))) return R.finish(rc);
+  if ((rc = reserve_chunk(c, (int)cols, c->Nc, col_bytes))) return R.finish(rc);
 
   int status = DYSON_OK;
   for (int64_t start = 0; start < n_src; start += chunk) {
@@ -958,8 +1005,7 @@ int dyson_solve_vector_columns(dyson_ctx* c, const int32_t* sites, const int32_t
   size_t col_bytes = 0;
   const int64_t chunk = chunk_columns(c, precision, GS, padded, &col_bytes);
   if (chunk < GS) return R.finish(ctx_fail(c, DYSON_ERR_OOM, "32 vector columns do not fit in device memory"));
-  if ((rc = ensure_work(c, (size_t)chunk * col_bytes))) return R.finish(rc);
-  if ((rc = ensure_cols(c, (int)chunk, (int)(chunk / GS)))) return R.finish(rc);
+  if ((rc = reserve_chunk(c, (int)chunk, GS, col_bytes))) return R.finish(rc);
   int status = DYSON_OK;
   for (int64_t start = 0; start < padded; start += chunk) {
     const int ncol = (int)std::min<int64_t>(chunk, padded - start);

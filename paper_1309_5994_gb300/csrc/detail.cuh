@@ -101,8 +101,12 @@ double rel_max(const unsigned long long* norm, const double* ref, int ng);
 double sweep_flops(const dyson_ctx* c, int ncol);         // algorithmic contour-GEMM flops of one sweep
 // reduced-precision copies of Lambda that the context's sweep variant needs (batch: those of the
 // fused sweep, whatever the variant); sets c->use_tc, c->use_oz, c->use_oz64 and c->Ns
-// columns: vector columns that the solve works on at once (0: not a solve of its own)
-int prepare_tables(dyson_ctx* c, int precision, double tol, int64_t columns = 0, bool batch = false);
+// columns: vector columns that the solve works on at once (0: not a solve of its own).  May free the scratch,
+// unless held.
+int prepare_tables(dyson_ctx* c, int precision, double tol, int64_t columns = 0, bool batch = false, bool hold = false);
+size_t scratch_bytes(const dyson_ctx* c);                 // held by the buffers that each solve sizes for itself
+void release_scratch(dyson_ctx* c);
+int reserve_chunk(dyson_ctx* c, int ncol, int gs, size_t bytes_per_col, bool batch = false);
 int enqueue_residual(dyson_ctx* c, int ncol, int gs, const double2* G, float* r32);
 // mixed-precision solve of the chunk whose sources are on the device (G in c->work)
 int solve_mixed(dyson_ctx* c, int ncol, int gs, int precision, double tol, int max_sweeps, double2** result,

@@ -8,6 +8,8 @@
 // right-hand side); bound: an upper bound of |in|, or 0 for none known; returns a DYSON_ERR_* code
 using MatvecFn = std::function<int(const float* zero, const float* in, float* out, double bound)>;
 
+// Bytes held by the Krylov basis.
+size_t gmres_bytes(const dyson_ctx* c);
 // Restart length that fits the free device memory for ncol columns (0: none fits).
 int gmres_restart_length(dyson_ctx* c, int ncol);
 // Solve (I - K) x = r per vector column of the chunk by restarted GMRES, starting

@@ -487,13 +487,16 @@ int gm_prepare(dyson_ctx* c, size_t vsz, int ncol, int m) {
 
 }  // namespace
 
+size_t gmres_bytes(const dyson_ctx* c) {
+  const GmState* st = static_cast<const GmState*>(c->gm);
+  return st ? (size_t)(st->m + 4) * st->vsz * sizeof(float) : 0;
+}
+
 int gmres_restart_length(dyson_ctx* c, int ncol) {
   const size_t vbytes = (size_t)c->Nr * ncol * 2 * c->Ns * sizeof(float);
-  GmState* st = static_cast<GmState*>(c->gm);
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return 0;
-  const size_t held = st ? (size_t)(st->m + 4) * st->vsz * sizeof(float) : 0;
-  const double budget = 0.8 * (double)(free_b + held);
+  const double budget = 0.8 * (double)(free_b + gmres_bytes(c));
   const int fit = (int)(budget / (double)vbytes) - 4;
   return std::max(0, std::min(c->gmres_restart > 0 ? c->gmres_restart : 40, std::min(fit, 60)));
 }

@@ -548,6 +548,29 @@ void oz_invalidate(dyson_ctx* c) {
   if (c->oz) static_cast<OzState*>(c->oz)->a_ready = false;
 }
 
+int oz_reserve(dyson_ctx* c, int ncol) {
+  OzState* st = state(c);
+  int rc;
+  if ((rc = grow(c, &st->xslices, &st->x_bytes, (size_t)S * c->Nr * ncol * 2 * c->Nc * 2, "Ozaki slices of X"))) return rc;
+  return grow(c, &st->tau, &st->tau_bytes, (size_t)c->Nr * ncol * sizeof(double), "Ozaki column scales");
+}
+
+size_t oz_x_bytes(const dyson_ctx* c) {
+  const OzState* st = static_cast<const OzState*>(c->oz);
+  return st ? st->x_bytes + st->tau_bytes : 0;
+}
+
+void oz_release_x(dyson_ctx* c) {
+  OzState* st = static_cast<OzState*>(c->oz);
+  if (!st) return;
+  cudaFree(st->xslices);
+  cudaFree(st->tau);
+  st->xslices = nullptr;
+  st->tau = nullptr;
+  st->x_bytes = st->tau_bytes = 0;
+  st->xmap_ptr = nullptr;
+}
+
 int oz_residual(dyson_ctx* c, int ncol, int gs, const double2* G, float* r32) {
   OzState* st = state(c);
   const int Nr = c->Nr, Nc = c->Nc, N2 = 2 * Nc;
@@ -570,9 +593,7 @@ int oz_residual(dyson_ctx* c, int ncol, int gs, const double2* G, float* r32) {
       return ctx_fail(c, DYSON_ERR_CUDA, "cuTensorMapEncodeTiled failed for the Lambda slices");
     st->a_ready = true;
   }
-  size_t xbytes = (size_t)S * Nr * ncol * N2 * 2;
-  if ((rc = grow(c, &st->xslices, &st->x_bytes, xbytes, "Ozaki slices of X"))) return rc;
-  if ((rc = grow(c, &st->tau, &st->tau_bytes, (size_t)Nr * ncol * sizeof(double), "Ozaki column scales"))) return rc;
+  if ((rc = oz_reserve(c, ncol))) return rc;
   if (st->xmap_ptr != st->xslices || st->xmap_ncol != ncol) {
     if (!make_map4(&st->xmap, st->xslices, N2, ncol, Nr, S, BN))
       return ctx_fail(c, DYSON_ERR_CUDA, "cuTensorMapEncodeTiled failed for the X slices");

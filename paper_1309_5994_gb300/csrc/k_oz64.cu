@@ -28,6 +28,7 @@
 #include <cuda_bf16.h>
 
 #include "common.cuh"
+#include "detail.cuh"
 #include "oz64.cuh"
 #include "ptx.cuh"
 
@@ -76,7 +77,7 @@ struct SliceRow {
 struct Oz64State {
   __nv_bfloat16* as = nullptr;        // tiles of the 2 Nc rows of every site (SliceRow)
   int* esig = nullptr;                // [Nr][2Nc] row scale exponents
-  size_t a_bytes = 0;
+  size_t a_bytes = 0, sig_bytes = 0;
   bool a_ready = false;
   __nv_bfloat16* xs = nullptr;        // tiles of the ncol columns of every site
   int* etau = nullptr;                // [Nr][ncol] column scale exponents
@@ -689,13 +690,37 @@ void launch_xprep(dyson_ctx* c, int ncol, const double2* G, Oz64State* st, const
 
 }  // namespace
 
-bool oz64_usable(dyson_ctx* c) {
+bool oz64_usable(dyson_ctx* c, size_t* more) {
+  *more = 0;
   if (!c->oz64_enabled) return false;
   Oz64State* st = static_cast<Oz64State*>(c->oz64);
   if (st && st->a_bytes >= a_slice_bytes(c)) return true;
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;
-  return a_slice_bytes(c) <= (free_b + c->work_bytes) / 3;
+  *more = a_slice_bytes(c);
+  return a_slice_bytes(c) <= (free_b + dyson_detail::scratch_bytes(c)) / 3;
+}
+
+int oz64_reserve(dyson_ctx* c, int ncol) {
+  Oz64State* st = state(c);
+  int rc;
+  if ((rc = grow(c, &st->xs, &st->x_bytes, (size_t)S * c->Nr * ncol * k_pad(c->Nc) * 2, "FP64 slices of X"))) return rc;
+  return grow(c, &st->etau, &st->tau_bytes, (size_t)c->Nr * ncol * sizeof(int), "FP64 column scales");
+}
+
+size_t oz64_x_bytes(const dyson_ctx* c) {
+  const Oz64State* st = static_cast<const Oz64State*>(c->oz64);
+  return st ? st->x_bytes + st->tau_bytes : 0;
+}
+
+void oz64_release_x(dyson_ctx* c) {
+  Oz64State* st = static_cast<Oz64State*>(c->oz64);
+  if (!st) return;
+  cudaFree(st->xs);
+  cudaFree(st->etau);
+  st->xs = nullptr;
+  st->etau = nullptr;
+  st->x_bytes = st->tau_bytes = 0;
 }
 
 double oz64_bytes_per_element(const dyson_ctx* c) {
@@ -731,7 +756,7 @@ int oz64_prepare(dyson_ctx* c) {
   if (rc) return rc;
   if (!st->a_ready) {
     if ((rc = grow(c, &st->as, &st->a_bytes, a_slice_bytes(c), "FP64 slices of Lambda"))) return rc;
-    if (!st->esig) DY_CUDA(c, cudaMalloc(&st->esig, (size_t)Nr * N2 * sizeof(int)));
+    if ((rc = grow(c, &st->esig, &st->sig_bytes, (size_t)Nr * N2 * sizeof(int), "FP64 row scales"))) return rc;
     const size_t rows = (size_t)Nr * Nc;
     k_oz64_aprep<<<(unsigned)((rows + 7) / 8), 256, 0, c->stream>>>(c->d_lam, uniform_hopping(c), Nr, c->Nt, c->Nm,
                                                                    c->dt, c->beta, Kp, st->as, st->esig);
@@ -748,8 +773,7 @@ int oz64_sweep(dyson_ctx* c, int ncol, int gs, const double2* Gin, double2* out,
   if (rc) return rc;
   Oz64State* st = state(c);
   const int Nr = c->Nr, Nc = c->Nc, N2 = 2 * Nc, Kp = k_pad(Nc);
-  if ((rc = grow(c, &st->xs, &st->x_bytes, (size_t)S * Nr * ncol * Kp * 2, "FP64 slices of X"))) return rc;
-  if ((rc = grow(c, &st->etau, &st->tau_bytes, (size_t)Nr * ncol * sizeof(int), "FP64 column scales"))) return rc;
+  if ((rc = oz64_reserve(c, ncol))) return rc;
   if (uniform_hopping(c)) launch_xprep<true>(c, ncol, Gin, st, run);
   else launch_xprep<false>(c, ncol, Gin, st, run);
   DY_CUDA(c, cudaGetLastError());

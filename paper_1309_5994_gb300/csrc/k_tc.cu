@@ -1590,6 +1590,20 @@ int tc_check_error(dyson_ctx* c) {
   return tc_error_status(c);
 }
 
+size_t tc_x_bytes(const dyson_ctx* c) {
+  const TcState* st = static_cast<const TcState*>(c->tc);
+  return st ? st->xbuf_bytes : 0;
+}
+
+void tc_release_x(dyson_ctx* c) {
+  TcState* st = static_cast<TcState*>(c->tc);
+  if (!st) return;
+  cudaFree(st->xbuf);
+  st->xbuf = nullptr;
+  st->xbuf_bytes = 0;
+  st->x_ptr = st->xh_ptr = nullptr;
+}
+
 void tc_release(dyson_ctx* c) {
   TcState* st = static_cast<TcState*>(c->tc);
   if (!st) return;

@@ -6,6 +6,10 @@
 bool oz_supported(dyson_ctx* c);
 // device bytes of X slices per complex state element
 size_t oz_bytes_per_element();
+// X slices for ncol columns (oz_residual makes them where they are missing); bytes held by them; give them back
+int oz_reserve(dyson_ctx* c, int ncol);
+size_t oz_x_bytes(const dyson_ctx* c);
+void oz_release_x(dyson_ctx* c);
 // forget the Lambda slices (after dyson_build_sigma)
 void oz_invalidate(dyson_ctx* c);
 // tolerances that the split serves; tighter ones need the residual of k_oz64

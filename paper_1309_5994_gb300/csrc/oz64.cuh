@@ -3,8 +3,13 @@
 #include "common.cuh"
 
 // true when the split-product FP64 sweep can serve this context: its slices of Lambda exist or
-// fit in a third of the free device memory (it takes every contour length)
-bool oz64_usable(dyson_ctx* c);
+// fit in a third of the device memory that is free or scratch (it takes every contour length); *more: bytes
+// that oz64_prepare would allocate
+bool oz64_usable(dyson_ctx* c, size_t* more);
+// X slices for ncol columns (oz64_sweep makes them where they are missing); bytes held by them; give them back
+int oz64_reserve(dyson_ctx* c, int ncol);
+size_t oz64_x_bytes(const dyson_ctx* c);
+void oz64_release_x(dyson_ctx* c);
 // device bytes of the X slices per complex state element
 double oz64_bytes_per_element(const dyson_ctx* c);
 // forget the Lambda slices (after Lambda changed)

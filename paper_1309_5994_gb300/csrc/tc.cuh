@@ -67,6 +67,9 @@ int tc_error_enqueue(dyson_ctx* c);
 // time limit (ns) of the pipeline waits of this file's kernels on the context's device
 int tc_set_wait_limit(dyson_ctx* c, unsigned long long ns);
 int tc_error_status(dyson_ctx* c);
+// bytes held by the unfused forms' gather buffer; give it back
+size_t tc_x_bytes(const dyson_ctx* c);
+void tc_release_x(dyson_ctx* c);
 // free tensor-core module state
 void tc_release(dyson_ctx* c);
 

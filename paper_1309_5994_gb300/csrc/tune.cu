@@ -93,7 +93,7 @@ int dyson_autotune(dyson_ctx* c, int32_t max_block_columns, dyson_tuning* out) {
     if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess) {
       const int m = c->gmres_restart > 0 ? c->gmres_restart : 40;
       const double per_block = (double)c->Nc * ((double)col_total + (m + 4.0) * c->Nr * 2.0 * c->Nc * sizeof(float));
-      const double avail = 0.8 * (double)(free_b + c->work_bytes);
+      const double avail = 0.8 * (double)(free_b + scratch_bytes(c));
       cap_gm = std::max<int64_t>(1, std::min<int64_t>(cap, (int64_t)(avail / per_block)));
     }
   }
@@ -120,7 +120,7 @@ int dyson_autotune(dyson_ctx* c, int32_t max_block_columns, dyson_tuning* out) {
     for (int v : variants) {
       c->tc_variant = v;
       double ms = 0.0;
-      if ((rc = prepare_tables(c, DYSON_PREC_TF32X3_F64REF, kOzTol)) || (rc = time_sweeps(c, nq, 2, 3, &ms))) {
+      if ((rc = prepare_tables(c, DYSON_PREC_TF32X3_F64REF, kOzTol, 0, false, true)) || (rc = time_sweeps(c, nq, 2, 3, &ms))) {
         c->tc_variant = saved_variant;
         return rc;
       }
