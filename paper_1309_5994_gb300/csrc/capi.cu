@@ -736,6 +736,9 @@ void release_scratch(dyson_ctx* c) {
   gmres_release(c);
 }
 
+// (site, vector column) pairs from which 64 contour points take the unfused sweep (prepare_tables)
+constexpr int64_t kManySiteColumns = 32768;
+
 // share of the free memory that cudaMalloc is taken to deliver in a few blocks
 constexpr double kFreeShare = 0.95;
 
@@ -763,9 +766,8 @@ int prepare_tables(dyson_ctx* c, int precision, double tol, int64_t columns, boo
   // A fused tile of 256 rows is half empty at 64 contour points (128 rows of the embedding), so from
   // kManySiteColumns on the unfused form is the faster one although its series waits for every sweep:
   // single CTA / fused, us a sweep: 8x8 sites, 512 columns 34 / 46, 1024 57 / 83; 12x12, 512 62 / 85;
-  // 16x16, 128 36 / 52; 5x5, 1024 33 / 43.
-  constexpr int64_t kManySiteColumns = 32768;
-  c->many_of_64 = c->Nc == 64 && c->Nr * columns >= kManySiteColumns;
+  // 16x16, 128 36 / 52; 5x5, 1024 33 / 43.  Only where no form was selected or tuned.
+  c->many_of_64 = c->tc_variant < 0 && c->Nc == 64 && c->Nr * columns >= kManySiteColumns;
   c->use_tc = c->use_oz = c->use_oz64 = false;
   c->Ns = c->Nc;
   if (precision == DYSON_PREC_F64) return prepare_oz64(c, hold);
@@ -851,6 +853,18 @@ int64_t chunk_columns(dyson_ctx* c, int precision, int64_t unit, int64_t want, s
   return cols;
 }
 
+// Tables for a solve of `want` columns, *cols of them at once where memory allows; *cols becomes what it allows.
+// The sweep is picked by the columns that really go through at once.
+int prepare_chunk(dyson_ctx* c, int precision, double tol, int64_t unit, int64_t want, int64_t* cols, size_t* bytes_per_col) {
+  int rc = prepare_tables(c, precision, tol, *cols);
+  if (rc) return rc;
+  *cols = chunk_columns(c, precision, unit, want, bytes_per_col);
+  if (!c->many_of_64 || c->Nr * *cols >= kManySiteColumns) return DYSON_OK;
+  if ((rc = prepare_tables(c, precision, tol, *cols))) return rc;
+  *cols = chunk_columns(c, precision, unit, want, bytes_per_col);
+  return DYSON_OK;
+}
+
 // Buffers of a chunk of ncol columns in groups of gs: work state, sources and norms, and what the sweeps and the
 // residual need besides, ahead of the GMRES basis, which takes most of what is left.  Where the residual's or the
 // FP64 sweep's slices cannot be had, the FP64-pipe kernel runs.
@@ -925,9 +939,9 @@ int solve_columns_impl(dyson_ctx* c, const int32_t* src, int64_t n_src, int prec
     if (src[q] < 0 || src[q] >= c->Nr) return R.finish(ctx_fail(c, DYSON_ERR_INVALID_ARG, "source site out of range"));
   DeviceGuard g(c->device);
   const int64_t at_once = c->chunk_override > 0 ? std::min<int64_t>(n_src, c->chunk_override) : n_src;
-  if ((rc = prepare_tables(c, precision, tol, at_once * c->Nc))) return R.finish(rc);
   size_t col_bytes = 0;
-  const int64_t cols = chunk_columns(c, precision, c->Nc, n_src * (int64_t)c->Nc, &col_bytes);
+  int64_t cols = at_once * c->Nc;
+  if ((rc = prepare_chunk(c, precision, tol, c->Nc, n_src * (int64_t)c->Nc, &cols, &col_bytes))) return R.finish(rc);
   if (cols < c->Nc) return R.finish(ctx_fail(c, DYSON_ERR_OOM, "one block column does not fit in device memory"));
   const int64_t chunk = cols / c->Nc;
   if ((rc = reserve_chunk(c, (int)cols, c->Nc, col_bytes))) return R.finish(rc);
@@ -999,11 +1013,11 @@ int dyson_solve_vector_columns(dyson_ctx* c, const int32_t* sites, const int32_t
     if (sites[q] < 0 || sites[q] >= c->Nr || times[q] < 0 || times[q] >= c->Nc)
       return R.finish(ctx_fail(c, DYSON_ERR_INVALID_ARG, "column source out of range"));
   DeviceGuard g(c->device);
-  if ((rc = prepare_tables(c, precision, tol, n))) return R.finish(rc);
   constexpr int GS = 32;                                   // norm group; columns padded to a multiple
   const int64_t padded = (n + GS - 1) / GS * GS;
   size_t col_bytes = 0;
-  const int64_t chunk = chunk_columns(c, precision, GS, padded, &col_bytes);
+  int64_t chunk = n;
+  if ((rc = prepare_chunk(c, precision, tol, GS, padded, &chunk, &col_bytes))) return R.finish(rc);
   if (chunk < GS) return R.finish(ctx_fail(c, DYSON_ERR_OOM, "32 vector columns do not fit in device memory"));
   if ((rc = reserve_chunk(c, (int)chunk, GS, col_bytes))) return R.finish(rc);
   int status = DYSON_OK;

@@ -123,3 +123,51 @@ def test_large_solves_of_64_points_take_the_unfused_form(torch_cuda, lib, n, unf
     for k in list(range(0, n, 97)) + [n - 1]:
         assert np.abs(got[k] - ref[sites[k], times[k]]).max() / big < 1e-11
     s.close()
+
+
+def _many_of_64(torch, binding, n, variant=None, leave=None):
+    """profile counts (gather, single-CTA or default, fused) of a solve of n vector columns on 6 sites"""
+    p = wl.random_tables(wl.small(L=3, Ly=2, Nt=24, Nm=16, dt=0.02, beta=1.0, trap_c=0.3, U0=14.0), seed=7, rel=0.1)
+    s = binding.Solver(p, device=0)
+    if variant is not None:
+        s.set_sweep_variant(variant)
+    s.build_sigma()
+    hog = None
+    if leave is not None:
+        torch.cuda.empty_cache()
+        hog = torch.empty(torch.cuda.mem_get_info()[0] - leave, dtype=torch.uint8, device="cuda:0")
+    s.profile(True)
+    res = s.solve_vectors([k % p.Nr for k in range(n)], [(7 * k) % p.Nc for k in range(n)],
+                          precision=binding.PREC_TF32X3_F64REF, tol=1e-6)
+    kinds = [s.profile_query(k)[0] for k in (binding.KERNEL_GATHER_TC, binding.KERNEL_SWEEP_TC, binding.KERNEL_SWEEP_TC_FUSED)]
+    s.close()
+    del hog
+    torch.cuda.empty_cache()
+    return kinds, res.report["chunks"]
+
+
+def test_a_selected_form_runs_at_64_points_too(torch_cuda, lib):
+    from paper_1309_5994_gb300 import binding
+    (gather, plain, fused), _ = _many_of_64(torch_cuda, binding, 5472, variant=binding.SWEEP_FUSED_PAIR)
+    assert gather == 0 and plain == 0 and fused > 0
+
+
+def test_the_line_at_64_points_counts_the_columns_of_a_chunk(torch_cuda, lib):
+    """5472 columns of 6 sites in 96 MB are several chunks below the line."""
+    from paper_1309_5994_gb300 import binding
+    (gather, plain, _), chunks = _many_of_64(torch_cuda, binding, 5472, leave=96 << 20)
+    assert chunks > 1 and gather == 0 and plain > 0
+
+
+def test_the_tuned_form_is_the_one_that_runs(torch_cuda, lib):
+    from paper_1309_5994_gb300 import binding
+    p = wl.small(L=8, Ly=8, Nt=24, Nm=16, dt=0.05, beta=2.0, trap_c=0.05, U0=20.0)
+    s = binding.Solver(p, device=0)
+    s.build_sigma()
+    t = s.autotune(16)
+    s.profile(True)
+    s.solve(list(range(16)), precision=binding.PREC_TF32X3_F64REF, tol=1e-6)
+    fused = binding.SWEEP_NAMES[t["sweep_variant"]].startswith("fused")
+    assert (s.profile_query(binding.KERNEL_SWEEP_TC_FUSED)[0] > 0) == fused
+    assert (s.profile_query(binding.KERNEL_GATHER_TC)[0] > 0) == (not fused)
+    s.close()
