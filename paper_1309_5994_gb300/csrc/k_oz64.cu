@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(256) k_oz64_aprep(const double2* __restrict__ 
 // Bound by the FP64 pipe (83 % busy): 8x8, Nc = 64, 4096 columns 0.259 ms with four additions per part,
 // 0.197 with the three it needs (floor of its bytes 0.118).
 template <bool UNIFORM, int PER_LANE>
-__global__ void __launch_bounds__(256) k_oz64_xprep(const double2* __restrict__ G, const double* __restrict__ Jtab,
+__global__ void __launch_bounds__(256) k_oz64_xprep(const double2* G, const double* __restrict__ Jtab,
                                                     const int* __restrict__ nbr, const int* __restrict__ nbond, int Nr,
                                                     int Nt, int Nc, int ncol, int Kp, __nv_bfloat16* __restrict__ xs,
                                                     int* __restrict__ etau, const int* __restrict__ run) {
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(256) k_oz64_xprep(const double2* __restrict__ 
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       if (!has[q]) continue;
-      const double2 g = col[q][z];
+      const double2 g = ptx::load_d2(col[q] + z);
       if (UNIFORM) {
         if (q == 0) {                                      // (x is still zero: one FP64 addition less)
           x = g;
@@ -389,7 +389,7 @@ __device__ __forceinline__ void flush_norm(float sq, unsigned long long* norm, i
 template <int MODE>
 __global__ void __launch_bounds__(THREADS, 1)
     k_oz64_gemm(const __nv_bfloat16* __restrict__ as, const __nv_bfloat16* __restrict__ xs,
-                const int* __restrict__ esig, const int* __restrict__ etau, const double* __restrict__ Gin,
+                const int* __restrict__ esig, const int* etau, const double* Gin,
                 const double2* __restrict__ lam, const int* __restrict__ src_site, const int* __restrict__ src_time,
                 int Nr, int Nc, int KB, int ncol, int gs, double* __restrict__ out, float* __restrict__ r32, int Ns,
                 unsigned long long* __restrict__ norm, int* __restrict__ err, const int* __restrict__ run) {
@@ -525,7 +525,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       const int cols = max(0, min(COLS_PER_WARP, ncol - n_first));
       // lane j < 16: scale exponent and source of the warp's column j (read by shuffle below)
       static_assert(COLS_PER_WARP == 16, "one column per lane of a half warp");
-      const int et_l = lane < cols ? __ldg(etau + (size_t)site * ncol + n_first + lane) : 0;
+      const int et_l = lane < cols ? load_i(etau + (size_t)site * ncol + n_first + lane) : 0;
       const unsigned src_here =
           __ballot_sync(0xffffffffu, MODE != 2 && lane < cols && __ldg(src_site + n_first + lane) == site);
       const size_t off0 = ((size_t)site * ncol + n_first) * N2 + (row_ok ? m : 0);
@@ -535,7 +535,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         const int c = 8 * h;
 #pragma unroll
         for (int j = 0; j < 8; ++j)
-          gin[h][j] = MODE != 2 && c + j < cols ? __ldg(Gin + off0 + (size_t)(c + j) * N2) : 0.0;
+          gin[h][j] = MODE != 2 && c + j < cols ? load_d(Gin + off0 + (size_t)(c + j) * N2) : 0.0;
       };
       load_g(0);
       long long V[COLS_PER_WARP];

@@ -782,7 +782,7 @@ template <class Cfg, bool RZERO>
 struct FusedEpilogue {
   static constexpr int NB = Cfg::NB, CH = 16, PER = NB / CH, CHUNKS = Cfg::GT * PER;
   const float* __restrict__ r;
-  const float* __restrict__ din;
+  const float* din;
   float* __restrict__ dout;
   int n_first, ncol, N2, row_gap;
   size_t base0;                                          // element of (site, column n_first, this lane's first row)
@@ -800,14 +800,14 @@ struct FusedEpilogue {
 #pragma unroll
       for (int j = 0; j < CH; ++j) {
         if (!RZERO) rv[B][j] = __ldcs(r + o + (size_t)j * N2);
-        dv[B][j] = __ldcs(din + o + (size_t)j * N2);
+        dv[B][j] = ptx::load_cs(din + o + (size_t)j * N2);
       }
     } else {
 #pragma unroll
       for (int j = 0; j < CH; ++j)
         if (j < left) {
           if (!RZERO) rv[B][j] = __ldcs(r + o + (size_t)j * N2);
-          dv[B][j] = __ldcs(din + o + (size_t)j * N2);
+          dv[B][j] = ptx::load_cs(din + o + (size_t)j * N2);
         }
     }
   }
@@ -830,7 +830,7 @@ struct FusedEpilogue {
       qcur = n / gs;
       qbeg = qcur * gs;
       qend = qbeg + gs;
-      down = adown * sc[qcur].down;
+      down = adown * ptx::load_f(&sc[qcur].down);
     };
     enter(n0);
     uint32_t v[CH];
@@ -1059,7 +1059,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
       const FTile T = fused_tile<Cfg>(I, tile, sweep);
       if (!T.active) continue;
       const int Ns = I.Ns, N2 = 2 * Ns, ncol = I.ncol, gs = I.gs;
-      const float* __restrict__ din = I.din;
+      const float* din = I.din;
       const float* __restrict__ Jz = I.Jz;
       const TcScale* sc = I.sc;
       int nb[4], bd[4];
@@ -1073,7 +1073,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
       const int ni = max(0, min(NB / 64, (ncol - col0 - c0 + 31) / 32));
       float up[NB / 64];
 #pragma unroll
-      for (int i = 0; i < NB / 64; ++i) up[i] = i < ni ? __ldg(&sc[(col0 + c0 + 32 * i) / gs].up) : 0.f;
+      for (int i = 0; i < NB / 64; ++i) up[i] = i < ni ? load_f(&sc[(col0 + c0 + 32 * i) / gs].up) : 0.f;
       // row of neighbour q at the first column (a valid address also where the neighbour is missing)
       const float* nbp[4];
 #pragma unroll
@@ -1093,8 +1093,8 @@ __global__ void __launch_bounds__(F_THREADS, 1)
             const int ci = GT == 2 ? i : 2 * h + i;
             const bool ok_qi = nb[q] >= 0 && ci < ni;
             const float* p = ok_qi ? nbp[q] + ci * cstride + kb * F_BK + (GT == 2 ? h * Ns : 0) : nbp[q];
-            v[q][i][0] = __ldg(reinterpret_cast<const float4*>(p));
-            v[q][i][1] = __ldg(reinterpret_cast<const float4*>(p + 32));
+            v[q][i][0] = load_f4(p);
+            v[q][i][1] = load_f4(p + 32);
           }
       };
       auto issue_j = [&](int kb) {
