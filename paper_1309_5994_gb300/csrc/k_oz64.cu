@@ -356,19 +356,35 @@ __device__ __forceinline__ double fixed_to_double_normal(long long V, int e) {
   return __hiloint2double((int)(((a == 0 ? 0u : h)) | ((unsigned int)(V >> 32) & 0x80000000u)), (int)(unsigned int)q);
 }
 
-// |d| as FP32 from its bits (truncated; no conversion on the FP64 pipe): 0 below 2^-126, inf from 2^127
-// and for NaN
-__device__ __forceinline__ float magnitude(double d) {
-  const unsigned int hi = (unsigned int)__double2hiint(d) & 0x7FFFFFFFu, lo = (unsigned int)__double2loint(d);
-  const unsigned int f = __funnelshift_l(lo, hi, 3) - (896u << 23);
-  return __uint_as_float(hi < 0x38100000u ? 0u : (hi >= 0x47E00000u ? 0x7F800000u : f));
-}
-// sqrt of a running maximum of squares (inf stays inf)
-__device__ __forceinline__ void flush_norm(float sq, unsigned long long* norm, int lane) {
-  for (int o = 16; o > 0; o >>= 1) sq = fmaxf(sq, __shfl_xor_sync(0xffffffffu, sq, o));
-  // (an FP64 square root, even of one lane, holds the SM's FP64 pipe for hundreds of cycles a warp)
-  if (lane == 0) atomicMax(norm, (unsigned long long)__double_as_longlong((double)sqrtf(sq)));
-}
+// The norms decide when an iteration stops, relative to a scale: they are held in FP32 in units of the power of two
+// below that scale (24 bits, from 2^-74 to 2^63 of it; the FP64 pipe has no room for their squares).
+struct NormUnit {
+  unsigned int least;                                      // high word of 2^-126 units
+  static constexpr unsigned int SPAN = (0x47E - 0x381) << 20;   // from there to 2^127 units
+  __device__ __forceinline__ explicit NormUnit(unsigned long long scale)
+      : least((unsigned int)(0x381 + (scale == 0ull ? 0 : max(-880, min(880, (int)(scale >> 52) - 1023)))) << 20) {}
+  // |d| in units as FP32, from its bits (truncated; no conversion on the FP64 pipe): 0 outside the span; top keeps
+  // the largest high word
+  __device__ __forceinline__ float magnitude(double d, unsigned int& top) const {
+    const unsigned int hi = (unsigned int)__double2hiint(d) & 0x7FFFFFFFu, lo = (unsigned int)__double2loint(d);
+    const unsigned int t = hi - least;
+    top = max(top, hi);
+    return t < SPAN ? __uint_as_float(__funnelshift_l(lo, t, 3) + 0x00800000u) : 0.f;
+  }
+  // max of the word with the square root of a running maximum of squares (infinite where an entry lay above the
+  // span, or was infinite or not a number)
+  __device__ __forceinline__ void flush(float sq, unsigned int top, unsigned long long* norm, int lane) const {
+    const float inf = __int_as_float(0x7f800000);
+    if (top >= least + SPAN) sq = inf;
+    for (int o = 16; o > 0; o >>= 1) sq = fmaxf(sq, __shfl_xor_sync(0xffffffffu, sq, o));
+    // (an FP64 square root, even of one lane, holds the SM's FP64 pipe for hundreds of cycles a warp)
+    if (lane != 0) return;
+    const float m = sqrtf(sq);
+    unsigned long long bits = (unsigned long long)__double_as_longlong((double)m);
+    if (m > 0.f && m < inf) bits += ((unsigned long long)least << 32) - (0x381ull << 52);
+    atomicMax(norm, bits);
+  }
+};
 
 // Persistent: one CTA per SM walks 128 x 64 output tiles (row tile fastest, then column tile, then
 // site).  A stage is a 32-deep k-block of all eight slices of both operands.  Per k16 step,
@@ -528,6 +544,9 @@ __global__ void __launch_bounds__(THREADS, 1)
       const int et_l = lane < cols ? load_i(etau + (size_t)site * ncol + n_first + lane) : 0;
       const unsigned src_here =
           __ballot_sync(0xffffffffu, MODE != 2 && lane < cols && __ldg(src_site + n_first + lane) == site);
+      int qcur = n_first / gs;
+      NormUnit unit(MODE != 2 && cols > 0 ? norm[ncol / gs + qcur] : 0ull);   // (the scales follow the norms)
+      unsigned int top = 0;
       const size_t off0 = ((size_t)site * ncol + n_first) * N2 + (row_ok ? m : 0);
       // G of this lane's row, eight columns at a time (the first ones before the wait)
       double gin[2][8];
@@ -576,7 +595,6 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
       if (!go) break;
       load_g(1);
-      int qcur = n_first / gs;
       int left = min(COLS_PER_WARP, (qcur + 1) * gs - n_first);   // columns to the next norm group
       float sq = 0.f;                                       // running max |d|^2 of the group
       // A whole tile without sources, in one norm group and far from the ends of the exponent range takes
@@ -592,13 +610,13 @@ __global__ void __launch_bounds__(THREADS, 1)
             const int et = __shfl_sync(0xffffffffu, et_l, j + u);
             const double y = fixed_to_double_normal(V[j + u], es + et - 53 + extra);
             out[off0 + (size_t)(j + u) * N2] = y;
-            const float a = magnitude(y - gin[j / 8][(j + u) % 8]);
+            const float a = unit.magnitude(y - gin[j / 8][(j + u) % 8], top);
             a2[u] = a * a;
           }
           const float other = __shfl_xor_sync(0xffffffffu, odd ? a2[0] : a2[1], 1);
           sq = fmaxf(sq, (odd ? a2[1] : a2[0]) + other);
         }
-        flush_norm(sq, norm + qcur, lane);
+        unit.flush(sq, top, norm + qcur, lane);
         continue;
       }
 #pragma unroll
@@ -611,8 +629,10 @@ __global__ void __launch_bounds__(THREADS, 1)
           continue;
         }
         if (j == left) {
-          flush_norm(sq, norm + qcur, lane);
+          unit.flush(sq, top, norm + qcur, lane);
           ++qcur;
+          unit = NormUnit(norm[ncol / gs + qcur]);
+          top = 0;
           left = j + gs;
           sq = 0.f;
         }
@@ -621,7 +641,7 @@ __global__ void __launch_bounds__(THREADS, 1)
           y += (m & 1) ? b.y : b.x;
         }
         const double d = y - gin[j / 8][j % 8];
-        const float a = row_ok ? magnitude(d) : 0.f;
+        const float a = row_ok ? unit.magnitude(d, top) : 0.f;
         if (row_ok) {
           if (MODE == 0) out[off0 + (size_t)j * N2] = y;
           else r32[((size_t)site * ncol + n_first + j) * 2 * Ns + (m >> 1) + ((m & 1) ? Ns : 0)] = (float)d;
@@ -629,7 +649,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         const float a2 = a * a;
         sq = fmaxf(sq, a2 + __shfl_xor_sync(0xffffffffu, a2, 1));
       }
-      if (MODE != 2 && cols > 0) flush_norm(sq, norm + qcur, lane);
+      if (MODE != 2 && cols > 0) unit.flush(sq, top, norm + qcur, lane);
     }
   }
 

@@ -16,7 +16,8 @@ double oz64_bytes_per_element(const dyson_ctx* c);
 void oz64_invalidate(dyson_ctx* c);
 // build the Lambda slices now (so that the free memory a caller sizes its chunk by is what is left)
 int oz64_prepare(dyson_ctx* c);
-// mode 0: out = B + K Gin, c->d_norm[q] = max |out - Gin| (complex modulus);
+// mode 0: out = B + K Gin, c->d_norm[q] = max |out - Gin| (complex modulus; 24 bits, relative to the scale
+// c->d_norm[ncol / gs + q]);
 // mode 1: r32 = B + K Gin - Gin (FP32 planar of stride c->Ns; only the Nc points are written), c->d_norm[q] = max |r|.
 // Groups of gs columns as launch_sweep_f64; two kernel launches, counted on the context.
 int oz64_sweep(dyson_ctx* c, int ncol, int gs, const double2* Gin, double2* out, float* r32, int mode,
