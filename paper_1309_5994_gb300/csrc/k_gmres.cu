@@ -24,6 +24,7 @@
 #include "common.cuh"
 #include "detail.cuh"
 #include "gmres.cuh"
+#include "sumsq.cuh"
 #include "tc.cuh"
 
 using namespace dyson_detail;
@@ -124,13 +125,16 @@ __device__ __forceinline__ void store_slab(const Slab<VEC, T>& x, float* __restr
   }
 }
 template <int VEC, int T>
-__device__ __forceinline__ float slab_norm2(const Slab<VEC, T>& x) {
-  float q = 0.f;
+__device__ __forceinline__ double slab_norm2(const Slab<VEC, T>& x) {
+  SumSq q;
 #pragma unroll
   for (int t = 0; t < T; ++t)
 #pragma unroll
-    for (int v = 0; v < VEC; ++v) q = fmaf(x.re[t][v], x.re[t][v], fmaf(x.im[t][v], x.im[t][v], q));
-  return q;
+    for (int v = 0; v < VEC; ++v) {
+      q.add(x.re[t][v]);
+      q.add(x.im[t][v]);
+    }
+  return q.value();
 }
 
 // Sum of eight FP64 values over a warp: halving exchanges (nine additions; the FP64 pipe takes 16 cycles
@@ -194,7 +198,7 @@ __global__ void __launch_bounds__(GM_THREADS, 2) k_gm_dots(const float* __restri
           w.im[t][v] -= q[1].im[t][v];
         }
     }
-    if (nrm0) sq += (double)slab_norm2(w);
+    if (nrm0) sq += slab_norm2(w);
     for (int g0 = 0; g0 < nvec; g0 += GM_GROUP) {
       double v8[2 * GM_GROUP];
 #pragma unroll
@@ -251,7 +255,7 @@ __global__ void __launch_bounds__(GM_THREADS) k_gm_norm2(const float* __restrict
   for (int item = i0 + (int)(threadIdx.x >> 5); item < i1; item += GM_THREADS / 32) {
     Slab<VEC, T> x;
     load_slab(x, a, item_pos<VEC, T>(item, nz, n, ncol, Ns, threadIdx.x & 31), Ns);
-    acc += (double)slab_norm2(x);
+    acc += slab_norm2(x);
   }
   block_add(acc, &nrm[n]);
 }
@@ -333,7 +337,7 @@ __global__ void __launch_bounds__(GM_THREADS) k_gm_update(const float* __restric
       fold(q[2], hs[i + 2]);
     }
     store_slab(x, w, at, Ns);
-    acc += (double)slab_norm2(x);
+    acc += slab_norm2(x);
   }
   if (nrm) block_add(acc, &nrm[n]);
 }
