@@ -406,7 +406,7 @@ int dyson_batch_solve(dyson_batch* b, const int32_t* const* src, const int32_t* 
         X.status = DYSON_ERR_DIVERGED;
         X.done = true;
       } else if (res <= tol) {
-        if (!refine_once_more(res, tol, X.prev_res, c->Nc, ref + 1 == max_ref)) {
+        if (!refine_once_more(res, tol, X.prev_res, c->accept, ref + 1 == max_ref)) {
           X.status = DYSON_OK;
           X.done = true;
         }

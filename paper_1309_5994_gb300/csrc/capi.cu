@@ -559,8 +559,7 @@ int solve_mixed(dyson_ctx* c, int ncol, int gs, int precision, double tol, int m
       status = DYSON_ERR_DIVERGED;
       break;
     }
-    if (res <= tol && !(c->use_tc && tc_uses_fused(c) &&
-                        refine_once_more(res, tol, prev_res, c->Nc, ref + 1 == c->max_refinements))) {
+    if (res <= tol && !refine_once_more(res, tol, prev_res, c->accept, ref + 1 == c->max_refinements)) {
       status = DYSON_OK;
       break;
     }
@@ -644,6 +643,13 @@ int dyson_init(dyson_ctx** out, const dyson_lattice* L, const dyson_contour* C, 
       return fail_noctx(DYSON_ERR_INVALID_ARG, "J table holds a non-finite value");
     }
   for (double v : c->J) c->j_max = std::max(c->j_max, (float)(std::fabs(v) * 1.000001));
+  double u_min = std::numeric_limits<double>::infinity(), eps_max = 0.0;
+  for (double v : c->U) u_min = std::min(u_min, std::fabs(v));
+  for (int i = 0; i < c->Nr; ++i) {
+    const double x = i % c->Lx - 0.5 * (c->Lx - 1), y = i / c->Lx - 0.5 * (c->Ly - 1);
+    eps_max = std::max(eps_max, std::fabs(c->curvature * (x * x + y * y) - 0.5 * c->U[(size_t)i * c->Nt] - c->mu));
+  }
+  c->accept = accept_share(c->dt, u_min, eps_max, c->j_max);
   c->j_uniform = true;
   for (int b = 1; b < c->Nb && c->j_uniform; ++b)
     c->j_uniform = std::equal(c->J.begin() + (size_t)b * c->Nt, c->J.begin() + (size_t)(b + 1) * c->Nt, c->J.begin());

@@ -193,6 +193,7 @@ struct dyson_ctx {
   int Ns = 0;                        // contour stride of the FP32 states of the current solve (contour_stride, or Nc)
   bool lam16_built = false;
   float j_max = 0.f;                 // max |J_b(t_k)|
+  double accept = 1.0;               // share of a loose tolerance below which a residual is accepted (accept_share)
   TcScale* d_xscale = nullptr;       // [norm_cap] scales of the FP16 X per column group
   double* d_obs = nullptr;           // [3][Nr][Nt]
   bool sigma_built = false;

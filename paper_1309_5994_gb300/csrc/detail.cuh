@@ -41,19 +41,6 @@ inline double inner_target(double floor_target, double tol, double prev_res) {
   const double t = kInnerSlack * tol / prev_res;
   return t > kInnerCap ? kInnerCap : (t > floor_target ? t : floor_target);
 }
-// A first refinement that ends just below a loose tolerance leaves errors of a few tolerances in quantities
-// that amplify the residual (the double occupancy's difference quotient, up to 4 times), where 3xTF32
-// inner solves, whose residuals are about twice as large, went on to a second refinement and 1e-9.  So at
-// tolerances of kLooseTol and above one more refinement follows unless the residual is below
-// kAcceptShare of the tolerance (0.43 was the least residual, in units of 1e-6, for which they did).
-constexpr double kLooseTol = 1e-8;
-// Contours of no multiple of 64 ran FP32 CUDA-core sweeps, whose residuals are 0.5 to 1 of the fused
-// sweep's (1.2 to 3.6 of 1e-7 up to 70 points): there below half of that.
-constexpr double kAcceptShare = 0.4, kAcceptShareOdd = 0.2;
-inline bool refine_once_more(double res, double tol, double prev_res, int Nc, bool last) {
-  const double share = Nc % 64 ? kAcceptShareOdd : kAcceptShare;
-  return res <= tol && tol >= kLooseTol && res > share * tol && prev_res > tol && !last;
-}
 // Refinement that grows the residual: a residual above kRefineContract times the
 // previous one, kRefineStrikes times, means the series of App. C does not
 // converge for this problem (spectral radius of K above 1); the solve ends with

@@ -103,4 +103,19 @@ SERIES_HD inline void series_step(SeriesState& S, double upd, int max_sweeps, do
 // relative residuals after it and before it (infinite before the first, whose solution is zero)
 inline bool plateau_served(double res, double prev_res) { return res <= kPlateauGain * (prev_res < 1.0 ? prev_res : 1.0); }
 
+// Observables amplify the residual.  The double occupancy D = (Re (G(t) - G(t - dt)) / dt - eps n - E_kin) / U has
+// up to 2 / (dt |U|) of it from the difference quotient and (|eps| + 4 |J|) / |U| from the rest (errors of G of the
+// residual's size).  An inner solve after the first aims at a tenth of the tolerance (kInnerSlack), but the first
+// refinement aims at no tolerance and may end just below a loose one; so at tolerances of kLooseTol and above (no
+// first refinement reaches lower ones) one more refinement follows unless the residual is below accept_share
+// of the tolerance.
+constexpr double kLooseTol = 1e-8;
+inline double accept_share(double dt, double u_min, double eps_max, double j_max) {
+  const double amplification = u_min > 0.0 ? (2.0 / dt + eps_max + 4.0 * j_max) / u_min : 1e300;
+  return amplification > 1.0 ? 1.0 / amplification : 1.0;
+}
+inline bool refine_once_more(double res, double tol, double prev_res, double share, bool last) {
+  return res <= tol && tol >= kLooseTol && res > share * tol && prev_res > tol && !last;
+}
+
 }  // namespace dyson_detail

@@ -18,6 +18,8 @@ extern "C" int run(const double* upd, int n, int max_sweeps, double target, doub
   return S.outcome;
 }
 extern "C" int served(double res, double prev) { return plateau_served(res, prev); }
+extern "C" double share(double dt, double u, double eps, double j) { return accept_share(dt, u, eps, j); }
+extern "C" int more(double res, double tol, double prev, double share, int last) { return refine_once_more(res, tol, prev, share, last); }
 """
 
 
@@ -33,12 +35,18 @@ def rule(tmp_path_factory):
                         ctypes.c_int, ctypes.POINTER(ctypes.c_int)]
     lib.served.argtypes = [ctypes.c_double, ctypes.c_double]
 
+    lib.share.argtypes = [ctypes.c_double] * 4
+    lib.share.restype = ctypes.c_double
+    lib.more.argtypes = [ctypes.c_double] * 4 + [ctypes.c_int]
+
     def go(upd, max_sweeps=400, target=4e-7, abort_peak=1e5, plateau=1):
         s = ctypes.c_int()
         out = lib.run((ctypes.c_double * len(upd))(*upd), len(upd), max_sweeps, target, abort_peak, plateau, ctypes.byref(s))
         return out, s.value
 
     go.served = lambda res, prev: bool(lib.served(res, prev))
+    go.share = lib.share
+    go.more = lambda *a: bool(lib.more(*a))
     return go
 
 
@@ -81,3 +89,15 @@ def test_other_ends_of_a_series(rule):
     assert rule([1.0, float("nan")]) == (NOT_FINITE, 2)
     assert rule([1.0, 0.9, 0.8], max_sweeps=3) == (EXHAUSTED, 3)
     assert rule([1.0, 1e-3, 1e-5, 1.1e-5, 1.2e-5, 1.1e-5, 1.2e-5])[0] == STOPPED
+
+
+def test_a_loose_tolerance_is_met_by_the_observables_too(rule):
+    """The share of the tolerance follows from how much the double occupancy amplifies a residual."""
+    assert rule.share(0.05, 20.0, 10.0, 1.0) == pytest.approx(20.0 / (2 / 0.05 + 10.0 + 4.0))
+    assert rule.share(0.005, 4.0, 2.0, 1.0) == pytest.approx(4.0 / (2 / 0.005 + 2.0 + 4.0))
+    assert rule.share(0.05, 0.0, 1.0, 1.0) < 1e-200 and rule.share(10.0, 50.0, 1.0, 1.0) == 1.0
+    inf = float("inf")
+    assert rule.more(0.5e-6, 1e-6, inf, 0.37, 0) and not rule.more(0.3e-6, 1e-6, inf, 0.37, 0)
+    assert rule.more(0.3e-6, 1e-6, inf, 0.01, 0)
+    assert not rule.more(0.5e-6, 1e-6, 0.9e-6, 0.37, 0)                # only one more
+    assert not rule.more(0.5e-6, 1e-6, inf, 0.37, 1) and not rule.more(0.5e-10, 1e-10, 1e-6, 0.37, 0)
