@@ -360,6 +360,14 @@ int dyson_set_sweep_variant(dyson_ctx* ctx, int variant);
  * run out of time and check that path.  INVALID_ARG for a limit outside [0, 60]. */
 int dyson_set_wait_limit(dyson_ctx* ctx, double seconds);
 
+/* Device memory for the BF16 slices that the FP64 sweeps, FP64-accurate residuals and
+ * the adjoint's site contraction multiply on the tensor cores: Lambda's slices (64 bytes
+ * per entry of Lambda) are made where they take at most `bytes`, the contraction works on
+ * as many sites at a time as fit in it.  What does not fit runs on the FP64 pipes, with the
+ * same results to FP64 rounding; 0: everything.  -1 (the default): a third of the free
+ * memory for Lambda's slices, a sixteenth for the contraction.  INVALID_ARG below -1. */
+int dyson_set_slice_memory(dyson_ctx* ctx, int64_t bytes);
+
 /* Sweeps of the inner series (App. C) on the fused tensor-core sweep that are enqueued at a
  * time, each followed by a one-warp kernel that applies the series' stopping rule on the
  * device and lets the remaining sweeps of a batch return at once (they take their sweep

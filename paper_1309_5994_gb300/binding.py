@@ -76,7 +76,7 @@ EXPORTS = ["dyson_init", "dyson_build_sigma", "dyson_copy_sigma", "dyson_solve_c
            "dyson_batch_create", "dyson_batch_solve", "dyson_batch_launch_count", "dyson_batch_last_error",
            "dyson_batch_destroy", "dyson_set_inner_solver", "dyson_autotune", "dyson_set_symmetry",
            "dyson_adjoint_obs", "dyson_extrapolate_dt", "dyson_set_support_truncation", "dyson_local_greens",
-           "dyson_selfenergy_step", "dyson_selfenergy_set_anderson"]
+           "dyson_selfenergy_step", "dyson_selfenergy_set_anderson", "dyson_set_slice_memory"]
 SYMMETRY_NONE, SYMMETRY_C4V = 0, 1
 INNER_SERIES, INNER_GMRES, INNER_AUTO = 0, 1, 2
 SWEEP_SINGLE_CTA, SWEEP_CTA_PAIR, SWEEP_FUSED_PAIR, SWEEP_FUSED_PAIR_WIDE = 0, 1, 2, 3
@@ -111,6 +111,7 @@ def load(path: str = _LIB_PATH):
     lib.dyson_set_sweep_variant.argtypes = [P, C.c_int]
     lib.dyson_set_wait_limit.argtypes = [P, C.c_double]
     lib.dyson_set_graph_sweeps.argtypes = [P, C.c_int]
+    lib.dyson_set_slice_memory.argtypes = [P, C.c_int64]
     lib.dyson_set_inner_solver.argtypes = [P, C.c_int, C.c_int32]
     lib.dyson_autotune.argtypes = [P, C.c_int32, C.POINTER(Tuning)]
     lib.dyson_set_symmetry.argtypes = [P, C.c_int]
@@ -375,6 +376,10 @@ class Solver:
     def set_wait_limit(self, seconds: float):
         """Time limit of the tensor-core pipelines' bounded waits on this device (0: the default 2 s)."""
         self._check(self.lib.dyson_set_wait_limit(self.h, float(seconds)))
+
+    def set_slice_memory(self, nbytes: int):
+        """Device memory for the slices of the FP64 path (0: FP64 pipes; -1: the default share of what is free)."""
+        self._check(self.lib.dyson_set_slice_memory(self.h, int(nbytes)))
 
     def set_graph_sweeps(self, sweeps: int):
         """Sweeps of the inner series per host synchronisation (0: one synchronisation per sweep)."""

@@ -777,7 +777,7 @@ int prepare_tables(dyson_ctx* c, int precision, double tol, int64_t columns, boo
   c->use_tc = c->use_oz = c->use_oz64 = false;
   c->Ns = c->Nc;
   if (precision == DYSON_PREC_F64) return prepare_oz64(c, hold);
-  const bool tc = c->tc_enabled && tc_supported(c);
+  const bool tc = tc_supported(c);
   const bool fused = tc && (batch || tc_uses_fused(c));
   if (tc) c->Ns = contour_stride(c);
   if (!tc && !c->lam32_built) {
@@ -805,7 +805,7 @@ int prepare_tables(dyson_ctx* c, int precision, double tol, int64_t columns, boo
     c->lam_split_built = true;
   }
   c->use_tc = tc;
-  c->use_oz = tc && tol >= kOzTol && c->oz_enabled && oz_supported(c);
+  c->use_oz = tc && tol >= kOzTol && c->slice_memory != 0 && oz_supported(c);
   return c->use_oz ? DYSON_OK : prepare_oz64(c, hold);
 }
 
@@ -1250,6 +1250,13 @@ int dyson_set_wait_limit(dyson_ctx* c, double seconds) {
   if (rc) return rc;
   if ((rc = oz_set_wait_limit(c, ns))) return rc;
   return oz64_set_wait_limit(c, ns);
+}
+
+int dyson_set_slice_memory(dyson_ctx* c, int64_t bytes) {
+  if (!c) return fail_noctx(DYSON_ERR_INVALID_ARG, "NULL context");
+  if (bytes < -1) return ctx_fail(c, DYSON_ERR_INVALID_ARG, "need a number of bytes, or -1");
+  c->slice_memory = bytes;
+  return DYSON_OK;
 }
 
 int dyson_set_graph_sweeps(dyson_ctx* c, int sweeps) {

@@ -212,7 +212,6 @@ struct dyson_ctx {
 
   bool lam32_built = false;
   bool lam_split_built = false;
-  bool tc_enabled = true;            // 3xTF32 tcgen05 sweep allowed where the contour fits it
   bool use_tc = false;               // chosen for the current solve
   int tc_variant = -1;               // DYSON_SWEEP_*; -1: none selected, the fused form
   bool many_of_64 = false;           // this solve is large and of 64 contour points (prepare_tables)
@@ -247,14 +246,13 @@ struct dyson_ctx {
   size_t act_bytes = 0;
   void* se = nullptr;                // self-energy step state (atomic G0, its pseudo-inverse, mixed T)
   bool se_installed = false;         // Lambda holds the local block of a self-energy step
-  bool oz_enabled = true;            // split-product residual allowed where 2 Nc <= 512
   bool use_oz = false;               // chosen for the current solve
   void* oz64 = nullptr;              // split-product FP64 sweep state (slices, scales, maps)
   bool overlap = false;              // series sweeps and checks are launched overlapped
   double* h_f64_upd = nullptr;       // pinned: update of each enqueued FP64 sweep (ring)
   int* d_f64_run = nullptr;          // 1 while the FP64 series goes on
   cudaEvent_t f64_ev[kF64Ahead] = {};
-  bool oz64_enabled = true;          // split-product FP64 sweeps allowed (memory permitting)
+  int64_t slice_memory = -1;         // dyson_set_slice_memory
   bool use_oz64 = false;             // chosen for the current solve: FP64 sweeps and residuals on the tensor cores
 
   std::string err;

@@ -712,13 +712,13 @@ void launch_xprep(dyson_ctx* c, int ncol, const double2* G, Oz64State* st, const
 
 bool oz64_usable(dyson_ctx* c, size_t* more) {
   *more = 0;
-  if (!c->oz64_enabled) return false;
+  if (c->slice_memory >= 0 && (int64_t)a_slice_bytes(c) > c->slice_memory) return false;
   Oz64State* st = static_cast<Oz64State*>(c->oz64);
   if (st && st->a_bytes >= a_slice_bytes(c)) return true;
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;
   *more = a_slice_bytes(c);
-  return a_slice_bytes(c) <= (free_b + dyson_detail::scratch_bytes(c)) / 3;
+  return c->slice_memory >= 0 || a_slice_bytes(c) <= (free_b + dyson_detail::scratch_bytes(c)) / 3;
 }
 
 int oz64_reserve(dyson_ctx* c, int ncol) {
@@ -812,17 +812,16 @@ int oz64_sweep(dyson_ctx* c, int ncol, int gs, const double2* Gin, double2* out,
 }
 
 int oz64_batched_product(dyson_ctx* c, int batch, int nk, int Nc, const double2* A, const double2* X, double2* out) {
-  if (!c->oz64_enabled) return DYSON_ERR_OOM;
   int rc = prepare_common(c);
   if (rc) return rc;
   Oz64State* st = state(c);
   const int Kp = (2 * nk + BK - 1) / BK * BK, N2 = 2 * Nc;
-  // scratch for as many entries at a time as fit in a sixteenth of the free memory
+  // scratch for as many entries at a time as fit in a sixteenth of the free memory, or in what the caller allows
   const size_t per_a = (size_t)S * N2 * Kp * 2, per_x = per_a / 2, per_e = (size_t)3 * Nc * sizeof(int);
   size_t free_b = 0, total_b = 0;
   DY_CUDA(c, cudaMemGetInfo(&free_b, &total_b));
   const size_t per = per_a + per_x + per_e;
-  const int step = (int)std::min<size_t>(batch, free_b / 16 / per);
+  const int step = (int)std::min<size_t>(batch, (c->slice_memory >= 0 ? (size_t)c->slice_memory : free_b / 16) / per);
   if (step < 1) return DYSON_ERR_OOM;
   char* buf = nullptr;
   if (cudaMalloc((void**)&buf, step * per) != cudaSuccess) {

@@ -54,3 +54,29 @@ def test_expired_pipeline_wait_returns_timeout_and_the_context_recovers(torch_cu
         s.set_wait_limit(-1.0)
     assert e.value.code == -1
     s.close()
+
+
+@pytest.mark.parametrize("Nt,Nm", [(24, 16), (72, 48), (38, 24), (80, 55)])
+def test_the_fused_form_returns_timeout_and_the_context_recovers(torch_cuda, lib, Nt, Nm):
+    """The default form on CTA pairs, in each of its four instances (Nc = 64, 192; 100, 215)."""
+    from paper_1309_5994_gb300 import binding
+    torch = torch_cuda
+    p = wl.random_tables(wl.small(L=2, Ly=2, Nt=Nt, Nm=Nm, trap_c=0.3, U0=20.0), seed=41, rel=0.2)
+    S = dyson.setup(p)
+    ref = dyson.dense_solve(S, dyson.rhs_block_columns(S, [0, 3]))
+    s = binding.Solver(p, device=0)
+    s.build_sigma()
+    g = torch.empty((2, p.Nr, p.Nc, p.Nc), dtype=torch.complex128, device="cuda:0")
+    try:
+        s.set_wait_limit(1e-9)
+        with pytest.raises(binding.DysonError) as e:
+            s.solve([0, 3], precision=binding.PREC_TF32X3_F64REF, tol=1e-12, g_out=g)
+        assert e.value.code == -5 and "time limit" in str(e.value)
+    finally:
+        s.set_wait_limit(0.0)
+    assert s.solve([0, 3], precision=binding.PREC_TF32X3_F64REF, tol=1e-12, g_out=g).status == 0
+    got = g.cpu().numpy()
+    for q in range(2):
+        want = ref[:, :, q * p.Nc:(q + 1) * p.Nc]
+        assert np.abs(got[q] - want).max() / np.abs(want).max() < 1e-11
+    s.close()
