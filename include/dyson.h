@@ -454,14 +454,13 @@ int dyson_set_support_truncation(dyson_ctx* ctx, int enable);
  * Each context keeps its own lattice, contour, trap, drive and Lambda, and its
  * block columns are solved exactly as dyson_solve_columns(precision =
  * DYSON_PREC_TF32X3_F64REF) solves them (the series of App. C refined with
- * FP64-accurate residuals).  What the instances share is the inner FP32
- * series.  Every sweep is one fused launch per instance still iterating, on
- * parallel branches, followed by a check
- * kernel that applies each instance's stopping rule on the device.  Blocks of
- * graph_sweeps sweeps are captured once as a CUDA graph and replayed with no
- * host round trip inside a block.  An instance whose series diverges (spectral
- * radius of Lambda W J above 1) is afterwards solved alone with the GMRES inner
- * solver of App. C, unless its context was set to DYSON_INNER_SERIES.
+ * FP64-accurate residuals).  The inner FP32 series of the instances run side by
+ * side on streams of the batch's own: graph_sweeps sweeps are enqueued at a time
+ * for every instance still iterating, each followed by a check kernel that applies
+ * the stopping rule on the device, and the host waits once for all of them.  An
+ * instance whose series diverges (spectral radius of Lambda W J above 1) is
+ * afterwards solved alone with the GMRES inner solver of App. C, unless its
+ * context was set to DYSON_INNER_SERIES.
  *
  * Requirements: every context is on the same device and stream, its Lambda is
  * built and upright, and its contour suits the tensor-core path with the
@@ -479,7 +478,7 @@ int dyson_batch_create(dyson_batch** out, dyson_ctx* const* ctxs, int32_t n);
 
 /* Solve the block columns src[k][0..n_src[k]) of instance k, for every k, to a
  * relative FP64 Dyson residual <= tol; max_sweeps bounds each inner series.
- * graph_sweeps = sweeps per graph replay (0 = 8; odd values are rounded up).
+ * graph_sweeps = sweeps enqueued at a time (0 = 8; odd values are rounded up).
  * g_out: NULL, or per instance NULL or a device buffer [n_src[k]][Nr][Nc][Nc]
  * complex128 (the layout of dyson_solve_columns).  reports: NULL or n entries.
  * Observables are read afterwards per context with dyson_observables.
@@ -488,7 +487,7 @@ int dyson_batch_create(dyson_batch** out, dyson_ctx* const* ctxs, int32_t n);
 int dyson_batch_solve(dyson_batch* b, const int32_t* const* src, const int32_t* n_src, double tol,
                       int32_t max_sweeps, int32_t graph_sweeps, double* const* g_out, dyson_report* reports);
 
-/* Kernels launched by the batch's sweep graphs (one per instance and one check per sweep; -1 for NULL). */
+/* Kernels launched for the batch's inner series (a sweep and its check each; -1 for NULL). */
 int64_t dyson_batch_launch_count(const dyson_batch* b);
 const char* dyson_batch_last_error(const dyson_batch* b);
 void dyson_batch_destroy(dyson_batch* b);

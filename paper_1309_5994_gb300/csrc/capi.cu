@@ -277,6 +277,62 @@ int tc_timed_sweep(dyson_ctx* c, int ncol, int gs, const float* r, const float* 
   return tc_sweep(c, ncol, gs, r, din, dout, TC_GEMM, act, sweep);
 }
 
+// the series starts from d = r: its scales come from the reference norms max|r| (c->d_rref)
+int seed_series(dyson_ctx* c, const std::vector<double>& rref) {
+  DY_CUDA(c, cudaMemcpyAsync(c->d_rref, rref.data(), rref.size() * sizeof(double), cudaMemcpyHostToDevice,
+                             c->stream));                  // pageable: complete when the call returns
+  return tc_seed_scale(c, (int)rref.size(), c->d_rref, 0.0);
+}
+
+// Start of a series on the fused sweep, da already holding r and the scales seeded.
+int SeriesRun::begin(bool plateau) {
+  if (!c->d_series) {
+    DY_CUDA(c, cudaMalloc(&c->d_series, sizeof(SeriesState)));
+    DY_CUDA(c, cudaMallocHost(&c->h_series, sizeof(SeriesState)));
+  }
+  SeriesState* hS = static_cast<SeriesState*>(c->h_series);
+  *hS = series_start(plateau);
+  int rc;
+  if ((rc = tc_prepare_sweep(c, ncol, true)) || (rc = tc_set_scale(c, ncol / gs))) return rc;
+  DY_CUDA(c, cudaMemcpyAsync(c->d_series, hS, sizeof(SeriesState), cudaMemcpyHostToDevice, c->stream));
+  DY_CUDA(c, cudaMemsetAsync(c->d_norm, 0, (size_t)(ncol / gs) * sizeof(unsigned long long), c->stream));
+  return DYSON_OK;
+}
+
+const SeriesState* SeriesRun::state() const { return static_cast<const SeriesState*>(c->h_series); }
+bool SeriesRun::running() const { return state()->run != 0; }
+
+// `sweeps` sweeps (even, so that every batch starts from da), each followed by its check, on the context's
+// stream, and the copies of the series' state and of the error flag behind them.
+int SeriesRun::enqueue(bool overlap) {
+  SeriesState* dS = static_cast<SeriesState*>(c->d_series);
+  int rc;
+  for (int k = 0; k < sweeps; ++k) {
+    c->overlap = overlap && k > 0;
+    rc = tc_fused_sweep(c, ncol, gs, r32, k % 2 ? db : da, k % 2 ? da : db, act, 0, rform, &dS->run, &dS->sweeps, c->stream);
+    c->overlap = false;
+    if (rc) return rc;
+    DY_CUDA(c, launch_overlapped(overlap, k_series_check, 1, 32, 0, c->stream, c->d_norm, c->d_rref, ncol / gs, max_sweeps,
+                                 target, abort_peak, dS, c->d_xscale, tc_jbound(c)));
+    c->launches += 1;
+  }
+  before = state()->sweeps;
+  if ((rc = tc_error_enqueue(c))) return rc;
+  DY_CUDA(c, cudaMemcpyAsync(c->h_series, dS, sizeof(SeriesState), cudaMemcpyDeviceToHost, c->stream));
+  return DYSON_OK;
+}
+
+// After the stream has been waited for: sweeps that ran; da: the state that the last one left.
+int SeriesRun::collect(int* rc) {
+  if ((*rc = tc_error_status(c))) return 0;
+  const int n_run = state()->sweeps - before;
+  rep->sweeps += n_run;
+  rep->gemm_flops += n_run * sweep_flops(c, ncol);
+  rep->update = state()->last;
+  if (!running() && n_run % 2) std::swap(da, db);          // the last sweep wrote db
+  return n_run;
+}
+
 // inner solve d <- r + K d in FP32 (SIMT or 3xTF32 tensor cores)
 // act (optional): support truncation of the tensor-core sweeps (tc_sweep), valid
 // while every column of r32 is zero off its source site
@@ -303,12 +359,7 @@ int inner_solve(dyson_ctx* c, int ncol, int gs, int precision, float* r32, float
   const int eager_until = batches ? 0 : max_sweeps;
   SeriesState S = series_start(plateau);
   int rc;
-  if (precision == DYSON_PREC_TF32X3_F64REF && c->use_tc && tc_uses_fused(c)) {
-    // the series starts from d = r: its scales come from the reference norms max|r|
-    DY_CUDA(c, cudaMemcpyAsync(c->d_rref, rref.data(), (size_t)ng * sizeof(double), cudaMemcpyHostToDevice,
-                               c->stream));                // pageable: complete when the call returns
-    if ((rc = tc_seed_scale(c, ng, c->d_rref, 0.0))) return rc;
-  }
+  if (precision == DYSON_PREC_TF32X3_F64REF && c->use_tc && tc_uses_fused(c) && (rc = seed_series(c, rref))) return rc;
   while (S.run && S.sweeps < std::min(max_sweeps, eager_until)) {
     const int sweep = S.sweeps + 1;
     DY_CUDA(c, cudaMemsetAsync(c->d_norm, 0, (size_t)ng * sizeof(unsigned long long), c->stream));
@@ -333,77 +384,33 @@ int inner_solve(dyson_ctx* c, int ncol, int gs, int precision, float* r32, float
     series_step(S, upd, max_sweeps, target, abort_peak);
   }
   if (S.run && batches) {
-    // batches of S_g sweeps (even, so that every batch starts from da), each followed by its check
-    const int Sg = c->graph_sweeps;
-    if (!c->d_series) {
-      DY_CUDA(c, cudaMalloc(&c->d_series, sizeof(SeriesState)));
-      DY_CUDA(c, cudaMallocHost(&c->h_series, sizeof(SeriesState)));
-    }
-    SeriesState* hS = static_cast<SeriesState*>(c->h_series);
-    SeriesState* dS = static_cast<SeriesState*>(c->d_series);
-    *hS = S;
-    if ((rc = tc_prepare_sweep(c, ncol))) return rc;     // (buffers and tensor maps)
-    if ((rc = tc_set_scale(c, ng))) return rc;
-    DY_CUDA(c, cudaMemcpyAsync(dS, hS, sizeof(SeriesState), cudaMemcpyHostToDevice, c->stream));
-    DY_CUDA(c, cudaMemsetAsync(c->d_norm, 0, (size_t)ng * sizeof(unsigned long long), c->stream));
-    auto enqueue = [&]() -> int {
-      const int64_t launches0 = c->launches;
-      int rc1 = DYSON_OK;
-      c->sweep_run = &dS->run;
-      c->sweep_count = &dS->sweeps;
-      for (int k = 0; k < Sg && rc1 == DYSON_OK; ++k) {
-        rc1 = tc_sweep(c, ncol, gs, r32, k % 2 ? db : da, k % 2 ? da : db, TC_GATHER | TC_GEMM, act, 0, rform);
-        if (rc1 == DYSON_OK)
-          launch_overlapped(true, k_series_check, 1, 32, 0, c->stream, c->d_norm, c->d_rref, ng, max_sweeps, target,
-                            abort_peak, dS, c->d_xscale, tc_jbound(c));
-        c->overlap = true;
-      }
-      c->overlap = false;
-      c->sweep_run = nullptr;
-      c->sweep_count = nullptr;
-      c->launches = launches0 + 2 * Sg;
-      return rc1;
-    };
+    SeriesRun run{c, ncol, gs, max_sweeps, c->graph_sweeps, r32, da, db, act, rform, target, abort_peak, rep};
+    if ((rc = run.begin(plateau))) return rc;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (c->profiling) {
       cudaEventCreate(&e0);
       cudaEventCreate(&e1);
     }
-    rc = DYSON_OK;
-    while (rc == DYSON_OK) {
-      const int before = hS->sweeps;
+    while (rc == DYSON_OK && run.running()) {
       if (e0) cudaEventRecord(e0, c->stream);
-      if ((rc = enqueue())) break;
-      cudaError_t le = cudaGetLastError();
+      rc = run.enqueue(true);
       if (e1) cudaEventRecord(e1, c->stream);
-      if (le == cudaSuccess && c->use_tc) rc = tc_error_enqueue(c);
-      if (le == cudaSuccess && rc == DYSON_OK)
-        le = cudaMemcpyAsync(hS, dS, sizeof(SeriesState), cudaMemcpyDeviceToHost, c->stream);
-      if (le == cudaSuccess && rc == DYSON_OK) le = cudaStreamSynchronize(c->stream);
-      if (le != cudaSuccess) {
-        rc = ctx_fail(c, DYSON_ERR_CUDA, std::string("inner series: ") + cudaGetErrorString(le));
-        break;
-      }
+      if (rc) break;
+      const cudaError_t e = cudaStreamSynchronize(c->stream);
+      if (e != cudaSuccess) rc = ctx_fail(c, DYSON_ERR_CUDA, std::string("inner series: ") + cudaGetErrorString(e));
       c->host_syncs += 1;
-      if (rc || (c->use_tc && (rc = tc_error_status(c)))) break;
-      const int n_run = hS->sweeps - before;
-      rep->sweeps += n_run;
-      rep->gemm_flops += n_run * sweep_flops(c, ncol);
-      rep->update = hS->last;
+      const int n_run = rc ? 0 : run.collect(&rc);
       float ms = 0.f;
       if (e0 && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess) {
         c->prof_ms[fused_kind(c)] += ms;                   // the batch, its checks included
         c->prof_launches[fused_kind(c)] += n_run;
       }
-      if (!hS->run) {
-        if (n_run % 2) std::swap(da, db);                  // the last sweep wrote db
-        break;
-      }
     }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     if (rc) return rc;
-    S = *hS;
+    S = *run.state();
+    da = run.da;
   }
   if (outcome) *outcome = S.outcome;
   if (S.outcome == SERIES_NOT_FINITE) return ctx_fail(c, DYSON_ERR_DIVERGED, "FP32 series update not finite");

@@ -164,11 +164,7 @@ struct dyson_ctx {
   double dt = 0, beta = 0, curvature = 0, mu = 0;
   std::vector<double> U, J;          // host copies of the drive tables
   bool j_uniform = false;            // every bond carries the same J(t) row
-  // inner series in batches: sweeps per batch (0: one host synchronisation per sweep); while a batch
-  // is enqueued, the flag its fused sweeps read (0: the series stopped) and the count of sweeps done
-  int graph_sweeps = 16;
-  const int* sweep_run = nullptr;
-  const int* sweep_count = nullptr;  // while capturing: the device count of sweeps done
+  int graph_sweeps = 16;             // sweeps of the inner series per host synchronisation (0: one)
   void* d_series = nullptr;          // device stopping state of the series
   void* h_series = nullptr;          // pinned mirror
   double* d_rref = nullptr;          // [norm_cap] reference norms of the current inner solve

@@ -1,6 +1,7 @@
 // Host helpers of the solve drivers (capi.cu), shared with the batched driver (batch.cu).
 #pragma once
 #include <string>
+#include <vector>
 
 #include "common.cuh"
 #include "series.cuh"
@@ -94,6 +95,26 @@ int prepare_tables(dyson_ctx* c, int precision, double tol, int64_t columns = 0,
 size_t scratch_bytes(const dyson_ctx* c);                 // held by the buffers that each solve sizes for itself
 void release_scratch(dyson_ctx* c);
 int reserve_chunk(dyson_ctx* c, int ncol, int gs, size_t bytes_per_col, bool batch = false);
+const int* support_table(dyson_ctx* c, int ncol);          // support truncation of the first right-hand side, or nullptr
+int seed_series(dyson_ctx* c, const std::vector<double>& rref);
+
+// An inner series on the fused sweep, enqueued on the context's stream a number of sweeps at a time; the rule that
+// ends it runs on the device, and the sweeps behind its end return at once.
+struct SeriesRun {
+  dyson_ctx* c;
+  int ncol, gs, max_sweeps, sweeps;
+  float *r32, *da, *db;
+  const int* act;
+  int rform;
+  double target, abort_peak;
+  dyson_report* rep;
+  int before = 0;
+  int begin(bool plateau);
+  int enqueue(bool overlap);
+  int collect(int* rc);
+  bool running() const;
+  const SeriesState* state() const;
+};
 int enqueue_residual(dyson_ctx* c, int ncol, int gs, const double2* G, float* r32);
 // mixed-precision solve of the chunk whose sources are on the device (G in c->work)
 int solve_mixed(dyson_ctx* c, int ncol, int gs, int precision, double tol, int max_sweeps, double2** result,

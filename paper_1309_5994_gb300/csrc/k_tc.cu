@@ -1519,9 +1519,8 @@ int tc_sweep(dyson_ctx* c, int ncol, int gs, const float* r, const float* din, f
   if (gt > 0) {
     // one launch gathers and multiplies: the gather phase alone launches nothing
     if (!(phases & TC_GEMM)) return tc_prepare_fused(c);
-    // (in a batch of sweeps the check kernel sets the scales)
-    if (!c->sweep_run && (rc = tc_set_scale(c, (ncol + gs - 1) / gs))) return rc;
-    return tc_fused_sweep(c, ncol, gs, r, din, dout, act, sweep, rform, c->sweep_run, c->sweep_count, c->stream);
+    if ((rc = tc_set_scale(c, (ncol + gs - 1) / gs))) return rc;
+    return tc_fused_sweep(c, ncol, gs, r, din, dout, act, sweep, rform, nullptr, nullptr, c->stream);
   }
   if ((rc = tc_prepare(c, ncol))) return rc;
   TcState* st = state(c);
