@@ -367,7 +367,7 @@ def batched_uneven_leg(args, dev, stream):
     """The seeded uneven batch (lattice sides 8..24, Nc in {128, 192, 256}, U, trap and
     drive phase drawn per instance): one block column per instance (the site next to
     the trap centre) solved to the same FP64 residual, once as one dyson_batch
-    (shared sweep launches under CUDA graphs) and once instance by instance."""
+    (their series side by side) and once instance by instance."""
     import torch
     import workloads as wl
     from paper_1309_5994_gb300 import binding
@@ -381,7 +381,7 @@ def batched_uneven_leg(args, dev, stream):
     batch = binding.Batch(solvers)
     # instances whose series diverges (spectral radius of Lambda W J above 1) end with
     # DIVERGED in the batch; the paper hands those to GMRES, which finishes them below
-    batch.solve(sources, tol=args.tol, allow=(0, -4))      # warm-up: tables, graph, buffers
+    batch.solve(sources, tol=args.tol, allow=(0, -4))      # warm-up: tables, buffers
     torch.cuda.synchronize(dev)
     l0 = batch.launch_count()
     t0 = time.perf_counter()

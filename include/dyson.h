@@ -332,7 +332,7 @@ int dyson_set_chunk(dyson_ctx* ctx, int32_t block_columns);
  *               operands under power-of-two scales (22 bits, as the TF32 pairs
  *               of the other forms);
  *   FUSED_PAIR_WIDE  the same kernel (kept as a name of its own; the tuner lists
- *               it where Nc % 256 == 0).
+ *               it where Nc % 256 == 0, with the rate of FUSED_PAIR).
  * A context that selects none runs the fused form.  SINGLE_CTA needs Nc % 64 == 0
  * and CTA_PAIR Nc % 128 == 0 (else the single-CTA form runs); the fused form
  * serves every contour of at least 24 points, padded to a multiple of 64 with

@@ -201,12 +201,12 @@ def test_fused_sweep_matches_dense(torch_cuda, lib, kw, sources, variant):
 
 @pytest.mark.parametrize("kw,sources,variant", FUSED_CASES[:2] + [(FUSED_CASES[1][0], list(range(12)), 2)])
 def test_graph_replayed_series_is_bit_identical(torch_cuda, lib, kw, sources, variant):
-    """The inner series replayed from captured graphs (its stopping rule applied on the
-    device, one host synchronisation per graph of sweeps) returns the same G bit for bit,
+    """The inner series enqueued a number of sweeps at a time (its stopping rule applied on the
+    device, one host synchronisation for all of them) returns the same G bit for bit,
     the same sweep and refinement counts and the same residual as the loop with one
     synchronisation per sweep: after truncated first sweeps (a few sources) and without
-    them (every site a source), and with a graph of 2 sweeps, where the series stops
-    inside a replay."""
+    them (every site a source), and two sweeps at a time, where the series stops
+    inside a pair."""
     p = wl.random_tables(wl.small(**kw), seed=23, rel=0.2)
     out, syncs = {}, {}
     for gsw in (0, 16, 2):
@@ -225,7 +225,7 @@ def test_graph_replayed_series_is_bit_identical(torch_cuda, lib, kw, sources, va
     for gsw in (16, 2):
         assert np.array_equal(out[gsw][0], out[0][0])
         assert out[gsw][1:] == out[0][1:]
-    # fewer waits for the device with graphs: one per replay instead of one per sweep
+    # fewer waits for the device: one per sixteen or two sweeps instead of one per sweep
     # (GMRES steps, where a case switches to them, wait once each in both)
     assert syncs[16] < syncs[0]
 
@@ -521,7 +521,7 @@ def test_trapped_16x16_sampled_columns_mixed(torch_cuda, lib):
 def test_trapped_16x16_bench_launch_shape_sampled_columns(torch_cuda, lib):
     """The benchmark's launch configuration on its workload: 16 block columns of the 16x16,
     Nc = 256 lattice in one chunk (the fused sweep on CTA pairs, as the tuner picks, support
-    truncation on, the inner series from replayed graphs of 16 sweeps), mixed precision at
+    truncation on, the inner series sixteen sweeps at a time), mixed precision at
     the benchmark's tolerance 1e-6, sources 112..127 (one of its batches).  Sampled vector columns of four block columns, and the densities of two
     sources at three times, against the oracle's complex128 series; bound 1e-6 relative."""
     torch = torch_cuda
@@ -537,7 +537,7 @@ def test_trapped_16x16_bench_launch_shape_sampled_columns(torch_cuda, lib):
     res = s.solve(sources, precision=binding.PREC_TF32X3_F64REF, tol=1e-6, max_sweeps=400, g_out=g)
     assert res.report["chunks"] == 1
     assert s.profile_query(binding.KERNEL_SWEEP_TC_FUSED)[0] > 0          # the fused sweep ran
-    assert res.report["host_syncs"] < res.report["sweeps"]                 # from replayed graphs
+    assert res.report["host_syncs"] < res.report["sweeps"]                 # sixteen at a time
     rng = np.random.default_rng(11)
     picks = [(q, int(z)) for q in (0, 5, 10, 15) for z in rng.choice(p.Nc, 2, replace=False)]
     dens = [(q, z) for q in (0, 7) for z in (0, p.Nt // 2, p.Nt - 1)]
