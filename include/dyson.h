@@ -337,8 +337,9 @@ int dyson_set_chunk(dyson_ctx* ctx, int32_t block_columns);
  * and CTA_PAIR Nc % 128 == 0 (else the single-CTA form runs); the fused form
  * serves every contour of at least 24 points, padded to a multiple of 64 with
  * zeros, and takes the place of the others on contours they do not fill; at
- * Nc = 64 solves of 32768 (site, vector column) pairs or more run the SINGLE_CTA
- * form in its place, which is faster there.  All
+ * Nc = 64, which fills half of its tiles, chunks of 32768 (site, vector column)
+ * pairs or more run the SINGLE_CTA form in its place, unless dyson_autotune
+ * chose it.  All
  * give the same results to FP32 rounding; which is fastest depends on the
  * shape, which is what dyson_autotune measures.  Returns INVALID_ARG for an
  * unknown variant. */

@@ -779,8 +779,8 @@ int prepare_tables(dyson_ctx* c, int precision, double tol, int64_t columns, boo
   // A fused tile of 256 rows is half empty at 64 contour points (128 rows of the embedding), so from
   // kManySiteColumns on the unfused form is the faster one although its series waits for every sweep:
   // single CTA / fused, us a sweep: 8x8 sites, 512 columns 34 / 46, 1024 57 / 83; 12x12, 512 62 / 85;
-  // 16x16, 128 36 / 52; 5x5, 1024 33 / 43.  Only where no form was selected or tuned.
-  c->many_of_64 = c->tc_variant < 0 && c->Nc == 64 && c->Nr * columns >= kManySiteColumns;
+  // 16x16, 128 36 / 52; 5x5, 1024 33 / 43.  A form that the tuner measured is the one that runs.
+  c->many_of_64 = !c->tc_tuned && c->Nc == 64 && c->Nr * columns >= kManySiteColumns;
   c->use_tc = c->use_oz = c->use_oz64 = false;
   c->Ns = c->Nc;
   if (precision == DYSON_PREC_F64) return prepare_oz64(c, hold);
@@ -1278,6 +1278,7 @@ int dyson_set_sweep_variant(dyson_ctx* c, int variant) {
   if (variant < DYSON_SWEEP_SINGLE_CTA || variant > DYSON_SWEEP_FUSED_PAIR_WIDE)
     return ctx_fail(c, DYSON_ERR_INVALID_ARG, "unknown sweep variant");
   c->tc_variant = variant;
+  c->tc_tuned = false;
   return DYSON_OK;
 }
 

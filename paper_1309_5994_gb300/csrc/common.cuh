@@ -210,6 +210,7 @@ struct dyson_ctx {
   bool lam_split_built = false;
   bool use_tc = false;               // chosen for the current solve
   int tc_variant = -1;               // DYSON_SWEEP_*; -1: none selected, the fused form
+  bool tc_tuned = false;             // chosen by the tuner
   bool many_of_64 = false;           // this solve is large and of 64 contour points (prepare_tables)
   int max_refinements = 12;
   int chunk_override = 0;

@@ -654,8 +654,8 @@ __global__ void __launch_bounds__(THREADS, 1)
 // 22 bits of every entry down to 2^-16 of the row's (group's) largest and 2^-39 of the
 // largest below that, under the FP32 accumulation's own rounding.
 // The kernel is bound by the latency of the loads through L2 at what an SM keeps in flight (10.4 TB/s of
-// L2 traffic; tensor pipe 29 %, L2 33 %, DRAM 50 % busy), so the two forms differ in what they read.  Both have two accumulator sets of 256 TMEM
-// columns, so that a tile's epilogue overlaps the next tile's MMAs:
+// L2 traffic; tensor pipe 29 %, L2 33 %, DRAM 50 % busy), so the two forms differ in what they read.  Both have two
+// accumulator sets of 256 TMEM columns, so that a tile's epilogue overlaps the next tile's MMAs:
 //   <2>  a tile is (site, 128 vector columns, 256 contour points z): its two accumulators are the
 //        real and the imaginary rows of those points.  A k-block is 64 complex points; the tiles
 //        Re and Im of Lambda are loaded once and serve both halves of the embedding
@@ -663,14 +663,16 @@ __global__ void __launch_bounds__(THREADS, 1)
 //        per ceil(Ns / 256) tiles.  Two stages of 96 KB.  Ns >= 192.
 //   <1>  a tile is (site, 256 vector columns, 256 rows of the embedding); a k-block is 64 real
 //        values, three stages of 64 KB.  Ns = 64 and 128, where <2> would fill half of its rows at most.
-// Bytes from L2 per sweep at 16x16, Nc = 256, 4096 columns: X 8.6 GB, Lambda 4.3, epilogue 4.3
-// and 2.1 written (<1>: X 17.2, Lambda 4.3; with the embedding in 512-row tiles: X 8.6, Lambda 8.6).
-// Measured there: 2.05 ms per sweep; 2.67 ms as <1> and 2.37 with the embedding in
+// Bytes from L2 per sweep at 16x16, Nc = 256, 4096 columns, by count: X 8.6 GB, Lambda 4.3, epilogue 4.3
+// and 2.1 written (<1>: X 17.2, Lambda 4.3; with the embedding in 512-row tiles: X 8.6, Lambda 8.6); the counters
+// say 25 GB in all.  Measured there, in the mean over a solve's launches, truncated ones among them:
+// 2.05 ms (2.15 per sweep that does work, with its check); 2.67 ms as <1> and 2.37 with the embedding in
 // 512-row tiles; 2.66 ms in 3xTF32 with the traffic of <1>.  Each gather step waits for one loaded
 // memory latency (about 2.3 us, 64 KB in flight per SM); fetching the next tile's neighbour rows
 // into L2 ahead adds requests and cost 25 %.
-// Error of one inner solve against the FP64 residual, 8x8 to 24x24, six contours: 0.45 to 0.95 of the
-// 3xTF32 form's in every case (fewer roundings: twice the products per MMA).
+// FP64 residual of one inner solve, 57 drawn problems on contours of 64 to 256 points: 0.39 to 1.21 of the 3xTF32
+// form's, 0.63 in the mean (fewer roundings: twice the products per MMA).  With the lo halves scaled by 2^11, 22 bits
+// down to 2^-29, it is the same: the range is no limit.
 // SPLIT: contours that are no multiple of 64, whose other form is the FP32 CUDA-core sweep (every product and
 // sum rounded to nearest).  The tensor memory accumulation truncates once per MMA, and with all three products in
 // one accumulator the residual of an inner solve was 1.1 to 2.8 times that sweep's (Nc 33 to 151; 0.4 to 1.2 from

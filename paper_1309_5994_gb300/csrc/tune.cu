@@ -144,6 +144,7 @@ int dyson_autotune(dyson_ctx* c, int32_t max_block_columns, dyson_tuning* out) {
       }
     }
   c->tc_variant = T.sweep_variant;
+  c->tc_tuned = true;
   c->chunk_override = T.chunk_block_columns;
   flush_timers(c);
   if (out) *out = T;

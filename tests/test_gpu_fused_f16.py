@@ -146,10 +146,12 @@ def _many_of_64(torch, binding, n, variant=None, leave=None):
     return kinds, res.report["chunks"]
 
 
-def test_a_selected_form_runs_at_64_points_too(torch_cuda, lib):
+@pytest.mark.parametrize("n,unfused", [(5440, False), (5472, True)])
+def test_the_line_at_64_points_with_the_fused_form_selected(torch_cuda, lib, n, unfused):
+    """As where none is selected: the fused form's tiles are half empty there."""
     from paper_1309_5994_gb300 import binding
-    (gather, plain, fused), _ = _many_of_64(torch_cuda, binding, 5472, variant=binding.SWEEP_FUSED_PAIR)
-    assert gather == 0 and plain == 0 and fused > 0
+    (gather, _, fused), _ = _many_of_64(torch_cuda, binding, n, variant=binding.SWEEP_FUSED_PAIR)
+    assert (gather > 0) == unfused and (fused > 0) == (not unfused)
 
 
 def test_the_line_at_64_points_counts_the_columns_of_a_chunk(torch_cuda, lib):
@@ -160,14 +162,17 @@ def test_the_line_at_64_points_counts_the_columns_of_a_chunk(torch_cuda, lib):
 
 
 def test_the_tuned_form_is_the_one_that_runs(torch_cuda, lib):
+    """Tuned on one block column of 6 sites (one launch a sweep beats two there), then used above the line."""
     from paper_1309_5994_gb300 import binding
-    p = wl.small(L=8, Ly=8, Nt=24, Nm=16, dt=0.05, beta=2.0, trap_c=0.05, U0=20.0)
+    p = wl.random_tables(wl.small(L=3, Ly=2, Nt=24, Nm=16, dt=0.02, beta=1.0, trap_c=0.3, U0=14.0), seed=7, rel=0.1)
     s = binding.Solver(p, device=0)
     s.build_sigma()
-    t = s.autotune(16)
+    fused = binding.SWEEP_NAMES[s.autotune(1)["sweep_variant"]].startswith("fused")
+    s.set_chunk(0)
     s.profile(True)
-    s.solve(list(range(16)), precision=binding.PREC_TF32X3_F64REF, tol=1e-6)
-    fused = binding.SWEEP_NAMES[t["sweep_variant"]].startswith("fused")
+    n = 5472
+    s.solve_vectors([k % p.Nr for k in range(n)], [(7 * k) % p.Nc for k in range(n)],
+                    precision=binding.PREC_TF32X3_F64REF, tol=1e-6)
     assert (s.profile_query(binding.KERNEL_SWEEP_TC_FUSED)[0] > 0) == fused
     assert (s.profile_query(binding.KERNEL_GATHER_TC)[0] > 0) == (not fused)
     s.close()
