@@ -11,7 +11,7 @@
 // GMRES of App. C (k_gmres.cu).
 // Six instances of 8x8 to 16x16 sites to 1e-10: 52.7 ms (one by one 62.5).  As a graph of S sweeps of all instances,
 // captured for every call, each sweep ended by a check of all, 60.4; twelve drawn batches of 2 to 8 instances were
-// 1.13 to 1.26 times as long so.
+// 1.14 to 1.27 times as long so.
 #include <algorithm>
 #include <chrono>
 #include <limits>
