@@ -68,9 +68,11 @@ enum {
 
 /* Arithmetic of the sweeps (App. C series). */
 enum {
-  DYSON_PREC_F64 = 0,           /* complex128 sweeps, FP64-accurate: BF16 slice products
-                                   on the tensor cores, or the FP64 pipes where the
-                                   slices of Lambda do not fit in device memory          */
+  DYSON_PREC_F64 = 0,           /* complex128 sweeps, FP64-accurate relative to the largest
+                                   entry of a row of Lambda and of a column: BF16 slice
+                                   products on the tensor cores, or the FP64 pipes where
+                                   the slices of Lambda do not fit (or may not be made,
+                                   dyson_set_slice_memory)                                */
   DYSON_PREC_TF32X3_F64REF = 1  /* complex FP32 sweeps as three tcgen05 products of FP16
                                    hi + lo (or, where selected, TF32 hi + lo) operands
                                    with FP32 accumulation, refined by FP64 Dyson residuals */

@@ -103,6 +103,24 @@ def test_gmres_item_shapes(torch_cuda, lib, Nt, Nm):
     s.close()
 
 
+def test_gmres_states_that_start_at_eight_bytes(torch_cuda, lib):
+    """Sites, columns and points all odd: the FP32 states of the CUDA-core stride start at a multiple of 8 bytes."""
+    from paper_1309_5994_gb300 import binding
+    torch = torch_cuda
+    p = wl.random_tables(wl.small(L=3, Ly=1, Nt=10, Nm=1, dt=0.01, beta=0.2, trap_c=0.3, U0=14.0), seed=9, rel=0.1)
+    S = dyson.setup(p)
+    assert p.Nr * p.Nc % 2 == 1
+    ref = dyson.dense_solve(S, dyson.rhs_block_columns(S, [1]))
+    s = binding.Solver(p, device=0)
+    s.set_inner_solver(1)
+    s.build_sigma()
+    g = torch.empty((1, p.Nr, p.Nc, p.Nc), dtype=torch.complex128, device="cuda:0")
+    res = s.solve([1], precision=binding.PREC_TF32X3_F64REF, tol=1e-12, g_out=g)
+    assert res.report["inner_gmres"] == 1
+    assert np.abs(g.cpu().numpy()[0] - ref).max() / np.abs(ref).max() < 1e-11
+    s.close()
+
+
 @pytest.mark.parametrize("n,unfused", [(5440, False), (5472, True)])
 def test_large_solves_of_64_points_take_the_unfused_form(torch_cuda, lib, n, unfused):
     """6 sites times n vector columns on either side of 32768, the rule's line at Nc = 64."""
