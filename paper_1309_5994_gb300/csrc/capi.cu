@@ -439,7 +439,7 @@ int matvec_f32(dyson_ctx* c, int ncol, int gs, int precision, const float* zero,
   return DYSON_OK;
 }
 
-// Support truncation (NEXT-2 of the build plan; Sec. IV.D): the first right-hand
+// Support truncation (Sec. IV.D): the first right-hand
 // side Lambda delta_s is non-zero only on the source site of each column, and a
 // sweep spreads an iterate by one hop, so after n sweeps a column is zero beyond
 // lattice distance n of its source.  act[i][t] = min over the columns of 256-column
